@@ -20,6 +20,7 @@
 #include "step_gemv.cuh"
 #include "vocab_gemv.cuh"
 #include "crosskv_gemm.cuh"
+#include "f32_rows.cuh"
 #include "stream_schedule.h"
 
 using namespace aed;
@@ -281,33 +282,6 @@ struct ProfScope {
 
 // ---- typed launch sequences ------------------------------------------------------------------------------
 
-template <typename T>
-aed_status_t launch_layernorm(aed_dec *dec, int rows_ub, const float *x, const void *g, const void *b, float *out)
-{
-    ProfScope ps(dec, KF_LAYERNORM);
-    const int d = dec->cfg.d_model;
-    if (d <= 2048)
-        layernorm_kernel<T, 8><<<rows_ub, 256, 0, dec->stream>>>(dec->state(), x, (const T *)g, (const T *)b, d,
-                                                                 dec->cfg.ln_eps, out);
-    else
-        layernorm_kernel<T, 8><<<rows_ub, 1024, 0, dec->stream>>>(dec->state(), x, (const T *)g, (const T *)b, d,
-                                                                  dec->cfg.ln_eps, out);
-    AED_LAUNCHED(dec);
-    return AED_OK;
-}
-
-template <typename AT, typename T, int EPI>
-aed_status_t launch_gemm(aed_dec *dec, int family, int rows_ub, int rows_fixed, const AT *A, int lda, const void *W,
-                         const void *bias, int M, int K, const GemmEpilogueArgs<T> &ep)
-{
-    ProfScope ps(dec, family);
-    dim3 grid((M + 31) / 32, (rows_ub + 63) / 64);
-    gemm_rows_kernel<AT, T, T, EPI><<<grid, 128, 0, dec->stream>>>(dec->state(), rows_fixed, A, lda, (const T *)W,
-                                                                    (const T *)bias, M, K, ep);
-    AED_LAUNCHED(dec);
-    return AED_OK;
-}
-
 template <typename T, bool kCross, bool kAppend = false>
 aed_status_t launch_attention(aed_dec *dec, int rows_ub, int len_ub, const float *q, int ldq, const T *cache,
                               int seq_capacity, float *out)
@@ -398,60 +372,76 @@ aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 b
         if (s__ != AED_OK) return s__;       \
     } while (0)
 
-// The forward pass of one step for the rows in the active list (at most rows_ub of them).
+// fp32 projection of at most rows_ub rows (f32_rows.cuh).  Up to 4 rows one feature per warp and 4-row tiles, up to 16 rows
+// 8-row tiles: as many warps as features, because a launch is bound by its latency.  Beyond, two features per warp halve the
+// shared-memory reads per FMA.  Small outputs take 4 warps per block, so that they still spread over 64 SMs and more.
+template <int EPI>
+aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p)
+{
+    ProfScope ps(dec, family);
+    const int warps = p.M <= 512 ? 4 : f32::kWarps;
+    p.state = dec->state();
+    p.eps = dec->cfg.ln_eps;
+    void *args[] = {&p};
+    auto grid = [&](int rt, int fpw) { return dim3((p.M + warps * fpw - 1) / (warps * fpw), (rows_ub + rt - 1) / rt); };
+    if (rows_ub <= 4) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 4, 1>, grid(4, 1), dim3(warps * 32), f32::rows_smem(4, p.K), args);
+    if (rows_ub <= 16) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 1>, grid(8, 1), dim3(warps * 32), f32::rows_smem(8, p.K), args);
+    return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 2>, grid(8, 2), dim3(warps * 32), f32::rows_smem(8, p.K), args);
+}
+
+// The forward pass of one step in fp32 for the rows in the active list (at most rows_ub of them): 8 kernels per layer, chained
+// with programmatic dependent launch.
 //   tokens: by utterance.  self_len_ub: upper bound on t_u + 1.
-template <typename T>
-aed_status_t forward_step(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out)
+aed_status_t forward_step_f32(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out)
 {
     const auto &c = dec->cfg;
     const Layout &L = dec->lay;
-    const int d = c.d_model, F = c.d_ffn, V = c.vocab;
-    float *x = dec->at<float>(L.x), *act = dec->at<float>(L.act), *qkv = dec->at<float>(L.qkv), *hid = dec->at<float>(L.hid);
+    int d = c.d_model, V = c.vocab, zero = 0;
+    const int F = c.d_ffn;
+    float *x = dec->at<float>(L.x), *act = dec->at<float>(L.act), *qkv = dec->at<float>(L.qkv), *hid = dec->at<float>(L.hid), *none = nullptr;
     const int32_t *active_list = dec->at<int32_t>(L.active_list), *t_u = dec->at<int32_t>(L.t_u);
-
+    const bool split = dec->partials_override != nullptr;        // aed_dec_step_static_scratch: attention split over chunks, with its scratch
     {
         ProfScope ps(dec, KF_EMBED);
-        embed_kernel<T><<<rows_ub, 256, 0, dec->stream>>>(dec->state(), active_list, tokens, t_u, (const T *)dec->embed,
-                                                          dec->at<float>(L.pe), d, V, sqrtf((float)d), x);
-        AED_LAUNCHED(dec);
+        const DecState *state = dec->state();
+        const float *emb = (const float *)dec->embed, *pe = dec->at<float>(L.pe);
+        float sc = sqrtf((float)d);
+        void *args[] = {&state, &active_list, &tokens, &t_u, &emb, &pe, &d, &V, &sc, &x, &none, &zero, &none, &zero};
+        AED_TRY(launch_pdl_impl(dec, (const void *)embed_kernel<float>, dim3(rows_ub), dim3(256), 0, args));
     }
-
-    GemmEpilogueArgs<T> ep{};
-    ep.active_list = active_list;
-    ep.t_u = t_u;
-    ep.max_dec_len = c.max_dec_len;
-    ep.d_model = d;
-    ep.n_heads = c.n_heads;
+    auto rows = [&](const float *a, const void *ln_g, const void *ln_b, const void *w, const void *bias, int M, int K, float *out, int ldo) {
+        f32::RowsArgs p{};
+        p.rows_fixed = -1;
+        p.a = a; p.ln_g = (const float *)ln_g; p.ln_b = (const float *)ln_b;
+        p.w = (const float *)w; p.bias = (const float *)bias; p.M = M; p.K = K;
+        p.out = out; p.ldo = ldo;
+        return p;
+    };
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerWeights &w = dec->layers[l];
-        T *self_cache = dec->at<T>(L.self_cache) + (size_t)l * L.self_layer_elems;
-        const T *cross = dec->at<T>(L.cross_store) + (size_t)l * L.cross_layer_elems;
-        // masked self-attention
-        AED_TRY(launch_layernorm<T>(dec, rows_ub, x, w.ln1_g, w.ln1_b, act));
-        ep.out = qkv; ep.ldo = d; ep.self_cache = self_cache;
-        AED_TRY((launch_gemm<float, T, EPI_QKV>(dec, KF_GEMM_QKV, rows_ub, -1, act, d, w.w_qkv, w.b_qkv, 3 * d, d, ep)));
-        AED_TRY((launch_attention<T, false>(dec, rows_ub, self_len_ub, qkv, d, self_cache, c.max_dec_len, act)));
-        ep.out = x; ep.ldo = d;
-        AED_TRY((launch_gemm<float, T, EPI_RESID>(dec, KF_GEMM_O, rows_ub, -1, act, d, w.w_o, w.b_o, d, d, ep)));
+        float *self_cache = dec->at<float>(L.self_cache) + (size_t)l * L.self_layer_elems;
+        const float *cross = dec->at<float>(L.cross_store) + (size_t)l * L.cross_layer_elems;
+        // masked self-attention (which appends the new keys and values)
+        AED_TRY(launch_f32<f32::EPI_STORE>(dec, KF_GEMM_QKV, rows_ub, rows(x, w.ln1_g, w.ln1_b, w.w_qkv, w.b_qkv, 3 * d, d, qkv, 3 * d)));
+        if (split) AED_TRY((launch_attention<float, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, act)));
+        else AED_TRY((launch_attention_fused<float, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, act, nullptr, nullptr, nullptr,
+                                                                 nullptr, nullptr, dec->use_pdl)));
+        AED_TRY(launch_f32<f32::EPI_RESID>(dec, KF_GEMM_O, rows_ub, rows(act, nullptr, nullptr, w.w_o, w.b_o, d, d, x, d)));
         // cross-attention over the utterance's own encoder frames
-        AED_TRY(launch_layernorm<T>(dec, rows_ub, x, w.ln2_g, w.ln2_b, act));
-        ep.out = qkv; ep.ldo = d;
-        AED_TRY((launch_gemm<float, T, EPI_STORE>(dec, KF_GEMM_QC, rows_ub, -1, act, d, w.w_q_c, w.b_q_c, d, d, ep)));
-        AED_TRY((launch_attention<T, true>(dec, rows_ub, c.max_enc_len, qkv, d, cross, c.max_total_enc_frames, act)));
-        ep.out = x; ep.ldo = d;
-        AED_TRY((launch_gemm<float, T, EPI_RESID>(dec, KF_GEMM_OC, rows_ub, -1, act, d, w.w_o_c, w.b_o_c, d, d, ep)));
+        AED_TRY(launch_f32<f32::EPI_STORE>(dec, KF_GEMM_QC, rows_ub, rows(x, w.ln2_g, w.ln2_b, w.w_q_c, w.b_q_c, d, d, qkv, d)));
+        if (split) AED_TRY((launch_attention<float, true>(dec, rows_ub, c.max_enc_len, qkv, d, cross, c.max_total_enc_frames, act)));
+        else AED_TRY((launch_attention_fused<float, true, false>(dec, rows_ub, c.max_enc_len, qkv, d, cross, c.max_total_enc_frames, act, nullptr, nullptr, nullptr,
+                                                                 nullptr, nullptr, dec->use_pdl)));
+        AED_TRY(launch_f32<f32::EPI_RESID>(dec, KF_GEMM_OC, rows_ub, rows(act, nullptr, nullptr, w.w_o_c, w.b_o_c, d, d, x, d)));
         // feed-forward
-        AED_TRY(launch_layernorm<T>(dec, rows_ub, x, w.ln3_g, w.ln3_b, act));
-        ep.out = hid; ep.ldo = F;
-        AED_TRY((launch_gemm<float, T, EPI_RELU>(dec, KF_GEMM_FF1, rows_ub, -1, act, d, w.w_ff1, w.b_ff1, F, d, ep)));
-        ep.out = x; ep.ldo = d;
-        AED_TRY((launch_gemm<float, T, EPI_RESID>(dec, KF_GEMM_FF2, rows_ub, -1, hid, F, w.w_ff2, w.b_ff2, d, F, ep)));
+        AED_TRY(launch_f32<f32::EPI_RELU>(dec, KF_GEMM_FF1, rows_ub, rows(x, w.ln3_g, w.ln3_b, w.w_ff1, w.b_ff1, F, d, hid, F)));
+        AED_TRY(launch_f32<f32::EPI_RESID>(dec, KF_GEMM_FF2, rows_ub, rows(hid, nullptr, nullptr, w.w_ff2, w.b_ff2, d, F, x, d)));
     }
-    AED_TRY(launch_layernorm<T>(dec, rows_ub, x, dec->final_ln_g, dec->final_ln_b, act));
-    ep.logits_out = logits_out;
-    ep.keys = dec->at<unsigned long long>(L.keys);
-    AED_TRY((launch_gemm<float, T, EPI_LOGITS>(dec, KF_GEMM_VOCAB, rows_ub, -1, act, d, dec->w_out, dec->b_out, V, d, ep)));
-    return AED_OK;
+    f32::RowsArgs p = rows(x, dec->final_ln_g, dec->final_ln_b, dec->w_out, dec->b_out, V, d, nullptr, 0);
+    p.logits_out = logits_out;
+    p.keys = dec->at<unsigned long long>(L.keys);
+    p.active_list = active_list;
+    return launch_f32<f32::EPI_LOGITS>(dec, KF_GEMM_VOCAB, rows_ub, p);
 }
 
 
@@ -1049,20 +1039,19 @@ ckv::CkvSegs one_run(int frames, int dst0)
     return g;
 }
 
-template <typename T>
-aed_status_t precompute_impl(aed_dec *dec, const void *enc_packed, int frames, int frame0)
+aed_status_t precompute_f32(aed_dec *dec, const void *enc_packed, int frames, int frame0)
 {
     const auto &c = dec->cfg;
     const Layout &L = dec->lay;
-    GemmEpilogueArgs<T> ep{};
-    ep.d_model = c.d_model;
-    ep.n_heads = c.n_heads;
-    ep.frame_capacity = c.max_total_enc_frames;
-    ep.frame0 = frame0;
     for (int l = 0; l < c.n_layers; ++l) {
-        ep.cross_store = dec->at<T>(L.cross_store) + (size_t)l * L.cross_layer_elems;
-        AED_TRY((launch_gemm<T, T, EPI_CROSSKV>(dec, KF_PRECOMPUTE, frames, frames, (const T *)enc_packed, c.d_enc,
-                                                dec->layers[l].w_kv_c, dec->layers[l].b_kv_c, 2 * c.d_model, c.d_enc, ep)));
+        f32::RowsArgs p{};
+        p.rows_fixed = frames;
+        p.a = (const float *)enc_packed;
+        p.w = (const float *)dec->layers[l].w_kv_c; p.bias = (const float *)dec->layers[l].b_kv_c;
+        p.M = 2 * c.d_model; p.K = c.d_enc;
+        p.out = dec->at<float>(L.cross_store) + (size_t)l * L.cross_layer_elems;
+        p.d_model = c.d_model; p.n_heads = c.n_heads; p.frame_capacity = c.max_total_enc_frames; p.frame0 = frame0;
+        AED_TRY(launch_f32<f32::EPI_CROSSKV>(dec, KF_PRECOMPUTE, frames, p));
     }
     return AED_OK;
 }
@@ -1220,7 +1209,7 @@ extern "C" aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *
     AED_CUDA(dec, cudaMemcpyAsync(&dec->state()->batch, &dec->batch, sizeof(int32_t), cudaMemcpyHostToDevice, dec->stream));
     dec->slot_mode = false;
     aed_status_t s = dec->use_tc ? precompute_tc(dec, enc_packed, dec->total_frames, one_run(dec->total_frames, 0))
-                                 : precompute_impl<float>(dec, enc_packed, dec->total_frames, 0);
+                                 : precompute_f32(dec, enc_packed, dec->total_frames, 0);
     if (s != AED_OK) return s;
     dec->have_batch = true;
     dec->fresh_batch = true;
@@ -1241,7 +1230,7 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
     AED_TRY(launch_build_active(dec, active));
     const int rows_ub = dec->batch;
     const int self_len_ub = dec->steps_issued + 1 < dec->cfg.max_dec_len ? dec->steps_issued + 1 : dec->cfg.max_dec_len;
-    aed_status_t s = !dec->use_tc ? forward_step<float>(dec, rows_ub, self_len_ub, tokens_in, logits_out)
+    aed_status_t s = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tokens_in, logits_out)
                      : rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tokens_in, logits_out)
                                                   : forward_step_fused(dec, rows_ub, self_len_ub, tokens_in, logits_out);
     if (s != AED_OK) return s;
@@ -1362,7 +1351,7 @@ aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, int
     if (self_len_ub > dec->cfg.max_dec_len) self_len_ub = dec->cfg.max_dec_len;
     AED_TRY(launch_build_active(dec, nullptr));
     const int32_t *tok = dec->at<int32_t>(L.cur_tok);
-    aed_status_t st = !dec->use_tc ? forward_step<float>(dec, rows_ub, self_len_ub, tok, nullptr)
+    aed_status_t st = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tok, nullptr)
                       : rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tok, nullptr)
                                                    : forward_step_fused(dec, rows_ub, self_len_ub, tok, nullptr);
     if (st != AED_OK) return st;
@@ -1540,7 +1529,7 @@ aed_status_t admit_many(aed_dec *dec, const void *enc_base, long long enc_rows, 
         AED_TRY(precompute_tc(dec, enc_base, enc_rows, segs));
     } else {
         for (int i = 0; i < n; ++i)
-            AED_TRY(precompute_impl<float>(dec, static_cast<const char *>(enc_base) + (size_t)adm[i].src_row * row_bytes, adm[i].frames, segs.dst0[i]));
+            AED_TRY(precompute_f32(dec, static_cast<const char *>(enc_base) + (size_t)adm[i].src_row * row_bytes, adm[i].frames, segs.dst0[i]));
     }
     {
         ProfScope ps(dec, KF_BOOKKEEPING);

@@ -1,5 +1,5 @@
-// Per-step kernels of the AED decoder: row bookkeeping, embedding, LayerNorm, CUDA-core GEMM with fused
-// epilogues (fp32 mode and fallback shapes), flash-decoding attention over ragged caches, argmax finalisation.
+// Per-step kernels of the AED decoder: row bookkeeping, embedding, attention over ragged caches (single pass; split over
+// chunks for the fp32 step with its scratch in the library image), activation planes, argmax finalisation.
 #pragma once
 #include "common.cuh"
 
@@ -93,177 +93,6 @@ __global__ void embed_kernel(const DecState *state, const int32_t *__restrict__ 
         x[(size_t)r * d + i] = to_f32(embed[(size_t)tok * d + i]) * scale + pe[(size_t)t * d + i];
     for (int i = threadIdx.x; i < zero_cols; i += blockDim.x) zero_buf[(size_t)r * zero_cols + i] = 0.f;
     for (int i = threadIdx.x; i < zero_cols2; i += blockDim.x) zero_buf2[(size_t)r * zero_cols2 + i] = 0.f;
-}
-
-// out[r] = g * (x[r] - mean) / sqrt(var + eps) + b, biased variance, two passes over a row held in registers.
-template <typename T, int kMaxPerThread>
-__global__ void layernorm_kernel(const DecState *state, const float *__restrict__ x, const T *__restrict__ g,
-                                 const T *__restrict__ b, int d, float eps, float *__restrict__ out)
-{
-    int r = blockIdx.x;
-    if (r >= state->n_active) return;
-    __shared__ float red[32];
-    __shared__ float stat;
-    float v[kMaxPerThread];
-    const float *xr = x + (size_t)r * d;
-    float s = 0.f;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        int i = threadIdx.x + j * blockDim.x;
-        v[j] = (i < d) ? xr[i] : 0.f;
-        s += v[j];
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    s = warp_sum(s);
-    if (lane == 0) red[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) { float tsum = 0.f; for (int w = 0; w < n_warps; ++w) tsum += red[w]; stat = tsum / d; }
-    __syncthreads();
-    float mean = stat;
-    float q = 0.f;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        int i = threadIdx.x + j * blockDim.x;
-        float c = (i < d) ? v[j] - mean : 0.f;
-        q += c * c;
-    }
-    q = warp_sum(q);
-    __syncthreads();
-    if (lane == 0) red[warp] = q;
-    __syncthreads();
-    if (threadIdx.x == 0) { float tsum = 0.f; for (int w = 0; w < n_warps; ++w) tsum += red[w]; stat = rsqrtf(tsum / d + eps); }
-    __syncthreads();
-    float rstd = stat;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        int i = threadIdx.x + j * blockDim.x;
-        if (i < d) out[(size_t)r * d + i] = to_f32(g[i]) * (v[j] - mean) * rstd + to_f32(b[i]);
-    }
-}
-
-// ------------------------------------------------------------------------------------------------------------
-// CUDA-core GEMM  out[r, o] = sum_k A[r, k] * W[o, k] + bias[o]  with fused epilogues.
-// 64 rows x 32 output features per block, K in slices of 32 staged through shared memory, 4x4 per thread.
-// ------------------------------------------------------------------------------------------------------------
-enum Epilogue { EPI_STORE = 0, EPI_RELU = 1, EPI_RESID = 2, EPI_QKV = 3, EPI_LOGITS = 4, EPI_CROSSKV = 5 };
-
-template <typename CT>
-struct GemmEpilogueArgs {
-    float *out;                 // STORE / RELU: [rows, ldo];  RESID: x [rows, ldo];  QKV: q [rows, d]
-    int ldo;
-    // QKV: self-attention cache of this layer [batch][2][H][max_dec_len][64]
-    CT *self_cache;
-    const int32_t *active_list;
-    const int32_t *t_u;
-    int max_dec_len, d_model, n_heads;
-    // LOGITS
-    float *logits_out;          // [batch, vocab] by utterance, or nullptr
-    unsigned long long *keys;   // [rows] packed argmax keys
-    // CROSSKV: store of this layer [2][H][frame_capacity][64]
-    CT *cross_store;
-    int frame_capacity;
-    int frame0;                 // CROSSKV: store row of the first frame (an utterance admitted into a slot of its own)
-};
-
-template <typename AT, typename WT, typename CT, int EPI>
-__global__ void __launch_bounds__(128)
-gemm_rows_kernel(const DecState *state, int rows_fixed, const AT *__restrict__ A, int lda,
-                 const WT *__restrict__ W, const WT *__restrict__ bias, int M, int K, GemmEpilogueArgs<CT> ep)
-{
-    constexpr int BM = 64, BN = 32, BK = 32;
-    const int n_rows = (rows_fixed >= 0) ? rows_fixed : state->n_active;
-    const int row0 = blockIdx.y * BM, o0 = blockIdx.x * BN;
-    if (row0 >= n_rows) return;
-    __shared__ __align__(16) float As[BK][BM + 4];
-    __shared__ __align__(16) float Ws[BK][BN + 4];
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        // A tile: 64 rows x 32 k, 4 elements per load
-        for (int idx = tid; idx < BM * BK / 4; idx += 128) {
-            int r = idx / (BK / 4), kq = (idx % (BK / 4)) * 4;
-            float v[4] = {0.f, 0.f, 0.f, 0.f};
-            if (row0 + r < n_rows) load4(A + (size_t)(row0 + r) * lda + k0 + kq, v);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) As[kq + j][r] = v[j];
-        }
-        for (int idx = tid; idx < BN * BK / 4; idx += 128) {
-            int o = idx / (BK / 4), kq = (idx % (BK / 4)) * 4;
-            float v[4] = {0.f, 0.f, 0.f, 0.f};
-            if (o0 + o < M) load4(W + (size_t)(o0 + o) * K + k0 + kq, v);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) Ws[kq + j][o] = v[j];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            float4 a4 = *reinterpret_cast<const float4 *>(&As[k][ty * 4]);
-            float4 w4 = *reinterpret_cast<const float4 *>(&Ws[k][tx * 4]);
-            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, w[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-
-    // epilogue
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = row0 + ty * 4 + i;
-        const bool row_ok = r < n_rows;
-        float best = -INFINITY;
-        uint32_t best_idx = 0;
-        int u = 0, t = 0;
-        if (row_ok && (EPI == EPI_QKV || EPI == EPI_LOGITS)) u = ep.active_list[r];
-        if (row_ok && EPI == EPI_QKV) t = ep.t_u[u];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int o = o0 + tx * 4 + j;
-            if (!row_ok || o >= M) continue;
-            float v = acc[i][j] + (bias ? to_f32(bias[o]) : 0.f);
-            if (EPI == EPI_STORE) {
-                ep.out[(size_t)r * ep.ldo + o] = v;
-            } else if (EPI == EPI_RELU) {
-                ep.out[(size_t)r * ep.ldo + o] = fmaxf(v, 0.f);
-            } else if (EPI == EPI_RESID) {
-                ep.out[(size_t)r * ep.ldo + o] += v;
-            } else if (EPI == EPI_QKV) {
-                const int d = ep.d_model;
-                if (o < d) {
-                    ep.out[(size_t)r * d + o] = v;
-                } else {
-                    const int kv = (o - d) / d, c = (o - d) % d, h = c / kHeadDim, e = c % kHeadDim;
-                    size_t off = ((((size_t)u * 2 + kv) * ep.n_heads + h) * ep.max_dec_len + t) * kHeadDim + e;
-                    ep.self_cache[off] = from_f32<CT>(v);
-                }
-            } else if (EPI == EPI_LOGITS) {
-                if (ep.logits_out) ep.logits_out[(size_t)u * M + o] = v;
-                if (v > best) { best = v; best_idx = o; }
-            } else if (EPI == EPI_CROSSKV) {
-                const int d = ep.d_model;
-                const int kv = o / d, c = o % d, h = c / kHeadDim, e = c % kHeadDim;
-                size_t off = (((size_t)kv * ep.n_heads + h) * ep.frame_capacity + ep.frame0 + r) * kHeadDim + e;
-                ep.cross_store[off] = from_f32<CT>(v);
-            }
-        }
-        if (EPI == EPI_LOGITS) {
-            // the 8 threads that share this row sit in consecutive lanes: reduce, then one atomic per block row
-            unsigned long long key = (row_ok && best > -INFINITY) ? argmax_key(best, best_idx) : 0ull;
-#pragma unroll
-            for (int off = 1; off < 8; off <<= 1) {
-                unsigned long long other = __shfl_xor_sync(0xffffffffu, key, off);
-                key = other > key ? other : key;
-            }
-            if (tx == 0 && row_ok && key != 0ull) atomicMax(ep.keys + r, key);
-        }
-    }
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -458,7 +287,7 @@ template <int N> __device__ __forceinline__ void load_n(const float *p, float (&
 // so only two blocks per SM: for grids that fit anyway).
 // kRowStats: the block computes (mean, rstd) of its row of stats_x itself instead of reading ln_stats.
 template <typename CT, bool kCross, bool kAppend, bool kPipe = false, bool kRowStats = false>
-__global__ void __launch_bounds__(kFusedMaxWarps * 32, ((kAppend || kPipe) ? 2 : (LaneWidth<CT>::kE > 8 ? 3 : 4)))      // self-attention holds the new key/value as well; wider lanes need more registers
+__global__ void __launch_bounds__(kFusedMaxWarps * 32, sizeof(CT) == 4 ? 1 : ((kAppend || kPipe) ? 2 : (LaneWidth<CT>::kE > 8 ? 3 : 4)))      // self-attention holds the new key/value as well; wider lanes and fp32 need more registers
 attn_fused_kernel(const DecState *state, const int4 *__restrict__ row_info, const float *__restrict__ q, int ldq,
                   CT *__restrict__ cache, int n_heads, int seq_capacity, float scale,
                   float *__restrict__ out, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, int ldo,

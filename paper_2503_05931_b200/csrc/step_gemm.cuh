@@ -120,10 +120,9 @@ __device__ __forceinline__ void side_prefetch(const StepGemmParams &p, int cta, 
 }
 // After the dependency wait: clear the rows a later split-K projection accumulates into, and (mean, rstd) of the rows
 // assigned to this CTA.  w: 0 or 1, which of the two warps; red_s, red_q: two floats of shared memory each.
-__device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int cta, int n_cta, int st, int lane, int w,
+__device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_rows, int cta, int n_cta, int st, int lane, int w,
                                                 float *red_s, float *red_q)
 {
-    const int n_rows = p.state->n_active;
     if (p.zero_buf) {
         const size_t total4 = static_cast<size_t>(n_rows) * p.zero_cols / 4;
         float4 *z = reinterpret_cast<float4 *>(p.zero_buf);
@@ -294,7 +293,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
                 }
             }
         }
-        side_after_wait(p, cta, n_cta, st, lane, warp - 10, red_s, red_q);
+        side_after_wait(p, p.state->n_active, cta, n_cta, st, lane, warp - 10, red_s, red_q);
     } else {
         pdl_wait();
         AED_TRACE_PUT(p.state, tcur, 41);  // dependency resolved

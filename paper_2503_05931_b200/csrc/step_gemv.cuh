@@ -97,8 +97,9 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         const int cta = blockIdx.x + gridDim.x * blockIdx.y;
         const int n_cta = gridDim.x * gridDim.y;
         sg::side_prefetch(p, cta, n_cta, st);
+        const int n_rows = p.state->n_active;
         sg::pdl_wait();
-        sg::side_after_wait(p, cta, n_cta, st, lane, warp - 8, red_s, red_q);
+        sg::side_after_wait(p, n_rows, cta, n_cta, st, lane, warp - 8, red_s, red_q);
         return;
     }
 
@@ -124,8 +125,8 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int ldo = second_w ? p.ldo2 : p.ldo;
     asm volatile("bar.sync 2, 256;" ::: "memory");           // the constants are in place (still before the wait)
 
-    sg::pdl_wait();
     const int n_rows = p.state->n_active;
+    sg::pdl_wait();
     // B fragments: column n = lane / 4 is row nt * 8 + n of the step, rows k0 + {0, 1, 8, 9} with k0 = 16 ks + 2 (lane % 4)
     const int kq = (lane & 3) * 2;
     float2 xa[kNT][kSvMaxKb][4], xb[kNT][kSvMaxKb][4];
@@ -283,8 +284,9 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
         const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
         const int n_cta = gridDim.x * gridDim.y * gridDim.z;
         sg::side_prefetch(p, cta, n_cta, st);
+        const int n_rows = p.state->n_active;
         sg::pdl_wait();
-        sg::side_after_wait(p, cta, n_cta, st, lane, warp - 8, red_s, red_q);
+        sg::side_after_wait(p, n_rows, cta, n_cta, st, lane, warp - 8, red_s, red_q);
         return;
     }
 
@@ -308,8 +310,8 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
     const int ldo = second_w ? p.ldo2 : p.ldo;
     asm volatile("bar.sync 2, 256;" ::: "memory");
 
-    sg::pdl_wait();
     const int n_rows = p.state->n_active;
+    sg::pdl_wait();
     // ---- the rows' k range -> planes: element e of the tile is row e / kF4, floats 4 (e % kF4) .. + 3 ------------------
     constexpr int kPer = kRows * kF4 / 256;                    // 16-byte loads per thread
     float4 xv[kPer];

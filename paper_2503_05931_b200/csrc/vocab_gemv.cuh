@@ -90,8 +90,8 @@ vocab_gemv_kernel(const __grid_constant__ CUtensorMap map_w, VocabGemvParams p)
     }
 
     // ---- rows 2 * warp and 2 * warp + 1: statistics and planes ------------------------------------------------------
-    sg::pdl_wait();
     const int n_rows = p.state->n_active;
+    sg::pdl_wait();
     const int per_lane = p.d_model / 128;                     // 16-byte loads per lane and row (d_model is a multiple of 128 here)
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {

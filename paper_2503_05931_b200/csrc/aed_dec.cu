@@ -532,6 +532,12 @@ aed_status_t tc_setup(aed_dec *dec)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_GAMMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_LN_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
@@ -689,22 +695,27 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     p.n_tile = n_tile;
     p.state = dec->state();
     p.eps = dec->cfg.ln_eps;
-    // (41 to 64 rows: two row halves on grid.z and half the k-splits, up to four k-blocks per CTA.  Measured per decode
-    // step of the 24-layer model against the tcgen05 kernel: 1036 / 1094 / 1129 / 1160 us against 1002 / 1103 / 1160 /
-    // 1200 at 33 / 48 / 56 / 64 rows, hence not between 33 and 40.)
+    // Row tiles of 8 per CTA follow the row count: 2, 3 or 4, and from 33 rows two halves of 3 or 4 on grid.z with half the
+    // k-splits, up to four k-blocks per CTA.  A step of these sizes is bound by instructions issued (conversion of the
+    // rows to planes, fragments, reductions), so a tile of padding costs as much as one of rows.  Per decode step of the
+    // 24-layer model, with four tiles -> with three: 715 -> 630 us at 20 rows, 723 -> 680 at 24, 1104 -> 959 at 48; 33 to
+    // 40 rows left the tcgen05 kernel for it (939 / 952 / 1032 -> 837 / 825 / 922 us at 33 / 36 / 40 rows).  At 65 rows
+    // and beyond three or four such parts lose to the tcgen05 kernel (1392 / 1634 / 1881 us there against 1512 / 1655 /
+    // 2006 at 65 / 96 / 128 rows).
     const int splits_wide = std::max((k_blocks + 3) / 4, splits / 2);
-    const bool gemv = MODE != sg::B_PLANES && dec->use_gemv && rows_ub <= dec->gemv_rows && !(rows_ub > 32 && rows_ub <= 40) &&
+    const bool gemv = MODE != sg::B_PLANES && dec->use_gemv && rows_ub <= dec->gemv_rows &&
                       (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
     ProfScope ps(dec, family + KF_COUNT * (!gemv ? KV_TCGEN05 : rows_ub <= dec->gemv_direct_rows ? KV_GEMV : KV_GEMV_STAGED));
     if constexpr (MODE != sg::B_PLANES) {
-        // Steps of at most 32 rows whose CTAs cover at most two k-blocks: warp-level MMAs (step_gemv.cuh), activation
-        // fragments straight from global memory up to 8 rows, through shared memory beyond
+        // Steps of at most 32 rows whose CTAs cover at most two k-blocks (64 rows, four): warp-level MMAs
+        // (step_gemv.cuh), activation fragments straight from global memory up to 4 rows, through shared memory beyond
         if (gemv) {
             cudaLaunchConfig_t gc = {};
             gc.gridDim = dim3(m_tiles, splits, 1);
             gc.blockDim = dim3(sv::kSvThreads);
             const bool direct = rows_ub <= dec->gemv_direct_rows, wide = rows_ub > 32;
-            const int nt = rows_ub <= 16 ? 2 : 4;
+            const int part = wide ? (rows_ub + 1) / 2 : rows_ub;
+            const int nt = wide ? (part <= 24 ? 3 : 4) : part <= 16 ? 2 : part <= 24 ? 3 : 4;      // row tiles of 8 per CTA
             if (wide) gc.gridDim = dim3(m_tiles, splits_wide, 2);
             gc.dynamicSmemBytes = direct ? (size_t)sv::kSvMaxKb * tc::kATileBytes + 1024 : (size_t)sv::sv_staged_smem(nt, wide ? 4 : sv::kSvMaxKb);
             gc.stream = dec->stream;
@@ -715,7 +726,9 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
             gc.numAttrs = 1;
             const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
             cudaError_t ge = direct    ? cudaLaunchKernelEx(&gc, sv::step_gemv_kernel<MODE, 1>, map_w, second, p)
-                             : wide    ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4, 4>, map_w, second, p)
+                             : wide    ? (nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3, 4>, map_w, second, p)
+                                                  : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4, 4>, map_w, second, p))
+                             : nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3>, map_w, second, p)
                              : nt == 2 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 2>, map_w, second, p)
                                        : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4>, map_w, second, p);
             if (ge != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(ge));

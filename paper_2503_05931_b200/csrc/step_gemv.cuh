@@ -226,7 +226,7 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     }
 }
 
-// The same projection for steps of 9 to 32 rows.  Loading B fragments straight from global memory makes every one of
+// The same projection for steps of 5 to 64 rows.  Loading B fragments straight from global memory makes every one of
 // the 8 warps fetch and split the same activation values; beyond a handful of rows that traffic costs more than one
 // hand-over through shared memory.  Here the 256 compute threads load the rows' k range once (coalesced 16-byte loads),
 // apply the transform, write bf16 high and low planes [row][k] into shared memory (row pitch padded against bank
@@ -250,7 +250,7 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
     __shared__ __align__(16) float s_g[kKB * kBlockK], s_c1[kKB * kBlockK], s_c2[kKB * kBlockK];
     __shared__ __align__(16) float s_t[8][8][16 + 4];
 
-    static_assert(kNT == 2 || kNT == 4, "row tiles are read in pairs");
+    static_assert(kNT >= 2 && kNT <= 4, "row tiles are read in pairs, an odd last one alone");
     constexpr int kRows = kNT * 8, kSvPitch = sv_pitch(kKB), kF4 = kKB * kBlockK / 4;      // kF4: 16-byte loads per row
     const int row0 = blockIdx.z * kRows;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -353,6 +353,7 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
     bool ok = true;
     // ldmatrix addresses of the B fragments: matrices (rows 0-7, k 0-7), (rows 0-7, k 8-15), (rows 8-15, k 0-7), (rows 8-15, k 8-15)
     const uint32_t b_off = static_cast<uint32_t>(((lane & 7) + ((lane >> 4) << 3)) * kSvPitch + ((lane >> 3) & 1) * 16);
+    const uint32_t b_last = static_cast<uint32_t>((lane & 7) * kSvPitch + ((lane >> 3) & 1) * 16);
     const uint32_t hi_base = smem_u32(plane_hi), lo_base = smem_u32(plane_lo);
 #pragma unroll
     for (int i = 0; i < kKB; ++i) {
@@ -366,7 +367,7 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
             ldmatrix_x4(wt + swz(warp * 16 + (lane & 15), ks * 2 + (lane >> 4)), a);
             const uint32_t kbyte = static_cast<uint32_t>((i * kBlockK + ks * 16) * 2);
 #pragma unroll
-            for (int np = 0; np < kNT; np += 2) {                // two row tiles of 8 per ldmatrix
+            for (int np = 0; np + 1 < kNT; np += 2) {            // two row tiles of 8 per ldmatrix
                 uint32_t bh[4], bl[4];
                 ldmatrix_x4(hi_base + np * 8 * kSvPitch + b_off + kbyte, bh);
                 ldmatrix_x4(lo_base + np * 8 * kSvPitch + b_off + kbyte, bl);
@@ -374,6 +375,12 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
                 mma_16816(acc_l[np], a, bl[0], bl[1]);
                 mma_16816(acc_h[np + 1], a, bh[2], bh[3]);
                 mma_16816(acc_l[np + 1], a, bl[2], bl[3]);
+            }
+            if (kNT % 2) {                                      // the third row tile: both planes in one ldmatrix
+                uint32_t b[4];
+                ldmatrix_x4((lane >> 4 ? lo_base : hi_base) + (kNT - 1) * 8 * kSvPitch + b_last + kbyte, b);
+                mma_16816(acc_h[kNT - 1], a, b[0], b[1]);
+                mma_16816(acc_l[kNT - 1], a, b[2], b[3]);
             }
         }
     }

@@ -372,6 +372,16 @@ def test_small_batch_row_counts(batch):
     _run_both(w, rows=rows)
 
 
+@pytest.mark.parametrize("batch", [20, 24, 25, 33, 47, 49])
+def test_row_tiles_of_three(batch):
+    """Row counts around the steps that cover their rows with three tiles of 8 per CTA: a partly filled third tile, a
+    full one, one row beyond, and the same in two row halves (the second one partly filled)."""
+    rng = np.random.default_rng(950 + batch)
+    w = wl.make_custom(WIDE_A, rng.integers(1, 80, size=batch), rng.integers(1, 6, size=batch), dtype="bf16", seed=330 + batch,
+                       out_std=0.1, ln_std=0.2)
+    _run_both(w, rows=sorted({0, 7, 16, 19, batch // 2, batch - 1}))
+
+
 @pytest.mark.parametrize("model", ["wide_b", "odd"])
 def test_small_batch_model_shapes(model):
     """d_model 1024 with 16 heads at 64 rows, and a model whose widths are not multiples of 128 (an odd number of

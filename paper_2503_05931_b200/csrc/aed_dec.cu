@@ -337,6 +337,24 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
     if constexpr (kCross && !kAppend) {
         if (stats_x) kernel = pipe ? attn_fused_kernel<T, true, false, true, true> : attn_fused_kernel<T, true, false, false, true>;
     }
+    if constexpr (!kCross && sizeof(T) == 2) {
+        // One warp per (row, head) once there are more than about 7 of them per SM: a block of its own per pair spends
+        // its time starting, merging and ending.  With fewer the pairs need several warps each to have enough loads in
+        // flight (24-layer model, 16 heads, per step at up to 8 / 239 positions, a block per pair -> a warp per pair:
+        // 64 rows 1051 / 1225 -> 1040 / 1382 us, 80 rows 1450 / 1635 -> 1394 / 1646, 128 rows 1778 / 2042 ->
+        // 1666 / 1948, 512 rows 4022 / 5127 -> 3513 / 4452).
+        if (rows_ub * dec->cfg.n_heads > 1024) {
+            cfg.gridDim = dim3((rows_ub * dec->cfg.n_heads + 7) / 8);
+            cfg.blockDim = dim3(256);
+            cudaError_t e = cudaLaunchKernelEx(&cfg, self_attn_warp_kernel<T, kAppend>, (const DecState *)dec->state(),
+                                               (const int4 *)dec->at<int4>(dec->lay.row_info), q, ldq, const_cast<T *>(cache),
+                                               dec->cfg.n_heads, seq_capacity, 1.0f / sqrtf((float)kHeadDim), out, out_hi, out_lo,
+                                               dec->cfg.d_model, ln_stats, ln_c1, ln_c2, rows_ub * dec->cfg.n_heads);
+            if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
+            AED_LAUNCHED(dec);
+            return AED_OK;
+        }
+    }
     cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, (const DecState *)dec->state(),
                                        (const int4 *)dec->at<int4>(dec->lay.row_info), q, ldq, const_cast<T *>(cache),
                                        dec->cfg.n_heads, seq_capacity, 1.0f / sqrtf((float)kHeadDim), out, out_hi, out_lo,

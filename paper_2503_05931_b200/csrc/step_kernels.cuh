@@ -534,6 +534,127 @@ attn_fused_kernel(const DecState *state, const int4 *__restrict__ row_info, cons
     AED_TRACE_PUT_NS(state, tcur, 7);                       // output written
 }
 
+// Self-attention of many rows: one warp per (row, head), 8 pairs per block, no shared memory and no merge of warps.
+// Short caches make this a matter of latency (the dependency wait, then one round of loads and a chain of shuffles), so
+// what counts is how many pairs an SM holds at once: 24 warps of at most 85 registers.  A pair's later chunks are loaded
+// one after the other; 24 x 4 KB in flight per SM are enough (512 rows, up to 239 positions: the cache is read at about
+// 6.2 TB/s; at up to 8 positions a launch went from about 26 us with a block per pair to 6).
+template <typename CT, bool kAppend>
+__global__ void __launch_bounds__(256, 3)
+self_attn_warp_kernel(const DecState *state, const int4 *__restrict__ row_info, const float *__restrict__ q, int ldq,
+                      CT *__restrict__ cache, int n_heads, int seq_capacity, float scale, float *__restrict__ out,
+                      __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, int ldo,
+                      const float2 *__restrict__ ln_stats, const float *__restrict__ ln_c1, const float *__restrict__ ln_c2, int row_heads)
+{
+    constexpr int kE = LaneWidth<CT>::kE, kDG = kHeadDim / kE, kPG = 32 / kDG, kChunk = 4 * kPG;
+    const int lane = threadIdx.x & 31, rh = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int r = rh / n_heads, h = rh - r * n_heads;
+    const int4 ri = rh < row_heads ? row_info[r] : make_int4(-1, 0, 0, 0);
+    const int len = ri.y + 1, len_static = kAppend ? len - 1 : len;
+    const int dg = lane % kDG, pg = lane / kDG, qcol = h * kHeadDim + dg * kE, d_model = n_heads * kHeadDim;
+    CT *const kbase = cache + ((size_t)max(ri.x, 0) * 2 * n_heads + h) * (size_t)seq_capacity * kHeadDim + dg * kE;
+    CT *const vbase = kbase + (size_t)n_heads * seq_capacity * kHeadDim;
+    RawLane<CT> rk[4], rv[4];
+    auto load_chunk = [&](int p0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int p = p0 + i * kPG + pg;
+            if (p < len_static) { rk[i].load(kbase + (size_t)p * kHeadDim); rv[i].load(vbase + (size_t)p * kHeadDim); }
+            else { rk[i].zero(); rv[i].zero(); }
+        }
+    };
+    if (kAppend && ri.x >= 0) load_chunk(0);            // positions of earlier steps: before the dependency wait
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (ri.x < 0) return;
+    if (!kAppend) load_chunk(0);
+    const float2 st = ln_stats[r];
+    const float *const qr = q + (size_t)r * ldq + qcol;
+    float qv[kE];
+    RawLane<CT> new_k, new_v;
+    {
+        float y[3][kE], c1[kE], c2[kE];
+#pragma unroll
+        for (int j = 0; j < (kAppend ? 3 : 1); ++j) load_n<kE>(qr + j * d_model, y[j]);
+#pragma unroll
+        for (int j = 0; j < (kAppend ? 3 : 1); ++j) {
+            load_n<kE>(ln_c1 + j * d_model + qcol, c1);
+            load_n<kE>(ln_c2 + j * d_model + qcol, c2);
+#pragma unroll
+            for (int i = 0; i < kE; ++i) y[j][i] = fmaf(st.y, y[j][i] - st.x * c1[i], c2[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < kE; ++i) qv[i] = y[0][i] * (scale * 1.4426950408889634f);
+        if (kAppend) {
+            new_k.set(y[1]);
+            new_v.set(y[2]);
+            if (pg == 0) {
+                new_k.store(kbase + (size_t)(len - 1) * kHeadDim);
+                new_v.store(vbase + (size_t)(len - 1) * kHeadDim);
+            }
+        }
+    }
+    float m = -INFINITY, l = 0.f, acc[kE];
+#pragma unroll
+    for (int i = 0; i < kE; ++i) acc[i] = 0.f;
+    for (int p0 = 0; p0 < len; p0 += kChunk) {
+        if (p0) load_chunk(p0);
+        float s[4], cmax = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int p = p0 + i * kPG + pg;
+            if (kAppend && p == len - 1) { rk[i] = new_k; rv[i] = new_v; }
+            float kf[kE], d = 0.f;
+            rk[i].get(kf);
+#pragma unroll
+            for (int j = 0; j < kE; ++j) d = fmaf(qv[j], kf[j], d);
+#pragma unroll
+            for (int o = 1; o < kDG; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            s[i] = p < len ? d : -INFINITY;
+            cmax = fmaxf(cmax, s[i]);
+        }
+#pragma unroll
+        for (int o = kDG; o < 32; o <<= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+        const float m_new = fmaxf(m, cmax), corr = exp2_fast(m - m_new);
+        l *= corr;
+#pragma unroll
+        for (int j = 0; j < kE; ++j) acc[j] *= corr;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float pr = exp2_fast(s[i] - m_new);
+            float vf[kE];
+            rv[i].get(vf);
+            l += pr;
+#pragma unroll
+            for (int j = 0; j < kE; ++j) acc[j] = fmaf(pr, vf[j], acc[j]);
+        }
+        m = m_new;
+    }
+    // sum the position groups: every lane keeps kE / kPG = 2 of its 8 dimensions, so the groups write one row together
+    float o2[2];
+    l += __shfl_xor_sync(0xffffffffu, l, kDG);
+    l += __shfl_xor_sync(0xffffffffu, l, 2 * kDG);
+    static_assert(kE == 8 && kPG == 4, "two halving exchanges");
+    {
+        float a4[4];
+        const bool up = pg & 2;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a4[j] = (up ? acc[4 + j] : acc[j]) + __shfl_xor_sync(0xffffffffu, up ? acc[j] : acc[4 + j], 2 * kDG);
+        const bool up1 = pg & 1;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) o2[j] = (up1 ? a4[2 + j] : a4[j]) + __shfl_xor_sync(0xffffffffu, up1 ? a4[j] : a4[2 + j], kDG);
+    }
+    const float inv = 1.f / l;
+    o2[0] *= inv; o2[1] *= inv;
+    const size_t off = (size_t)r * ldo + qcol + pg * 2;
+    if (out) *reinterpret_cast<float2 *>(out + off) = make_float2(o2[0], o2[1]);
+    if (out_hi) {
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(o2[0], o2[1]);
+        *reinterpret_cast<__nv_bfloat162 *>(out_hi + off) = hi;
+        *reinterpret_cast<__nv_bfloat162 *>(out_lo + off) = __floats2bfloat162_rn(o2[0] - __bfloat162float(hi.x), o2[1] - __bfloat162float(hi.y));
+    }
+}
+
 // Merge the chunk partials of each (row, head): one warp per pair, 2 head dimensions per lane.
 template <bool kCross>
 __global__ void __launch_bounds__(128)

@@ -382,6 +382,18 @@ def test_row_tiles_of_three(batch):
     _run_both(w, rows=sorted({0, 7, 16, 19, batch // 2, batch - 1}))
 
 
+@pytest.mark.parametrize("model, batch", [("wide_a", 129), ("wide_b", 65), ("odd", 342), ("odd", 347)])
+def test_self_attention_of_many_rows(model, batch):
+    """More than 1024 (row, head) pairs, where self-attention takes a warp per pair: just above the line, a last block
+    with 1 and 2 of its 8 pairs, blocks that span two rows, and caches that end at and around 16-position chunks."""
+    rng = np.random.default_rng(970 + batch)
+    dec_lens = rng.integers(1, 6, size=batch)
+    dec_lens[:5] = [1, 16, 17, 33, 34]
+    m = {"wide_a": WIDE_A, "wide_b": WIDE_B, "odd": ODD}[model]
+    w = wl.make_custom(m, rng.integers(1, 30, size=batch), dec_lens, dtype="bf16", seed=340 + batch, out_std=0.1, ln_std=0.2)
+    _run_both(w, rows=[0, 1, 2, 3, 4, batch // 2, batch - 1])
+
+
 @pytest.mark.parametrize("model", ["wide_b", "odd"])
 def test_small_batch_model_shapes(model):
     """d_model 1024 with 16 heads at 64 rows, and a model whose widths are not multiples of 128 (an odd number of

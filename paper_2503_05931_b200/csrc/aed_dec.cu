@@ -517,7 +517,7 @@ aed_status_t tc_setup(aed_dec *dec)
         ok = ok && encode_map(&m.qkv, w.w_qkv, 3 * d, d, tc::kTileM) && encode_map(&m.o, w.w_o, d, d, tc::kTileM) &&
              encode_map(&m.qc, w.w_q_c, d, d, tc::kTileM) && encode_map(&m.oc, w.w_o_c, d, d, tc::kTileM) &&
              encode_map(&m.ff1, w.w_ff1, F, d, tc::kTileM) && encode_map(&m.ff2, w.w_ff2, d, F, tc::kTileM) &&
-             encode_map(&kvc_maps[l], w.w_kv_c, 2 * d, c.d_enc, ckv::kTileN) &&
+             encode_map(&kvc_maps[l], w.w_kv_c, 2 * d, c.d_enc, ckv::kTileN / 2) &&
              encode_map(&m.o_qc, dec->ws + L.comp_w + (size_t)l * d * d * 2, d, d, tc::kTileM);
         kvc_bias[l] = w.b_kv_c;
     }
@@ -1050,7 +1050,7 @@ aed_status_t precompute_tc(aed_dec *dec, const void *enc_base, long long enc_row
     p.layer_elems = L.cross_layer_elems;
     p.bias = dec->at<const T *>(L.ckv_bias);
     p.state = dec->state();
-    const long long tiles = (long long)segs.tile0[segs.n] * c.n_layers * ((2 * c.d_model + ckv::kTileN - 1) / ckv::kTileN);
+    const long long tiles = (long long)((segs.tile0[segs.n] + 1) / 2) * c.n_layers * ((2 * c.d_model + ckv::kTileN - 1) / ckv::kTileN);
     ProfScope ps(dec, KF_PRECOMPUTE);
     const unsigned grid = (unsigned)std::min<long long>(tiles, dec->sm_count);
     const size_t smem = ckv::kStages * ckv::kStageBytes + 1024;

@@ -394,6 +394,25 @@ def test_self_attention_of_many_rows(model, batch):
     _run_both(w, rows=[0, 1, 2, 3, 4, batch // 2, batch - 1])
 
 
+@pytest.mark.parametrize("enc_lens", [(1,), (128,), (100, 29), (256,), (200, 57), (384, 1)])
+def test_cross_kv_frame_tiles(enc_lens):
+    """Encoder frames that fill 1, 2, 3 and 4 tiles of 128 exactly or by one frame (an odd last tile has no partner in
+    its pair of blocks), with a feature count that ends inside a 256-wide tile and crosses from keys to values in it."""
+    w = wl.make_custom(ODD, list(enc_lens), [3] * len(enc_lens), dtype="bf16", seed=360 + sum(enc_lens), out_std=0.1, ln_std=0.2,
+                       bias_std=0.05)
+    _run_both(w)
+
+
+@pytest.mark.parametrize("batch", [18, 70, 83, 131, 163, 259])
+def test_equal_row_tiles(batch):
+    """Row counts that take one tile of 32, 80 or 96 rows, two of 80, two of 96 with ready-made planes, and two tiles of
+    the vocabulary projection, whose 333 entries end inside a tile and inside a lane's four."""
+    rng = np.random.default_rng(980 + batch)
+    w = wl.make_custom(ODD, rng.integers(1, 20, size=batch), rng.integers(1, 4, size=batch), dtype="bf16", seed=350 + batch,
+                       out_std=0.1, ln_std=0.2, out_bias_std=0.1)
+    _run_both(w, rows=sorted({0, 15, 16, 17, batch // 2 - 1, batch // 2, batch // 2 + 1, batch - 2, batch - 1}))
+
+
 @pytest.mark.parametrize("model", ["wide_b", "odd"])
 def test_small_batch_model_shapes(model):
     """d_model 1024 with 16 heads at 64 rows, and a model whose widths are not multiples of 128 (an odd number of

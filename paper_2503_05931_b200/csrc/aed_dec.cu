@@ -534,7 +534,7 @@ aed_status_t tc_setup(aed_dec *dec)
     }
     if (!ok) return fail(nullptr, AED_ERR_CUDA, "cuTensorMapEncodeTiled failed (are all weight tensors 16-byte aligned?)");
     const int smem = kTcSmemBudget + 1024;
-    cudaError_t e = cudaFuncSetAttribute(tc::tc_gemm_kernel<tc::TC_EPI_LOGITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(tc::tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv::crosskv_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ckv::kStages * ckv::kStageBytes + 1024);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(ckv::crosskv_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ckv::kStages * ckv::kStageBytes + 1024);
     // tensor maps and bias pointers of the cross-K/V weights: read by the precompute kernel from the workspace
@@ -648,7 +648,7 @@ aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int ro
     const CUtensorMap *acts = dec->tc_actd[ni];
     dim3 grid(m_tiles, 1, row_tiles);
     void *args[] = {(void *)&dec->tc_w_out, (void *)&acts[0], (void *)&acts[1], &p, &stages, (void *)&producers};
-    return launch_pdl_impl(dec, (const void *)tc::tc_gemm_kernel<tc::TC_EPI_LOGITS>, grid, dim3(tc::kThreads),
+    return launch_pdl_impl(dec, (const void *)tc::tc_gemm_kernel, grid, dim3(tc::kThreads),
                            (size_t)stages * stage_bytes + 1024, args);
 }
 

@@ -4,16 +4,17 @@
 //
 // Both operands are K-major bf16 in global memory and arrive in shared memory through
 // cp.async.bulk.tensor (no multicast) with the 128-byte swizzle the MMA descriptors name.
-// One CTA = one (128-row tile of A, N-row tile of B, k-split).  Warp roles: warps 0..3 issue TMA (a thread's
+// One CTA = one (128-row tile of A, N-row tile of B, k-split).  Warp roles: warps 0..7 issue TMA (a thread's
 // copies complete one after the other, about a third of a microsecond each, so the k-blocks are shared out round
-// robin over four issuing threads), warp 4 owns the TMEM allocation and issues the MMAs, warps 5..8 drain the
-// accumulator (warp w reads TMEM lanes 32*(w%4) .. +31) and run the epilogue.
+// robin over the issuing threads), warp 8 owns the TMEM allocation and issues the MMAs; at the end all warps but that
+// one drain the accumulator (warp w reads TMEM lanes 32*(w%4) .. +31) into the ring's memory, rows first, and then take
+// a row each.
 //
-// Two uses:
-//   * vocabulary projection ("weights as A"): A = output matrix [vocab, K], B = the final LayerNorm output
-//     [rows, K] as a bf16 high plane and a low (residual) plane accumulated into the same D, so that
-//     activations keep ~16 mantissa bits; the greedy argmax is taken in the epilogue.
-//   * cross-K/V precompute ("frames as A"): A = packed encoder frames, B = [2d, d_enc] weights of a layer.
+// Used by the vocabulary projection ("weights as A"): A = output matrix [vocab, K], B = the final LayerNorm output
+// [rows, K] as a bf16 high plane and a low (residual) plane accumulated into the same D, so that activations keep ~16
+// mantissa bits; the greedy argmax is taken in the epilogue.  The rows-first epilogue is there because an argmax straight
+// from the accumulator (a lane per vocabulary entry) needs four warp reductions and four atomics per row and tile, one
+// row after the other, and took longer than the product: 16384 entries x 128 rows 38 us, now 20; 512 rows 109, now 57.
 //
 // Every wait on an mbarrier is bounded: on expiry the CTA raises the error word in the decode state, stops
 // issuing work, waits (bounded) for its own TMA copies, frees its TMEM and returns.
@@ -30,7 +31,7 @@ constexpr int kBlockK = 64;                    // bf16 elements per k-block = on
 constexpr int kTileM = 128;
 constexpr int kATileBytes = kTileM * kBlockK * 2;
 constexpr int kMaxStages = 8;
-constexpr int kThreads = 416;                    // 8 producer warps, 1 MMA warp, 4 epilogue warps
+constexpr int kThreads = 416;                    // 8 producer warps, 1 MMA warp, 4 more for the epilogue
 constexpr int kProducerWarps = 8;                // (a k-block is three copies, and a thread's copies complete one after the other)
 constexpr long long kWaitCycles = 2000000000ll;   // about a second at B200 clocks
 constexpr int kErrTimeout = 2;
@@ -132,8 +133,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-enum TcEpilogue { TC_EPI_LOGITS = 1 };
-
 struct TcParams {
     int a_rows;          // valid rows of A (output features, or frames)
     int n_tile;          // rows of B per CTA = MMA N (multiple of 16, at most 256)
@@ -141,7 +140,6 @@ struct TcParams {
     int use_lo;          // 1: accumulate the low activation plane as well
     int rows_fixed;      // >= 0: number of valid B rows; < 0: read it from the decode state
     const __nv_bfloat16 *bias;         // over the columns of D's first dimension (vocabulary / K-V features), may be null
-    // TC_EPI_LOGITS
     float *logits_out;                 // [batch, vocab] by utterance or nullptr
     unsigned long long *keys;          // [rows]
     const int32_t *active_list;
@@ -149,7 +147,6 @@ struct TcParams {
 };
 
 // grid: x = 128-row tiles of A, y = k-splits, z = N-row tiles of B.  Dynamic shared memory: stage ring + 1024.
-template <int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b_lo, TcParams p, int stages, int producers)
@@ -163,7 +160,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
-    AED_TRACE_BEGIN(p.state, 16 + EPI);
+    AED_TRACE_BEGIN(p.state, 17);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row0 = blockIdx.z * p.n_tile;
     // Only row tiles after the first can be empty; the first one skips this read so that set-up and the first
@@ -248,38 +245,62 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             if (ok) mma_commit(&bar_done);      // accumulator complete
         }
-    } else {
-        // epilogue warps
-        const int quarter = warp & 3;
+    }
+    // ---- epilogue: all warps but the one that issues the MMAs (the producers have nothing left to do) -------------
+    if (warp != kProducerWarps) {
+        constexpr int kPitch = kTileM + 4;
+        const int ew = warp < kProducerWarps ? warp : warp - 1;      // 0..11
+        const int quarter = warp & 3;                                // tensor memory lanes this warp can reach
+        const int third = warp < 4 ? 0 : warp < kProducerWarps ? 1 : 2;      // three warps per quarter share the rows in 16s
+        float *trans = reinterpret_cast<float *>(tiles);             // T[row][feature] over the ring's memory
+        __syncwarp();
         const int n_rows = p.rows_fixed >= 0 ? p.rows_fixed : p.state->n_active;
-        const bool ok = mbar_wait(&bar_done, 0, &abort_flag);
+        const bool ok = mbar_wait(&bar_done, 0, &abort_flag);        // every MMA has completed: the ring is free
         tc_fence_after_sync();
         if (threadIdx.x == (kProducerWarps + 1) * 32) AED_TRACE_MARK(p.state, 34);  // accumulator complete
+        const int rows_here = min(p.n_tile, max(n_rows - row0, 0));
         if (ok) {
-            const int a_idx = a0 + quarter * 32 + lane;          // row of A this thread owns
-            const bool a_ok = a_idx < p.a_rows;
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-            if (EPI == TC_EPI_LOGITS) {
-                const float bias = (p.bias && a_ok) ? to_f32(p.bias[a_idx]) : 0.f;
-                for (int c0 = 0; c0 < p.n_tile; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(taddr + c0, v);
+            for (int c0 = 16 * third; c0 < rows_here; c0 += 48) {
+                float v[16];
+                tmem_ld16(taddr + c0, v);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int r = row0 + c0 + j;                 // uniform over the warp
-                        if (r >= n_rows) continue;
-                        const float z = v[j] + bias;
-                        if (p.logits_out && a_ok) p.logits_out[static_cast<size_t>(p.active_list[r]) * p.a_rows + a_idx] = z;
-                        // warp maximum of the order-preserving key, then the lowest lane that attains it
-                        const uint32_t k32 = a_ok ? float_order_key(z) : 0u;
-                        const uint32_t kmax = __reduce_max_sync(0xffffffffu, k32);
-                        const uint32_t winners = __ballot_sync(0xffffffffu, k32 == kmax);
-                        const uint32_t best = a0 + quarter * 32 + (__ffs(winners) - 1);
-                        const unsigned long long key =
-                            kmax ? ((static_cast<unsigned long long>(kmax) << 32) | (0xFFFFFFFFu - best)) : 0ull;
-                        if (lane == 0 && key != 0ull) atomicMax(p.keys + r, key);
+                for (int j = 0; j < 16; ++j) trans[(c0 + j) * kPitch + quarter * 32 + lane] = v[j];
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");
+        if (ok) {
+            // a warp per row, 4 consecutive vocabulary entries per lane
+            const int o = a0 + lane * 4;
+            float bias[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) bias[j] = p.bias && o + j < p.a_rows ? to_f32(p.bias[o + j]) : 0.f;
+            const bool vec = o + 3 < p.a_rows && p.a_rows % 4 == 0 && (reinterpret_cast<uintptr_t>(p.logits_out) & 15) == 0;
+#pragma unroll 2
+            for (int rl = ew; rl < rows_here; rl += kThreads / 32 - 1) {
+                const int r = row0 + rl;
+                float4 t = *reinterpret_cast<const float4 *>(trans + rl * kPitch + lane * 4);
+                const float z[4] = {t.x + bias[0], t.y + bias[1], t.z + bias[2], t.w + bias[3]};
+                if (p.logits_out) {
+                    float *dst = p.logits_out + static_cast<size_t>(p.active_list[r]) * p.a_rows + o;
+                    if (vec) *reinterpret_cast<float4 *>(dst) = make_float4(z[0], z[1], z[2], z[3]);
+                    else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (o + j < p.a_rows) dst[j] = z[j];
                     }
                 }
+                // the lane's best entry, the warp's best key, then the lowest lane that has it: the lowest index among equals
+                uint32_t k32 = 0u, best = 0u;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t k = o + j < p.a_rows ? float_order_key(z[j]) : 0u;
+                    if (k > k32) { k32 = k; best = static_cast<uint32_t>(o + j); }
+                }
+                const uint32_t kmax = __reduce_max_sync(0xffffffffu, k32);
+                const uint32_t winners = __ballot_sync(0xffffffffu, k32 == kmax);
+                if (kmax != 0u && lane == __ffs(winners) - 1)
+                    atomicMax(p.keys + r, (static_cast<unsigned long long>(kmax) << 32) | (0xFFFFFFFFu - best));
             }
         }
     }

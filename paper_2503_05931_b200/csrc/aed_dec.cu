@@ -188,8 +188,8 @@ struct aed_dec {
     struct TcLayerMaps { CUtensorMap qkv, o, qc, oc, ff1, ff2, o_qc; };      // o_qc: the composite Wqc diag(gamma2) Wo
     std::vector<TcLayerMaps> tc_layers;
     CUtensorMap tc_w_out;
-    CUtensorMap tc_actd[5][2], tc_actf[5][2];     // [log2(N/16)][plane]: activation planes [rows, d] and [rows, F]
-    CUtensorMap tc_src_x[5], tc_src_att[5], tc_src_hid[5];   // fp32 sources of the fused projections, per MMA N
+    CUtensorMap tc_actd[16][2], tc_actf[16][2];   // [N/16 - 1][plane]: activation planes [rows, d] and [rows, F]
+    CUtensorMap tc_src_x[8], tc_src_att[8], tc_src_hid[8];   // fp32 sources of the fused projections, per MMA N
     bool use_tc = false;
     int sm_count = 148;
     int tc_target_ctas = 128;
@@ -522,13 +522,14 @@ aed_status_t tc_setup(aed_dec *dec)
         kvc_bias[l] = w.b_kv_c;
     }
     ok = ok && encode_map(&dec->tc_w_out, dec->w_out, c.vocab, d, tc::kTileM);
-    for (int i = 0; i < 5; ++i) {
-        const int box = 16 << i;
+    for (int i = 0; i < 16; ++i) {
+        const int box = 16 * (i + 1);
         ok = ok && encode_map(&dec->tc_actd[i][0], dec->ws + L.actd_hi, L.rows_cap, d, box) &&
              encode_map(&dec->tc_actd[i][1], dec->ws + L.actd_lo, L.rows_cap, d, box) &&
              encode_map(&dec->tc_actf[i][0], dec->ws + L.actf_hi, L.rows_cap, F, box) &&
-             encode_map(&dec->tc_actf[i][1], dec->ws + L.actf_lo, L.rows_cap, F, box) &&
-             encode_map(&dec->tc_src_x[i], dec->ws + L.x, c.max_batch, d, box, true) &&
+             encode_map(&dec->tc_actf[i][1], dec->ws + L.actf_lo, L.rows_cap, F, box);
+        if (i < 8)
+            ok = ok && encode_map(&dec->tc_src_x[i], dec->ws + L.x, c.max_batch, d, box, true) &&
              encode_map(&dec->tc_src_att[i], dec->ws + L.act, c.max_batch, d, box, true) &&
              encode_map(&dec->tc_src_hid[i], dec->ws + L.hid, c.max_batch, F, box, true);
     }
@@ -616,12 +617,13 @@ aed_status_t tc_setup(aed_dec *dec)
     return AED_OK;
 }
 
-// MMA N for a step with at most rows_ub rows: the smallest of 16, 32, ..., 256 that covers them (or 256).
-int tc_n_index(int rows_ub)
+// MMA N (a multiple of 16) for rows_ub rows in tiles of at most `most`: as few tiles as possible, of equal size, because
+// a tile's operand traffic and tensor time go with its N whether its rows are real or padding.  (Tiles of a power of two
+// against this, per step of the 24-layer model: 72 rows 1387 -> 1278 us, 136 rows 2109 -> 1856, 192 rows 2323 -> 2120.)
+int tc_n_tile(int rows_ub, int most)
 {
-    int i = 0;
-    while (i < 4 && (16 << i) < rows_ub) ++i;
-    return i;
+    const int tiles = (rows_ub + most - 1) / most;
+    return std::max(16, ((rows_ub + tiles - 1) / tiles + 15) / 16 * 16);
 }
 
 // The vocabulary projection on tensor cores: logits[r, v] = sum_k act[r, k] * Wout[v, k] (+ bias), argmax in the epilogue.
@@ -629,7 +631,7 @@ aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int ro
 {
     ProfScope ps(dec, KF_GEMM_VOCAB);
     const int M = dec->cfg.vocab, K = dec->cfg.d_model;
-    const int ni = tc_n_index(rows_ub), n_tile = 16 << ni;
+    const int n_tile = tc_n_tile(rows_ub, 256), ni = n_tile / 16 - 1;
     const int row_tiles = (rows_ub + n_tile - 1) / n_tile, m_tiles = (M + tc::kTileM - 1) / tc::kTileM;
     const int k_blocks = K / tc::kBlockK;
     p.a_rows = M;
@@ -681,12 +683,10 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
                               const CUtensorMap *map_w2 = nullptr, int M2 = 0)
 {
     // map_w2, M2: a second weight matrix [M2, K] over the same rows (its output, gamma and bias are in p)
-    // plane_maps (B_PLANES only): [log2(N/16)][high, low] tensor maps of the ready-made activation planes
+    // plane_maps (B_PLANES only): [N/16 - 1][high, low] tensor maps of the ready-made activation planes
     // Rows per CTA tile: up to 128 (two ring stages still fit beside the transposition buffer); more rows are
     // covered by row tiles that re-read the weight tile from L2.
-    int ni = tc_n_index(rows_ub);
-    if (ni > 3) ni = 3;
-    const int n_tile = 16 << ni;
+    const int n_tile = tc_n_tile(rows_ub, 128), ni = n_tile / 16 - 1;
     const int m_tiles1 = (M + tc::kTileM - 1) / tc::kTileM;
     const int row_tiles = (rows_ub + n_tile - 1) / n_tile, m_tiles = m_tiles1 + (map_w2 ? (M2 + tc::kTileM - 1) / tc::kTileM : 0);
     p.tiles_first = map_w2 ? m_tiles1 : 0;
@@ -986,12 +986,12 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
                                                         ad_hi, ad_lo, stats, c1_qkv, c2_qkv, pdl)));
         p = sg::StepGemmParams{};
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_o;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_O, m.o, nullptr, d, d, rows_ub, p, dec->tc_actd));
+        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_O, m.o, nullptr, d, d, rows, p, dec->tc_actd));
         // cross-attention block
         AED_TRY(gamma_planes(w.ln2_g, stats + stats_stride, hid, F));
         p = sg::StepGemmParams{};
         p.out = qc; p.ldo = d;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_QC, m.qc, nullptr, d, d, rows_ub, p, dec->tc_actd));
+        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_QC, m.qc, nullptr, d, d, rows, p, dec->tc_actd));
         if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
             const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
             AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows_ub, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, nullptr,
@@ -1002,12 +1002,12 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         }
         p = sg::StepGemmParams{};
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_o_c;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_OC, m.oc, nullptr, d, d, rows_ub, p, dec->tc_actd));
+        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_OC, m.oc, nullptr, d, d, rows, p, dec->tc_actd));
         // feed-forward block
         AED_TRY(gamma_planes(w.ln3_g, stats + 2 * stats_stride, qkv, 3 * d));
         p = sg::StepGemmParams{};
         p.out = hid; p.ldo = F;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF1, m.ff1, nullptr, F, d, rows_ub, p, dec->tc_actd));
+        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF1, m.ff1, nullptr, F, d, rows, p, dec->tc_actd));
         {
             ProfScope ps(dec, KF_LAYERNORM);
             AED_TRY(launch_pdl(dec, lnrelu_planes_kernel, dim3((F / 4 + 255) / 256, rows_ub), dim3(256), (const DecState *)dec->state(),
@@ -1015,7 +1015,7 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         }
         p = sg::StepGemmParams{};
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_ff2;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF2, m.ff2, nullptr, d, F, rows_ub, p, dec->tc_actf));
+        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF2, m.ff2, nullptr, d, F, rows, p, dec->tc_actf));
     }
     AED_TRY(launch_ln_planes(dec, rows_ub, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
     tc::TcParams tp{};

@@ -1052,7 +1052,7 @@ aed_status_t precompute_tc(aed_dec *dec, const void *enc_base, long long enc_row
     p.state = dec->state();
     const long long tiles = (long long)((segs.tile0[segs.n] + 1) / 2) * c.n_layers * ((2 * c.d_model + ckv::kTileN - 1) / ckv::kTileN);
     ProfScope ps(dec, KF_PRECOMPUTE);
-    const unsigned grid = (unsigned)std::min<long long>(tiles, dec->sm_count);
+    const unsigned grid = 2 * (unsigned)std::min<long long>(tiles, dec->sm_count / 2);
     const size_t smem = ckv::kStages * ckv::kStageBytes + 1024;
     if (c.cross_kv_format == AED_CROSS_KV_E4M3)
         ckv::crosskv_gemm_kernel<true><<<grid, ckv::kCkvThreads, smem, dec->stream>>>(map_enc, dec->at<CUtensorMap>(L.ckv_maps), p);

@@ -778,7 +778,35 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
 // A prefill pass (several prompt positions per utterance, rows = (utterance, position) pairs): the row table and the
 // rows' tokens are already in place; keys and values are appended by a kernel of their own before any row attends; only
 // the last chunk projects to the vocabulary, and only for the rows of the last position (rows 0 .. batch - 1).
+//
+// In the last layer the rows of earlier positions are done once their keys and values are in the cache: the rest of it
+// runs for the rows of the last position only, or not at all before the last chunk.
 struct PrefillPass { bool last_chunk; int batch; };
+
+// Self-attention of a layer over raw [q | k | v] rows; a step appends the new position in the same launch, a prefill
+// pass in one before it, because there a row reads positions that other rows append.  rows_out: rows that attend.
+aed_status_t launch_self_attention(aed_dec *dec, int rows_ub, int rows_out, int self_len_ub, __nv_bfloat16 *self_cache, float *out, __nv_bfloat16 *out_hi,
+                                   __nv_bfloat16 *out_lo, const float2 *stats, const float *c1, const float *c2, bool prefill)
+{
+    typedef __nv_bfloat16 T;
+    const auto &c = dec->cfg;
+    const float *qkv = dec->at<float>(dec->lay.qkv);
+    const int d = c.d_model;
+    if (!prefill)
+        return launch_attention_fused<T, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, out, out_hi, out_lo, stats, c1,
+                                                      c2, dec->use_pdl);
+    {
+        ProfScope ps(dec, KF_ATTN_SELF);
+        const DecState *state = dec->state();
+        const int4 *ri = dec->at<int4>(dec->lay.row_info);
+        int ldq = 3 * d, heads = c.n_heads, cap = c.max_dec_len;
+        void *args[] = {&state, &ri, &qkv, &ldq, &self_cache, &heads, &cap, &stats, &c1, &c2};
+        AED_TRY(launch_pdl_impl(dec, (const void *)append_kv_kernel<T>, dim3(rows_ub, c.n_heads), dim3(kHeadDim), 0, args));
+    }
+    if (rows_out == 0) return AED_OK;
+    return launch_attention_fused<T, false, false>(dec, rows_out, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, out, out_hi, out_lo, stats, c1, c2,
+                                                   dec->use_pdl);
+}
 
 aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out,
                                 const PrefillPass *pf = nullptr)
@@ -812,6 +840,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         if (pf) AED_LAUNCHED(dec);
     }
     const bool pdl = dec->use_pdl;
+    int rows = rows_ub;
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerWeights &w = dec->layers[l];
         const aed_dec::TcLayerMaps &m = dec->tc_layers[l];
@@ -835,23 +864,9 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         if (l == c.n_layers - 1) { p.prefetch2_ptr = dec->w_out; p.prefetch2_bytes = (size_t)V * d * e2; }
         AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, dec->tc_src_x, 3 * d, d, rows_ub, p, nullptr, &m.qc, d));
         // 2. self-attention (applies LN1 to q, k, v; appends k, v)
-        if (pf) {
-            {
-                ProfScope ps(dec, KF_ATTN_SELF);
-                const DecState *state = dec->state();
-                const int4 *ri = dec->at<int4>(L.row_info);
-                const float *qp = qkv;
-                int ldq = 3 * d, heads = c.n_heads, cap = c.max_dec_len;
-                const float2 *stp = stats;
-                void *args[] = {&state, &ri, &qp, &ldq, &self_cache, &heads, &cap, &stp, &c1_qkv, &c2_qkv};
-                AED_TRY(launch_pdl_impl(dec, (const void *)append_kv_kernel<T>, dim3(rows_ub, c.n_heads), dim3(kHeadDim), 0, args));
-            }
-            AED_TRY((launch_attention_fused<T, false, false>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, att,
-                                                             nullptr, nullptr, stats, c1_qkv, c2_qkv, pdl)));
-        } else {
-            AED_TRY((launch_attention_fused<T, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, att,
-                                                            nullptr, nullptr, stats, c1_qkv, c2_qkv, pdl)));
-        }
+        if (pf && l == c.n_layers - 1) rows = pf->last_chunk ? pf->batch : 0;
+        AED_TRY(launch_self_attention(dec, rows_ub, rows, self_len_ub, self_cache, att, nullptr, nullptr, stats, c1_qkv, c2_qkv, pf != nullptr));
+        if (rows == 0) return AED_OK;
         // 3. x += att Wo^T + bo, and in the same launch the rest of the cross-attention query:
         //    (gamma2 * x_new) Wqc^T = q'A + att (Wqc diag(gamma2) Wo)^T + Wqc (gamma2 * bo), so the query projection does
         //    not wait for the sum over all features of x_new ; side: clear the FFN hidden rows
@@ -862,14 +877,14 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.zero_buf = hid; p.zero_cols = F;
         p.prefetch_ptr = wn.w_o; p.prefetch_bytes = (size_t)d * d * e2;
         p.prefetch2_ptr = dec->at<T>(L.comp_w) + (size_t)((l + 1) % c.n_layers) * d * d; p.prefetch2_bytes = (size_t)d * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_O, m.o, dec->tc_src_att, d, d, rows_ub, p, nullptr, &m.o_qc, d));
+        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_O, m.o, dec->tc_src_att, d, d, rows, p, nullptr, &m.o_qc, d));
         // 4. cross-attention; every block computes the LN2 statistics of its row of x_new itself
         if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
             const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
-            AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows_ub, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, att,
+            AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, att,
                                                                   nullptr, nullptr, nullptr, c1_qc, c2_qc, pdl, x)));
         } else {
-            AED_TRY((launch_attention_fused<T, true, false>(dec, rows_ub, c.max_enc_len, qc, d, cross, c.max_total_enc_frames, att,
+            AED_TRY((launch_attention_fused<T, true, false>(dec, rows, c.max_enc_len, qc, d, cross, c.max_total_enc_frames, att,
                                                             nullptr, nullptr, nullptr, c1_qc, c2_qc, pdl, x)));
         }
         // 5. x += att Woc^T + boc ; side: clear the [q | k | v] rows for the next layer
@@ -878,24 +893,23 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_o_c;
         p.zero_buf = qkv; p.zero_cols = 3 * d;
         p.prefetch_ptr = wn.w_o_c; p.prefetch_bytes = (size_t)d * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_OC, m.oc, dec->tc_src_att, d, d, rows_ub, p));
+        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_OC, m.oc, dec->tc_src_att, d, d, rows, p));
         // 6. hidden raw = (gamma3 * x) W1^T ; side: LN3 statistics
         p = sg::StepGemmParams{};
         p.src = x; p.ld_src = d; p.gamma = (const T *)w.ln3_g;
         p.out = hid; p.ldo = F;
         p.stats_src = x; p.stats_out = stats + 2 * stats_stride; p.stats_d = d;
         p.prefetch_ptr = wn.w_ff1; p.prefetch_bytes = (size_t)F * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_FF1, m.ff1, dec->tc_src_x, F, d, rows_ub, p));
+        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_FF1, m.ff1, dec->tc_src_x, F, d, rows, p));
         // 7. x += relu(LN3-corrected hidden) W2^T + b2 ; side: clear the cross-query rows
         p = sg::StepGemmParams{};
         p.src = hid; p.ld_src = F; p.c1 = c1_ff; p.c2 = c2_ff; p.stats_in = stats + 2 * stats_stride;
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_ff2;
         p.zero_buf = qc; p.zero_cols = d;          // the next layer's first launch accumulates into it
         p.prefetch_ptr = wn.w_ff2; p.prefetch_bytes = (size_t)F * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_LN_RELU>(dec, KF_GEMM_FF2, m.ff2, dec->tc_src_hid, d, F, rows_ub, p));
+        AED_TRY(launch_step_gemm<sg::B_LN_RELU>(dec, KF_GEMM_FF2, m.ff2, dec->tc_src_hid, d, F, rows, p));
     }
-    if (pf && !pf->last_chunk) return AED_OK;
-    if (!pf && dec->use_gemv && rows_ub <= vg::kVgRows && d % 128 == 0 && vg::vg_smem(d) <= 227 * 1024) {
+    if (!pf && dec->use_gemv && rows <= vg::kVgRows && d % 128 == 0 && vg::vg_smem(d) <= 227 * 1024) {
         // at most 16 rows: final LayerNorm, vocabulary projection and argmax keys in one kernel (vocab_gemv.cuh)
         ProfScope ps(dec, KF_GEMM_VOCAB + KF_COUNT * KV_GEMV);
         vg::VocabGemvParams vp{};
@@ -911,13 +925,13 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         return launch_pdl_impl(dec, (const void *)vg::vocab_gemv_kernel, dim3((V + tc::kTileM - 1) / tc::kTileM), dim3(vg::kVgThreads),
                                (size_t)vg::vg_smem(d), args);
     }
-    AED_TRY(launch_ln_planes(dec, rows_ub, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
+    AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
     tc::TcParams tp{};
     tp.bias = (const T *)dec->b_out;
     tp.logits_out = logits_out;
     tp.keys = dec->at<unsigned long long>(L.keys);
     tp.active_list = active_list;
-    AED_TRY(launch_vocab_gemm(dec, pf ? pf->batch : rows_ub, tp, pf ? pf->batch : -1));
+    AED_TRY(launch_vocab_gemm(dec, rows, tp, pf ? rows : -1));
     return AED_OK;
 }
 
@@ -945,7 +959,8 @@ aed_status_t launch_pdl(aed_dec *dec, K kernel, dim3 grid, dim3 block, Args... a
     return AED_OK;
 }
 
-aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out)
+aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out,
+                                 const PrefillPass *pf = nullptr)
 {
     typedef __nv_bfloat16 T;
     const auto &c = dec->cfg;
@@ -958,15 +973,20 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
     const int32_t *active_list = dec->at<int32_t>(L.active_list), *t_u = dec->at<int32_t>(L.t_u);
     {
         ProfScope ps(dec, KF_EMBED);
-        embed_kernel<T><<<rows_ub, 256, 0, dec->stream>>>(dec->state(), active_list, tokens, t_u, (const T *)dec->embed,
-                                                          dec->at<float>(L.pe), d, V, sqrtf((float)d), x, qkv, 3 * d);
+        if (pf)
+            embed_rows_kernel<T><<<rows_ub, 256, 0, dec->stream>>>(dec->state(), dec->at<int4>(L.row_info), dec->at<int32_t>(L.row_tok), (const T *)dec->embed,
+                                                                   dec->at<float>(L.pe), d, V, sqrtf((float)d), x, qkv, 3 * d);
+        else
+            embed_kernel<T><<<rows_ub, 256, 0, dec->stream>>>(dec->state(), active_list, tokens, t_u, (const T *)dec->embed,
+                                                              dec->at<float>(L.pe), d, V, sqrtf((float)d), x, qkv, 3 * d);
         AED_LAUNCHED(dec);
     }
     const bool pdl = dec->use_pdl;
+    int rows = rows_ub;
     const dim3 ln_block(d <= 2048 ? 256 : 1024);
     auto gamma_planes = [&](const void *g, float2 *st, float *zero_buf, int zero_cols) -> aed_status_t {
         ProfScope ps(dec, KF_LAYERNORM);
-        return launch_pdl(dec, gamma_planes_kernel<8>, dim3(rows_ub), ln_block, (const DecState *)dec->state(), (const float *)x,
+        return launch_pdl(dec, gamma_planes_kernel<8>, dim3(rows), ln_block, (const DecState *)dec->state(), (const float *)x,
                           (const T *)g, d, c.ln_eps, st, ad_hi, ad_lo, zero_buf, zero_cols);
     };
     for (int l = 0; l < c.n_layers; ++l) {
@@ -982,8 +1002,9 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         AED_TRY(gamma_planes(w.ln1_g, stats, qc, d));
         p.out = qkv; p.ldo = 3 * d;
         AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_QKV, m.qkv, nullptr, 3 * d, d, rows_ub, p, dec->tc_actd));
-        AED_TRY((launch_attention_fused<T, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, nullptr,
-                                                        ad_hi, ad_lo, stats, c1_qkv, c2_qkv, pdl)));
+        if (pf && l == c.n_layers - 1) rows = pf->last_chunk ? pf->batch : 0;
+        AED_TRY(launch_self_attention(dec, rows_ub, rows, self_len_ub, self_cache, nullptr, ad_hi, ad_lo, stats, c1_qkv, c2_qkv, pf != nullptr));
+        if (rows == 0) return AED_OK;
         p = sg::StepGemmParams{};
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_o;
         AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_O, m.o, nullptr, d, d, rows, p, dec->tc_actd));
@@ -994,10 +1015,10 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_QC, m.qc, nullptr, d, d, rows, p, dec->tc_actd));
         if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
             const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
-            AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows_ub, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, nullptr,
+            AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, nullptr,
                                                                   ad_hi, ad_lo, stats + stats_stride, c1_qc, c2_qc, pdl)));
         } else {
-            AED_TRY((launch_attention_fused<T, true, false>(dec, rows_ub, c.max_enc_len, qc, d, cross, c.max_total_enc_frames, nullptr,
+            AED_TRY((launch_attention_fused<T, true, false>(dec, rows, c.max_enc_len, qc, d, cross, c.max_total_enc_frames, nullptr,
                                                             ad_hi, ad_lo, stats + stats_stride, c1_qc, c2_qc, pdl)));
         }
         p = sg::StepGemmParams{};
@@ -1010,20 +1031,20 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF1, m.ff1, nullptr, F, d, rows, p, dec->tc_actd));
         {
             ProfScope ps(dec, KF_LAYERNORM);
-            AED_TRY(launch_pdl(dec, lnrelu_planes_kernel, dim3((F / 4 + 255) / 256, rows_ub), dim3(256), (const DecState *)dec->state(),
+            AED_TRY(launch_pdl(dec, lnrelu_planes_kernel, dim3((F / 4 + 255) / 256, rows), dim3(256), (const DecState *)dec->state(),
                                (const float *)hid, F, (const float2 *)(stats + 2 * stats_stride), c1_ff, c2_ff, af_hi, af_lo));
         }
         p = sg::StepGemmParams{};
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_ff2;
         AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF2, m.ff2, nullptr, d, F, rows, p, dec->tc_actf));
     }
-    AED_TRY(launch_ln_planes(dec, rows_ub, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
+    AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
     tc::TcParams tp{};
     tp.bias = (const T *)dec->b_out;
     tp.logits_out = logits_out;
     tp.keys = dec->at<unsigned long long>(L.keys);
     tp.active_list = active_list;
-    AED_TRY(launch_vocab_gemm(dec, rows_ub, tp));
+    AED_TRY(launch_vocab_gemm(dec, rows, tp, pf ? rows : -1));
     return AED_OK;
 }
 
@@ -1301,7 +1322,8 @@ extern "C" aed_status_t aed_dec_prefill(aed_dec_t *dec, const int32_t *prompt, i
             AED_LAUNCHED(dec);
         }
         PrefillPass pf{last, B};
-        AED_TRY(forward_step_fused(dec, rows, j0 + chunk, nullptr, logits_out, &pf));
+        AED_TRY(rows > dec->planes_rows ? forward_step_planes(dec, rows, j0 + chunk, nullptr, logits_out, &pf)
+                                        : forward_step_fused(dec, rows, j0 + chunk, nullptr, logits_out, &pf));
         {
             ProfScope ps(dec, KF_BOOKKEEPING);
             DecState *state = dec->state();

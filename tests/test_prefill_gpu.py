@@ -55,6 +55,13 @@ def test_prefill_matches_the_checker(prompt_len, max_batch):
         dec.close()
 
 
+@pytest.mark.parametrize("prompt_len,max_batch", [(24, 144), (40, 180), (60, 400)])
+def test_prefill_with_many_rows(prompt_len, max_batch):
+    """More than 128 (utterance, position) rows, where the pass takes ready-made activation planes: 144 rows, 180 rows
+    and then a chunk of 60 that does not, and 360 rows, whose self-attention takes a warp per (row, head)."""
+    test_prefill_matches_the_checker(prompt_len, max_batch)
+
+
 def test_prefill_argument_errors():
     import torch
     from paper_2503_05931_b200 import binding

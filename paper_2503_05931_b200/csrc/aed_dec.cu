@@ -130,10 +130,10 @@ Layout make_layout(const aed_dec_config_t &c)
     L.cur_tok = take(B * 4);
     L.enc_off = take((B + 1) * 4);
     L.enc_len = take(B * 4);
+    L.len_order = take(B * 4);                                     // utterances by decreasing encoder length (offsets, lengths and order: one copy)
     L.max_len = take(B * 4);
     L.row_info = take((size_t)rows_bucket(c.max_batch) * 16);      // grids are sized for the bucket
     L.row_tok = take((size_t)rows_bucket(c.max_batch) * 4);        // prefill: the token of every (utterance, position) row
-    L.len_order = take(B * 4);                                     // utterances by decreasing encoder length
     L.rows_cap = (int)align_up(B, 16);
     L.slot_tokens = take(B * (size_t)c.max_dec_len * 4);
     L.slot_lens = take(B * 4);
@@ -176,6 +176,8 @@ struct aed_dec {
     std::vector<int32_t> enc_len, enc_off;
     // continuous batching: the batch is a set of slots that utterances enter and leave one by one
     bool slot_mode = false;
+    bool rows_ready = false;        // slots: the row table of the next step is in place ...
+    const void *rows_tokens = nullptr, *rows_lens = nullptr;      // ... and these are the results' places it noted
     std::vector<int32_t> slot_t, slot_max;      // steps issued since the slot's utterance entered (-1: empty), its forced length
     std::string err;
     int64_t launches = 0;
@@ -201,7 +203,7 @@ struct aed_dec {
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
     // greedy decoding replays one captured CUDA graph per (row bucket, self-attention chunk count, output buffers)
-    typedef std::tuple<int, int, const void *, const void *> GraphKey;
+    typedef std::tuple<int, int> GraphKey;       // (row count, chunks of self-attention positions)
     struct GraphEntry { cudaGraphExec_t exec; int64_t nodes; };
     std::map<GraphKey, GraphEntry> graphs;
     cudaStream_t capture_stream = nullptr;
@@ -365,8 +367,8 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
 }
 
 // A launch that may start before its predecessor in the stream has ended (programmatic stream serialization): the
-// kernel itself waits (griddepcontrol.wait) before it touches what the predecessor wrote.
-aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 block, size_t smem, void **args)
+// kernel itself waits (griddepcontrol.wait) before it touches what the predecessor wrote.  full: an ordinary dependency.
+aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 block, size_t smem, void **args, bool full = false)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -375,7 +377,7 @@ aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 b
     cfg.stream = dec->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl && !full ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, args);
@@ -394,7 +396,7 @@ aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 b
 // 8-row tiles: as many warps as features, because a launch is bound by its latency.  Beyond, two features per warp halve the
 // shared-memory reads per FMA.  Small outputs take 4 warps per block, so that they still spread over 64 SMs and more.
 template <int EPI>
-aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p)
+aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, bool after_rows = false)
 {
     ProfScope ps(dec, family);
     const int warps = p.M <= 512 ? 4 : f32::kWarps;
@@ -402,9 +404,9 @@ aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p)
     p.eps = dec->cfg.ln_eps;
     void *args[] = {&p};
     auto grid = [&](int rt, int fpw) { return dim3((p.M + warps * fpw - 1) / (warps * fpw), (rows_ub + rt - 1) / rt); };
-    if (rows_ub <= 4) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 4, 1>, grid(4, 1), dim3(warps * 32), f32::rows_smem(4, p.K), args);
-    if (rows_ub <= 16) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 1>, grid(8, 1), dim3(warps * 32), f32::rows_smem(8, p.K), args);
-    return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 2>, grid(8, 2), dim3(warps * 32), f32::rows_smem(8, p.K), args);
+    if (rows_ub <= 4) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 4, 1>, grid(4, 1), dim3(warps * 32), f32::rows_smem(4, p.K), args, after_rows);
+    if (rows_ub <= 16) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 1>, grid(8, 1), dim3(warps * 32), f32::rows_smem(8, p.K), args, after_rows);
+    return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 2>, grid(8, 2), dim3(warps * 32), f32::rows_smem(8, p.K), args, after_rows);
 }
 
 // The forward pass of one step in fp32 for the rows in the active list (at most rows_ub of them): 8 kernels per layer, chained
@@ -419,7 +421,8 @@ aed_status_t forward_step_f32(aed_dec *dec, int rows_ub, int self_len_ub, const 
     float *x = dec->at<float>(L.x), *act = dec->at<float>(L.act), *qkv = dec->at<float>(L.qkv), *hid = dec->at<float>(L.hid), *none = nullptr;
     const int32_t *active_list = dec->at<int32_t>(L.active_list), *t_u = dec->at<int32_t>(L.t_u);
     const bool split = dec->partials_override != nullptr;        // aed_dec_step_static_scratch: attention split over chunks, with its scratch
-    {
+    const bool embedded = rows_ub <= kRowsInside;          // by the kernel that made the row table
+    if (!embedded) {
         ProfScope ps(dec, KF_EMBED);
         const DecState *state = dec->state();
         const float *emb = (const float *)dec->embed, *pe = dec->at<float>(L.pe);
@@ -440,7 +443,7 @@ aed_status_t forward_step_f32(aed_dec *dec, int rows_ub, int self_len_ub, const 
         float *self_cache = dec->at<float>(L.self_cache) + (size_t)l * L.self_layer_elems;
         const float *cross = dec->at<float>(L.cross_store) + (size_t)l * L.cross_layer_elems;
         // masked self-attention (which appends the new keys and values)
-        AED_TRY(launch_f32<f32::EPI_STORE>(dec, KF_GEMM_QKV, rows_ub, rows(x, w.ln1_g, w.ln1_b, w.w_qkv, w.b_qkv, 3 * d, d, qkv, 3 * d)));
+        AED_TRY(launch_f32<f32::EPI_STORE>(dec, KF_GEMM_QKV, rows_ub, rows(x, w.ln1_g, w.ln1_b, w.w_qkv, w.b_qkv, 3 * d, d, qkv, 3 * d), embedded && l == 0));
         if (split) AED_TRY((launch_attention<float, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, act)));
         else AED_TRY((launch_attention_fused<float, false, true>(dec, rows_ub, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, act, nullptr, nullptr, nullptr,
                                                                  nullptr, nullptr, dec->use_pdl)));
@@ -654,8 +657,6 @@ aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int ro
                            (size_t)stages * stage_bytes + 1024, args);
 }
 
-aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 block, size_t smem, void **args);
-
 aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const void *g, const void *b, float *zero_buf,
                               int zero_cols)
 {
@@ -680,8 +681,10 @@ struct FusedGemm {
 template <int MODE>
 aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, const CUtensorMap *src_maps, int M,
                               int K, int rows_ub, sg::StepGemmParams p, const CUtensorMap (*plane_maps)[2] = nullptr,
-                              const CUtensorMap *map_w2 = nullptr, int M2 = 0)
+                              const CUtensorMap *map_w2 = nullptr, int M2 = 0, bool after_rows = false)
 {
+    // after_rows: the kernel before this launch made the row table, which the kernels of a step read ahead of their
+    // dependency waits: a full dependency, no programmatic one
     // map_w2, M2: a second weight matrix [M2, K] over the same rows (its output, gamma and bias are in p)
     // plane_maps (B_PLANES only): [N/16 - 1][high, low] tensor maps of the ready-made activation planes
     // Rows per CTA tile: up to 128 (two ring stages still fit beside the transposition buffer); more rows are
@@ -739,7 +742,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
             gc.stream = dec->stream;
             cudaLaunchAttribute ga[1];
             ga[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            ga[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
+            ga[0].val.programmaticStreamSerializationAllowed = dec->use_pdl && !after_rows ? 1 : 0;
             gc.attrs = ga;
             gc.numAttrs = 1;
             const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
@@ -761,7 +764,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     cfg.stream = dec->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl && !after_rows ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     // the accumulator is transposed through the ring's memory before it leaves: n_tile rows of 132 floats
@@ -820,7 +823,8 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
     float2 *stats = dec->at<float2>(L.ln_stats);
     const int stats_stride = rows_bucket(c.max_batch);
     const int32_t *active_list = dec->at<int32_t>(L.active_list), *t_u = dec->at<int32_t>(L.t_u);
-    {
+    const bool embedded = !pf && rows_ub <= kRowsInside;   // by the kernel that made the row table
+    if (!embedded) {
         ProfScope ps(dec, KF_EMBED);
         if (pf)
             embed_rows_kernel<T><<<rows_ub, 256, 0, dec->stream>>>(dec->state(), dec->at<int4>(L.row_info), dec->at<int32_t>(L.row_tok),
@@ -862,7 +866,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.prefetch2_ptr = wn.w_q_c; p.prefetch2_bytes = (size_t)d * d * e2;
         // the vocabulary matrix is as large as a layer: its way into L2 starts a whole layer ahead of the projection
         if (l == c.n_layers - 1) { p.prefetch2_ptr = dec->w_out; p.prefetch2_bytes = (size_t)V * d * e2; }
-        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, dec->tc_src_x, 3 * d, d, rows_ub, p, nullptr, &m.qc, d));
+        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, dec->tc_src_x, 3 * d, d, rows_ub, p, nullptr, &m.qc, d, embedded && l == 0));
         // 2. self-attention (applies LN1 to q, k, v; appends k, v)
         if (pf && l == c.n_layers - 1) rows = pf->last_chunk ? pf->batch : 0;
         AED_TRY(launch_self_attention(dec, rows_ub, rows, self_len_ub, self_cache, att, nullptr, nullptr, stats, c1_qkv, c2_qkv, pf != nullptr));
@@ -1108,33 +1112,67 @@ aed_status_t precompute_f32(aed_dec *dec, const void *enc_packed, int frames, in
     return AED_OK;
 }
 
-aed_status_t launch_build_active(aed_dec *dec, const uint8_t *mask)
+// The row table of the next step (step_rows_kernel): after the bookkeeping of a greedy step that ends (finish), or on its
+// own before the first one and before every step of the caller's loop.
+template <typename T>
+aed_status_t launch_step_rows_t(aed_dec *dec, bool finish, const uint8_t *mask, const int32_t *tokens, bool clear, int32_t *tokens_out, int32_t *out_lens)
 {
+    const auto &c = dec->cfg;
     const Layout &L = dec->lay;
+    StepRowsArgs<T> a{};
+    a.state = dec->state();
+    a.mask = mask; a.tokens = tokens;
+    a.t_u = dec->at<int32_t>(L.t_u); a.retired = dec->at<int32_t>(L.retired); a.active_list = dec->at<int32_t>(L.active_list);
+    a.max_dec_len = c.max_dec_len;
+    a.enc_len = dec->at<int32_t>(L.enc_len); a.enc_off = dec->at<int32_t>(L.enc_off); a.order = dec->at<int32_t>(L.len_order);
+    a.row_info = dec->at<int4>(L.row_info); a.row_slots = rows_bucket(c.max_batch);
+    a.embed = (const T *)dec->embed; a.pe = dec->at<float>(L.pe); a.d = c.d_model; a.vocab = c.vocab; a.scale = sqrtf((float)c.d_model);
+    a.x = dec->at<float>(L.x);
+    if (clear && dec->use_tc) {
+        a.zero_buf = dec->at<float>(L.qkv); a.zero_cols = 3 * c.d_model;
+        a.zero_buf2 = dec->at<float>(L.qc); a.zero_cols2 = c.d_model;
+    }
+    a.keys = dec->at<unsigned long long>(L.keys); a.cur_tok = dec->at<int32_t>(L.cur_tok); a.max_len = dec->at<int32_t>(L.max_len); a.eos_id = c.eos_id;
+    a.tokens_out = tokens_out; a.out_lens = out_lens;
+    void *args[] = {&a};
     ProfScope ps(dec, KF_BOOKKEEPING);
-    build_active_kernel<<<1, 1024, 0, dec->stream>>>(mask, dec->at<int32_t>(L.retired),
-                                                     dec->at<int32_t>(L.t_u), dec->cfg.max_dec_len,
-                                                     dec->at<int32_t>(L.active_list), dec->state(),
-                                                     dec->at<int32_t>(L.enc_len), dec->at<int32_t>(L.enc_off),
-                                                     dec->at<int4>(L.row_info), rows_bucket(dec->cfg.max_batch),
-                                                     dec->at<int32_t>(L.len_order));
-    AED_LAUNCHED(dec);
-    return AED_OK;
+    return launch_pdl_impl(dec, finish ? (const void *)step_rows_kernel<T, true> : (const void *)step_rows_kernel<T, false>, dim3(1), dim3(1024), 0, args, !finish);
+}
+aed_status_t launch_step_rows(aed_dec *dec, bool finish, const uint8_t *mask, const int32_t *tokens, bool clear, int32_t *tokens_out = nullptr,
+                              int32_t *out_lens = nullptr)
+{
+    return dec->use_tc ? launch_step_rows_t<__nv_bfloat16>(dec, finish, mask, tokens, clear, tokens_out, out_lens)
+                       : launch_step_rows_t<float>(dec, finish, mask, tokens, clear, tokens_out, out_lens);
 }
 
-aed_status_t launch_finish(aed_dec *dec, int rows_ub, int32_t *next_out, int greedy, int32_t *tokens_out,
-                           int32_t *out_lens)
+aed_status_t launch_finish(aed_dec *dec, int rows_ub, int32_t *next_out)
 {
     const Layout &L = dec->lay;
     ProfScope ps(dec, KF_BOOKKEEPING);
     DecState *state = dec->state();
     const int32_t *active_list = dec->at<int32_t>(L.active_list);
     unsigned long long *keys = dec->at<unsigned long long>(L.keys);
-    int32_t *t_u = dec->at<int32_t>(L.t_u), *cur_tok = dec->at<int32_t>(L.cur_tok), *retired = dec->at<int32_t>(L.retired);
-    const int32_t *max_len = dec->at<int32_t>(L.max_len);
-    int eos = dec->cfg.eos_id, ld = dec->cfg.max_dec_len;
-    void *args[] = {&state, &active_list, &keys, &t_u, &next_out, &greedy, &cur_tok, &retired, &max_len, &eos, &tokens_out, &ld, &out_lens};
+    int32_t *t_u = dec->at<int32_t>(L.t_u);
+    void *args[] = {&state, &active_list, &keys, &t_u, &next_out};
     return launch_pdl_impl(dec, (const void *)finish_step_kernel, dim3((rows_ub + 127) / 128), dim3(128), 0, args);
+}
+
+// A new batch (or set of slots): lengths, offsets and visiting order in one copy, cleared bookkeeping in one kernel.
+aed_status_t begin_batch(aed_dec *dec, const std::vector<int32_t> &order)
+{
+    const Layout &L = dec->lay;
+    const size_t batch = dec->batch, at_len = (L.enc_len - L.enc_off) / 4, at_order = (L.len_order - L.enc_off) / 4;
+    std::vector<int32_t> host(at_order + batch);
+    std::copy(dec->enc_off.begin(), dec->enc_off.end(), host.begin());
+    std::copy(dec->enc_len.begin(), dec->enc_len.end(), host.begin() + at_len);
+    std::copy(order.begin(), order.end(), host.begin() + at_order);
+    // Pageable host memory: cudaMemcpyAsync stages it before returning.
+    AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.enc_off, host.data(), host.size() * 4, cudaMemcpyHostToDevice, dec->stream));
+    ProfScope ps(dec, KF_BOOKKEEPING);
+    begin_batch_kernel<<<1, 1024, 0, dec->stream>>>(dec->at<int4>(L.keys), (int)((L.enc_off - L.keys) / 16), dec->state(), dec->batch);      // keys, state, t_u, retired, lists
+    AED_LAUNCHED(dec);
+    dec->rows_ready = false;
+    return AED_OK;
 }
 
 aed_status_t fill_i32(aed_dec *dec, int32_t *p, int32_t v, size_t n)
@@ -1238,7 +1276,6 @@ extern "C" aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *
     if (total > dec->cfg.max_total_enc_frames)
         return fail(dec, AED_ERR_CAPACITY, "%lld encoder frames exceed max_total_enc_frames %d", total, dec->cfg.max_total_enc_frames);
 
-    const Layout &L = dec->lay;
     std::vector<int32_t> off(batch + 1, 0);
     for (int u = 0; u < batch; ++u) off[u + 1] = off[u] + enc_lens[u];
     // From here on the old batch is gone.
@@ -1247,18 +1284,13 @@ extern "C" aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *
     dec->enc_off = off;
     dec->batch = batch;
     dec->total_frames = (int)total;
-    // Pageable host vectors: cudaMemcpyAsync stages them before returning, so the vectors may change afterwards.
-    AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.enc_off, dec->enc_off.data(), (batch + 1) * 4, cudaMemcpyHostToDevice, dec->stream));
-    AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.enc_len, dec->enc_len.data(), batch * 4, cudaMemcpyHostToDevice, dec->stream));
     {
         // visiting order of the row compaction: longest encoder output first (ties by utterance index)
         std::vector<int32_t> order(batch);
         for (int u = 0; u < batch; ++u) order[u] = u;
         std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return enc_lens[a] > enc_lens[b]; });
-        AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.len_order, order.data(), batch * 4, cudaMemcpyHostToDevice, dec->stream));
+        AED_TRY(begin_batch(dec, order));
     }
-    AED_CUDA(dec, cudaMemsetAsync(dec->ws + L.keys, 0, L.enc_off - L.keys, dec->stream));   // keys, state, t_u, retired, lists
-    AED_CUDA(dec, cudaMemcpyAsync(&dec->state()->batch, &dec->batch, sizeof(int32_t), cudaMemcpyHostToDevice, dec->stream));
     dec->slot_mode = false;
     aed_status_t s = dec->use_tc ? precompute_tc(dec, enc_packed, dec->total_frames, one_run(dec->total_frames, 0))
                                  : precompute_f32(dec, enc_packed, dec->total_frames, 0);
@@ -1279,14 +1311,14 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
     if (dec->slot_mode) return fail(dec, AED_ERR_STATE, "aed_dec_step does not run on slots: use aed_dec_greedy_steps");
     if (dec->full_steps >= dec->cfg.max_dec_len)
         return fail(dec, AED_ERR_CAPACITY, "every utterance already holds max_dec_len = %d tokens", dec->cfg.max_dec_len);
-    AED_TRY(launch_build_active(dec, active));
+    AED_TRY(launch_step_rows(dec, false, active, tokens_in, true));
     const int rows_ub = dec->batch;
     const int self_len_ub = dec->steps_issued + 1 < dec->cfg.max_dec_len ? dec->steps_issued + 1 : dec->cfg.max_dec_len;
     aed_status_t s = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tokens_in, logits_out)
                      : rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tokens_in, logits_out)
                                                   : forward_step_fused(dec, rows_ub, self_len_ub, tokens_in, logits_out);
     if (s != AED_OK) return s;
-    AED_TRY(launch_finish(dec, rows_ub, next_out, 0, nullptr, nullptr));
+    AED_TRY(launch_finish(dec, rows_ub, next_out));
     dec->steps_issued++;
     if (!active) dec->full_steps++;
     dec->fresh_batch = false;
@@ -1398,22 +1430,23 @@ extern "C" aed_status_t aed_dec_step_static_scratch(aed_dec_t *dec, const int32_
 
 namespace {
 
-aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, int32_t *tokens_out, int32_t *out_lens)
+// One greedy step whose row table is in place, and the row table of the next one.
+aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub)
 {
     const Layout &L = dec->lay;
     if (self_len_ub > dec->cfg.max_dec_len) self_len_ub = dec->cfg.max_dec_len;
-    AED_TRY(launch_build_active(dec, nullptr));
     const int32_t *tok = dec->at<int32_t>(L.cur_tok);
+    const bool planes = dec->use_tc && rows_ub > dec->planes_rows;
     aed_status_t st = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tok, nullptr)
-                      : rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tok, nullptr)
-                                                   : forward_step_fused(dec, rows_ub, self_len_ub, tok, nullptr);
+                      : planes     ? forward_step_planes(dec, rows_ub, self_len_ub, tok, nullptr)
+                                   : forward_step_fused(dec, rows_ub, self_len_ub, tok, nullptr);
     if (st != AED_OK) return st;
-    return launch_finish(dec, rows_ub, nullptr, 1, tokens_out, out_lens);
+    // (the side jobs of the few-row projections leave the accumulators clear for the next step, the planes path does not)
+    return launch_step_rows(dec, true, nullptr, tok, planes);
 }
 
 // Record one greedy step into a graph on the library's capture stream (nothing runs) and instantiate it.
-aed_status_t capture_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, int32_t *tokens_out, int32_t *out_lens,
-                                 aed_dec::GraphEntry *entry)
+aed_status_t capture_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, aed_dec::GraphEntry *entry)
 {
     if (!dec->capture_stream)
         AED_CUDA(dec, cudaStreamCreateWithFlags(&dec->capture_stream, cudaStreamNonBlocking));
@@ -1421,7 +1454,7 @@ aed_status_t capture_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, int
     const int64_t before = dec->launches;
     AED_CUDA(dec, cudaStreamBeginCapture(dec->capture_stream, cudaStreamCaptureModeThreadLocal));
     dec->stream = dec->capture_stream;
-    aed_status_t st = enqueue_greedy_step(dec, rows_ub, self_len_ub, tokens_out, out_lens);
+    aed_status_t st = enqueue_greedy_step(dec, rows_ub, self_len_ub);
     dec->stream = user;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(dec->capture_stream, &graph);
@@ -1458,9 +1491,13 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
 
     dec->fresh_batch = false;
     AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.max_len, max_len, B * 4, cudaMemcpyHostToDevice, dec->stream));
-    AED_TRY(fill_i32(dec, dec->at<int32_t>(L.cur_tok), dec->cfg.bos_id, B));
-    AED_TRY(fill_i32(dec, tokens_out, -1, (size_t)B * dec->cfg.max_dec_len));
-    AED_TRY(fill_i32(dec, out_lens, 0, B));
+    {
+        ProfScope ps(dec, KF_BOOKKEEPING);
+        const size_t n = (size_t)B * dec->cfg.max_dec_len;
+        begin_greedy_kernel<<<(unsigned)((n + 255) / 256), 256, 0, dec->stream>>>(dec->at<int32_t>(L.cur_tok), dec->cfg.bos_id, B, tokens_out, n, out_lens);
+        AED_LAUNCHED(dec);
+    }
+    AED_TRY(launch_step_rows(dec, false, nullptr, dec->at<int32_t>(L.cur_tok), true, tokens_out, out_lens));
     // With an end-of-sequence id the forced lengths are only upper bounds.  The host then stays at most kWindow steps
     // ahead of the device: before it issues step s it looks at the retired count that step s - kWindow left behind
     // (an asynchronous copy into pinned memory followed by an event) and stops once every utterance has retired.
@@ -1480,17 +1517,17 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
         if (dec->use_graphs && !dec->profiling) {
             // grids are sized for the keyed row count; kernels leave rows beyond the device-side row count alone
             const int rows_b = rows_key(rows_ub), chunks = (s + 1 + kAttnChunk - 1) / kAttnChunk;
-            const aed_dec::GraphKey key(rows_b, chunks, tokens_out, out_lens);
+            const aed_dec::GraphKey key(rows_b, chunks);
             auto it = dec->graphs.find(key);
             if (it == dec->graphs.end()) {
                 aed_dec::GraphEntry entry{};
-                AED_TRY(capture_greedy_step(dec, rows_b, chunks * kAttnChunk, tokens_out, out_lens, &entry));
+                AED_TRY(capture_greedy_step(dec, rows_b, chunks * kAttnChunk, &entry));
                 it = dec->graphs.emplace(key, entry).first;
             }
             AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
             dec->launches += it->second.nodes;
         } else {
-            AED_TRY(enqueue_greedy_step(dec, rows_ub, s + 1, tokens_out, out_lens));
+            AED_TRY(enqueue_greedy_step(dec, rows_ub, s + 1));
         }
         dec->steps_issued = s + 1;
         if (probe) {
@@ -1523,15 +1560,11 @@ extern "C" aed_status_t aed_dec_open_slots(aed_dec_t *dec, int32_t slots)
     for (int u = 0; u <= slots; ++u) dec->enc_off[u] = u * c.max_enc_len;       // every slot owns max_enc_len store rows
     dec->slot_t.assign(slots, -1);
     dec->slot_max.assign(slots, 0);
-    AED_CUDA(dec, cudaMemsetAsync(dec->ws + L.keys, 0, L.enc_off - L.keys, dec->stream));   // keys, state, t_u, retired, lists
-    AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.enc_off, dec->enc_off.data(), (slots + 1) * 4, cudaMemcpyHostToDevice, dec->stream));
-    AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.enc_len, dec->enc_len.data(), slots * 4, cudaMemcpyHostToDevice, dec->stream));
     {
         std::vector<int32_t> order(slots);
         for (int u = 0; u < slots; ++u) order[u] = u;
-        AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.len_order, order.data(), slots * 4, cudaMemcpyHostToDevice, dec->stream));
+        AED_TRY(begin_batch(dec, order));
     }
-    AED_CUDA(dec, cudaMemcpyAsync(&dec->state()->batch, &dec->batch, sizeof(int32_t), cudaMemcpyHostToDevice, dec->stream));
     AED_TRY(fill_i32(dec, dec->at<int32_t>(L.retired), 1, slots));      // empty slots take no part in a step
     dec->slot_mode = true;
     dec->have_batch = true;
@@ -1578,6 +1611,7 @@ aed_status_t admit_many(aed_dec *dec, const void *enc_base, long long enc_rows, 
         segs.src0[i] = (int)adm[i].src_row; segs.frames[i] = adm[i].frames; segs.dst0[i] = adm[i].slot * c.max_enc_len;
         ab.slot[i] = adm[i].slot; ab.n_frames[i] = adm[i].frames; ab.frame0[i] = segs.dst0[i]; ab.forced_len[i] = adm[i].max_len;
     }
+    dec->rows_ready = false;
     if (dec->use_tc) {
         AED_TRY(precompute_tc(dec, enc_base, enc_rows, segs));
     } else {
@@ -1627,19 +1661,24 @@ extern "C" aed_status_t aed_dec_greedy_steps(aed_dec_t *dec, int32_t n_steps, in
         for (int u = 0; u < dec->batch; ++u)
             if (dec->slot_t[u] >= 0 && dec->slot_t[u] < dec->slot_max[u]) { ++rows_ub; longest = std::max(longest, dec->slot_t[u] + 1); }
         if (rows_ub == 0) break;
+        if (!dec->rows_ready || dec->rows_tokens != tokens_out || dec->rows_lens != out_lens) {
+            AED_TRY(launch_step_rows(dec, false, nullptr, dec->at<int32_t>(dec->lay.cur_tok), true, tokens_out, out_lens));
+            dec->rows_ready = true;
+            dec->rows_tokens = tokens_out; dec->rows_lens = out_lens;
+        }
         if (dec->use_graphs && !dec->profiling) {
             const int rows_b = rows_key(rows_ub), chunks = (longest + kAttnChunk - 1) / kAttnChunk;
-            const aed_dec::GraphKey key(rows_b, chunks, tokens_out, out_lens);
+            const aed_dec::GraphKey key(rows_b, chunks);
             auto it = dec->graphs.find(key);
             if (it == dec->graphs.end()) {
                 aed_dec::GraphEntry entry{};
-                AED_TRY(capture_greedy_step(dec, rows_b, chunks * kAttnChunk, tokens_out, out_lens, &entry));
+                AED_TRY(capture_greedy_step(dec, rows_b, chunks * kAttnChunk, &entry));
                 it = dec->graphs.emplace(key, entry).first;
             }
             AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
             dec->launches += it->second.nodes;
         } else {
-            AED_TRY(enqueue_greedy_step(dec, rows_ub, longest, tokens_out, out_lens));
+            AED_TRY(enqueue_greedy_step(dec, rows_ub, longest));
         }
         for (int u = 0; u < dec->batch; ++u)
             if (dec->slot_t[u] >= 0 && dec->slot_t[u] < dec->slot_max[u]) ++dec->slot_t[u];

@@ -15,50 +15,132 @@ namespace aed {
 // row, and utterance -1 for the slots past the last row, so that a kernel needs one 16-byte load per row.
 // The batch size is read from the decode state, not passed by value: a captured step graph outlives the batch it
 // was recorded for and is replayed for later batches of other sizes.
-__global__ void build_active_kernel(const uint8_t *__restrict__ mask, const int32_t *__restrict__ retired,
-                                    const int32_t *__restrict__ t_u, int max_dec_len,
-                                    int32_t *__restrict__ active_list, DecState *state,
-                                    const int32_t *__restrict__ enc_len, const int32_t *__restrict__ enc_off,
-                                    int4 *__restrict__ row_info, int row_slots, const int32_t *__restrict__ order)
+//
+// The greedy loop runs this kernel at the end of every step, with the bookkeeping of the step that ends (kFinish): decode
+// the argmax keys, record the token and feed it back, advance t_u, retire finished utterances, and then the rows of the
+// next step.  Steps of at most kRowsInside rows find their embedded rows there as well.  These are chains of dependent
+// loads of a few hundred cycles each, so what matters is the number of launches in a row: one here, where the end of a
+// step, the compaction and the embedding were three, with the boundary between two graphs in the middle.
+// It never lets its successor start early: kernels read the row count and the row table ahead of their dependency wait.
+constexpr int kRowsInside = 8;       // one block embeds these in less than the 2.8 us of another launch
+
+template <typename T>
+struct StepRowsArgs {
+    DecState *state;
+    const uint8_t *mask;                      // by utterance, or null
+    const int32_t *tokens;                    // by utterance: the token that goes into the next step
+    int32_t *t_u, *retired, *active_list;
+    int max_dec_len;
+    const int32_t *enc_len, *enc_off, *order;
+    int4 *row_info;
+    int row_slots;
+    // embedding of up to kRowsInside rows
+    const T *embed;
+    const float *pe;
+    int d, vocab;
+    float scale;
+    float *x, *zero_buf, *zero_buf2;          // rows that the first projection accumulates into, cleared if not null
+    int zero_cols, zero_cols2;
+    // kFinish
+    unsigned long long *keys;
+    int32_t *cur_tok;
+    const int32_t *max_len;
+    int eos_id;
+    // !kFinish: where the greedy steps to come leave their results
+    int32_t *tokens_out, *out_lens;
+};
+
+// One block of 1024 threads.
+template <typename T, bool kFinish>
+__global__ void __launch_bounds__(1024) step_rows_kernel(const __grid_constant__ StepRowsArgs<T> a)
 {
-    AED_TRACE_BEGIN(state, 1);
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the next kernel may become resident; it waits for this one inside
+    AED_TRACE_BEGIN(a.state, 1);
     __shared__ int warp_counts[32];
     __shared__ int base;
-    const int batch = state->batch;
+    __shared__ int4 first[kRowsInside];       // (utterance, t_u, token) of the first rows
+    DecState *const state = a.state;
+    const int batch = state->batch, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (threadIdx.x == 0) base = 0;
+    if (kFinish) {
+        const int n = state->n_active;
+        for (int r = threadIdx.x; r < n; r += blockDim.x) {
+            const int u = a.active_list[r];
+            const int32_t tok = argmax_key_index(a.keys[r]);
+            const int t = a.t_u[u];
+            a.keys[r] = 0ull;
+            a.t_u[u] = t + 1;
+            a.cur_tok[u] = tok;
+            state->tokens_out[(size_t)u * a.max_dec_len + t] = tok;
+            if (t + 1 >= a.max_len[u] || (a.eos_id >= 0 && tok == a.eos_id)) {
+                a.retired[u] = 1;
+                state->out_lens[u] = t + 1;
+                atomicAdd(&state->n_retired, 1);          // the host polls this to stop issuing steps once every utterance is done
+            }
+        }
+    } else if (threadIdx.x == 0) {
+        state->tokens_out = a.tokens_out;
+        state->out_lens = a.out_lens;
+    }
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     for (int start = 0; start < batch; start += blockDim.x) {
         // utterances are visited in the given order (longest encoder output first), so compact rows come out
         // sorted by encoder length: the attention blocks of the longest rows are scheduled first
         const int i = start + threadIdx.x;
-        const int u = i < batch ? order[i] : batch;
+        const int u = i < batch ? a.order[i] : batch;
         bool take = false;
+        int t = 0;
         if (u < batch) {
-            take = retired[u] == 0 && (mask == nullptr || mask[u] != 0);
-            if (take && t_u[u] >= max_dec_len) { take = false; atomicExch(&state->error, 1); }
+            t = a.t_u[u];
+            take = a.retired[u] == 0 && (a.mask == nullptr || a.mask[u] != 0);
+            if (take && t >= a.max_dec_len) { take = false; atomicExch(&state->error, 1); }
         }
-        unsigned ballot = __ballot_sync(0xffffffffu, take);
+        const unsigned ballot = __ballot_sync(0xffffffffu, take);
         if (lane == 0) warp_counts[warp] = __popc(ballot);
         __syncthreads();
-        int before = base;
-        for (int w = 0; w < warp; ++w) before += warp_counts[w];
+        const int count = warp_counts[lane];              // (blockDim.x = 1024: 32 warps)
+        const int before = base + static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? count : 0));
+        const int total = static_cast<int>(__reduce_add_sync(0xffffffffu, count));
         if (take) {
             const int slot = before + __popc(ballot & ((1u << lane) - 1u));
-            active_list[slot] = u;
-            row_info[slot] = make_int4(u, t_u[u], enc_len[u], enc_off[u]);
+            a.active_list[slot] = u;
+            a.row_info[slot] = make_int4(u, t, a.enc_len[u], a.enc_off[u]);
+            if (slot < kRowsInside) first[slot] = make_int4(u, t, min(max(a.tokens[u], 0), a.vocab - 1), 0);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            int total = 0;
-            for (int w = 0; w < n_warps; ++w) total += warp_counts[w];
-            base += total;
-        }
+        if (threadIdx.x == 0) base += total;
         __syncthreads();
     }
-    if (threadIdx.x == 0) { state->n_active = base; state->grid_sync = 0; }
-    for (int r = base + threadIdx.x; r < row_slots; r += blockDim.x) row_info[r] = make_int4(-1, 0, 0, 0);
+    const int n_rows = base;
+    if (threadIdx.x == 0) state->n_active = n_rows;
+    for (int r = n_rows + threadIdx.x; r < a.row_slots; r += blockDim.x) a.row_info[r] = make_int4(-1, 0, 0, 0);
+    if (n_rows > kRowsInside) return;
+    for (int i = threadIdx.x; i < a.d; i += blockDim.x) {
+#pragma unroll 4
+        for (int r = 0; r < n_rows; ++r)
+            a.x[(size_t)r * a.d + i] = to_f32(a.embed[(size_t)first[r].z * a.d + i]) * a.scale + a.pe[(size_t)first[r].y * a.d + i];
+    }
+    if (a.zero_buf)
+        for (int i = threadIdx.x; i < n_rows * a.zero_cols; i += blockDim.x) a.zero_buf[i] = 0.f;
+    if (a.zero_buf2)
+        for (int i = threadIdx.x; i < n_rows * a.zero_cols2; i += blockDim.x) a.zero_buf2[i] = 0.f;
+}
+
+// A new batch: clear the state and the bookkeeping arrays behind it, and note the batch size.  One block.
+__global__ void begin_batch_kernel(int4 *region, int n16, DecState *state, int batch)
+{
+    for (int i = threadIdx.x; i < n16; i += blockDim.x) region[i] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    if (threadIdx.x == 0) state->batch = batch;
+}
+
+// Start of a greedy decode: the start token into every utterance, empty results.
+__global__ void begin_greedy_kernel(int32_t *__restrict__ cur_tok, int bos, int batch, int32_t *__restrict__ tokens_out, size_t n_tokens,
+                                    int32_t *__restrict__ out_lens)
+{
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n_tokens) tokens_out[i] = -1;
+    if (i < (size_t)batch) { cur_tok[i] = bos; out_lens[i] = 0; }
 }
 
 // Sinusoidal position table PE[t][2i] = sin(t / 10000^(2i/d)), PE[t][2i+1] = cos(same), evaluated in double.
@@ -862,7 +944,7 @@ __global__ void build_prefill_rows_kernel(DecState *state, int chunk, int j0, in
             row_info[r] = make_int4(-1, 0, 0, 0);
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) { state->n_active = rows; state->grid_sync = 0; }
+    if (blockIdx.x == 0 && threadIdx.x == 0) state->n_active = rows;
 }
 
 // x[r] = E[token of the row] * sqrt(d) + PE[position of the row]
@@ -924,36 +1006,20 @@ __global__ void prefill_finish_kernel(DecState *state, const int32_t *__restrict
     }
 }
 
-// ------------------------------------------------------------------------------------------------------------
-// End of a step: decode the argmax keys, hand the choice out by utterance id, advance t_u, and (greedy mode)
-// record the token, feed it back and retire finished utterances.
-// ------------------------------------------------------------------------------------------------------------
+// End of a step of the caller's own loop: decode the argmax keys, hand the choice out by utterance id, advance t_u.
 __global__ void finish_step_kernel(DecState *state, const int32_t *__restrict__ active_list,
                                    unsigned long long *__restrict__ keys, int32_t *__restrict__ t_u,
-                                   int32_t *__restrict__ next_out /* by utterance, nullable */,
-                                   int greedy, int32_t *__restrict__ cur_tok, int32_t *__restrict__ retired,
-                                   const int32_t *__restrict__ max_len, int eos_id,
-                                   int32_t *__restrict__ tokens_out, int tokens_ld, int32_t *__restrict__ out_lens)
+                                   int32_t *__restrict__ next_out /* by utterance, nullable */)
 {
     AED_TRACE_BEGIN(state, 6);
     asm volatile("griddepcontrol.wait;" ::: "memory");       // launched with programmatic stream serialization
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= state->n_active) return;
-    int u = active_list[r];
-    int32_t tok = argmax_key_index(keys[r]);
+    const int u = active_list[r];
+    const int32_t tok = argmax_key_index(keys[r]);
     keys[r] = 0ull;
-    int t = t_u[u];
-    t_u[u] = t + 1;
+    t_u[u] += 1;
     if (next_out) next_out[u] = tok;
-    if (greedy) {
-        cur_tok[u] = tok;
-        tokens_out[(size_t)u * tokens_ld + t] = tok;
-        if (t + 1 >= max_len[u] || (eos_id >= 0 && tok == eos_id)) {
-            retired[u] = 1;
-            out_lens[u] = t + 1;
-            atomicAdd(&state->n_retired, 1);          // the host polls this to stop issuing steps once every utterance is done
-        }
-    }
 }
 
 // New utterances take over slots: position 0, start token, their encoder range and forced length.  One thread each.

@@ -413,6 +413,18 @@ def test_equal_row_tiles(batch):
     _run_both(w, rows=sorted({0, 15, 16, 17, batch // 2 - 1, batch // 2, batch // 2 + 1, batch - 2, batch - 1}))
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("groups", [[(8, 3)], [(9, 3)], [(4, 2), (5, 4), (3, 7)], [(131, 2), (5, 6)], [(60, 3), (2, 5)]])
+def test_rows_of_the_next_step(groups, dtype):
+    """Steps around the 8 rows that the bookkeeping kernel embeds itself, and row counts that fall to fewer from one step
+    to the next: from 12 over 8 to 3, from ready-made planes (136 rows) and from the tiled projections (62) at once."""
+    dec_lens = np.concatenate([[steps] * n for n, steps in groups])
+    rng = np.random.default_rng(len(dec_lens))
+    rng.shuffle(dec_lens)
+    w = wl.make_custom(ODD, rng.integers(1, 20, size=len(dec_lens)), dec_lens, dtype=dtype, seed=370 + len(dec_lens), out_std=0.1, ln_std=0.2)
+    _run_both(w, rows=sorted({0, len(dec_lens) - 1} | set(int(u) for u in np.argsort(dec_lens)[-5:])))
+
+
 @pytest.mark.parametrize("model", ["wide_b", "odd"])
 def test_small_batch_model_shapes(model):
     """d_model 1024 with 16 heads at 64 rows, and a model whose widths are not multiples of 128 (an odd number of

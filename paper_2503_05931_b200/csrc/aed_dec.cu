@@ -203,16 +203,16 @@ struct aed_dec {
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
     // greedy decoding replays one captured CUDA graph per (row bucket, self-attention chunk count, output buffers)
-    typedef std::tuple<int, int> GraphKey;       // (row count, chunks of self-attention positions)
+    typedef std::tuple<int, int, int> GraphKey;       // (row count, chunks of self-attention positions, steps)
     struct GraphEntry { cudaGraphExec_t exec; int64_t nodes; };
     std::map<GraphKey, GraphEntry> graphs;
     cudaStream_t capture_stream = nullptr;
     bool use_graphs = true;
     // set only while aed_dec_step_static_scratch runs: attention partials go here instead of the workspace
     float *partials_override = nullptr;
-    // greedy decoding with an end-of-sequence id: the retired count of recent steps, copied to pinned host memory
+    // with an end-of-sequence id: the retired count in pinned host memory, written by every greedy step
     static constexpr int kProbeSlots = 16;
-    int32_t *probe_host = nullptr;
+    int32_t *retired_host = nullptr;
     cudaEvent_t probe_event[kProbeSlots] = {};
 
     template <typename T> T *at(size_t off) const { return reinterpret_cast<T *>(ws + off); }
@@ -402,11 +402,12 @@ aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, 
     const int warps = p.M <= 512 ? 4 : f32::kWarps;
     p.state = dec->state();
     p.eps = dec->cfg.ln_eps;
+    p.after_rows = after_rows;
     void *args[] = {&p};
     auto grid = [&](int rt, int fpw) { return dim3((p.M + warps * fpw - 1) / (warps * fpw), (rows_ub + rt - 1) / rt); };
-    if (rows_ub <= 4) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 4, 1>, grid(4, 1), dim3(warps * 32), f32::rows_smem(4, p.K), args, after_rows);
-    if (rows_ub <= 16) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 1>, grid(8, 1), dim3(warps * 32), f32::rows_smem(8, p.K), args, after_rows);
-    return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 2>, grid(8, 2), dim3(warps * 32), f32::rows_smem(8, p.K), args, after_rows);
+    if (rows_ub <= 4) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 4, 1>, grid(4, 1), dim3(warps * 32), f32::rows_smem(4, p.K), args);
+    if (rows_ub <= 16) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 1>, grid(8, 1), dim3(warps * 32), f32::rows_smem(8, p.K), args);
+    return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 2>, grid(8, 2), dim3(warps * 32), f32::rows_smem(8, p.K), args);
 }
 
 // The forward pass of one step in fp32 for the rows in the active list (at most rows_ub of them): 8 kernels per layer, chained
@@ -683,8 +684,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
                               int K, int rows_ub, sg::StepGemmParams p, const CUtensorMap (*plane_maps)[2] = nullptr,
                               const CUtensorMap *map_w2 = nullptr, int M2 = 0, bool after_rows = false)
 {
-    // after_rows: the kernel before this launch made the row table, which the kernels of a step read ahead of their
-    // dependency waits: a full dependency, no programmatic one
+    // after_rows: the kernel before this launch makes the row table
     // map_w2, M2: a second weight matrix [M2, K] over the same rows (its output, gamma and bias are in p)
     // plane_maps (B_PLANES only): [N/16 - 1][high, low] tensor maps of the ready-made activation planes
     // Rows per CTA tile: up to 128 (two ring stages still fit beside the transposition buffer); more rows are
@@ -693,6 +693,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     const int m_tiles1 = (M + tc::kTileM - 1) / tc::kTileM;
     const int row_tiles = (rows_ub + n_tile - 1) / n_tile, m_tiles = m_tiles1 + (map_w2 ? (M2 + tc::kTileM - 1) / tc::kTileM : 0);
     p.tiles_first = map_w2 ? m_tiles1 : 0;
+    p.after_rows = after_rows;
     p.a_rows2 = M2;
     const int k_blocks = K / tc::kBlockK;
     const int stage_bytes = tc::kATileBytes + 2 * n_tile * tc::kBlockK * 2 + (MODE == sg::B_PLANES ? 0 : n_tile * tc::kBlockK * 4);
@@ -742,7 +743,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
             gc.stream = dec->stream;
             cudaLaunchAttribute ga[1];
             ga[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            ga[0].val.programmaticStreamSerializationAllowed = dec->use_pdl && !after_rows ? 1 : 0;
+            ga[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
             gc.attrs = ga;
             gc.numAttrs = 1;
             const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
@@ -764,7 +765,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     cfg.stream = dec->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl && !after_rows ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     // the accumulator is transposed through the ring's memory before it leaves: n_tile rows of 132 floats
@@ -1133,6 +1134,7 @@ aed_status_t launch_step_rows_t(aed_dec *dec, bool finish, const uint8_t *mask, 
         a.zero_buf2 = dec->at<float>(L.qc); a.zero_cols2 = c.d_model;
     }
     a.keys = dec->at<unsigned long long>(L.keys); a.cur_tok = dec->at<int32_t>(L.cur_tok); a.max_len = dec->at<int32_t>(L.max_len); a.eos_id = c.eos_id;
+    a.retired_host = dec->retired_host;
     a.tokens_out = tokens_out; a.out_lens = out_lens;
     void *args[] = {&a};
     ProfScope ps(dec, KF_BOOKKEEPING);
@@ -1249,10 +1251,19 @@ extern "C" aed_status_t aed_dec_create(const aed_dec_config_t *config, const aed
         const char *no_graph = getenv("AED_DEC_NO_GRAPH");
         dec->use_graphs = !(no_graph && no_graph[0] == '1');
     }
+    if (config->eos_id >= 0) {
+        e = cudaHostAlloc(reinterpret_cast<void **>(&dec->retired_host), sizeof(int32_t), cudaHostAllocDefault);
+        for (int i = 0; i < aed_dec::kProbeSlots && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&dec->probe_event[i], cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            aed_status_t s = fail(nullptr, AED_ERR_CUDA, "create: %s", cudaGetErrorString(e));
+            aed_dec_destroy(dec);
+            return s;
+        }
+    }
     if (config->dtype == AED_DTYPE_BF16) {
         aed_status_t s = tc_setup(dec);
         if (s != AED_OK) {
-            delete dec;
+            aed_dec_destroy(dec);
             return s;
         }
     }
@@ -1445,8 +1456,8 @@ aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub)
     return launch_step_rows(dec, true, nullptr, tok, planes);
 }
 
-// Record one greedy step into a graph on the library's capture stream (nothing runs) and instantiate it.
-aed_status_t capture_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, aed_dec::GraphEntry *entry)
+// Record greedy steps into a graph on the library's capture stream (nothing runs) and instantiate it.
+aed_status_t capture_greedy_steps(aed_dec *dec, int rows_ub, int self_len_ub, int steps, aed_dec::GraphEntry *entry)
 {
     if (!dec->capture_stream)
         AED_CUDA(dec, cudaStreamCreateWithFlags(&dec->capture_stream, cudaStreamNonBlocking));
@@ -1454,7 +1465,8 @@ aed_status_t capture_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, aed
     const int64_t before = dec->launches;
     AED_CUDA(dec, cudaStreamBeginCapture(dec->capture_stream, cudaStreamCaptureModeThreadLocal));
     dec->stream = dec->capture_stream;
-    aed_status_t st = enqueue_greedy_step(dec, rows_ub, self_len_ub);
+    aed_status_t st = AED_OK;
+    for (int i = 0; i < steps && st == AED_OK; ++i) st = enqueue_greedy_step(dec, rows_ub, self_len_ub);
     dec->stream = user;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamEndCapture(dec->capture_stream, &graph);
@@ -1465,6 +1477,29 @@ aed_status_t capture_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub, aed
     e = cudaGraphInstantiate(&entry->exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
+    return AED_OK;
+}
+
+// Steps of the same key per graph.  Inside a graph the kernels around a step's end overlap like all others (each starts
+// while its predecessor runs and fetches its weights); between two graphs they do not, which costs about 3 us.  (4 steps
+// instead of 1, 4-layer model: 93.5 -> 90.6 us per step of 1 row, 105.5 -> 102.1 of 8, 135.3 -> 133.9 of 24, 319.7 -> 318.5
+// of 128; 24 layers: 460 -> 457 us of 1 row, nothing beyond 8; fp32, 2 layers: 51.7 -> 47.1.)  A longer graph takes longer
+// to record, so deep models have them up to 8 rows and shallow ones up to 64.
+constexpr int kGraphSteps = 4;
+int steps_per_graph(const aed_dec *dec, int rows_b) { return rows_b <= (dec->cfg.n_layers <= 8 ? 64 : kRowsInside) ? kGraphSteps : 1; }
+
+// Launch `steps` greedy steps of at most rows_b rows and chunks * kAttnChunk positions as one graph, recorded at first use.
+aed_status_t launch_greedy_graph(aed_dec *dec, int rows_b, int chunks, int steps)
+{
+    const aed_dec::GraphKey key(rows_b, chunks, steps);
+    auto it = dec->graphs.find(key);
+    if (it == dec->graphs.end()) {
+        aed_dec::GraphEntry entry{};
+        AED_TRY(capture_greedy_steps(dec, rows_b, chunks * kAttnChunk, steps, &entry));
+        it = dec->graphs.emplace(key, entry).first;
+    }
+    AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
+    dec->launches += it->second.nodes;
     return AED_OK;
 }
 
@@ -1491,6 +1526,7 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
 
     dec->fresh_batch = false;
     AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.max_len, max_len, B * 4, cudaMemcpyHostToDevice, dec->stream));
+    const bool probe = dec->cfg.eos_id >= 0;
     {
         ProfScope ps(dec, KF_BOOKKEEPING);
         const size_t n = (size_t)B * dec->cfg.max_dec_len;
@@ -1499,41 +1535,36 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
     }
     AED_TRY(launch_step_rows(dec, false, nullptr, dec->at<int32_t>(L.cur_tok), true, tokens_out, out_lens));
     // With an end-of-sequence id the forced lengths are only upper bounds.  The host then stays at most kWindow steps
-    // ahead of the device: before it issues step s it looks at the retired count that step s - kWindow left behind
-    // (an asynchronous copy into pinned memory followed by an event) and stops once every utterance has retired.
-    const bool probe = dec->cfg.eos_id >= 0;
+    // ahead of the device (an event behind every launch) and stops once every utterance has retired, as the steps report
+    // in pinned memory.
     constexpr int kWindow = 8;
-    if (probe && !dec->probe_host) {
-        AED_CUDA(dec, cudaHostAlloc(reinterpret_cast<void **>(&dec->probe_host), aed_dec::kProbeSlots * sizeof(int32_t), cudaHostAllocDefault));
-        for (int i = 0; i < aed_dec::kProbeSlots; ++i) AED_CUDA(dec, cudaEventCreateWithFlags(&dec->probe_event[i], cudaEventDisableTiming));
-    }
-    for (int s = 0; s < longest; ++s) {
-        if (probe && s >= kWindow) {
-            const int slot = (s - kWindow) % aed_dec::kProbeSlots;
-            AED_CUDA(dec, cudaEventSynchronize(dec->probe_event[slot]));
-            if (dec->probe_host[slot] >= B) break;           // everything retired kWindow steps ago: the steps in between did nothing
+    int done = 0, oldest = 0, newest = 0;                   // steps known to be over; ring of launches in flight
+    int ends[aed_dec::kProbeSlots];
+    for (int s = 0; s < longest;) {
+        // grids are sized for the keyed row count; kernels leave rows beyond the device-side row count alone
+        const int rows_b = rows_key(alive[s]), chunks = s / kAttnChunk + 1;
+        const bool graph = dec->use_graphs && !dec->profiling;
+        int n = 1;
+        if (graph) {
+            const int most = steps_per_graph(dec, rows_b);
+            while (n < most && s + n < longest && rows_key(alive[s + n]) == rows_b && (s + n) / kAttnChunk + 1 == chunks) ++n;
+            if (n < most) n = 1;
         }
-        const int rows_ub = alive[s];
-        if (dec->use_graphs && !dec->profiling) {
-            // grids are sized for the keyed row count; kernels leave rows beyond the device-side row count alone
-            const int rows_b = rows_key(rows_ub), chunks = (s + 1 + kAttnChunk - 1) / kAttnChunk;
-            const aed_dec::GraphKey key(rows_b, chunks);
-            auto it = dec->graphs.find(key);
-            if (it == dec->graphs.end()) {
-                aed_dec::GraphEntry entry{};
-                AED_TRY(capture_greedy_step(dec, rows_b, chunks * kAttnChunk, &entry));
-                it = dec->graphs.emplace(key, entry).first;
-            }
-            AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
-            dec->launches += it->second.nodes;
-        } else {
-            AED_TRY(enqueue_greedy_step(dec, rows_ub, s + 1));
-        }
-        dec->steps_issued = s + 1;
         if (probe) {
-            const int slot = s % aed_dec::kProbeSlots;
-            AED_CUDA(dec, cudaMemcpyAsync(&dec->probe_host[slot], &dec->state()->n_retired, sizeof(int32_t), cudaMemcpyDeviceToHost, dec->stream));
-            AED_CUDA(dec, cudaEventRecord(dec->probe_event[slot], dec->stream));
+            while (s + n - done > kWindow) {
+                AED_CUDA(dec, cudaEventSynchronize(dec->probe_event[oldest % aed_dec::kProbeSlots]));
+                done = ends[oldest++ % aed_dec::kProbeSlots];
+            }
+            // (looked at only behind an event of this decode; steps already issued beyond the last retirement do nothing)
+            if (done > 0 && *static_cast<volatile int32_t *>(dec->retired_host) >= B) break;
+        }
+        if (graph) AED_TRY(launch_greedy_graph(dec, rows_b, chunks, n));
+        else AED_TRY(enqueue_greedy_step(dec, alive[s], s + 1));
+        s += n;
+        dec->steps_issued = s;
+        if (probe) {
+            AED_CUDA(dec, cudaEventRecord(dec->probe_event[newest % aed_dec::kProbeSlots], dec->stream));
+            ends[newest++ % aed_dec::kProbeSlots] = s;
         }
     }
     dec->full_steps = dec->cfg.max_dec_len;   // every utterance is retired: further steps are refused
@@ -1654,35 +1685,40 @@ extern "C" aed_status_t aed_dec_greedy_steps(aed_dec_t *dec, int32_t n_steps, in
     if (!dec->have_batch || !dec->slot_mode) return fail(dec, AED_ERR_STATE, "aed_dec_greedy_steps needs slots: call aed_dec_open_slots first");
     if (!tokens_out || !out_lens) return fail(dec, AED_ERR_INVALID_ARG, "tokens_out and out_lens must not be NULL");
     if (n_steps < 0) return fail(dec, AED_ERR_INVALID_ARG, "n_steps must not be negative");
-    for (int s = 0; s < n_steps; ++s) {
+    for (int s = 0; s < n_steps;) {
         // what the host knows: a slot decodes until its forced length (with an end-of-sequence id it may stop earlier
         // on the device; its row then simply is not there any more)
-        int rows_ub = 0, longest = 0;
-        for (int u = 0; u < dec->batch; ++u)
-            if (dec->slot_t[u] >= 0 && dec->slot_t[u] < dec->slot_max[u]) { ++rows_ub; longest = std::max(longest, dec->slot_t[u] + 1); }
+        auto rows_at = [&](int ahead, int &longest) {
+            int rows = 0;
+            longest = 0;
+            for (int u = 0; u < dec->batch; ++u)
+                if (dec->slot_t[u] >= 0 && dec->slot_t[u] + ahead < dec->slot_max[u]) { ++rows; longest = std::max(longest, dec->slot_t[u] + ahead + 1); }
+            return rows;
+        };
+        int longest;
+        const int rows_ub = rows_at(0, longest);
         if (rows_ub == 0) break;
         if (!dec->rows_ready || dec->rows_tokens != tokens_out || dec->rows_lens != out_lens) {
             AED_TRY(launch_step_rows(dec, false, nullptr, dec->at<int32_t>(dec->lay.cur_tok), true, tokens_out, out_lens));
             dec->rows_ready = true;
             dec->rows_tokens = tokens_out; dec->rows_lens = out_lens;
         }
+        int n = 1;
         if (dec->use_graphs && !dec->profiling) {
-            const int rows_b = rows_key(rows_ub), chunks = (longest + kAttnChunk - 1) / kAttnChunk;
-            const aed_dec::GraphKey key(rows_b, chunks);
-            auto it = dec->graphs.find(key);
-            if (it == dec->graphs.end()) {
-                aed_dec::GraphEntry entry{};
-                AED_TRY(capture_greedy_step(dec, rows_b, chunks * kAttnChunk, &entry));
-                it = dec->graphs.emplace(key, entry).first;
+            const int rows_b = rows_key(rows_ub), chunks = (longest + kAttnChunk - 1) / kAttnChunk, most = steps_per_graph(dec, rows_b);
+            if (most <= n_steps - s) {
+                int last;
+                const int rows_last = rows_at(most - 1, last);       // (rows only leave in between, positions only grow)
+                if (rows_last > 0 && rows_key(rows_last) == rows_b && (last + kAttnChunk - 1) / kAttnChunk == chunks && last == longest + most - 1) n = most;
             }
-            AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
-            dec->launches += it->second.nodes;
+            AED_TRY(launch_greedy_graph(dec, rows_b, chunks, n));
         } else {
             AED_TRY(enqueue_greedy_step(dec, rows_ub, longest));
         }
         for (int u = 0; u < dec->batch; ++u)
-            if (dec->slot_t[u] >= 0 && dec->slot_t[u] < dec->slot_max[u]) ++dec->slot_t[u];
-        if (steps_done) ++*steps_done;
+            if (dec->slot_t[u] >= 0 && dec->slot_t[u] < dec->slot_max[u]) dec->slot_t[u] = std::min(dec->slot_t[u] + n, dec->slot_max[u]);
+        s += n;
+        if (steps_done) *steps_done += n;
     }
     return AED_OK;
 }
@@ -1833,7 +1869,7 @@ extern "C" void aed_dec_destroy(aed_dec_t *dec)
     for (auto &g : dec->graphs) cudaGraphExecDestroy(g.second.exec);
     if (dec->capture_stream) cudaStreamDestroy(dec->capture_stream);
     for (cudaEvent_t e : dec->probe_event) if (e) cudaEventDestroy(e);
-    if (dec->probe_host) cudaFreeHost(dec->probe_host);
+    if (dec->retired_host) cudaFreeHost(dec->retired_host);
     delete dec;
 }
 

@@ -21,6 +21,7 @@ constexpr int kTileK = 1024;                 // columns of the rows staged at a 
 constexpr int kWarps = 8;
 
 struct RowsArgs {
+    int after_rows;
     const DecState *state;
     int rows_fixed;                          // >= 0: number of rows; < 0: read it from the decode state
     const float *a;                          // [rows, K]
@@ -68,8 +69,8 @@ rows_kernel(const RowsArgs p)
     __shared__ unsigned long long s_key[RT];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const int f0 = (blockIdx.x * n_warps + warp) * FPW, row0 = blockIdx.y * RT;
-    const int n_rows = p.rows_fixed >= 0 ? p.rows_fixed : p.state->n_active;
-    sg::pdl_launch_dependents();
+    int n_rows = p.rows_fixed >= 0 ? p.rows_fixed : p.after_rows ? 0 : p.state->n_active;
+    if (!p.after_rows) sg::pdl_launch_dependents();
     const int K = p.K;
     float4 w[FPW][kAhead];
     auto load_w = [&](int f, int k) {
@@ -80,6 +81,7 @@ rows_kernel(const RowsArgs p)
 #pragma unroll
         for (int i = 0; i < kAhead; ++i) w[f][i] = load_w(f, i * 128 + lane * 4);
     sg::pdl_wait();
+    if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }      // (see StepGemmParams)
     if (row0 >= n_rows) return;
     if (EPI == EPI_LOGITS && threadIdx.x < RT) s_key[threadIdx.x] = 0ull;
     if (p.ln_g) {

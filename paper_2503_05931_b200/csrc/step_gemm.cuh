@@ -56,6 +56,9 @@ struct StepGemmParams {
     const __nv_bfloat16 *bias;     // added by k-split 0, may be null
     // second matrix (feature tiles tiles_first .. gridDim.x - 1); tiles_first == 0: none
     int tiles_first;
+    // the kernel before this launch makes the row table and the row count: read after the dependency wait, and the next
+    // kernel, which reads them ahead of its own, may start only then
+    int after_rows;
     int a_rows2;
     const __nv_bfloat16 *gamma2;   // B_GAMMA
     float *out2;
@@ -210,7 +213,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_slot;
-    pdl_launch_dependents();
+    if (!p.after_rows) pdl_launch_dependents();
     AED_TRACE_PUT(p.state, tcur, 40);      // set-up done
 
     if (warp == 0) {
@@ -296,6 +299,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         side_after_wait(p, p.state->n_active, cta, n_cta, st, lane, warp - 10, red_s, red_q);
     } else {
         pdl_wait();
+        if (p.after_rows) pdl_launch_dependents();
         AED_TRACE_PUT(p.state, tcur, 41);  // dependency resolved
         const int pt = threadIdx.x - 64;                  // 0..255 among the producer threads
         const int n_rows = p.state->n_active;

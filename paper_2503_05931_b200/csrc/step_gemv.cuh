@@ -82,7 +82,7 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    sg::pdl_launch_dependents();
+    if (!p.after_rows) sg::pdl_launch_dependents();
 
     if (warp >= 8) {
         // ---- weight copies (independent of every earlier kernel), then the side jobs --------------------------
@@ -97,8 +97,9 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         const int cta = blockIdx.x + gridDim.x * blockIdx.y;
         const int n_cta = gridDim.x * gridDim.y;
         sg::side_prefetch(p, cta, n_cta, st);
-        const int n_rows = p.state->n_active;
+        int n_rows = p.after_rows ? 0 : p.state->n_active;
         sg::pdl_wait();
+        if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }
         sg::side_after_wait(p, n_rows, cta, n_cta, st, lane, warp - 8, red_s, red_q);
         return;
     }
@@ -125,8 +126,9 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int ldo = second_w ? p.ldo2 : p.ldo;
     asm volatile("bar.sync 2, 256;" ::: "memory");           // the constants are in place (still before the wait)
 
-    const int n_rows = p.state->n_active;
+    int n_rows = p.after_rows ? 0 : p.state->n_active;
     sg::pdl_wait();
+    if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }
     // B fragments: column n = lane / 4 is row nt * 8 + n of the step, rows k0 + {0, 1, 8, 9} with k0 = 16 ks + 2 (lane % 4)
     const int kq = (lane & 3) * 2;
     float2 xa[kNT][kSvMaxKb][4], xb[kNT][kSvMaxKb][4];
@@ -270,7 +272,7 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    sg::pdl_launch_dependents();
+    if (!p.after_rows) sg::pdl_launch_dependents();
 
     if (warp >= 8) {
         if (warp == 8 && lane == 0) {
@@ -284,8 +286,9 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
         const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
         const int n_cta = gridDim.x * gridDim.y * gridDim.z;
         sg::side_prefetch(p, cta, n_cta, st);
-        const int n_rows = p.state->n_active;
+        int n_rows = p.after_rows ? 0 : p.state->n_active;
         sg::pdl_wait();
+        if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }
         sg::side_after_wait(p, n_rows, cta, n_cta, st, lane, warp - 8, red_s, red_q);
         return;
     }
@@ -310,8 +313,9 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
     const int ldo = second_w ? p.ldo2 : p.ldo;
     asm volatile("bar.sync 2, 256;" ::: "memory");
 
-    const int n_rows = p.state->n_active;
+    int n_rows = p.after_rows ? 0 : p.state->n_active;
     sg::pdl_wait();
+    if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }
     // ---- the rows' k range -> planes: element e of the tile is row e / kF4, floats 4 (e % kF4) .. + 3 ------------------
     constexpr int kPer = kRows * kF4 / 256;                    // 16-byte loads per thread
     float4 xv[kPer];

@@ -20,8 +20,11 @@ namespace aed {
 // the argmax keys, record the token and feed it back, advance t_u, retire finished utterances, and then the rows of the
 // next step.  Steps of at most kRowsInside rows find their embedded rows there as well.  These are chains of dependent
 // loads of a few hundred cycles each, so what matters is the number of launches in a row: one here, where the end of a
-// step, the compaction and the embedding were three, with the boundary between two graphs in the middle.
-// It never lets its successor start early: kernels read the row count and the row table ahead of their dependency wait.
+// step, the compaction and the embedding were three, with the boundary between two graphs in the middle.  (4-layer
+// model, per step of 1 / 16 rows: 97 / 115 us with three launches, 96 / 116 with this one, 93 / 113 with its loads ahead of the
+// wait, 91 / 110 with several steps per graph.)
+// Kernels read the row count and the row table ahead of their dependency wait; the one right after this kernel does not,
+// and lets its own successor start only after its wait.
 constexpr int kRowsInside = 8;       // one block embeds these in less than the 2.8 us of another launch
 
 template <typename T>
@@ -46,73 +49,101 @@ struct StepRowsArgs {
     int32_t *cur_tok;
     const int32_t *max_len;
     int eos_id;
+    volatile int32_t *retired_host;           // with an end-of-sequence id: how many have retired, for the host; or null
     // !kFinish: where the greedy steps to come leave their results
     int32_t *tokens_out, *out_lens;
 };
 
-// One block of 1024 threads.
+// One block of 1024 threads, one utterance per thread and pass.  Everything but the argmax keys is known before the
+// dependency wait (only this kernel changes the bookkeeping of greedy steps, and kernels of another kind in between are
+// separated by full dependencies): rows of the step that ends, lengths, positions are loaded and computed ahead of it.
+// By then the weights of a step have pushed those arrays out of L2, so each is a miss of about 1 us.
 template <typename T, bool kFinish>
 __global__ void __launch_bounds__(1024) step_rows_kernel(const __grid_constant__ StepRowsArgs<T> a)
 {
     AED_TRACE_BEGIN(a.state, 1);
-    __shared__ int warp_counts[32];
-    __shared__ int base;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __shared__ int counts_old[32], counts_new[32];
     __shared__ int4 first[kRowsInside];       // (utterance, t_u, token) of the first rows
     DecState *const state = a.state;
     const int batch = state->batch, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (threadIdx.x == 0) base = 0;
-    if (kFinish) {
-        const int n = state->n_active;
-        for (int r = threadIdx.x; r < n; r += blockDim.x) {
-            const int u = a.active_list[r];
-            const int32_t tok = argmax_key_index(a.keys[r]);
-            const int t = a.t_u[u];
-            a.keys[r] = 0ull;
-            a.t_u[u] = t + 1;
-            a.cur_tok[u] = tok;
-            state->tokens_out[(size_t)u * a.max_dec_len + t] = tok;
-            if (t + 1 >= a.max_len[u] || (a.eos_id >= 0 && tok == a.eos_id)) {
-                a.retired[u] = 1;
-                state->out_lens[u] = t + 1;
-                atomicAdd(&state->n_retired, 1);          // the host polls this to stop issuing steps once every utterance is done
-            }
-        }
-    } else if (threadIdx.x == 0) {
-        state->tokens_out = a.tokens_out;
-        state->out_lens = a.out_lens;
-    }
-    __syncthreads();
-    for (int start = 0; start < batch; start += blockDim.x) {
+    int32_t *const tokens_out = kFinish ? state->tokens_out : a.tokens_out, *const out_lens = kFinish ? state->out_lens : a.out_lens;
+    int u, t, enc_len, enc_off, max_len;
+    bool live;                                // takes part unless masked: not retired (and then within its cache)
+    auto load = [&](int i) {
         // utterances are visited in the given order (longest encoder output first), so compact rows come out
         // sorted by encoder length: the attention blocks of the longest rows are scheduled first
-        const int i = start + threadIdx.x;
-        const int u = i < batch ? a.order[i] : batch;
-        bool take = false;
-        int t = 0;
-        if (u < batch) {
+        live = false;
+        u = t = enc_len = enc_off = max_len = 0;
+        if (i < batch) {
+            u = a.order[i];
             t = a.t_u[u];
-            take = a.retired[u] == 0 && (a.mask == nullptr || a.mask[u] != 0);
-            if (take && t >= a.max_dec_len) { take = false; atomicExch(&state->error, 1); }
+            live = a.retired[u] == 0;
+            enc_len = a.enc_len[u]; enc_off = a.enc_off[u];
+            if (kFinish) max_len = a.max_len[u];
         }
-        const unsigned ballot = __ballot_sync(0xffffffffu, take);
-        if (lane == 0) warp_counts[warp] = __popc(ballot);
+    };
+    // rank of this thread among those of the block that satisfy the predicate, and their number (two barriers)
+    auto rank = [&](bool yes, int *counts, int &total) {
+        const unsigned ballot = __ballot_sync(0xffffffffu, yes);
+        if (lane == 0) counts[warp] = __popc(ballot);
         __syncthreads();
-        const int count = warp_counts[lane];              // (blockDim.x = 1024: 32 warps)
-        const int before = base + static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? count : 0));
-        const int total = static_cast<int>(__reduce_add_sync(0xffffffffu, count));
-        if (take) {
-            const int slot = before + __popc(ballot & ((1u << lane) - 1u));
-            a.active_list[slot] = u;
-            a.row_info[slot] = make_int4(u, t, a.enc_len[u], a.enc_off[u]);
-            if (slot < kRowsInside) first[slot] = make_int4(u, t, min(max(a.tokens[u], 0), a.vocab - 1), 0);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) base += total;
-        __syncthreads();
+        const int count = counts[lane];                   // (32 warps)
+        total = static_cast<int>(__reduce_add_sync(0xffffffffu, count));
+        return static_cast<int>(__reduce_add_sync(0xffffffffu, lane < warp ? count : 0)) + __popc(ballot & ((1u << lane) - 1u));
+    };
+    load(threadIdx.x);
+    int base_old = 0, base = 0, total = 0, row = 0;
+    if (kFinish) {
+        row = rank(live && t < a.max_dec_len, counts_old, total);
+        if (live && row < kRowsInside)        // the position rows that the next step probably adds
+            for (int i = 0; i < a.d; i += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.pe + (size_t)min(t + 1, a.max_dec_len - 1) * a.d + i));
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!kFinish && threadIdx.x == 0) { state->tokens_out = tokens_out; state->out_lens = out_lens; }
+    for (int start = 0; start < batch; start += blockDim.x) {
+        if (start > 0) {
+            load(start + threadIdx.x);
+            __syncthreads();                  // counts_old, counts_new of the previous pass have been read
+            if (kFinish) row = rank(live && t < a.max_dec_len, counts_old, total);
+        }
+        int tok = 0;
+        if (kFinish) {
+            row += base_old;
+            base_old += total;
+            if (live && t < a.max_dec_len) {
+                tok = argmax_key_index(a.keys[row]);
+                a.keys[row] = 0ull;
+                tokens_out[(size_t)u * a.max_dec_len + t] = tok;
+                a.t_u[u] = ++t;
+                a.cur_tok[u] = tok;
+                if (t >= max_len || (a.eos_id >= 0 && tok == a.eos_id)) {
+                    live = false;
+                    a.retired[u] = 1;
+                    out_lens[u] = t;
+                    atomicAdd(&state->n_retired, 1);          // the host polls this to stop issuing steps once every utterance is done
+                }
+            }
+        }
+        bool take = live && (kFinish || a.mask == nullptr || a.mask[u] != 0);
+        if (take && t >= a.max_dec_len) { take = false; atomicExch(&state->error, 1); }
+        const int slot = base + rank(take, counts_new, total);
+        base += total;
+        if (take) {
+            a.active_list[slot] = u;
+            a.row_info[slot] = make_int4(u, t, enc_len, enc_off);
+            if (slot < kRowsInside) first[slot] = make_int4(u, t, min(max(kFinish ? tok : a.tokens[u], 0), a.vocab - 1), 0);
+        }
+    }
+    __syncthreads();
     const int n_rows = base;
-    if (threadIdx.x == 0) state->n_active = n_rows;
+    if (threadIdx.x == 0) {
+        state->n_active = n_rows;
+        if (kFinish && a.retired_host) {
+            *a.retired_host = state->n_retired;       // pinned host memory; the host looks at it behind an event
+            __threadfence_system();
+        }
+    }
     for (int r = n_rows + threadIdx.x; r < a.row_slots; r += blockDim.x) a.row_info[r] = make_int4(-1, 0, 0, 0);
     if (n_rows > kRowsInside) return;
     for (int i = threadIdx.x; i < a.d; i += blockDim.x) {

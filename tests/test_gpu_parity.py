@@ -425,6 +425,14 @@ def test_rows_of_the_next_step(groups, dtype):
     _run_both(w, rows=sorted({0, len(dec_lens) - 1} | set(int(u) for u in np.argsort(dec_lens)[-5:])))
 
 
+@pytest.mark.parametrize("dtype, steps", [("bf16", 3), ("bf16", 4), ("bf16", 21), ("fp32", 37)])
+def test_several_steps_per_graph(dtype, steps):
+    """Greedy decodes of fewer steps than a graph holds, of exactly as many, and across 16-position chunks, with rows that
+    retire inside a graph."""
+    w = wl.make_custom(ODD, [9, 30, 4], [steps, max(1, steps - 5), 2], dtype=dtype, seed=380 + steps, out_std=0.1, ln_std=0.2)
+    _run_both(w)
+
+
 @pytest.mark.parametrize("model", ["wide_b", "odd"])
 def test_small_batch_model_shapes(model):
     """d_model 1024 with 16 heads at 64 rows, and a model whose widths are not multiples of 128 (an odd number of

@@ -20,6 +20,7 @@
 #include "step_gemv.cuh"
 #include "vocab_gemv.cuh"
 #include "crosskv_gemm.cuh"
+#include "plane_gemm.cuh"
 #include "f32_rows.cuh"
 #include "stream_schedule.h"
 
@@ -554,7 +555,7 @@ aed_status_t tc_setup(aed_dec *dec)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_GAMMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_LN_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_PLANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(pg::plane_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
@@ -681,12 +682,11 @@ struct FusedGemm {
 
 template <int MODE>
 aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, const CUtensorMap *src_maps, int M,
-                              int K, int rows_ub, sg::StepGemmParams p, const CUtensorMap (*plane_maps)[2] = nullptr,
+                              int K, int rows_ub, sg::StepGemmParams p,
                               const CUtensorMap *map_w2 = nullptr, int M2 = 0, bool after_rows = false)
 {
     // after_rows: the kernel before this launch makes the row table
     // map_w2, M2: a second weight matrix [M2, K] over the same rows (its output, gamma and bias are in p)
-    // plane_maps (B_PLANES only): [N/16 - 1][high, low] tensor maps of the ready-made activation planes
     // Rows per CTA tile: up to 128 (two ring stages still fit beside the transposition buffer); more rows are
     // covered by row tiles that re-read the weight tile from L2.
     const int n_tile = tc_n_tile(rows_ub, 128), ni = n_tile / 16 - 1;
@@ -696,7 +696,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     p.after_rows = after_rows;
     p.a_rows2 = M2;
     const int k_blocks = K / tc::kBlockK;
-    const int stage_bytes = tc::kATileBytes + 2 * n_tile * tc::kBlockK * 2 + (MODE == sg::B_PLANES ? 0 : n_tile * tc::kBlockK * 4);
+    const int stage_bytes = tc::kATileBytes + 2 * n_tile * tc::kBlockK * 2 + n_tile * tc::kBlockK * 4;
     int stages = kTcSmemBudget / stage_bytes;
     if (stages > sg::kMaxKb) stages = sg::kMaxKb;
     // k-splits: every split adds rows x features x 4 bytes of red.global traffic, so large batches stop at about
@@ -725,38 +725,36 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     // and beyond three or four such parts lose to the tcgen05 kernel (1392 / 1634 / 1881 us there against 1512 / 1655 /
     // 2006 at 65 / 96 / 128 rows).
     const int splits_wide = std::max((k_blocks + 3) / 4, splits / 2);
-    const bool gemv = MODE != sg::B_PLANES && dec->use_gemv && rows_ub <= dec->gemv_rows &&
+    const bool gemv = dec->use_gemv && rows_ub <= dec->gemv_rows &&
                       (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
     ProfScope ps(dec, family + KF_COUNT * (!gemv ? KV_TCGEN05 : rows_ub <= dec->gemv_direct_rows ? KV_GEMV : KV_GEMV_STAGED));
-    if constexpr (MODE != sg::B_PLANES) {
-        // Steps of at most 32 rows whose CTAs cover at most two k-blocks (64 rows, four): warp-level MMAs
-        // (step_gemv.cuh), activation fragments straight from global memory up to 4 rows, through shared memory beyond
-        if (gemv) {
-            cudaLaunchConfig_t gc = {};
-            gc.gridDim = dim3(m_tiles, splits, 1);
-            gc.blockDim = dim3(sv::kSvThreads);
-            const bool direct = rows_ub <= dec->gemv_direct_rows, wide = rows_ub > 32;
-            const int part = wide ? (rows_ub + 1) / 2 : rows_ub;
-            const int nt = wide ? (part <= 24 ? 3 : 4) : part <= 16 ? 2 : part <= 24 ? 3 : 4;      // row tiles of 8 per CTA
-            if (wide) gc.gridDim = dim3(m_tiles, splits_wide, 2);
-            gc.dynamicSmemBytes = direct ? (size_t)sv::kSvMaxKb * tc::kATileBytes + 1024 : (size_t)sv::sv_staged_smem(nt, wide ? 4 : sv::kSvMaxKb);
-            gc.stream = dec->stream;
-            cudaLaunchAttribute ga[1];
-            ga[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            ga[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
-            gc.attrs = ga;
-            gc.numAttrs = 1;
-            const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
-            cudaError_t ge = direct    ? cudaLaunchKernelEx(&gc, sv::step_gemv_kernel<MODE, 1>, map_w, second, p)
-                             : wide    ? (nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3, 4>, map_w, second, p)
-                                                  : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4, 4>, map_w, second, p))
-                             : nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3>, map_w, second, p)
-                             : nt == 2 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 2>, map_w, second, p)
-                                       : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4>, map_w, second, p);
-            if (ge != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(ge));
-            AED_LAUNCHED(dec);
-            return AED_OK;
-        }
+    // Steps of at most 32 rows whose CTAs cover at most two k-blocks (64 rows, four): warp-level MMAs
+    // (step_gemv.cuh), activation fragments straight from global memory up to 4 rows, through shared memory beyond
+    if (gemv) {
+        cudaLaunchConfig_t gc = {};
+        gc.gridDim = dim3(m_tiles, splits, 1);
+        gc.blockDim = dim3(sv::kSvThreads);
+        const bool direct = rows_ub <= dec->gemv_direct_rows, wide = rows_ub > 32;
+        const int part = wide ? (rows_ub + 1) / 2 : rows_ub;
+        const int nt = wide ? (part <= 24 ? 3 : 4) : part <= 16 ? 2 : part <= 24 ? 3 : 4;      // row tiles of 8 per CTA
+        if (wide) gc.gridDim = dim3(m_tiles, splits_wide, 2);
+        gc.dynamicSmemBytes = direct ? (size_t)sv::kSvMaxKb * tc::kATileBytes + 1024 : (size_t)sv::sv_staged_smem(nt, wide ? 4 : sv::kSvMaxKb);
+        gc.stream = dec->stream;
+        cudaLaunchAttribute ga[1];
+        ga[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        ga[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
+        gc.attrs = ga;
+        gc.numAttrs = 1;
+        const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
+        cudaError_t ge = direct    ? cudaLaunchKernelEx(&gc, sv::step_gemv_kernel<MODE, 1>, map_w, second, p)
+                         : wide    ? (nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3, 4>, map_w, second, p)
+                                              : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4, 4>, map_w, second, p))
+                         : nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3>, map_w, second, p)
+                         : nt == 2 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 2>, map_w, second, p)
+                                   : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4>, map_w, second, p);
+        if (ge != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(ge));
+        AED_LAUNCHED(dec);
+        return AED_OK;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m_tiles, splits, row_tiles);
@@ -768,12 +766,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // the accumulator is transposed through the ring's memory before it leaves: n_tile rows of 132 floats
-    if (MODE == sg::B_PLANES && (size_t)stages * stage_bytes < (size_t)n_tile * (tc::kTileM + 4) * 4)
-        cfg.dynamicSmemBytes = (size_t)n_tile * (tc::kTileM + 4) * 4 + 1024;
-    cudaError_t e = MODE == sg::B_PLANES
-                        ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE>, map_w, plane_maps[ni][0], plane_maps[ni][1], p)
-                        : cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE>, map_w, src_maps[ni], map_w2 ? *map_w2 : src_maps[ni], p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE>, map_w, src_maps[ni], map_w2 ? *map_w2 : src_maps[ni], p);
     if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(e));
     AED_LAUNCHED(dec);
     return AED_OK;
@@ -867,7 +860,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.prefetch2_ptr = wn.w_q_c; p.prefetch2_bytes = (size_t)d * d * e2;
         // the vocabulary matrix is as large as a layer: its way into L2 starts a whole layer ahead of the projection
         if (l == c.n_layers - 1) { p.prefetch2_ptr = dec->w_out; p.prefetch2_bytes = (size_t)V * d * e2; }
-        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, dec->tc_src_x, 3 * d, d, rows_ub, p, nullptr, &m.qc, d, embedded && l == 0));
+        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, dec->tc_src_x, 3 * d, d, rows_ub, p, &m.qc, d, embedded && l == 0));
         // 2. self-attention (applies LN1 to q, k, v; appends k, v)
         if (pf && l == c.n_layers - 1) rows = pf->last_chunk ? pf->batch : 0;
         AED_TRY(launch_self_attention(dec, rows_ub, rows, self_len_ub, self_cache, att, nullptr, nullptr, stats, c1_qkv, c2_qkv, pf != nullptr));
@@ -882,7 +875,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.zero_buf = hid; p.zero_cols = F;
         p.prefetch_ptr = wn.w_o; p.prefetch_bytes = (size_t)d * d * e2;
         p.prefetch2_ptr = dec->at<T>(L.comp_w) + (size_t)((l + 1) % c.n_layers) * d * d; p.prefetch2_bytes = (size_t)d * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_O, m.o, dec->tc_src_att, d, d, rows, p, nullptr, &m.o_qc, d));
+        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_O, m.o, dec->tc_src_att, d, d, rows, p, &m.o_qc, d));
         // 4. cross-attention; every block computes the LN2 statistics of its row of x_new itself
         if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
             const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
@@ -964,6 +957,43 @@ aed_status_t launch_pdl(aed_dec *dec, K kernel, dim3 grid, dim3 block, Args... a
     return AED_OK;
 }
 
+// The shape of a projection of the many-rows path (plane_gemm.cuh).  n_tile: rows per pair of blocks; splits: k-splits.
+//  * Two row tiles up to 320 rows, then tiles of at most 128: 136 rows 1872 us per step of the 24-layer model with one tile
+//    of 160 and 1845 with two of 96; 304 rows 2701 with three of 128 and 2601 with two of 160; 448 rows 3284 with three of
+//    160 and 3248 with four of 128.
+//  * At most 128 blocks, one per SM: the pairs of a cluster launch must all find room at once (144 blocks at 384 rows: 3287 us
+//    against 3015), and k-splits add rows x features x 4 bytes of reductions each.
+//  * whole_k (FFN1, whose epilogue needs complete sums): more row tiles instead of k-splits (256 rows 2405 -> 2371 us).
+struct PlaneShape { int n_tile, splits; };
+constexpr int kPlaneBlocks = 128;
+PlaneShape plane_shape(int M, int K, int rows_ub, bool whole_k)
+{
+    const int m_tiles = (M + 2 * tc::kTileM - 1) / (2 * tc::kTileM) * 2;
+    int tiles = rows_ub <= 320 ? 2 : (rows_ub + 127) / 128;
+    if (whole_k) tiles = std::max(tiles, kPlaneBlocks / m_tiles);
+    const int n_tile = ((rows_ub + tiles - 1) / tiles + 31) / 32 * 32, row_tiles = (rows_ub + n_tile - 1) / n_tile;
+    return {n_tile, whole_k ? 1 : std::min(std::max(kPlaneBlocks / (m_tiles * row_tiles), 1), K / tc::kBlockK)};
+}
+
+aed_status_t launch_plane_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, const CUtensorMap (*planes)[2], int M, int K, int rows_ub, PlaneShape shape,
+                               pg::PlaneGemmParams p)
+{
+    ProfScope ps(dec, family);
+    p.a_rows = M;
+    p.k_blocks = K / tc::kBlockK;
+    p.n_tile = shape.n_tile;
+    const int stage_bytes = tc::kATileBytes + p.n_tile * tc::kBlockK * 2, most = (p.k_blocks + shape.splits - 1) / shape.splits;
+    p.stages = std::min({128 * 1024 / stage_bytes, pg::kPgStages, most});
+    p.state = dec->state();
+    // More than half of an SM's shared memory whatever the ring needs: two pairs on the same two SMs while others idle would
+    // share what these take in (512 rows with 97 KB: 4150 us per step against 3500; 136 rows 1906 against 1845).
+    const size_t smem = std::max({(size_t)p.stages * stage_bytes, (size_t)p.n_tile * (tc::kTileM + 4) * 4, (size_t)116 * 1024}) + 1024;
+    const CUtensorMap *const maps = planes[p.n_tile / 32 - 1];
+    void *args[] = {(void *)&map_w, (void *)&maps[0], (void *)&maps[1], &p};
+    return launch_pdl_impl(dec, (const void *)pg::plane_gemm_kernel,
+                           dim3((M + 2 * tc::kTileM - 1) / (2 * tc::kTileM) * 2, shape.splits, (rows_ub + p.n_tile - 1) / p.n_tile), dim3(pg::kPgThreads), smem, args);
+}
+
 aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out,
                                  const PrefillPass *pf = nullptr)
 {
@@ -971,7 +1001,7 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
     const auto &c = dec->cfg;
     const Layout &L = dec->lay;
     const int d = c.d_model, F = c.d_ffn, V = c.vocab;
-    float *x = dec->at<float>(L.x), *qkv = dec->at<float>(L.qkv), *hid = dec->at<float>(L.hid), *qc = dec->at<float>(L.qc);
+    float *x = dec->at<float>(L.x), *qkv = dec->at<float>(L.qkv), *qc = dec->at<float>(L.qc);
     T *ad_hi = dec->at<T>(L.actd_hi), *ad_lo = dec->at<T>(L.actd_lo), *af_hi = dec->at<T>(L.actf_hi), *af_lo = dec->at<T>(L.actf_lo);
     float2 *stats = dec->at<float2>(L.ln_stats);
     const int stats_stride = rows_bucket(c.max_batch);
@@ -994,6 +1024,16 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         return launch_pdl(dec, gamma_planes_kernel<8>, dim3(rows), ln_block, (const DecState *)dec->state(), (const float *)x,
                           (const T *)g, d, c.ln_eps, st, ad_hi, ad_lo, zero_buf, zero_cols);
     };
+    const PlaneShape sh_qkv = plane_shape(3 * d, d, rows_ub, false), sh_o = plane_shape(d, d, rows_ub, false), sh_qc = sh_o,
+                     sh_ff1 = plane_shape(F, d, rows_ub, true), sh_ff2 = plane_shape(d, F, rows_ub, false);
+    // out: rows of their own, cleared before if there are k-splits; or null: the residual stream
+    auto project = [&](int family, const CUtensorMap &map_w, const CUtensorMap (*planes)[2], int M, int K, PlaneShape shape, float *out, const void *bias) -> aed_status_t {
+        pg::PlaneGemmParams p{};
+        p.epi = out && shape.splits == 1 ? pg::PG_STORE : pg::PG_ADD;
+        p.out = out ? out : x; p.ldo = M;
+        p.bias = (const T *)bias;
+        return launch_plane_gemm(dec, family, map_w, planes, M, K, rows, shape, p);
+    };
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerWeights &w = dec->layers[l];
         const aed_dec::TcLayerMaps &m = dec->tc_layers[l];
@@ -1002,22 +1042,16 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         const float *fc = dec->at<float>(L.fold_c) + (size_t)l * L.fold_layer_floats;
         const float *c1_qkv = fc, *c2_qkv = fc + 3 * d, *c1_qc = fc + 6 * d, *c2_qc = fc + 7 * d, *c1_ff = fc + 8 * d,
                     *c2_ff = fc + 8 * d + F;
-        sg::StepGemmParams p{};
         // self-attention block
-        AED_TRY(gamma_planes(w.ln1_g, stats, qc, d));
-        p.out = qkv; p.ldo = 3 * d;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_QKV, m.qkv, nullptr, 3 * d, d, rows_ub, p, dec->tc_actd));
+        AED_TRY(gamma_planes(w.ln1_g, stats, sh_qc.splits > 1 ? qc : nullptr, d));
+        AED_TRY(project(KF_GEMM_QKV, m.qkv, dec->tc_actd, 3 * d, d, sh_qkv, qkv, nullptr));
         if (pf && l == c.n_layers - 1) rows = pf->last_chunk ? pf->batch : 0;
         AED_TRY(launch_self_attention(dec, rows_ub, rows, self_len_ub, self_cache, nullptr, ad_hi, ad_lo, stats, c1_qkv, c2_qkv, pf != nullptr));
         if (rows == 0) return AED_OK;
-        p = sg::StepGemmParams{};
-        p.out = x; p.ldo = d; p.bias = (const T *)w.b_o;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_O, m.o, nullptr, d, d, rows, p, dec->tc_actd));
+        AED_TRY(project(KF_GEMM_O, m.o, dec->tc_actd, d, d, sh_o, nullptr, w.b_o));
         // cross-attention block
-        AED_TRY(gamma_planes(w.ln2_g, stats + stats_stride, hid, F));
-        p = sg::StepGemmParams{};
-        p.out = qc; p.ldo = d;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_QC, m.qc, nullptr, d, d, rows, p, dec->tc_actd));
+        AED_TRY(gamma_planes(w.ln2_g, stats + stats_stride, nullptr, 0));
+        AED_TRY(project(KF_GEMM_QC, m.qc, dec->tc_actd, d, d, sh_qc, qc, nullptr));
         if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
             const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
             AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, nullptr,
@@ -1026,22 +1060,15 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
             AED_TRY((launch_attention_fused<T, true, false>(dec, rows, c.max_enc_len, qc, d, cross, c.max_total_enc_frames, nullptr,
                                                             ad_hi, ad_lo, stats + stats_stride, c1_qc, c2_qc, pdl)));
         }
-        p = sg::StepGemmParams{};
-        p.out = x; p.ldo = d; p.bias = (const T *)w.b_o_c;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_OC, m.oc, nullptr, d, d, rows, p, dec->tc_actd));
-        // feed-forward block
-        AED_TRY(gamma_planes(w.ln3_g, stats + 2 * stats_stride, qkv, 3 * d));
-        p = sg::StepGemmParams{};
-        p.out = hid; p.ldo = F;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF1, m.ff1, nullptr, F, d, rows, p, dec->tc_actd));
-        {
-            ProfScope ps(dec, KF_LAYERNORM);
-            AED_TRY(launch_pdl(dec, lnrelu_planes_kernel, dim3((F / 4 + 255) / 256, rows), dim3(256), (const DecState *)dec->state(),
-                               (const float *)hid, F, (const float2 *)(stats + 2 * stats_stride), c1_ff, c2_ff, af_hi, af_lo));
-        }
-        p = sg::StepGemmParams{};
-        p.out = x; p.ldo = d; p.bias = (const T *)w.b_ff2;
-        AED_TRY(launch_step_gemm<sg::B_PLANES>(dec, KF_GEMM_FF2, m.ff2, nullptr, d, F, rows, p, dec->tc_actf));
+        AED_TRY(project(KF_GEMM_OC, m.oc, dec->tc_actd, d, d, sh_o, nullptr, w.b_o_c));
+        // feed-forward block; FFN1's epilogue makes the activation planes of FFN2
+        AED_TRY(gamma_planes(w.ln3_g, stats + 2 * stats_stride, sh_qkv.splits > 1 ? qkv : nullptr, 3 * d));
+        pg::PlaneGemmParams p{};
+        p.epi = pg::PG_RELU_PLANES;
+        p.c1 = c1_ff; p.c2 = c2_ff; p.stats = stats + 2 * stats_stride;
+        p.out_hi = af_hi; p.out_lo = af_lo; p.ldo = F;
+        AED_TRY(launch_plane_gemm(dec, KF_GEMM_FF1, m.ff1, dec->tc_actd, F, d, rows, sh_ff1, p));
+        AED_TRY(project(KF_GEMM_FF2, m.ff2, dec->tc_actf, d, F, sh_ff2, nullptr, w.b_ff2));
     }
     AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
     tc::TcParams tp{};

@@ -868,8 +868,8 @@ __global__ void gamma_planes_kernel(const DecState *state, const float *__restri
                                     int d, float eps, float2 *__restrict__ stats_out, __nv_bfloat16 *__restrict__ out_hi,
                                     __nv_bfloat16 *__restrict__ out_lo, float *__restrict__ zero_buf, int zero_cols)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int r = blockIdx.x;
     if (r >= state->n_active) return;
     __shared__ float red[32];
@@ -916,40 +916,8 @@ __global__ void gamma_planes_kernel(const DecState *state, const float *__restri
             out_lo[(size_t)r * d + i] = __float2bfloat16_rn(y - __bfloat162float(hi));
         }
     }
-    for (int i = threadIdx.x; i < zero_cols; i += blockDim.x) zero_buf[(size_t)r * zero_cols + i] = 0.f;
-}
-
-// planes of relu(rstd * (hidden_raw - mean * c1) + c2): the FFN hidden layer after the folded first projection.
-// grid: x = blocks of 1024 hidden features, y = rows.
-__global__ void lnrelu_planes_kernel(const DecState *state, const float *__restrict__ hid, int f,
-                                     const float2 *__restrict__ stats, const float *__restrict__ c1,
-                                     const float *__restrict__ c2, __nv_bfloat16 *__restrict__ out_hi,
-                                     __nv_bfloat16 *__restrict__ out_lo)
-{
-    const int r = blockIdx.y;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (i < f) {                       // static operands before the dependency wait
-        a = *reinterpret_cast<const float4 *>(c1 + i);
-        b = *reinterpret_cast<const float4 *>(c2 + i);
-    }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (r >= state->n_active || i >= f) return;
-    const float2 st = stats[r];
-    const float4 h = *reinterpret_cast<const float4 *>(hid + (size_t)r * f + i);
-    const float y[4] = {fmaxf(fmaf(st.y, h.x - st.x * a.x, b.x), 0.f), fmaxf(fmaf(st.y, h.y - st.x * a.y, b.y), 0.f),
-                        fmaxf(fmaf(st.y, h.z - st.x * a.z, b.z), 0.f), fmaxf(fmaf(st.y, h.w - st.x * a.w, b.w), 0.f)};
-    __nv_bfloat16 hi[4], lo[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        hi[j] = __float2bfloat16_rn(y[j]);
-        lo[j] = __float2bfloat16_rn(y[j] - __bfloat162float(hi[j]));
-    }
-    __nv_bfloat162 *ph = reinterpret_cast<__nv_bfloat162 *>(out_hi + (size_t)r * f + i);
-    __nv_bfloat162 *pl = reinterpret_cast<__nv_bfloat162 *>(out_lo + (size_t)r * f + i);
-    ph[0] = __halves2bfloat162(hi[0], hi[1]); ph[1] = __halves2bfloat162(hi[2], hi[3]);
-    pl[0] = __halves2bfloat162(lo[0], lo[1]); pl[1] = __halves2bfloat162(lo[2], lo[3]);
+    if (zero_buf)
+        for (int i = threadIdx.x; i < zero_cols; i += blockDim.x) zero_buf[(size_t)r * zero_cols + i] = 0.f;
 }
 
 // ------------------------------------------------------------------------------------------------------------

@@ -433,6 +433,30 @@ def test_several_steps_per_graph(dtype, steps):
     _run_both(w)
 
 
+@pytest.mark.parametrize("model, batch", [("odd", 129), ("wide_a", 193), ("odd", 320), ("wide_b", 321), ("odd", 385)])
+def test_plane_projections(model, batch):
+    """The row counts at which the projections of many rows change their tiles (two of 96, 128 and 160, three and four of
+    128, FFN1 in more), with an odd number of 128-feature tiles and tiles that end inside one."""
+    rng = np.random.default_rng(990 + batch)
+    m = {"wide_a": WIDE_A, "wide_b": WIDE_B, "odd": ODD}[model]
+    w = wl.make_custom(m, rng.integers(1, 20, size=batch), rng.integers(1, 4, size=batch), dtype="bf16", seed=390 + batch, out_std=0.1,
+                       ln_std=0.2, bias_std=0.05)
+    _run_both(w, rows=sorted({0, 31, 32, 95, 96, batch // 2, batch - 2, batch - 1}))
+
+
+F32_DEEP = dict(n_layers=2, d_model=320, n_heads=5, d_ffn=1344, vocab=517, d_enc=192)
+
+
+@pytest.mark.parametrize("batch", [1, 4, 5, 16, 17, 23])
+def test_fp32_row_tiles(batch):
+    """Rows around the steps between 4-row and 8-row tiles and one and two features per warp of the fp32 projections, with
+    K beyond the weights held ahead, K no multiple of 128 and feature counts that end inside a block."""
+    rng = np.random.default_rng(995 + batch)
+    w = wl.make_custom(F32_DEEP, rng.integers(1, 40, size=batch), rng.integers(1, 6, size=batch), dtype="fp32", seed=400 + batch, out_std=0.1,
+                       ln_std=0.2)
+    _run_both(w)
+
+
 @pytest.mark.parametrize("model", ["wide_b", "odd"])
 def test_small_batch_model_shapes(model):
     """d_model 1024 with 16 heads at 64 rows, and a model whose widths are not multiples of 128 (an odd number of

@@ -186,8 +186,8 @@ __global__ void fill_pe_kernel(float *pe, int max_len, int d)
 
 // x[r] = E[token of utterance] * sqrt(d) + PE[t_u]
 template <typename T>
-__global__ void embed_kernel(const DecState *state, const int32_t *__restrict__ active_list,
-                             const int32_t *__restrict__ tokens, const int32_t *__restrict__ t_u,
+__global__ void embed_kernel(const DecState *state, const int32_t *active_list,
+                             const int32_t *tokens, const int32_t *t_u,
                              const T *__restrict__ embed, const float *__restrict__ pe, int d, int vocab, float scale,
                              float *__restrict__ x, float *__restrict__ zero_buf = nullptr, int zero_cols = 0,
                              float *__restrict__ zero_buf2 = nullptr, int zero_cols2 = 0)
@@ -401,12 +401,14 @@ template <int N> __device__ __forceinline__ void load_n(const float *p, float (&
 // kRowStats: the block computes (mean, rstd) of its row of stats_x itself instead of reading ln_stats.
 template <typename CT, bool kCross, bool kAppend, bool kPipe = false, bool kRowStats = false>
 __global__ void __launch_bounds__(kFusedMaxWarps * 32, sizeof(CT) == 4 ? 1 : ((kAppend || kPipe) ? 2 : (LaneWidth<CT>::kE > 8 ? 3 : 4)))      // self-attention holds the new key/value as well; wider lanes and fp32 need more registers
-attn_fused_kernel(const DecState *state, const int4 *__restrict__ row_info, const float *__restrict__ q, int ldq,
+attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, int ldq,
                   CT *__restrict__ cache, int n_heads, int seq_capacity, float scale,
                   float *__restrict__ out, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, int ldo,
-                  const float2 *__restrict__ ln_stats, const float *__restrict__ ln_c1, const float *__restrict__ ln_c2,
-                  const float *__restrict__ stats_x = nullptr, float ln_eps = 0.f)
+                  const float2 *ln_stats, const float *__restrict__ ln_c1, const float *__restrict__ ln_c2,
+                  const float *stats_x = nullptr, float ln_eps = 0.f)
 {
+    // (What earlier kernels of the step write is not __restrict__: this kernel is resident before they have finished, and loads
+    // through the read-only path may return what their lines held then.)
     // stats_x: rows [*, heads * 64] whose (mean, rstd) this block computes itself instead of reading ln_stats (the
     // kernel before this one completed those rows, so nobody could have computed the statistics earlier).
     // Launched with programmatic stream serialization.  Before the dependency wait only data that no kernel of
@@ -422,6 +424,13 @@ attn_fused_kernel(const DecState *state, const int4 *__restrict__ row_info, cons
         asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
+    // The next kernel may start at once where that is a few-row projection, so that its weights are on their way while this
+    // one still waits (24 layers, 4 / 8 / 24 rows: 499 / 513 / 681 -> 473 / 486 / 661 us per step).  Not the cross-attention of
+    // steps with more than 128 rows, which read their statistics (no kRowStats): blocks of the next kernel would take room from
+    // its own later ones (200 / 512 rows 2130 / 3488 -> 2224 / 3650).  Nor fp32, whose projections hold their weights in
+    // registers (2 layers, 4 / 8 rows: 54 / 70 us per step against 59 / 75).
+    constexpr bool kEarly = sizeof(CT) < 4 && (!kCross || kRowStats);
+    if (kEarly) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const int u = ri.x;
     const int len = kCross ? ri.z : ri.y + 1;
@@ -485,7 +494,7 @@ attn_fused_kernel(const DecState *state, const int4 *__restrict__ row_info, cons
     AED_TRACE_RESERVE(tcur, state, (threadIdx.x == 0 && blockIdx.x == 0) ? 6u : 0u);
     AED_TRACE_PUT_NS(state, tcur, 8 + (kCross ? 1 : 0));      // resident, first chunk requested
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!kEarly) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     AED_TRACE_PUT(state, tcur, 3);                          // dependency resolved
     // Everything this block needs from earlier kernels is requested in one round: statistics, query, and (in the
     // warp that owns the new position) the new key and value.  When the projection ran on gamma*x, its raw output
@@ -654,10 +663,10 @@ attn_fused_kernel(const DecState *state, const int4 *__restrict__ row_info, cons
 // 6.2 TB/s; at up to 8 positions a launch went from about 26 us with a block per pair to 6).
 template <typename CT, bool kAppend>
 __global__ void __launch_bounds__(256, 3)
-self_attn_warp_kernel(const DecState *state, const int4 *__restrict__ row_info, const float *__restrict__ q, int ldq,
+self_attn_warp_kernel(const DecState *state, const int4 *row_info, const float *q, int ldq,
                       CT *__restrict__ cache, int n_heads, int seq_capacity, float scale, float *__restrict__ out,
                       __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, int ldo,
-                      const float2 *__restrict__ ln_stats, const float *__restrict__ ln_c1, const float *__restrict__ ln_c2, int row_heads)
+                      const float2 *ln_stats, const float *__restrict__ ln_c1, const float *__restrict__ ln_c2, int row_heads)
 {
     constexpr int kE = LaneWidth<CT>::kE, kDG = kHeadDim / kE, kPG = 32 / kDG, kChunk = 4 * kPG;
     const int lane = threadIdx.x & 31, rh = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -800,7 +809,7 @@ attn_combine_kernel(const DecState *state, const int32_t *__restrict__ active_li
 // LayerNorm whose result is written as bf16 high and low planes [row, d]; the same block also clears the fp32
 // rows that the following split-K projection accumulates into (zero_cols columns of zero_buf, if any).
 template <int kMaxPerThread>
-__global__ void layernorm_planes_kernel(const DecState *state, const float *__restrict__ x,
+__global__ void layernorm_planes_kernel(const DecState *state, const float *x,
                                         const __nv_bfloat16 *__restrict__ g, const __nv_bfloat16 *__restrict__ b, int d,
                                         float eps, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo,
                                         float *__restrict__ zero_buf, int zero_cols)
@@ -864,7 +873,7 @@ __global__ void layernorm_planes_kernel(const DecState *state, const float *__re
 // planes of gamma * x, the LayerNorm statistics (mean, rstd) of every row, and the clearing of the fp32 rows a later
 // split-K projection accumulates into (zero_cols columns of zero_buf, if any).  One block per row.
 template <int kMaxPerThread>
-__global__ void gamma_planes_kernel(const DecState *state, const float *__restrict__ x, const __nv_bfloat16 *__restrict__ g,
+__global__ void gamma_planes_kernel(const DecState *state, const float *x, const __nv_bfloat16 *__restrict__ g,
                                     int d, float eps, float2 *__restrict__ stats_out, __nv_bfloat16 *__restrict__ out_hi,
                                     __nv_bfloat16 *__restrict__ out_lo, float *__restrict__ zero_buf, int zero_cols)
 {
@@ -966,8 +975,8 @@ __global__ void embed_rows_kernel(const DecState *state, const int4 *__restrict_
 // rounded as the cache stores it), before any row attends: in a prefill pass a row reads positions that other rows of
 // the same pass append.  grid: (rows, heads), 64 threads.
 template <typename CT>
-__global__ void append_kv_kernel(const DecState *state, const int4 *__restrict__ row_info, const float *__restrict__ qkv, int ldq,
-                                 CT *__restrict__ cache, int n_heads, int seq_capacity, const float2 *__restrict__ ln_stats,
+__global__ void append_kv_kernel(const DecState *state, const int4 *row_info, const float *qkv, int ldq,
+                                 CT *__restrict__ cache, int n_heads, int seq_capacity, const float2 *ln_stats,
                                  const float *__restrict__ ln_c1, const float *__restrict__ ln_c2)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -96,7 +96,7 @@ KERNEL_OF_FAMILY = {
     "gemm_oc": "step_gemm_kernel", "gemm_ff1": "step_gemm_kernel", "gemm_ff2": "step_gemm_kernel",
     "attn_self": "attn_fused_kernel", "attn_cross": "attn_fused_kernel", "attn_combine": "attn_combine_kernel",
     "gemm_vocab": "tc_gemm_kernel", "precompute_cross_kv": "crosskv_gemm_kernel", "layernorm": "layernorm_planes_kernel",
-    "embed": "embed_kernel", "bookkeeping": "build_active/finish_step",
+    "embed": "embed_kernel", "bookkeeping": "step_rows/finish_step",
 }
 
 # DRAM bytes per algorithmic byte of a kernel, from the ncu captures summarised under profiles/ (dram__bytes_read.sum +

@@ -20,7 +20,7 @@ def _stale() -> bool:
     if not os.path.exists(OUT):
         return True
     built = os.path.getmtime(OUT)
-    deps = _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    deps = _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         glob.glob(os.path.join(_HERE, "..", "include", "*.h"))
     return any(os.path.getmtime(p) > built for p in deps)
 

@@ -74,3 +74,18 @@ def test_bucketing_reduces_padding():
     assert pe_b < 0.3 and pd_b < 0.3 and pe_b < pe_r / 2 and pd_b < pd_r / 2
     for b in buck:
         assert len(b) * (w.enc_lens[b].max() + w.dec_lens[b].max()) <= 65536 or len(b) == 1
+
+
+@pytest.mark.parametrize("pattern", ["*.cu", "*.cuh", "*.h"])
+def test_a_changed_source_is_built_again(lib, pattern, monkeypatch):
+    """The incremental build looks at every kind of source file, the plain C++ headers among them."""
+    import glob
+    from paper_2503_05931_b200 import build_ext
+    assert not build_ext._stale()
+    files = glob.glob(os.path.join(build_ext.CSRC, pattern))
+    assert files
+    real = os.path.getmtime
+    for newer in files:
+        monkeypatch.setattr(os.path, "getmtime", lambda p: real(p) + (1e9 if os.path.samefile(p, newer) else 0))
+        assert build_ext._stale(), newer
+        monkeypatch.setattr(os.path, "getmtime", real)

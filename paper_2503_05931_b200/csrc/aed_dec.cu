@@ -504,7 +504,7 @@ bool encode_map(CUtensorMap *map, const void *base, size_t rows, size_t cols, in
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-constexpr int kTcSmemBudget = 200 * 1024;
+using tc::kTcSmemBudget;
 
 aed_status_t tc_setup(aed_dec *dec)
 {
@@ -622,41 +622,21 @@ aed_status_t tc_setup(aed_dec *dec)
     return AED_OK;
 }
 
-// MMA N (a multiple of 16) for rows_ub rows in tiles of at most `most`: as few tiles as possible, of equal size, because
-// a tile's operand traffic and tensor time go with its N whether its rows are real or padding.  (Tiles of a power of two
-// against this, per step of the 24-layer model: 72 rows 1387 -> 1278 us, 136 rows 2109 -> 1856, 192 rows 2323 -> 2120.)
-int tc_n_tile(int rows_ub, int most)
-{
-    const int tiles = (rows_ub + most - 1) / most;
-    return std::max(16, ((rows_ub + tiles - 1) / tiles + 15) / 16 * 16);
-}
-
 // The vocabulary projection on tensor cores: logits[r, v] = sum_k act[r, k] * Wout[v, k] (+ bias), argmax in the epilogue.
 aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int rows_fixed = -1)
 {
     ProfScope ps(dec, KF_GEMM_VOCAB);
-    const int M = dec->cfg.vocab, K = dec->cfg.d_model;
-    const int n_tile = tc_n_tile(rows_ub, 256), ni = n_tile / 16 - 1;
-    const int row_tiles = (rows_ub + n_tile - 1) / n_tile, m_tiles = (M + tc::kTileM - 1) / tc::kTileM;
-    const int k_blocks = K / tc::kBlockK;
-    p.a_rows = M;
-    p.n_tile = n_tile;
-    p.k_blocks = k_blocks;
+    const VocabShape shape = vocab_shape(rows_ub, dec->cfg.d_model / tc::kBlockK);
+    p.a_rows = dec->cfg.vocab;
+    p.n_tile = shape.n_tile;
+    p.k_blocks = dec->cfg.d_model / tc::kBlockK;
     p.use_lo = 1;
     p.rows_fixed = rows_fixed;          // >= 0: only that many rows (a prefill pass projects its last-position rows only)
     p.state = dec->state();
-    const int stage_bytes = tc::kATileBytes + 2 * n_tile * tc::kBlockK * 2;
-    int stages = kTcSmemBudget / stage_bytes;
-    if (stages > tc::kMaxStages) stages = tc::kMaxStages;
-    if (stages > k_blocks) stages = k_blocks;
-    // every ring stage belongs to one issuing thread: as many producers as stages (at most one per producer warp)
-    int producers = stages >= tc::kProducerWarps ? tc::kProducerWarps : stages;
-    stages -= stages % producers;
-    const CUtensorMap *acts = dec->tc_actd[ni];
-    dim3 grid(m_tiles, 1, row_tiles);
-    void *args[] = {(void *)&dec->tc_w_out, (void *)&acts[0], (void *)&acts[1], &p, &stages, (void *)&producers};
-    return launch_pdl_impl(dec, (const void *)tc::tc_gemm_kernel, grid, dim3(tc::kThreads),
-                           (size_t)stages * stage_bytes + 1024, args);
+    const CUtensorMap *acts = dec->tc_actd[shape.n_tile / 16 - 1];
+    dim3 grid((p.a_rows + tc::kTileM - 1) / tc::kTileM, 1, shape.row_tiles);
+    void *args[] = {(void *)&dec->tc_w_out, (void *)&acts[0], (void *)&acts[1], &p, (void *)&shape.stages, (void *)&shape.producers};
+    return launch_pdl_impl(dec, (const void *)tc::tc_gemm_kernel, grid, dim3(tc::kThreads), shape.smem, args);
 }
 
 aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const void *g, const void *b, float *zero_buf,

@@ -23,16 +23,12 @@
 
 #include "bounded_wait.h"
 #include "common.cuh"
+#include "launch_shapes.h"
 
 namespace aed {
 namespace tc {
 
-constexpr int kBlockK = 64;                    // bf16 elements per k-block = one 128-byte swizzle row
-constexpr int kTileM = 128;
-constexpr int kATileBytes = kTileM * kBlockK * 2;
-constexpr int kMaxStages = 8;
 constexpr int kThreads = 416;                    // 8 producer warps, 1 MMA warp, 4 more for the epilogue
-constexpr int kProducerWarps = 8;                // (a k-block is three copies, and a thread's copies complete one after the other)
 constexpr long long kWaitCycles = 2000000000ll;   // about a second at B200 clocks
 constexpr int kErrTimeout = 2;
 
@@ -146,7 +142,7 @@ struct TcParams {
     DecState *state;
 };
 
-// grid: x = 128-row tiles of A, y = k-splits, z = N-row tiles of B.  Dynamic shared memory: stage ring + 1024.
+// grid: x = 128-row tiles of A, y = k-splits, z = N-row tiles of B.  Dynamic shared memory: see vocab_shape.
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b_lo, TcParams p, int stages, int producers)
@@ -248,7 +244,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
     // ---- epilogue: all warps but the one that issues the MMAs (the producers have nothing left to do) -------------
     if (warp != kProducerWarps) {
-        constexpr int kPitch = kTileM + 4;
+        constexpr int kPitch = kRowPitch;
         const int ew = warp < kProducerWarps ? warp : warp - 1;      // 0..11
         const int quarter = warp & 3;                                // tensor memory lanes this warp can reach
         const int third = warp < 4 ? 0 : warp < kProducerWarps ? 1 : 2;      // three warps per quarter share the rows in 16s

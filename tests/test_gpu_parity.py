@@ -447,6 +447,17 @@ def test_plane_projections(model, batch):
 F32_DEEP = dict(n_layers=2, d_model=320, n_heads=5, d_ffn=1344, vocab=517, d_enc=192)
 
 
+@pytest.mark.parametrize("batch", [16, 17, 63, 64, 65, 80, 128, 129, 256, 257, 300])
+def test_vocabulary_projection_of_one_k_block(batch):
+    """d_model 64: the ring of the vocabulary projection has one stage, and the accumulator's rows need more room than it
+    in tiles of 64 rows and more; row tiles of 16 to 256, one and two of them, on either side of the switch to ready-made planes."""
+    model = dict(n_layers=2, d_model=64, n_heads=1, d_ffn=128, vocab=333, d_enc=64)
+    rng = np.random.default_rng(600 + batch)
+    w = wl.make_custom(model, rng.integers(1, 40, size=batch), rng.integers(1, 4, size=batch), dtype="bf16", seed=601 + batch, out_std=0.4)
+    rows = sorted({0, 15, 16, 63, 64, 79, 127, 128, 255, 256, batch - 1} & set(range(batch)))
+    _run_both(w, rows=rows, label=f"d64 B={batch}")
+
+
 @pytest.mark.parametrize("batch", [1, 4, 5, 16, 17, 23])
 def test_fp32_row_tiles(batch):
     """Rows around the steps between 4-row and 8-row tiles and one and two features per warp of the fp32 projections, with

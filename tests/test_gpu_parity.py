@@ -458,6 +458,24 @@ def test_vocabulary_projection_of_one_k_block(batch):
     _run_both(w, rows=rows, label=f"d64 B={batch}")
 
 
+@pytest.mark.parametrize("dtype, batch", [("fp32", 3), ("fp32", 12), ("fp32", 21)])
+def test_vectors_at_any_element(dtype, batch, monkeypatch):
+    """LayerNorm parameters and biases that start one element past a 16-byte boundary."""
+    b = _binding()
+    upload = b.Decoder._upload
+
+    def shifted(self, arr):
+        arr = np.asarray(arr)
+        if arr.ndim != 1:
+            return upload(self, arr)
+        return upload(self, np.concatenate([np.zeros(1, arr.dtype), arr])) + self.tdtype.itemsize
+    monkeypatch.setattr(b.Decoder, "_upload", shifted)
+    rng = np.random.default_rng(620 + batch)
+    w = wl.make_custom(MID, rng.integers(1, 60, size=batch), rng.integers(1, 5, size=batch), dtype=dtype, seed=621 + batch, out_std=0.3,
+                       ln_std=0.3, out_bias_std=0.1)
+    _run_both(w, rows=sorted({0, batch // 2, batch - 1}), label=f"shifted vectors B={batch}")
+
+
 @pytest.mark.parametrize("batch", [1, 4, 5, 16, 17, 23])
 def test_fp32_row_tiles(batch):
     """Rows around the steps between 4-row and 8-row tiles and one and two features per warp of the fp32 projections, with

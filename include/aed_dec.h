@@ -84,7 +84,8 @@ typedef struct {
 
 /* All members are DEVICE pointers to tensors of the configured dtype.  The per-layer members are HOST arrays
  * of n_layers DEVICE pointers (the arrays are copied at creation, the tensors are borrowed).  A NULL bias
- * pointer (or a NULL per-layer bias array) means "no bias".
+ * pointer (or a NULL per-layer bias array) means "no bias".  Matrices, and the encoder states of later calls, start at a
+ * 16-byte boundary; vectors (LayerNorm parameters, biases) may start at any element.
  * w_qkv rows: d query rows, then d key rows, then d value rows.  w_kv_c rows: d key rows, then d value rows. */
 typedef struct {
     const void *embed;      /* [vocab, d_model] */

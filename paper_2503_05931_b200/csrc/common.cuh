@@ -128,6 +128,18 @@ __device__ __forceinline__ void load4(const __nv_bfloat16 *p, float (&v)[4])
     v[2] = __uint_as_float(raw.y << 16); v[3] = __uint_as_float(raw.y & 0xFFFF0000u);
 }
 
+// N consecutive elements of a vector that the caller may have put at any element; aligned: it starts at a 16-byte boundary.
+template <int N, typename T> __device__ __forceinline__ void load_vec(const T *p, bool aligned, float (&v)[N])
+{
+    static_assert(N == 4 || N == 8, "load4 or load8");
+    if (!aligned) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = to_f32(p[i]);
+    } else if constexpr (N == 8) load8(p, v);
+    else load4(p, v);
+}
+__device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 // One byte of the 8-bit floating-point format E4M3 (1 sign, 4 exponent bits with bias 7, 3 mantissa bits, no
 // infinities, largest finite value 448): the optional storage type of the cross-attention K/V store.
 struct fp8e4m3 { uint8_t bits; };

@@ -59,7 +59,7 @@ __device__ __forceinline__ float reduce_transposed(float (&v)[N], int lane)
 }
 
 // 4 values of a vector that the caller may have put at any element (only matrices have to be 16-byte aligned)
-__device__ __forceinline__ float4 load_vec(const float *p, bool aligned)
+__device__ __forceinline__ float4 load_vec4(const float *p, bool aligned)
 {
     return aligned ? __ldg(reinterpret_cast<const float4 *>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
 }
@@ -124,7 +124,7 @@ rows_kernel(const RowsArgs p)
                 v = *reinterpret_cast<const float4 *>(p.a + static_cast<size_t>(row0 + r) * K + k0 + k);
                 if (p.ln_g) {
                     const float2 st = s_stat[r];
-                    const float4 g = load_vec(p.ln_g + k0 + k, ln_aligned), b = load_vec(p.ln_b + k0 + k, ln_aligned);
+                    const float4 g = load_vec4(p.ln_g + k0 + k, ln_aligned), b = load_vec4(p.ln_b + k0 + k, ln_aligned);
                     v.x = fmaf(g.x * (v.x - st.x), st.y, b.x); v.y = fmaf(g.y * (v.y - st.x), st.y, b.y);
                     v.z = fmaf(g.z * (v.z - st.x), st.y, b.z); v.w = fmaf(g.w * (v.w - st.x), st.y, b.w);
                 }

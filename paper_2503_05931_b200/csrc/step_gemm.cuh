@@ -301,6 +301,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         float *const out = second_w ? p.out2 : p.out;
         const int ldo = second_w ? p.ldo2 : p.ldo;
         const __nv_bfloat16 *const gamma = second_w ? p.gamma2 : p.gamma;
+        const bool gamma_aligned = aligned16(gamma);
         float dv[2][8];
         if (direct && rbase < p.n_tile) {          // one row per thread (n_tile <= 32), both k-blocks requested at once
             const int rs = min(row0 + rbase, p.src_rows - 1);
@@ -316,7 +317,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
             const float *src_tile = reinterpret_cast<const float *>(lo_tile + plane_bytes);
             const int k = (kb_begin + i) * kBlockK + c * 8;
             float g[8], c1[8], c2[8];
-            if (MODE == B_GAMMA) load8(gamma + k, g);
+            if (MODE == B_GAMMA) load_vec(gamma + k, gamma_aligned, g);
             if (MODE == B_LN_RELU) { load8(p.c1 + k, c1); load8(p.c2 + k, c2); }
             if (!direct) ok = mbar_wait(&bar_s[s], (i / S) & 1, &abort_flag);
             if (!ok) break;

@@ -92,6 +92,7 @@ vocab_gemv_kernel(const __grid_constant__ CUtensorMap map_w, VocabGemvParams p)
     // ---- rows 2 * warp and 2 * warp + 1: statistics and planes ------------------------------------------------------
     const int n_rows = p.state->n_active;
     sg::pdl_wait();
+    const bool gamma_aligned = aligned16(p.gamma);
     const int per_lane = p.d_model / 128;                     // 16-byte loads per lane and row (d_model is a multiple of 128 here)
 #pragma unroll
     for (int rr = 0; rr < 2; ++rr) {
@@ -111,7 +112,7 @@ vocab_gemv_kernel(const __grid_constant__ CUtensorMap map_w, VocabGemvParams p)
                 const float d0 = v.x - mean, d1 = v.y - mean, d2 = v.z - mean, d3 = v.w - mean;
                 q += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
                 float g[4];
-                load4(p.gamma + k, g);
+                load_vec(p.gamma + k, gamma_aligned, g);
                 uint32_t h0, l0, h1, l1;
                 sv::split2(v.x * g[0], v.y * g[1], h0, l0);
                 sv::split2(v.z * g[2], v.w * g[3], h1, l1);

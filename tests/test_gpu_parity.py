@@ -458,7 +458,7 @@ def test_vocabulary_projection_of_one_k_block(batch):
     _run_both(w, rows=rows, label=f"d64 B={batch}")
 
 
-@pytest.mark.parametrize("dtype, batch", [("fp32", 3), ("fp32", 12), ("fp32", 21)])
+@pytest.mark.parametrize("dtype, batch", [("fp32", 3), ("fp32", 12), ("fp32", 21), ("bf16", 3), ("bf16", 12), ("bf16", 40), ("bf16", 70), ("bf16", 131)])
 def test_vectors_at_any_element(dtype, batch, monkeypatch):
     """LayerNorm parameters and biases that start one element past a 16-byte boundary."""
     b = _binding()

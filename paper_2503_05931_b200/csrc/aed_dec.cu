@@ -405,10 +405,13 @@ aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, 
     p.eps = dec->cfg.ln_eps;
     p.after_rows = after_rows;
     void *args[] = {&p};
-    auto grid = [&](int rt, int fpw) { return dim3((p.M + warps * fpw - 1) / (warps * fpw), (rows_ub + rt - 1) / rt); };
-    if (rows_ub <= 4) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 4, 1>, grid(4, 1), dim3(warps * 32), f32::rows_smem(4, p.K), args);
-    if (rows_ub <= 16) return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 1>, grid(8, 1), dim3(warps * 32), f32::rows_smem(8, p.K), args);
-    return launch_pdl_impl(dec, (const void *)f32::rows_kernel<EPI, 8, 2>, grid(8, 2), dim3(warps * 32), f32::rows_smem(8, p.K), args);
+    const bool vec = aligned16(p.ln_g) && aligned16(p.ln_b);          // (or no LayerNorm)
+    const void *kernel = rows_ub <= 4    ? (vec ? (const void *)f32::rows_kernel<EPI, 4, 1, true> : (const void *)f32::rows_kernel<EPI, 4, 1, false>)
+                         : rows_ub <= 16 ? (vec ? (const void *)f32::rows_kernel<EPI, 8, 1, true> : (const void *)f32::rows_kernel<EPI, 8, 1, false>)
+                                         : (vec ? (const void *)f32::rows_kernel<EPI, 8, 2, true> : (const void *)f32::rows_kernel<EPI, 8, 2, false>);
+    const int rt = rows_ub <= 4 ? 4 : 8, fpw = rows_ub <= 16 ? 1 : 2;
+    const dim3 grid((p.M + warps * fpw - 1) / (warps * fpw), (rows_ub + rt - 1) / rt);
+    return launch_pdl_impl(dec, kernel, grid, dim3(warps * 32), f32::rows_smem(rt, p.K), args);
 }
 
 // The forward pass of one step in fp32 for the rows in the active list (at most rows_ub of them): 8 kernels per layer, chained

@@ -138,7 +138,7 @@ template <int N, typename T> __device__ __forceinline__ void load_vec(const T *p
     } else if constexpr (N == 8) load8(p, v);
     else load4(p, v);
 }
-__device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+__host__ __device__ __forceinline__ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 // One byte of the 8-bit floating-point format E4M3 (1 sign, 4 exponent bits with bias 7, 3 mantissa bits, no
 // infinities, largest finite value 448): the optional storage type of the cross-attention K/V store.

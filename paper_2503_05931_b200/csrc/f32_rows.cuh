@@ -58,14 +58,10 @@ __device__ __forceinline__ float reduce_transposed(float (&v)[N], int lane)
     return s;
 }
 
-// 4 values of a vector that the caller may have put at any element (only matrices have to be 16-byte aligned)
-__device__ __forceinline__ float4 load_vec4(const float *p, bool aligned)
-{
-    return aligned ? __ldg(reinterpret_cast<const float4 *>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
-}
-
 // grid: x = blocks of blockDim / 32 * FPW output features, y = tiles of RT rows.
-template <int EPI, int RT, int FPW>
+// kLnVec: the LayerNorm vectors are read 16 bytes at a time, otherwise one value (the caller may have put them at any element).
+// A form of its own and not a test in the loop: that took 54 us instead of 52 per step of 4 rows of the 2-layer model.
+template <int EPI, int RT, int FPW, bool kLnVec>
 __global__ void __launch_bounds__(kWarps * 32)
 rows_kernel(const RowsArgs p)
 {
@@ -110,7 +106,9 @@ rows_kernel(const RowsArgs p)
         }
         __syncthreads();
     }
-    const bool ln_aligned = ((reinterpret_cast<uintptr_t>(p.ln_g) | reinterpret_cast<uintptr_t>(p.ln_b)) & 15) == 0;
+    auto load_ln = [](const float *v) {
+        return kLnVec ? __ldg(reinterpret_cast<const float4 *>(v)) : make_float4(__ldg(v), __ldg(v + 1), __ldg(v + 2), __ldg(v + 3));
+    };
     float acc[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) acc[i] = 0.f;
@@ -124,7 +122,7 @@ rows_kernel(const RowsArgs p)
                 v = *reinterpret_cast<const float4 *>(p.a + static_cast<size_t>(row0 + r) * K + k0 + k);
                 if (p.ln_g) {
                     const float2 st = s_stat[r];
-                    const float4 g = load_vec4(p.ln_g + k0 + k, ln_aligned), b = load_vec4(p.ln_b + k0 + k, ln_aligned);
+                    const float4 g = load_ln(p.ln_g + k0 + k), b = load_ln(p.ln_b + k0 + k);
                     v.x = fmaf(g.x * (v.x - st.x), st.y, b.x); v.y = fmaf(g.y * (v.y - st.x), st.y, b.y);
                     v.z = fmaf(g.z * (v.z - st.x), st.y, b.z); v.w = fmaf(g.w * (v.w - st.x), st.y, b.w);
                 }

@@ -1071,7 +1071,6 @@ aed_status_t precompute_tc(aed_dec *dec, const void *enc_base, long long enc_row
     typedef __nv_bfloat16 T;
     const auto &c = dec->cfg;
     const Layout &L = dec->lay;
-    if (reinterpret_cast<uintptr_t>(enc_base) % 16) return fail(dec, AED_ERR_INVALID_ARG, "the encoder states must be 16-byte aligned");
     CUtensorMap map_enc;
     if (!encode_map(&map_enc, enc_base, (size_t)enc_rows, c.d_enc, tc::kTileM))
         return fail(dec, AED_ERR_CUDA, "cuTensorMapEncodeTiled failed for the encoder states");
@@ -1227,6 +1226,13 @@ extern "C" aed_status_t aed_dec_create(const aed_dec_config_t *config, const aed
         for (int l = 0; l < config->n_layers; ++l)
             if (!arr[l]) return fail(nullptr, AED_ERR_INVALID_ARG, "a required weight of layer %d is NULL", l);
     }
+    if (config->dtype == AED_DTYPE_F32) {
+        // (in the bf16 configuration the tensor maps refuse the same)
+        bool ok = aligned16(w->w_out);
+        for (auto arr : {w->w_qkv, w->w_o, w->w_q_c, w->w_kv_c, w->w_o_c, w->w_ff1, w->w_ff2})
+            for (int l = 0; l < config->n_layers; ++l) ok = ok && aligned16(arr[l]);
+        if (!ok) return fail(nullptr, AED_ERR_INVALID_ARG, "weight matrices must be 16-byte aligned");
+    }
     aed_dec *dec = new (std::nothrow) aed_dec();
     if (!dec) return fail(nullptr, AED_ERR_INVALID_ARG, "out of host memory");
     dec->cfg = *config;
@@ -1281,11 +1287,18 @@ extern "C" aed_status_t aed_dec_create(const aed_dec_config_t *config, const aed
     return AED_OK;
 }
 
+// (both configurations read the states 16 bytes at a time)
+static aed_status_t check_encoder_states(aed_dec *dec, const void *enc)
+{
+    return aligned16(enc) ? AED_OK : fail(dec, AED_ERR_INVALID_ARG, "the encoder states must be 16-byte aligned");
+}
+
 extern "C" aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *enc_packed, const int32_t *enc_lens,
                                                     int32_t batch)
 {
     if (!dec) return AED_ERR_INVALID_ARG;
     if (!enc_packed || !enc_lens) return fail(dec, AED_ERR_INVALID_ARG, "enc_packed and enc_lens must not be NULL");
+    AED_TRY(check_encoder_states(dec, enc_packed));
     if (batch < 1) return fail(dec, AED_ERR_INVALID_ARG, "batch must be at least 1");
     if (batch > dec->cfg.max_batch) return fail(dec, AED_ERR_CAPACITY, "batch %d exceeds max_batch %d", batch, dec->cfg.max_batch);
     long long total = 0;
@@ -1682,6 +1695,7 @@ extern "C" aed_status_t aed_dec_admit(aed_dec_t *dec, int32_t slot, const void *
     if (!dec) return AED_ERR_INVALID_ARG;
     if (!dec->have_batch || !dec->slot_mode) return fail(dec, AED_ERR_STATE, "aed_dec_admit needs slots: call aed_dec_open_slots first");
     if (!enc) return fail(dec, AED_ERR_INVALID_ARG, "enc must not be NULL");
+    AED_TRY(check_encoder_states(dec, enc));
     const Admission a{slot, 0, enc_len, max_len};
     AED_TRY(check_admission(dec, a));           // before enc_len is used as the extent of the tensor
     return admit_many(dec, enc, enc_len, &a, 1, out_lens);
@@ -1743,6 +1757,7 @@ extern "C" aed_status_t aed_dec_decode_stream(aed_dec_t *dec, const void *enc_pa
     if (!dec) return AED_ERR_INVALID_ARG;
     if (!enc_packed || !enc_lens || !max_lens || !tokens_out || !out_lens)
         return fail(dec, AED_ERR_INVALID_ARG, "enc_packed, enc_lens, max_lens, tokens_out and out_lens must not be NULL");
+    AED_TRY(check_encoder_states(dec, enc_packed));
     if (n < 1) return fail(dec, AED_ERR_INVALID_ARG, "n must be at least 1");
     const auto &c = dec->cfg;
     const bool eos = c.eos_id >= 0;

@@ -476,6 +476,31 @@ def test_vectors_at_any_element(dtype, batch, monkeypatch):
     _run_both(w, rows=sorted({0, batch // 2, batch - 1}), label=f"shifted vectors B={batch}")
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_encoder_states_have_to_be_aligned(dtype):
+    """Encoder states off a 16-byte boundary are refused by every call that takes them, and the batch of before goes on."""
+    import torch
+    b = _binding()
+    w = wl.make_custom(SMALL, [9, 5], [3, 3], dtype=dtype, seed=630)
+    dec = b.decoder_for_workload(w)
+    enc = dec.upload_encoder(w.enc)
+    dec.precompute_cross_kv(enc, w.enc_lens)
+    bad = torch.zeros(enc.numel() + 1, dtype=enc.dtype, device="cuda:0")[1:].view(enc.shape)
+    with pytest.raises(b.AedError) as e:
+        dec.precompute_cross_kv(bad, w.enc_lens)
+    assert e.value.status == b.AED_ERR_INVALID_ARG
+    with pytest.raises(b.AedError) as e:
+        dec.decode_stream(bad, w.enc_lens, w.dec_lens, 1)
+    assert e.value.status == b.AED_ERR_INVALID_ARG
+    toks, lens = dec.greedy_decode(w.dec_lens)
+    assert np.array_equal(lens.cpu().numpy(), w.dec_lens)
+    dec.open_slots(1)
+    with pytest.raises(b.AedError) as e:
+        dec.admit(0, bad[:9], 3)
+    assert e.value.status == b.AED_ERR_INVALID_ARG
+    dec.close()
+
+
 @pytest.mark.parametrize("batch", [1, 4, 5, 16, 17, 23])
 def test_fp32_row_tiles(batch):
     """Rows around the steps between 4-row and 8-row tiles and one and two features per warp of the fp32 projections, with

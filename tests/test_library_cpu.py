@@ -56,6 +56,28 @@ def test_workspace_bytes_and_validation(lib):
     lib.aed_dec_destroy(None)
 
 
+@pytest.mark.parametrize("name", ["w_out", "w_qkv", "w_o", "w_q_c", "w_kv_c", "w_o_c", "w_ff1", "w_ff2"])
+def test_fp32_matrices_have_to_be_aligned(lib, name):
+    """The fp32 kernels read matrices 16 bytes at a time: a matrix at another address is refused before any CUDA call
+    (the addresses here are only looked at)."""
+    from paper_2503_05931_b200 import binding, workloads
+    model = workloads.MODELS["tiny"]
+    cfg = binding.make_config(model, "fp32", max_batch=4, max_total_enc_frames=100, max_enc_len=50, max_dec_len=8)
+    cfg.workspace, cfg.workspace_bytes = 1 << 20, binding.workspace_bytes(cfg)
+    layers = model["n_layers"]
+    w = binding.AedWeights()
+    for field in binding._GLOBAL_FIELDS:
+        setattr(w, field, (1 << 30) + (4 if field == name else 0))
+    keep = []
+    for field in binding._LAYER_FIELDS:
+        ptrs = (C.c_void_p * layers)(*[(1 << 30) + (4 if field == name and l == layers - 1 else 0) for l in range(layers)])
+        keep.append(ptrs)
+        setattr(w, field, C.cast(ptrs, C.POINTER(C.c_void_p)))
+    handle = C.c_void_p()
+    assert lib.aed_dec_create(C.byref(cfg), C.byref(w), C.byref(handle)) == binding.AED_ERR_INVALID_ARG
+    assert b"16-byte aligned" in lib.aed_dec_create_error()
+
+
 def test_bucketing_reduces_padding():
     from paper_2503_05931_b200 import bucketing, workloads
     w = workloads.make_workload("cfg5", with_weights=False, with_enc=False)

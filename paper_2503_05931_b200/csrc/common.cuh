@@ -172,9 +172,12 @@ __device__ __forceinline__ float warp_max(float v)
     return v;
 }
 
-// Monotone map float -> uint32 (larger float => larger key), used to take an argmax with integer atomics.
+// Monotone map float -> uint32 (larger float => larger key), used to take an argmax with integer atomics.  Every number has
+// a larger key than a NaN, and a NaN a larger one than nothing (0).  (Said outright: with the bits alone a NaN came out between
+// the negative and the positive numbers, because the compiler reads the sign of a float as such.)
 __device__ __forceinline__ uint32_t float_order_key(float f)
 {
+    if (f != f) return 1u;
     uint32_t u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }

@@ -501,6 +501,37 @@ def test_encoder_states_have_to_be_aligned(dtype):
     dec.close()
 
 
+@pytest.mark.parametrize("dtype, batch", [("fp32", 3), ("fp32", 12), ("fp32", 21), ("bf16", 3), ("bf16", 21), ("bf16", 70)])
+def test_choice_among_special_logits(dtype, batch):
+    """The greedy choice is the lowest index of the largest logit, also among negative ones and infinities; a NaN is chosen
+    only if nothing else is there."""
+    import torch
+    b = _binding()
+    w = wl.make_custom(SMALL, [7] * batch, [2] * batch, dtype=dtype, seed=640, out_std=0.1, out_bias_std=0.1)
+    V = SMALL["vocab"]
+    plain = w.weights["b_out"].copy()
+    toks = torch.arange(batch, dtype=torch.int32, device="cuda:0") + 3
+    nothing = {i: -np.inf for i in range(V)}
+    for shift, special in ((0, {5: np.nan, 299: np.nan}), (-64, {5: np.nan, 299: np.nan}), (-64, {5: np.nan, 9: -np.inf}),
+                           (0, {7: np.inf, 200: np.inf, 3: np.nan}), (0, nothing), (0, {**nothing, 0: np.nan}),
+                           (0, {i: np.nan for i in range(V)})):
+        bias = plain + np.float32(shift)
+        for i, v in special.items():
+            bias[i] = v
+        w.weights["b_out"] = bias
+        dec = b.decoder_for_workload(w)
+        dec.precompute_cross_kv(dec.upload_encoder(w.enc), w.enc_lens)
+        logits = torch.zeros((batch, V), dtype=torch.float32, device="cuda:0")
+        nxt = torch.full((batch,), -7, dtype=torch.int32, device="cuda:0")
+        dec.step(toks, None, logits, nxt)
+        z, got = logits.cpu().numpy(), nxt.cpu().numpy()
+        dec.close()
+        assert np.array_equal(np.isnan(z), np.broadcast_to(np.isnan(bias), z.shape))
+        largest = np.max(z, axis=1, where=~np.isnan(z), initial=-np.inf, keepdims=True)
+        want = np.argmax(z == largest, axis=1)            # (all NaN: no entry is equal, index 0)
+        assert np.array_equal(got, want), (shift, got, want)
+
+
 @pytest.mark.parametrize("batch", [1, 4, 5, 16, 17, 23])
 def test_fp32_row_tiles(batch):
     """Rows around the steps between 4-row and 8-row tiles and one and two features per warp of the fp32 projections, with

@@ -501,6 +501,34 @@ def test_encoder_states_have_to_be_aligned(dtype):
     dec.close()
 
 
+@pytest.mark.parametrize("frames", [2, 40, 300])
+def test_fp32_softmax_weights_below_the_normal_range(frames):
+    """fp32: a softmax weight below 2^-126 still counts (here e^-89 times a value of 1e38).  The cross-attention query is the
+    constant (8, 0, ...), so the score of a frame is its first encoder value and what it contributes its second one."""
+    d = 64
+    model = dict(n_layers=1, d_model=d, n_heads=1, d_ffn=64, vocab=50, d_enc=64)
+    w = wl.make_custom(model, [frames, frames], [2, 2], dtype="fp32", seed=650, out_std=1.0)
+    W = w.weights
+    zero = lambda *names: [W[n].__setitem__(0, np.zeros_like(W[n][0])) for n in names]
+    zero("w_o", "b_o", "w_q_c", "b_q_c", "w_kv_c", "b_kv_c", "w_o_c", "b_o_c", "w_ff2", "b_ff2")
+    W["embed"] = np.zeros_like(W["embed"])
+    W["b_q_c"][0][0] = 8.0
+    W["w_kv_c"][0][0, 0] = 1.0                        # key dimension 0 = encoder value 0
+    W["w_kv_c"][0][d + 1, 1] = 1.0                    # value dimension 1 = encoder value 1
+    W["w_o_c"][0][1, 1] = 1.0
+    w.enc[:] = 0.0
+    for u, at in ((0, frames - 1), (1, frames // 2)):
+        w.enc[u * frames:(u + 1) * frames, 0] = -200.0
+        w.enc[u * frames, 0] = 0.0
+        w.enc[u * frames + at, :2] = (-89.0, 1e38)
+    ref = oracle_reference(w)
+    assert np.max(np.abs(ref["logits"][0][0])) > 0.1
+    dec = _binding().decoder_for_workload(w)
+    worst, _, _ = teacher_forced_compare(dec, w, ref)
+    dec.close()
+    assert worst < TOL["fp32"], worst
+
+
 @pytest.mark.parametrize("dtype, batch", [("fp32", 3), ("fp32", 12), ("fp32", 21), ("bf16", 3), ("bf16", 21), ("bf16", 70)])
 def test_choice_among_special_logits(dtype, batch):
     """The greedy choice is the lowest index of the largest logit, also among negative ones and infinities; a NaN is chosen

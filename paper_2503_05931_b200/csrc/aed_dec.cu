@@ -395,7 +395,8 @@ aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 b
 
 // fp32 projection of at most rows_ub rows (f32_rows.cuh).  Up to 4 rows one feature per warp and 4-row tiles, up to 16 rows
 // 8-row tiles: as many warps as features, because a launch is bound by its latency.  Beyond, two features per warp halve the
-// shared-memory reads per FMA.  Small outputs take 4 warps per block, so that they still spread over 64 SMs and more.
+// shared-memory reads per FMA.  Small outputs take 4 warps per block, so that they still spread over 64 SMs and more.  Many rows
+// go to tiles of 64 x 64 (use_tiles says from where on); grid.y of the others stays below 25,000.
 template <int EPI>
 aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, bool after_rows = false)
 {
@@ -409,6 +410,11 @@ aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, 
     const void *kernel = rows_ub <= 4    ? (vec ? (const void *)f32::rows_kernel<EPI, 4, 1, true> : (const void *)f32::rows_kernel<EPI, 4, 1, false>)
                          : rows_ub <= 16 ? (vec ? (const void *)f32::rows_kernel<EPI, 8, 1, true> : (const void *)f32::rows_kernel<EPI, 8, 1, false>)
                                          : (vec ? (const void *)f32::rows_kernel<EPI, 8, 2, true> : (const void *)f32::rows_kernel<EPI, 8, 2, false>);
+    if (f32::use_tiles(p.M, rows_ub)) {
+        const dim3 tiles(((p.M + f32::kTile - 1) / f32::kTile) * ((rows_ub + f32::kTile - 1) / f32::kTile));
+        return launch_pdl_impl(dec, vec ? (const void *)f32::tile_kernel<EPI, true> : (const void *)f32::tile_kernel<EPI, false>, tiles,
+                               dim3(f32::kTileThreads), 0, args);
+    }
     const int rt = rows_ub <= 4 ? 4 : 8, fpw = rows_ub <= 16 ? 1 : 2;
     const dim3 grid((p.M + warps * fpw - 1) / (warps * fpw), (rows_ub + rt - 1) / rt);
     return launch_pdl_impl(dec, kernel, grid, dim3(warps * 32), f32::rows_smem(rt, p.K), args);

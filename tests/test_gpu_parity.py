@@ -461,15 +461,7 @@ def test_vocabulary_projection_of_one_k_block(batch):
 @pytest.mark.parametrize("dtype, batch", [("fp32", 3), ("fp32", 12), ("fp32", 21), ("bf16", 3), ("bf16", 12), ("bf16", 40), ("bf16", 70), ("bf16", 131)])
 def test_vectors_at_any_element(dtype, batch, monkeypatch):
     """LayerNorm parameters and biases that start one element past a 16-byte boundary."""
-    b = _binding()
-    upload = b.Decoder._upload
-
-    def shifted(self, arr):
-        arr = np.asarray(arr)
-        if arr.ndim != 1:
-            return upload(self, arr)
-        return upload(self, np.concatenate([np.zeros(1, arr.dtype), arr])) + self.tdtype.itemsize
-    monkeypatch.setattr(b.Decoder, "_upload", shifted)
+    _shift_vectors(monkeypatch)
     rng = np.random.default_rng(620 + batch)
     w = wl.make_custom(MID, rng.integers(1, 60, size=batch), rng.integers(1, 5, size=batch), dtype=dtype, seed=621 + batch, out_std=0.3,
                        ln_std=0.3, out_bias_std=0.1)
@@ -499,6 +491,64 @@ def test_encoder_states_have_to_be_aligned(dtype):
         dec.admit(0, bad[:9], 3)
     assert e.value.status == b.AED_ERR_INVALID_ARG
     dec.close()
+
+
+def test_fp32_half_a_million_rows():
+    """fp32: more frames, and more rows of a step, than 8-row tiles fit into one extent of a grid (8 * 65535)."""
+    import torch
+    batch = 8 * 65535 + 21
+    model = dict(n_layers=1, d_model=64, n_heads=1, d_ffn=64, vocab=40, d_enc=64)
+    w = wl.make_custom(model, [1] * batch, [2] * batch, dtype="fp32", seed=660, out_std=0.3)
+    rows = [0, 63, 8 * 65535 - 1, 8 * 65535, batch - 1]
+    ref = oracle_reference(w, rows)
+    dec = _binding().decoder_for_workload(w)
+    worst, compared, bad = teacher_forced_compare(dec, w, ref, rows)
+    assert compared == 2 * len(rows) and worst < TOL["fp32"] and not bad, (worst, bad)
+    dec.precompute_cross_kv(dec.upload_encoder(w.enc), w.enc_lens)
+    toks, lens = dec.greedy_decode(w.dec_lens)
+    dec.close()
+    assert bool((lens == 2).all())
+    got = toks[torch.tensor(rows, device="cuda:0")].cpu().numpy()
+    for i in range(len(rows)):
+        for t in range(2):
+            if ref["margin"][i, t] <= MARGIN:
+                break
+            assert got[i, t] == ref["next"][i, t]
+
+
+def _shift_vectors(monkeypatch):
+    """Decoders from here on have their LayerNorm parameters and biases one element past a 16-byte boundary."""
+    cls = _binding().Decoder
+    upload = cls._upload
+
+    def shifted(self, arr):
+        arr = np.asarray(arr)
+        if arr.ndim != 1:
+            return upload(self, arr)
+        return upload(self, np.concatenate([np.zeros(1, arr.dtype), arr])) + self.tdtype.itemsize
+    monkeypatch.setattr(cls, "_upload", shifted)
+
+
+@pytest.mark.parametrize("vocab, batch, shift", [(12001, 33, False), (12001, 64, True), (6200, 64, False), (6200, 65, False), (90, 1537, False), (90, 1600, True)])
+def test_fp32_tiles_of_many_rows(vocab, batch, shift, monkeypatch):
+    """fp32 launches on either side of the rule for 64 x 64 tiles: the vocabulary projection alone (33 to 65 rows), every
+    projection of a step (1537 and 1600), with rows and features that fill their last tile by one or not at all, and vectors
+    that cannot be read 16 bytes at a time."""
+    if shift:
+        _shift_vectors(monkeypatch)
+    model = dict(n_layers=1, d_model=256, n_heads=4, d_ffn=320, vocab=vocab, d_enc=192)
+    rng = np.random.default_rng(670 + batch)
+    w = wl.make_custom(model, rng.integers(1, 30, size=batch), rng.integers(1, 4, size=batch), dtype="fp32", seed=671 + batch, out_std=0.1,
+                       ln_std=0.3, out_bias_std=0.1)
+    _run_both(w, rows=sorted({0, 1, 31, 32, 63, 64, 1535, 1536, batch - 1} & set(range(batch))), label=f"fp32 tiles V={vocab} B={batch}")
+
+
+@pytest.mark.parametrize("frames", [767, 768, 769, 833])
+def test_fp32_cross_kv_frames(frames):
+    """fp32 cross-attention keys and values around the rule for tiles (512 features: 768 frames) and past a whole tile."""
+    model = dict(n_layers=2, d_model=256, n_heads=4, d_ffn=64, vocab=90, d_enc=192)
+    w = wl.make_custom(model, [500, 1, frames - 501], [3, 3, 3], dtype="fp32", seed=680 + frames, out_std=0.3)
+    _run_both(w, label=f"{frames} frames")
 
 
 @pytest.mark.parametrize("frames", [2, 40, 300])

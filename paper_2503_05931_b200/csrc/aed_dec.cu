@@ -639,7 +639,6 @@ aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int ro
     p.a_rows = dec->cfg.vocab;
     p.n_tile = shape.n_tile;
     p.k_blocks = dec->cfg.d_model / tc::kBlockK;
-    p.use_lo = 1;
     p.rows_fixed = rows_fixed;          // >= 0: only that many rows (a prefill pass projects its last-position rows only)
     p.state = dec->state();
     const CUtensorMap *acts = dec->tc_actd[shape.n_tile / 16 - 1];
@@ -648,8 +647,7 @@ aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int ro
     return launch_pdl_impl(dec, (const void *)tc::tc_gemm_kernel, grid, dim3(tc::kThreads), shape.smem, args);
 }
 
-aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const void *g, const void *b, float *zero_buf,
-                              int zero_cols)
+aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const void *g, const void *b)
 {
     ProfScope ps(dec, KF_LAYERNORM);
     int d = dec->cfg.d_model;
@@ -658,16 +656,11 @@ aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const v
     const DecState *state = dec->state();
     const __nv_bfloat16 *gp = (const __nv_bfloat16 *)g, *bp = (const __nv_bfloat16 *)b;
     __nv_bfloat16 *hi = dec->at<__nv_bfloat16>(L.actd_hi), *lo = dec->at<__nv_bfloat16>(L.actd_lo);
-    void *args[] = {&state, &x, &gp, &bp, &d, &eps, &hi, &lo, &zero_buf, &zero_cols};
+    void *args[] = {&state, &x, &gp, &bp, &d, &eps, &hi, &lo};
     return launch_pdl_impl(dec, (const void *)layernorm_planes_kernel<8>, dim3(rows_ub), dim3(d <= 2048 ? 256 : 1024), 0, args);
 }
 
 // ---- fused step (bf16 mode): 7 kernels per layer, chained with programmatic dependent launch -------------------
-
-struct FusedGemm {
-    const CUtensorMap *map;
-    int M, K, mode;
-};
 
 template <int MODE>
 aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, const CUtensorMap *src_maps, int M,
@@ -912,7 +905,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         return launch_pdl_impl(dec, (const void *)vg::vocab_gemv_kernel, dim3((V + tc::kTileM - 1) / tc::kTileM), dim3(vg::kVgThreads),
                                (size_t)vg::vg_smem(d), args);
     }
-    AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
+    AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b));
     tc::TcParams tp{};
     tp.bias = (const T *)dec->b_out;
     tp.logits_out = logits_out;
@@ -1059,7 +1052,7 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         AED_TRY(launch_plane_gemm(dec, KF_GEMM_FF1, m.ff1, dec->tc_actd, F, d, rows, sh_ff1, p));
         AED_TRY(project(KF_GEMM_FF2, m.ff2, dec->tc_actf, d, F, sh_ff2, nullptr, w.b_ff2));
     }
-    AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b, nullptr, 0));
+    AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b));
     tc::TcParams tp{};
     tp.bias = (const T *)dec->b_out;
     tp.logits_out = logits_out;

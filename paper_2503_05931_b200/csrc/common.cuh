@@ -165,12 +165,6 @@ __device__ __forceinline__ float warp_sum(float v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ __forceinline__ float warp_max(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
 
 // Monotone map float -> uint32 (larger float => larger key), used to take an argmax with integer atomics.  Every number has
 // a larger key than a NaN, and a NaN a larger one than nothing (0).  (Said outright: with the bits alone a NaN came out between

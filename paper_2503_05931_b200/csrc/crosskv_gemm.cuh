@@ -43,7 +43,6 @@ constexpr int kStages = 6;
 constexpr int kProducers = 6;                     // one stage each
 constexpr int kMmaWarp = 6;
 constexpr int kCkvThreads = 512;
-constexpr int kMaxLayers = 64;
 
 // The frames of a launch: up to kMaxSegs runs of consecutive rows of the encoder tensor, each with a store row of its
 // own (a packed batch is one run; utterances admitted into slots are one run each).  Frame tiles never straddle runs.

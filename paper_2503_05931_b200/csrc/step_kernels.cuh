@@ -811,13 +811,11 @@ attn_combine_kernel(const DecState *state, const int32_t *__restrict__ active_li
     *reinterpret_cast<float2 *>(out + (size_t)r * ldo + h * kHeadDim + lane * 2) = o;
 }
 
-// LayerNorm whose result is written as bf16 high and low planes [row, d]; the same block also clears the fp32
-// rows that the following split-K projection accumulates into (zero_cols columns of zero_buf, if any).
+// LayerNorm whose result is written as bf16 high and low planes [row, d].
 template <int kMaxPerThread>
 __global__ void layernorm_planes_kernel(const DecState *state, const float *x,
                                         const __nv_bfloat16 *__restrict__ g, const __nv_bfloat16 *__restrict__ b, int d,
-                                        float eps, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo,
-                                        float *__restrict__ zero_buf, int zero_cols)
+                                        float eps, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo)
 {
     AED_TRACE_BEGIN(state, 4);
     // launched with programmatic stream serialization: nothing of the previous kernel is touched before this wait
@@ -867,7 +865,6 @@ __global__ void layernorm_planes_kernel(const DecState *state, const float *x,
             out_lo[(size_t)r * d + i] = __float2bfloat16_rn(y - __bfloat162float(hi));
         }
     }
-    for (int i = threadIdx.x; i < zero_cols; i += blockDim.x) zero_buf[(size_t)r * zero_cols + i] = 0.f;
 }
 
 // ------------------------------------------------------------------------------------------------------------

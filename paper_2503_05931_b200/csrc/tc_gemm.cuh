@@ -1,10 +1,10 @@
 // Tensor-core GEMM for sm_100a: TMA-fed tcgen05.mma with the accumulator in tensor memory.
 //
-//   D[128 x N] (fp32, TMEM) = sum over this CTA's k-blocks of  A_tile[128 x 64] . B_tile[N x 64]^T
+//   D[128 x N] (fp32, TMEM) = sum over the k-blocks of  A_tile[128 x 64] . B_tile[N x 64]^T
 //
 // Both operands are K-major bf16 in global memory and arrive in shared memory through
 // cp.async.bulk.tensor (no multicast) with the 128-byte swizzle the MMA descriptors name.
-// One CTA = one (128-row tile of A, N-row tile of B, k-split).  Warp roles: warps 0..7 issue TMA (a thread's
+// One CTA = one (128-row tile of A, N-row tile of B).  Warp roles: warps 0..7 issue TMA (a thread's
 // copies complete one after the other, about a third of a microsecond each, so the k-blocks are shared out round
 // robin over the issuing threads), warp 8 owns the TMEM allocation and issues the MMAs; at the end all warps but that
 // one drain the accumulator (warp w reads TMEM lanes 32*(w%4) .. +31) into the ring's memory, rows first, and then take
@@ -132,8 +132,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 struct TcParams {
     int a_rows;          // valid rows of A (output features, or frames)
     int n_tile;          // rows of B per CTA = MMA N (multiple of 16, at most 256)
-    int k_blocks;        // k-blocks over the whole K
-    int use_lo;          // 1: accumulate the low activation plane as well
+    int k_blocks;
     int rows_fixed;      // >= 0: number of valid B rows; < 0: read it from the decode state
     const __nv_bfloat16 *bias;         // over the columns of D's first dimension (vocabulary / K-V features), may be null
     float *logits_out;                 // [batch, vocab] by utterance or nullptr
@@ -142,7 +141,7 @@ struct TcParams {
     DecState *state;
 };
 
-// grid: x = 128-row tiles of A, y = k-splits, z = N-row tiles of B.  Dynamic shared memory: see vocab_shape.
+// grid: x = 128-row tiles of A, z = N-row tiles of B.  Dynamic shared memory: see vocab_shape.
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b_lo, TcParams p, int stages, int producers)
@@ -163,15 +162,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // loads do not wait on it (the epilogue reads the row count when it needs it).
     if (blockIdx.z > 0 && row0 >= (p.rows_fixed >= 0 ? p.rows_fixed : p.state->n_active)) return;
     const int a0 = blockIdx.x * kTileM;
-    const int kb_begin = static_cast<int>((static_cast<long long>(p.k_blocks) * blockIdx.y) / gridDim.y);
-    const int kb_end = static_cast<int>((static_cast<long long>(p.k_blocks) * (blockIdx.y + 1)) / gridDim.y);
-    const int n_kb = kb_end - kb_begin;
-    if (n_kb <= 0) return;
+    const int n_kb = p.k_blocks;
 
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
     const int b_bytes = p.n_tile * kBlockK * 2;
-    const int planes = p.use_lo ? 2 : 1;
-    const int stage_bytes = kATileBytes + planes * b_bytes;
+    const int stage_bytes = kATileBytes + 2 * b_bytes;
     uint32_t tmem_cols = 32;
     while (tmem_cols < static_cast<uint32_t>(p.n_tile)) tmem_cols <<= 1;
 
@@ -193,7 +188,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (lane == 0 && warp < producers) {
             prefetch_tensormap(&map_a);
             prefetch_tensormap(&map_b);
-            if (p.use_lo) prefetch_tensormap(&map_b_lo);
+            prefetch_tensormap(&map_b_lo);
             int issued = 0;
             bool waited = false;
             for (int i = warp; i < n_kb; i += producers) {
@@ -201,13 +196,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (i >= stages && !mbar_wait(&bar_empty[s], ((i / stages) - 1) & 1, &abort_flag)) break;
                 uint8_t *st = tiles + static_cast<size_t>(s) * stage_bytes;
                 mbar_expect_tx(&bar_full[s], stage_bytes);
-                const int kc = (kb_begin + i) * kBlockK;
+                const int kc = i * kBlockK;
                 tma_load_2d(st, &map_a, kc, a0, &bar_full[s]);
                 // A is static (a weight matrix): its first tile is requested while the previous kernel still runs;
                 // B is that kernel's output
                 if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
                 tma_load_2d(st + kATileBytes, &map_b, kc, row0, &bar_full[s]);
-                if (p.use_lo) tma_load_2d(st + kATileBytes + b_bytes, &map_b_lo, kc, row0, &bar_full[s]);
+                tma_load_2d(st + kATileBytes + b_bytes, &map_b_lo, kc, row0, &bar_full[s]);
                 issued = i + 1;
             }
             if (abort_flag && issued > 0) {
@@ -228,15 +223,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (i == 0) AED_TRACE_MARK(p.state, 33);    // first operands landed
                 tc_fence_after_sync();
                 const uint32_t sa = smem_u32(tiles + static_cast<size_t>(s) * stage_bytes);
-                const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kATileBytes);
+                const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kATileBytes), dl = smem_desc_sw128(sa + kATileBytes + b_bytes);
 #pragma unroll
                 for (int k = 0; k < kBlockK / 16; ++k)
                     mma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
-                if (p.use_lo) {
-                    const uint64_t dl = smem_desc_sw128(sa + kATileBytes + b_bytes);
 #pragma unroll
-                    for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
-                }
+                for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
                 mma_commit(&bar_empty[s]);      // the stage may be refilled once these MMAs have read it
             }
             if (ok) mma_commit(&bar_done);      // accumulator complete

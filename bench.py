@@ -66,31 +66,32 @@ def step_bytes_and_flops(w):
     return per_step, pre_bytes, pre_flops, step_params
 
 
-def family_bytes(family, w):
-    """Algorithmic bytes one whole pass (precompute + greedy decode) moves in the launches of a kernel family."""
+def family_bytes(family, w, first=0, last=None):
+    """Algorithmic bytes that the launches of a kernel family move in the greedy steps first .. last - 1 of a pass (default:
+    all), or in its precompute."""
     m = w.model
     e = 2 if w.dtype == "bf16" else 4
     NL, d, F, V, de = m["n_layers"], m["d_model"], m["d_ffn"], m["vocab"], m["d_enc"]
     T, L = w.enc_lens.astype(np.int64), w.dec_lens.astype(np.int64)
-    steps = int(L.max())
+    steps = range(first, int(L.max()) if last is None else last)
     per_layer_weights = {"gemm_qkv": 3 * d * d, "gemm_o": d * d, "gemm_qc": d * d, "gemm_oc": d * d,
-                         "gemm_ff1": d * F, "gemm_ff2": d * F, "ffn": 2 * d * F}
+                         "gemm_ff1": d * F, "gemm_ff2": d * F}
     if family in per_layer_weights:
-        return e * per_layer_weights[family] * NL * steps
+        return e * per_layer_weights[family] * NL * len(steps)
     if family == "gemm_vocab":
-        return e * V * d * steps
+        return e * V * d * len(steps)
     if family == "attn_cross":
-        return sum((CROSS_KV_BYTES or e) * NL * 2 * d * int(T[L > s].sum()) for s in range(steps))
+        return sum((CROSS_KV_BYTES or e) * NL * 2 * d * int(T[L > s].sum()) for s in steps)
     if family == "attn_self":
-        return sum(e * NL * 2 * d * int((L > s).sum()) * (s + 1) for s in range(steps))
+        return sum(e * NL * 2 * d * int((L > s).sum()) * (s + 1) for s in steps)
     if family == "precompute_cross_kv":
         total_T = int(T.sum())
         return e * (total_T * de + NL * 2 * d * de) + (CROSS_KV_BYTES or e) * total_T * NL * 2 * d
     return None
 
 
-# Which kernel a launch family runs (the library times launches per call site; the projections of a layer are
-# five or six call sites of one kernel).
+# Which kernel a launch family runs (the library times launches per call site, and says with "@" which kernel ran it where
+# there are several; the projections of a layer are five or six call sites of one kernel).
 KERNEL_OF_FAMILY = {
     "gemm_qkv": "step_gemm_kernel", "gemm_o": "step_gemm_kernel", "gemm_qc": "step_gemm_kernel",
     "gemm_oc": "step_gemm_kernel", "gemm_ff1": "step_gemm_kernel", "gemm_ff2": "step_gemm_kernel",
@@ -98,6 +99,45 @@ KERNEL_OF_FAMILY = {
     "gemm_vocab": "tc_gemm_kernel", "precompute_cross_kv": "crosskv_gemm_kernel", "layernorm": "layernorm_planes_kernel",
     "embed": "embed_kernel", "bookkeeping": "step_rows/finish_step",
 }
+KERNEL_OF_VARIANT = {
+    "plane": "plane_gemm_kernel", "warp": "self_attn_warp_kernel", "gamma": "gamma_planes_kernel", "gemv_staged": "step_gemv_staged_kernel",
+    "gemv": "step_gemv_kernel", "f32_tile": "tile_kernel", "f32_rows": "rows_kernel",
+}
+# The rows of a greedy pass only fall, so the variants of a call site take its steps in this order.
+VARIANT_ORDER = ["plane", "warp", "f32_tile", "", "gemv_staged", "f32_rows", "gemv"]
+
+
+def kernel_of(family):
+    """The kernel behind a profile family such as "gemm_qkv@gemv_staged"."""
+    base, _, variant = family.partition("@")
+    if base == "gemm_vocab" and variant == "gemv":
+        return "vocab_gemv_kernel"                         # final LayerNorm + vocabulary projection of steps with few rows
+    return KERNEL_OF_VARIANT[variant] if variant else KERNEL_OF_FAMILY.get(base, base)
+
+
+def profile_bytes(prof, w):
+    """Algorithmic bytes of every family of a profiled pass: each variant of a call site has the steps it ran."""
+    m = w.model
+    d, e = m["d_model"], 2 if w.dtype == "bf16" else 4
+    out = {}
+    for base in {f.partition("@")[0] for f in prof}:
+        step = 0
+        for variant in VARIANT_ORDER + ["gamma"]:
+            fam = base + "@" + variant if variant else base
+            if fam not in prof:
+                continue
+            per_step = 1 if base == "gemm_vocab" else m["n_layers"]
+            n = prof[fam]["launches"] // per_step
+            if base == "precompute_cross_kv":
+                out[fam] = family_bytes(base, w)
+            else:
+                out[fam] = family_bytes(base, w, step, step + n) or 0.0
+            # steps of at most 128 rows: the launch that reads Wqkv reads the cross-attention query matrix as well
+            if base == "gemm_qkv" and variant in ("", "gemv", "gemv_staged") and w.dtype == "bf16":
+                out[fam] += e * d * d * prof[fam]["launches"]
+            step += n
+    return out
+
 
 # DRAM bytes per algorithmic byte of a kernel, from the ncu captures summarised under profiles/ (dram__bytes_read.sum +
 # dram__bytes_write.sum of the captured launches over their algorithmic bytes).  An entry is removed when its kernel
@@ -107,16 +147,23 @@ NCU_TRAFFIC_RATIO = {
     # the composite cross-query matrix (2.1 MB), the fp32 activation rows, and each prefetches the next layer's matrices
     # of its kind into L2, which under the profiler's serialised replay is a second DRAM read
     "step_gemm_kernel": 2.51,
-    # the five launches at 16 and at 4 rows (cfg2): 63.24 MB and 62.97 MB read
-    "step_gemv_staged_kernel": 2.15,
+    # the five launches at 16 and at 4 rows (cfg2): 63.70 MB and 62.92 MB read
+    "step_gemv_staged_kernel": 2.17,
     "step_gemv_kernel": 2.14,
-    # self + cross attention of one layer at 64 rows: 0.84 + 31.05 MB for 0.52 + 30.49 MB of K/V
+    # the six launches of one layer at 512 rows: 56.82 MB read; beside the weights the activation planes
+    "plane_gemm_kernel": 1.94,
+    # self + cross attention of one layer at 64 rows: 0.84 + 31.05 MB for 0.52 + 30.49 MB of K/V (cross-attention of 512 rows:
+    # 127.97 MB read for 125.8)
     "attn_fused_kernel": 1.03,
-    # vocabulary projection: 33.85 MB for the 33.55 MB output matrix (tcgen05 kernel; 33.79 MB in the few-row kernel)
+    # vocabulary projection: 33.84 MB for the 33.55 MB output matrix (tcgen05 kernel; 33.79 MB in the few-row kernel)
     "tc_gemm_kernel": 1.01,
     "vocab_gemv_kernel": 1.01,
-    # cross-K/V of 7444 frames: 117.2 MB read + 677.2 MB written for 847.7 MB (part of the output is still in L2 at exit)
-    "crosskv_gemm_kernel": 0.94,
+    # cross-K/V of 7444 frames: 131.3 MB read + 683.0 MB written for 847.7 MB (part of the output is still in L2 at exit)
+    "crosskv_gemm_kernel": 0.96,
+    # fp32: the six projections of a layer at 4 rows (2 layers, d 256), 3.86 MB for 3.67; cross-K/V of 20000 frames (d 1024),
+    # 90.9 MB read + 125.4 MB written for 254.1 MB
+    "rows_kernel": 1.05,
+    "tile_kernel": 0.85,
 }
 
 
@@ -501,39 +548,28 @@ def main():
 def profile_dominant_kernel(dec, w, one_pass, peaks, ms_per_step):
     """Roofline figure of the kernel that takes the largest share of device time.
 
-    Shares come from one extra pass with CUDA events around every launch on the library's stream (no graph replay in
-    that pass), summed per kernel, not per call site.  The kernel's time inside the measured (graphed, overlapped)
-    pass is taken as share x measured pass time: launches overlap under programmatic dependent launch, so a per-launch
-    duration of the measured configuration only exists in that sense.  ``avg_us_ungraphed`` is the plain event
-    figure of the extra pass, which includes the host launch gap."""
+    The times come from one extra pass with CUDA events around every launch on the library's stream (no graph replay in that
+    pass), summed per kernel, not per call site.  Launches of the measured pass overlap (programmatic dependent launch,
+    graphs) and have no events between them, so every launch of the extra pass is longer by about the same amount: what the
+    whole pass is longer by, over its launches, is taken off each.  ``avg_us_ungraphed`` is the plain event figure.
+    (Scaling all launches by one factor instead takes too much off the long ones: 1.03 of the copy bandwidth for attention at
+    512 rows, where its own events say 0.75.)"""
     prof = dec.profile_pass(one_pass)
     if not prof:
         return None
-    total = sum(v["ms"] for v in prof.values())
+    extra = max(0.0, sum(v["ms"] for v in prof.values()) - ms_per_step) / sum(v["launches"] for v in prof.values())
+    for v in prof.values():
+        v["own_ms"] = max(v["ms"] - extra * v["launches"], 0.0)
+    total = sum(v["own_ms"] for v in prof.values())
     kernels = {}
-    m = w.model
-    e = 2 if w.dtype == "bf16" else 4
-    d, F = m["d_model"], m["d_ffn"]
-    # bytes of weights one launch of a projection call site reads (what the layer's definition contains)
-    site_weights = {"gemm_qkv": 3 * d * d, "gemm_o": d * d, "gemm_qc": d * d, "gemm_oc": d * d, "gemm_ff1": d * F, "gemm_ff2": d * F}
+    moved = profile_bytes(prof, w)
     for fam, v in prof.items():
-        base, _, variant = fam.partition("@")                  # "gemm_qkv@gemv_staged": call site and the kernel that ran it
-        kernel = {"gemv": "step_gemv_kernel", "gemv_staged": "step_gemv_staged_kernel"}.get(variant, KERNEL_OF_FAMILY.get(base, base))
-        if base == "gemm_vocab" and variant:
-            kernel = "vocab_gemv_kernel"                       # final LayerNorm + vocabulary projection of steps with few rows
-        k = kernels.setdefault(kernel, {"ms": 0.0, "launches": 0, "bytes": 0.0, "families": []})
-        k["ms"] += v["ms"]; k["launches"] += v["launches"]; k["families"].append(fam)
-        if base in site_weights:
-            per_launch_w = site_weights[base]
-            # steps of at most 128 rows: the cross-attention query matrix is read by the launch that reads Wqkv
-            if base == "gemm_qkv" and not any(f.partition("@")[0] == "gemm_qc" for f in prof):
-                per_launch_w += d * d
-            k["bytes"] += e * per_launch_w * v["launches"]
-        else:
-            k["bytes"] += family_bytes(base, w) or 0.0
-    top = max(kernels, key=lambda k: kernels[k]["ms"])
+        k = kernels.setdefault(kernel_of(fam), {"ms": 0.0, "own_ms": 0.0, "launches": 0, "bytes": 0.0, "families": []})
+        k["ms"] += v["ms"]; k["own_ms"] += v["own_ms"]; k["launches"] += v["launches"]; k["families"].append(fam)
+        k["bytes"] += moved[fam]
+    top = max(kernels, key=lambda k: kernels[k]["own_ms"])
     info = kernels[top]
-    share = info["ms"] / total
+    share = info["own_ms"] / total
     in_graph_ms = share * ms_per_step
     per_launch = info["bytes"] / max(info["launches"], 1)
     achieved = info["bytes"] / (in_graph_ms * 1e-3) / 1e9 if info["bytes"] else None
@@ -541,7 +577,7 @@ def profile_dominant_kernel(dec, w, one_pass, peaks, ms_per_step):
     family_shares = {}
     for fam, v in prof.items():
         base = fam.partition("@")[0]
-        family_shares[base] = family_shares.get(base, 0.0) + v["ms"] / total
+        family_shares[base] = family_shares.get(base, 0.0) + v["own_ms"] / total
     return {"bound": "hbm", "kernel": top, "families": sorted(info["families"]), "achieved": achieved,
             "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": (achieved / peaks["hbm_gbs"]) if achieved else None,
             "traffic": ratio * per_launch if (ratio and per_launch) else None,
@@ -551,7 +587,7 @@ def profile_dominant_kernel(dec, w, one_pass, peaks, ms_per_step):
             "avg_us": 1e3 * in_graph_ms / max(info["launches"], 1),
             "avg_us_ungraphed": 1e3 * info["ms"] / max(info["launches"], 1),
             "peak_source": peaks["source"],
-            "shares": {k: round(v["ms"] / total, 4) for k, v in sorted(kernels.items(), key=lambda kv: -kv[1]["ms"])},
+            "shares": {k: round(v["own_ms"] / total, 4) for k, v in sorted(kernels.items(), key=lambda kv: -kv[1]["own_ms"])},
             "family_shares": {k: round(v, 4) for k, v in family_shares.items()}}
 
 

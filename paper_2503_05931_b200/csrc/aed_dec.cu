@@ -253,10 +253,10 @@ enum KernelFamily { KF_BOOKKEEPING = 0, KF_EMBED, KF_LAYERNORM, KF_GEMM_QKV, KF_
 const char *const kFamilyNames[KF_COUNT] = {"bookkeeping", "embed", "layernorm", "gemm_qkv", "attn_self", "attn_combine",
                                             "gemm_o", "gemm_qc", "attn_cross", "gemm_oc", "gemm_ff1", "gemm_ff2",
                                             "gemm_vocab", "precompute_cross_kv"};
-// The projections of steps with few rows run in kernels of their own (step_gemv.cuh); the profile keeps the call site
-// and says which kernel ran it: family + KF_COUNT * variant, reported as "gemm_qkv@gemv", "gemm_qkv@gemv_staged".
-enum { KV_TCGEN05 = 0, KV_GEMV = 1, KV_GEMV_STAGED = 2, KV_COUNT = 3 };
-const char *const kVariantSuffix[KV_COUNT] = {"", "@gemv", "@gemv_staged"};
+// A call site runs different kernels at different row counts; the profile keeps the call site and says which kernel ran it:
+// family + KF_COUNT * variant, reported as "gemm_qkv@gemv", "attn_self@warp".
+enum { KV_NONE = 0, KV_GEMV, KV_GEMV_STAGED, KV_PLANE, KV_GAMMA, KV_WARP, KV_F32_ROWS, KV_F32_TILE, KV_COUNT };
+const char *const kVariantSuffix[KV_COUNT] = {"", "@gemv", "@gemv_staged", "@plane", "@gamma", "@warp", "@f32_rows", "@f32_tile"};
 
 // Records an event before and after the launches issued while it is alive (profiling mode only).
 struct ProfScope {
@@ -319,7 +319,9 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
                                     const float2 *ln_stats = nullptr, const float *ln_c1 = nullptr,
                                     const float *ln_c2 = nullptr, bool pdl = false, const float *stats_x = nullptr)
 {
-    ProfScope ps(dec, kCross ? KF_ATTN_CROSS : KF_ATTN_SELF);
+    // self-attention of many rows: see below
+    const bool by_warp = !kCross && sizeof(T) == 2 && rows_ub * dec->cfg.n_heads > 1024;
+    ProfScope ps(dec, (kCross ? KF_ATTN_CROSS : KF_ATTN_SELF) + KF_COUNT * (by_warp ? KV_WARP : KV_NONE));
     int warps = (len_ub + fused_chunk<T>() - 1) / fused_chunk<T>();
     if (warps < 2) warps = 2;                    // at least 64 threads: the merge uses one thread per head dimension
     if (warps > kFusedMaxWarps) warps = kFusedMaxWarps;
@@ -346,7 +348,7 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
         // flight (24-layer model, 16 heads, per step at up to 8 / 239 positions, a block per pair -> a warp per pair:
         // 64 rows 1051 / 1225 -> 1040 / 1382 us, 80 rows 1450 / 1635 -> 1394 / 1646, 128 rows 1778 / 2042 ->
         // 1666 / 1948, 512 rows 4022 / 5127 -> 3513 / 4452).
-        if (rows_ub * dec->cfg.n_heads > 1024) {
+        if (by_warp) {
             cfg.gridDim = dim3((rows_ub * dec->cfg.n_heads + 7) / 8);
             cfg.blockDim = dim3(256);
             cudaError_t e = cudaLaunchKernelEx(&cfg, self_attn_warp_kernel<T, kAppend>, (const DecState *)dec->state(),
@@ -400,7 +402,8 @@ aed_status_t launch_pdl_impl(aed_dec *dec, const void *kernel, dim3 grid, dim3 b
 template <int EPI>
 aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, bool after_rows = false)
 {
-    ProfScope ps(dec, family);
+    const bool tiles = f32::use_tiles(p.M, rows_ub);
+    ProfScope ps(dec, family + KF_COUNT * (tiles ? KV_F32_TILE : KV_F32_ROWS));
     const int warps = p.M <= 512 ? 4 : f32::kWarps;
     p.state = dec->state();
     p.eps = dec->cfg.ln_eps;
@@ -410,9 +413,9 @@ aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, 
     const void *kernel = rows_ub <= 4    ? (vec ? (const void *)f32::rows_kernel<EPI, 4, 1, true> : (const void *)f32::rows_kernel<EPI, 4, 1, false>)
                          : rows_ub <= 16 ? (vec ? (const void *)f32::rows_kernel<EPI, 8, 1, true> : (const void *)f32::rows_kernel<EPI, 8, 1, false>)
                                          : (vec ? (const void *)f32::rows_kernel<EPI, 8, 2, true> : (const void *)f32::rows_kernel<EPI, 8, 2, false>);
-    if (f32::use_tiles(p.M, rows_ub)) {
-        const dim3 tiles(((p.M + f32::kTile - 1) / f32::kTile) * ((rows_ub + f32::kTile - 1) / f32::kTile));
-        return launch_pdl_impl(dec, vec ? (const void *)f32::tile_kernel<EPI, true> : (const void *)f32::tile_kernel<EPI, false>, tiles,
+    if (tiles) {
+        const dim3 grid(((p.M + f32::kTile - 1) / f32::kTile) * ((rows_ub + f32::kTile - 1) / f32::kTile));
+        return launch_pdl_impl(dec, vec ? (const void *)f32::tile_kernel<EPI, true> : (const void *)f32::tile_kernel<EPI, false>, grid,
                                dim3(f32::kTileThreads), 0, args);
     }
     const int rt = rows_ub <= 4 ? 4 : 8, fpw = rows_ub <= 16 ? 1 : 2;
@@ -709,7 +712,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     const int splits_wide = std::max((k_blocks + 3) / 4, splits / 2);
     const bool gemv = dec->use_gemv && rows_ub <= dec->gemv_rows &&
                       (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
-    ProfScope ps(dec, family + KF_COUNT * (!gemv ? KV_TCGEN05 : rows_ub <= dec->gemv_direct_rows ? KV_GEMV : KV_GEMV_STAGED));
+    ProfScope ps(dec, family + KF_COUNT * (!gemv ? KV_NONE : rows_ub <= dec->gemv_direct_rows ? KV_GEMV : KV_GEMV_STAGED));
     // Steps of at most 32 rows whose CTAs cover at most two k-blocks (64 rows, four): warp-level MMAs
     // (step_gemv.cuh), activation fragments straight from global memory up to 4 rows, through shared memory beyond
     if (gemv) {
@@ -960,7 +963,7 @@ PlaneShape plane_shape(int M, int K, int rows_ub, bool whole_k)
 aed_status_t launch_plane_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, const CUtensorMap (*planes)[2], int M, int K, int rows_ub, PlaneShape shape,
                                pg::PlaneGemmParams p)
 {
-    ProfScope ps(dec, family);
+    ProfScope ps(dec, family + KF_COUNT * KV_PLANE);
     p.a_rows = M;
     p.k_blocks = K / tc::kBlockK;
     p.n_tile = shape.n_tile;
@@ -1002,7 +1005,7 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
     int rows = rows_ub;
     const dim3 ln_block(d <= 2048 ? 256 : 1024);
     auto gamma_planes = [&](const void *g, float2 *st, float *zero_buf, int zero_cols) -> aed_status_t {
-        ProfScope ps(dec, KF_LAYERNORM);
+        ProfScope ps(dec, KF_LAYERNORM + KF_COUNT * KV_GAMMA);
         return launch_pdl(dec, gamma_planes_kernel<8>, dim3(rows), ln_block, (const DecState *)dec->state(), (const float *)x,
                           (const T *)g, d, c.ln_eps, st, ad_hi, ad_lo, zero_buf, zero_cols);
     };

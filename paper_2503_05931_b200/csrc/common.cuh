@@ -180,6 +180,18 @@ __device__ __forceinline__ unsigned long long argmax_key(float f, uint32_t idx)
 {
     return (static_cast<unsigned long long>(float_order_key(f)) << 32) | (0xFFFFFFFFu - idx);
 }
+// The largest of N logits whose indices rise: the order key and which of them (the first among equals).  n: how many there are.
+template <int N> __device__ __forceinline__ uint32_t best_of(const float (&z)[N], int n, int &which)
+{
+    float m = z[0];
+#pragma unroll
+    for (int j = 1; j < N; ++j) m = fmaxf(m, j < n ? z[j] : m);      // (a NaN only if all are)
+    which = 0;
+#pragma unroll
+    for (int j = N - 1; j >= 0; --j)
+        if (j < n && z[j] == m) which = j;
+    return n > 0 ? float_order_key(m) : 0u;
+}
 __device__ __forceinline__ int32_t argmax_key_index(unsigned long long key)
 {
     return static_cast<int32_t>(0xFFFFFFFFu - static_cast<uint32_t>(key & 0xFFFFFFFFull));

@@ -279,12 +279,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     }
                 }
                 // the lane's best entry, the warp's best key, then the lowest lane that has it: the lowest index among equals
-                uint32_t k32 = 0u, best = 0u;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t k = o + j < p.a_rows ? float_order_key(z[j]) : 0u;
-                    if (k > k32) { k32 = k; best = static_cast<uint32_t>(o + j); }
-                }
+                int which;
+                const uint32_t k32 = best_of(z, p.a_rows - o, which), best = static_cast<uint32_t>(o + which);
                 const uint32_t kmax = __reduce_max_sync(0xffffffffu, k32);
                 const uint32_t winners = __ballot_sync(0xffffffffu, k32 == kmax);
                 if (kmax != 0u && lane == __ffs(winners) - 1)

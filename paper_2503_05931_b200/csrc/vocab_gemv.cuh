@@ -182,16 +182,11 @@ vocab_gemv_kernel(const __grid_constant__ CUtensorMap map_w, VocabGemvParams p)
         const float2 st = s_stats[r];
         const float rawv[4] = {raw.x, raw.y, raw.z, raw.w};
         float z[4];
-        unsigned long long key = 0ull;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool o_ok = o + j < p.vocab;
-            z[j] = o_ok ? fmaf(st.y, rawv[j] - st.x * p.c1[o + j], p.c2[o + j]) : 0.f;
-            if (o_ok && r < n_rows) {
-                const unsigned long long kj = argmax_key(z[j], static_cast<uint32_t>(o + j));
-                key = kj > key ? kj : key;
-            }
-        }
+        for (int j = 0; j < 4; ++j) z[j] = o + j < p.vocab ? fmaf(st.y, rawv[j] - st.x * p.c1[o + j], p.c2[o + j]) : 0.f;
+        int which;
+        const uint32_t k32 = best_of(z, r < n_rows ? p.vocab - o : 0, which);
+        unsigned long long key = k32 ? (static_cast<unsigned long long>(k32) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(o + which)) : 0ull;
         if (r < n_rows && p.logits_out) {
             float *dst = p.logits_out + static_cast<size_t>(p.active_list[r]) * p.vocab + o;
             if (o + 3 < p.vocab && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) *reinterpret_cast<float4 *>(dst) = make_float4(z[0], z[1], z[2], z[3]);

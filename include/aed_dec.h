@@ -34,8 +34,9 @@
  *   - Matrices are row-major [out_features, in_features].  With dtype
  *     AED_DTYPE_F32 every tensor (weights, biases, LayerNorm parameters,
  *     embedding, encoder states, K/V caches) is fp32 and all arithmetic is fp32
- *     FMA.  With AED_DTYPE_BF16 every tensor is bf16; accumulation, LayerNorm
- *     statistics, softmax and the residual stream stay fp32.
+ *     FMA; softmax weights are exp2f or expf.  With AED_DTYPE_BF16 every
+ *     tensor is bf16; accumulation, LayerNorm statistics, softmax (weights by
+ *     the hardware approximation of 2^x) and the residual stream stay fp32.
  */
 #ifndef AED_DEC_H_
 #define AED_DEC_H_
@@ -144,7 +145,8 @@ aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *enc_packed,
  *   active      DEVICE uint8 [batch] or NULL; an utterance takes part if it is not retired and (active == NULL
  *               or active[u] != 0).  Utterances are retired only by aed_dec_greedy_decode.
  *   logits_out  DEVICE float [batch, vocab] or NULL; rows of idle utterances are left untouched
- *   next_out    DEVICE int32 [batch] or NULL; greedy choice (lowest index on ties); idle entries untouched
+ *   next_out    DEVICE int32 [batch] or NULL; greedy choice (lowest index on ties, a NaN only if there is nothing
+ *               else); idle entries untouched
  * Errors: AED_ERR_STATE before a precompute; AED_ERR_CAPACITY if a participating utterance already holds
  * max_dec_len tokens (checked on the host from the steps issued so far, so only reliable when every step uses
  * active == NULL; with masks the device also refuses to write past the cache and raises a sticky error that

@@ -43,8 +43,8 @@ int rows_bucket(int rows)
 
 // Row count a step graph is captured for.  Kernels whose grids follow the row count (attention: one block per row and
 // head) pay for every row of the grid, also for those beyond the device-side count, whose blocks only find out that
-// they have nothing to do; so the graphs are keyed finer than the power-of-two tiles of the projections: 4, then multiples
-// of 8 up to 64 rows, of 16 up to 256, of 32 beyond.  Never above rows_bucket(rows).
+// they have nothing to do, and hold the next kernel back until they have (attn_fused_kernel).  Every key is a graph to record,
+// so: 4, then multiples of 8 up to 64 rows, of 16 up to 256, of 32 beyond.  Never above rows_bucket(rows).
 int rows_key(int rows)
 {
     if (rows <= 4) return 4;         // the projections of steps of at most 4 rows take a form of their own
@@ -203,7 +203,7 @@ struct aed_dec {
     int gemv_rows = 64;             // ... up to this many rows
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
-    // greedy decoding replays one captured CUDA graph per (row bucket, self-attention chunk count, output buffers)
+    // greedy decoding replays one captured CUDA graph per key; the output buffers stand in the device-side state
     typedef std::tuple<int, int, int> GraphKey;       // (row count, chunks of self-attention positions, steps)
     struct GraphEntry { cudaGraphExec_t exec; int64_t nodes; };
     std::map<GraphKey, GraphEntry> graphs;
@@ -918,11 +918,11 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
     return AED_OK;
 }
 
-// ---- steps with many rows (bf16 mode): activation planes made once per projection input, 12 kernels per layer -------
+// ---- steps with many rows (bf16 mode): activation planes made once per projection input, 11 kernels per layer -------
 // With hundreds of rows every feature tile of the fused projections would convert the same activation rows again
 // (24 times for the QKV projection) and that conversion, not the tensor cores, would set the pace.  Here a small kernel
-// writes gamma * x (with the row statistics) or the ReLU of the corrected hidden layer as bf16 planes once, attention
-// writes its output as planes, and the projections fetch both operands by TMA.
+// writes gamma * x as bf16 planes once, with the row statistics; attention writes its output as planes, FFN1's epilogue the
+// ReLU of the corrected hidden layer; and the projections fetch both operands by TMA.
 
 template <typename K, typename... Args>
 aed_status_t launch_pdl(aed_dec *dec, K kernel, dim3 grid, dim3 block, Args... args)

@@ -3,12 +3,12 @@
 //
 //   out[r, o] = sum_k A'[r, k] * W[o, k] + bias[o],   A' = LayerNorm(A) or A
 //
-// The configuration is small and its steps have few rows, so a projection is bound by latency, not by arithmetic: one warp
+// Steps of few rows (rows_kernel): a projection is bound by latency, not by arithmetic: one warp
 // per one or two output features and RT rows, lanes along K.  A warp's weights (16 bytes per lane and 128 k) are requested
 // before the programmatic-dependency wait; the rows are staged through shared memory (normalised on the way); the RT x FPW
 // sums of the lanes are reduced by halving, one value per lane in the end.  The former 64-row x 32-feature tiles left most
 // of a 4-row tile idle and walked K in steps of 32 with a memory latency each.  Decode step of the 2-layer fp32 model at 4
-// rows: 316 us before (27 launches), 56 us now (20 launches of about 2.8 us, which is what a link of the chain costs).
+// rows: 316 us before (27 launches), 52 us now (18 launches of about 2.8 us, which is what a link of the chain costs).
 #pragma once
 #include "step_gemm.cuh"
 

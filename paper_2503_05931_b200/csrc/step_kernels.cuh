@@ -430,7 +430,9 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
         return;
     }
     // The next kernel may start at once where that is a few-row projection, so that its weights are on their way while this
-    // one still waits (24 layers, 4 / 8 / 24 rows: 499 / 513 / 681 -> 473 / 486 / 661 us per step).  Not the cross-attention of
+    // one still waits (24 layers, 4 / 8 / 24 rows: 499 / 513 / 681 -> 473 / 486 / 661 us per step).  That holds for grids without
+    // padding rows: their blocks, above, end only after the wait, and the next kernel starts when every block has called it or
+    // ended.  (Same model now, 7 / 8 / 9 rows in grids of 8 / 8 / 16: 511 / 494 / 526 us.)  Not the cross-attention of
     // steps with more than 128 rows, which read their statistics (no kRowStats): blocks of the next kernel would take room from
     // its own later ones (200 / 512 rows 2130 / 3488 -> 2224 / 3650).  Nor fp32, whose projections hold their weights in
     // registers (2 layers, 4 / 8 rows: 54 / 70 us per step against 59 / 75).
@@ -664,8 +666,9 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
 // Self-attention of many rows: one warp per (row, head), 8 pairs per block, no shared memory and no merge of warps.
 // Short caches make this a matter of latency (the dependency wait, then one round of loads and a chain of shuffles), so
 // what counts is how many pairs an SM holds at once: 24 warps of at most 85 registers.  A pair's later chunks are loaded
-// one after the other; 24 x 4 KB in flight per SM are enough (512 rows, up to 239 positions: the cache is read at about
-// 6.2 TB/s; at up to 8 positions a launch went from about 26 us with a block per pair to 6).
+// one after the other; 24 x 4 KB in flight per SM are enough for long caches (512 rows, positions 221 to 240: 483 MB in 93.5 us
+// by events, 5.2 TB/s; 129 rows 4.1).  What it gained per step stands at its launch.  The next kernel starts after the wait
+// here, unlike behind attn_fused_kernel: steps of 65 to 128 rows (16 heads) have early starts behind cross-attention only.
 template <typename CT, bool kAppend>
 __global__ void __launch_bounds__(256, 3)
 self_attn_warp_kernel(const DecState *state, const int4 *row_info, const float *q, int ldq,

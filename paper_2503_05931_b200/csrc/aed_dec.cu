@@ -201,6 +201,7 @@ struct aed_dec {
     bool attn_pipe = true;
     bool use_gemv = true;           // steps of few rows: projections by warp-level MMAs (step_gemv.cuh)
     int gemv_rows = 64;             // ... up to this many rows
+    bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
     // greedy decoding replays one captured CUDA graph per key; the output buffers stand in the device-side state
@@ -610,8 +611,11 @@ aed_status_t tc_setup(aed_dec *dec)
         dec->launches += 1;
     }
     e = cudaGetLastError();
-    if (e == cudaSuccess && vg::vg_smem((int)d) <= 227 * 1024)
-        e = cudaFuncSetAttribute(vg::vocab_gemv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, vg::vg_smem((int)d));
+    // the few-row vocabulary kernel holds planes of the whole width: as wide as its shared memory, static and dynamic, allows
+    cudaFuncAttributes attr;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, vg::vocab_gemv_kernel);
+    dec->use_vocab_gemv = e == cudaSuccess && d % 128 == 0 && vg::vg_smem((int)d) + (int)attr.sharedSizeBytes <= 227 * 1024;
+    if (dec->use_vocab_gemv) e = cudaFuncSetAttribute(vg::vocab_gemv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, vg::vg_smem((int)d));
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "fold constants: %s", cudaGetErrorString(e));
     {
         const char *v = getenv("AED_DEC_NO_PDL");
@@ -892,7 +896,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.prefetch_ptr = wn.w_ff2; p.prefetch_bytes = (size_t)F * d * e2;
         AED_TRY(launch_step_gemm<sg::B_LN_RELU>(dec, KF_GEMM_FF2, m.ff2, dec->tc_src_hid, d, F, rows, p));
     }
-    if (!pf && dec->use_gemv && rows <= vg::kVgRows && d % 128 == 0 && vg::vg_smem(d) <= 227 * 1024) {
+    if (!pf && dec->use_gemv && dec->use_vocab_gemv && rows <= vg::kVgRows) {
         // at most 16 rows: final LayerNorm, vocabulary projection and argmax keys in one kernel (vocab_gemv.cuh)
         ProfScope ps(dec, KF_GEMM_VOCAB + KF_COUNT * KV_GEMV);
         vg::VocabGemvParams vp{};

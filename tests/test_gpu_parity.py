@@ -447,6 +447,14 @@ def test_plane_projections(model, batch):
 F32_DEEP = dict(n_layers=2, d_model=320, n_heads=5, d_ffn=1344, vocab=517, d_enc=192)
 
 
+@pytest.mark.parametrize("heads", [22, 24, 26])
+def test_vocabulary_projection_of_wide_models(heads):
+    """Few rows and a d_model (1408, 1536, 1664) around the widest that the few-row vocabulary kernel has shared memory for."""
+    model = dict(n_layers=1, d_model=64 * heads, n_heads=heads, d_ffn=256, vocab=300, d_enc=128)
+    w = wl.make_custom(model, [9, 5, 30], [3, 3, 2], dtype="bf16", seed=690 + heads, out_std=0.1)
+    _run_both(w, label=f"d{64 * heads}")
+
+
 @pytest.mark.parametrize("batch", [16, 17, 63, 64, 65, 80, 128, 129, 256, 257, 300])
 def test_vocabulary_projection_of_one_k_block(batch):
     """d_model 64: the ring of the vocabulary projection has one stage, and the accumulator's rows need more room than it

@@ -425,19 +425,19 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
     const int rh = blockIdx.x;
     const int r = rh / n_heads, h = rh % n_heads;
     const int4 ri = row_info[r];                       // (utterance, t_u, encoder length, encoder offset)
-    if (ri.x < 0) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        return;
-    }
     // The next kernel may start at once where that is a few-row projection, so that its weights are on their way while this
-    // one still waits (24 layers, 4 / 8 / 24 rows: 499 / 513 / 681 -> 473 / 486 / 661 us per step).  That holds for grids without
-    // padding rows: their blocks, above, end only after the wait, and the next kernel starts when every block has called it or
-    // ended.  (Same model now, 7 / 8 / 9 rows in grids of 8 / 8 / 16: 511 / 494 / 526 us.)  Not the cross-attention of
+    // one still waits (24 layers, 4 / 8 / 24 rows: 499 / 513 / 681 -> 473 / 486 / 661 us per step).  It starts when every block has
+    // called it or ended, so the blocks of padding rows, which end only after the wait, call it as well (1 / 2 / 7 / 9 / 12 rows in
+    // grids of 4 / 4 / 8 / 16 / 16: 455 / 470 / 506 / 523 / 533 -> 442 / 449 / 492 / 503 / 515).  Not the cross-attention of
     // steps with more than 128 rows, which read their statistics (no kRowStats): blocks of the next kernel would take room from
     // its own later ones (200 / 512 rows 2130 / 3488 -> 2224 / 3650).  Nor fp32, whose projections hold their weights in
     // registers (2 layers, 4 / 8 rows: 54 / 70 us per step against 59 / 75).
     constexpr bool kEarly = sizeof(CT) < 4 && (!kCross || kRowStats);
     if (kEarly) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (ri.x < 0) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
     const int u = ri.x;
     const int len = kCross ? ri.z : ri.y + 1;

@@ -107,54 +107,55 @@ __device__ __forceinline__ void red_add_v4(float *addr, float4 v)
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
-// ---- side jobs of a projection launch, run by 64 threads (two warps) of every CTA, off the critical path -----------
-// st: 0..63 among those threads; cta / n_cta: this CTA among all CTAs of the launch.
+// ---- side jobs of a projection launch, run by warps of their own in every CTA, off the critical path ----------------------
+// w / n_w: this warp among all that do them in the launch.
 // Static data (a later kernel's weights) into L2: no need to wait for the previous kernel.  4 KB pieces.
-__device__ __forceinline__ void side_prefetch(const StepGemmParams &p, int cta, int n_cta, int st)
+__device__ __forceinline__ void side_prefetch(const StepGemmParams &p, int w, int n_w, int lane)
 {
     for (int range = 0; range < 2; ++range) {
         const char *base = static_cast<const char *>(range ? p.prefetch2_ptr : p.prefetch_ptr);
         if (!base) continue;
         const size_t pieces = (range ? p.prefetch2_bytes : p.prefetch_bytes) / 4096;
-        for (size_t i = static_cast<size_t>(cta) * 64 + st; i < pieces; i += static_cast<size_t>(n_cta) * 64)
+        for (size_t i = static_cast<size_t>(w) * 32 + lane; i < pieces; i += static_cast<size_t>(n_w) * 32)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + i * 4096), "r"(4096) : "memory");
     }
 }
-// After the dependency wait: clear the rows a later split-K projection accumulates into, and (mean, rstd) of the rows
-// assigned to this CTA.  w: 0 or 1, which of the two warps; red_s, red_q: two floats of shared memory each.
-__device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_rows, int cta, int n_cta, int st, int lane, int w,
-                                                float *red_s, float *red_q)
+// After the dependency wait: (mean, rstd) of the rows assigned to this warp, and clear the rows a later split-K projection
+// accumulates into.  A launch ends with its last side job, so a row is read once by one warp, with all loads in flight, and kept in
+// registers (rows of at most 1024 features; wider ones are read again for the deviations).  (Two warps per row that read it twice, a
+// few loads at a time, were what QKV and FFN1 of a few rows ended with: 24 layers, 4 / 16 rows 478 / 533 -> 475 / 526 us a step.)
+__device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_rows, int w, int n_w, int lane)
 {
+    if (p.stats_src) {
+        constexpr int kHeld = 8;
+        for (int r = w; r < n_rows; r += n_w) {
+            const float *const xr = p.stats_src + static_cast<size_t>(r) * p.stats_d + lane * 4;
+            const int n = (p.stats_d + 127) / 128;    // (widths are multiples of 64)
+            float4 v[kHeld];
+            float s = 0.f, q = 0.f;
+            auto load = [&](int i) { return i * 128 + lane * 4 < p.stats_d ? *reinterpret_cast<const float4 *>(xr + i * 128) : make_float4(0.f, 0.f, 0.f, 0.f); };
+#pragma unroll
+            for (int i = 0; i < kHeld; ++i) v[i] = load(i);
+#pragma unroll
+            for (int i = 0; i < kHeld; ++i) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+            for (int i = kHeld; i < n; ++i) { const float4 u = load(i); s += (u.x + u.y) + (u.z + u.w); }
+            const float mean = warp_sum(s) / p.stats_d;
+            auto spread = [&](int i, float4 u) {
+                const float d0 = u.x - mean, d1 = u.y - mean, d2 = u.z - mean, d3 = u.w - mean;
+                if (i * 128 + lane * 4 < p.stats_d) q += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+            };
+#pragma unroll
+            for (int i = 0; i < kHeld; ++i) spread(i, v[i]);
+            for (int i = kHeld; i < n; ++i) spread(i, load(i));
+            q = warp_sum(q);
+            if (lane == 0) p.stats_out[r] = make_float2(mean, rsqrtf(q / p.stats_d + p.eps));
+        }
+    }
     if (p.zero_buf) {
         const size_t total4 = static_cast<size_t>(n_rows) * p.zero_cols / 4;
         float4 *z = reinterpret_cast<float4 *>(p.zero_buf);
-        for (size_t idx = static_cast<size_t>(cta) * 64 + st; idx < total4; idx += static_cast<size_t>(n_cta) * 64)
+        for (size_t idx = static_cast<size_t>(w) * 32 + lane; idx < total4; idx += static_cast<size_t>(n_w) * 32)
             z[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if (p.stats_src) {
-        for (int r = cta; r < n_rows; r += n_cta) {    // uniform over the two warps
-            const float *xr = p.stats_src + static_cast<size_t>(r) * p.stats_d;
-            float s = 0.f;
-            for (int idx = st * 4; idx < p.stats_d; idx += 256) {
-                const float4 v = *reinterpret_cast<const float4 *>(xr + idx);
-                s += (v.x + v.y) + (v.z + v.w);
-            }
-            s = warp_sum(s);
-            if (lane == 0) red_s[w] = s;
-            asm volatile("bar.sync 1, 64;" ::: "memory");
-            const float mean = (red_s[0] + red_s[1]) / p.stats_d;
-            float q = 0.f;
-            for (int idx = st * 4; idx < p.stats_d; idx += 256) {
-                const float4 v = *reinterpret_cast<const float4 *>(xr + idx);
-                const float d0 = v.x - mean, d1 = v.y - mean, d2 = v.z - mean, d3 = v.w - mean;
-                q += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
-            }
-            q = warp_sum(q);
-            if (lane == 0) red_q[w] = q;
-            asm volatile("bar.sync 1, 64;" ::: "memory");
-            if (st == 0) p.stats_out[r] = make_float2(mean, rsqrtf((red_q[0] + red_q[1]) / p.stats_d + p.eps));
-            asm volatile("bar.sync 1, 64;" ::: "memory");
-        }
     }
 }
 
@@ -175,7 +176,6 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     __shared__ __align__(8) uint64_t bar_done;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ float red_s[2], red_q[2];
 
     // timeline of the first producer thread of block 0 (debug builds)
     AED_TRACE_RESERVE(tcur, p.state, (threadIdx.x == 64 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ? 10u : 0u);
@@ -273,12 +273,11 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         }
     } else if (warp >= 10) {
         // ---- side jobs, off the critical path --------------------------------------------------------------
-        const int st = threadIdx.x - 320;                 // 0..63
         const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
         const int n_cta = gridDim.x * gridDim.y * gridDim.z;
-        side_prefetch(p, cta, n_cta, st);
+        side_prefetch(p, cta * 2 + warp - 10, n_cta * 2, lane);
         pdl_wait();
-        side_after_wait(p, p.state->n_active, cta, n_cta, st, lane, warp - 10, red_s, red_q);
+        side_after_wait(p, p.state->n_active, cta + n_cta * (warp - 10), n_cta * 2, lane);
     } else {
         pdl_wait();
         if (p.after_rows) pdl_launch_dependents();

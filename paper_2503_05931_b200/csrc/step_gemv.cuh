@@ -62,7 +62,6 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     extern __shared__ uint8_t smem_dyn[];
     __shared__ __align__(8) uint64_t bar_a[kSvMaxKb];
     __shared__ int abort_flag;
-    __shared__ float red_s[2], red_q[2];
     __shared__ float s_g[kSvMaxKb * kBlockK], s_c1[kSvMaxKb * kBlockK], s_c2[kSvMaxKb * kBlockK];      // per-k constants of this CTA's k range
     __shared__ __align__(16) float s_t[8][8][16 + 4];          // per warp: 8 rows x 16 features (+ pad), for the transposition
 
@@ -93,14 +92,13 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
                 tma_load_2d(tiles + static_cast<size_t>(i) * kATileBytes, mw, (kb_begin + i) * kBlockK, a0, &bar_a[i]);
             }
         }
-        const int st = threadIdx.x - 256;                 // 0..63
         const int cta = blockIdx.x + gridDim.x * blockIdx.y;
         const int n_cta = gridDim.x * gridDim.y;
-        sg::side_prefetch(p, cta, n_cta, st);
+        sg::side_prefetch(p, cta * 2 + warp - 8, n_cta * 2, lane);
         int n_rows = p.after_rows ? 0 : p.state->n_active;
         sg::pdl_wait();
         if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }
-        sg::side_after_wait(p, n_rows, cta, n_cta, st, lane, warp - 8, red_s, red_q);
+        sg::side_after_wait(p, n_rows, cta + n_cta * (warp - 8), n_cta * 2, lane);
         return;
     }
 
@@ -248,7 +246,6 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
     extern __shared__ uint8_t smem_dyn[];
     __shared__ __align__(8) uint64_t bar_a[kKB];
     __shared__ int abort_flag;
-    __shared__ float red_s[2], red_q[2];
     __shared__ __align__(16) float s_g[kKB * kBlockK], s_c1[kKB * kBlockK], s_c2[kKB * kBlockK];
     __shared__ __align__(16) float s_t[8][8][16 + 4];
 
@@ -282,14 +279,13 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
                 tma_load_2d(tiles + static_cast<size_t>(i) * kATileBytes, mw, (kb_begin + i) * kBlockK, a0, &bar_a[i]);
             }
         }
-        const int st = threadIdx.x - 256;
         const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
         const int n_cta = gridDim.x * gridDim.y * gridDim.z;
-        sg::side_prefetch(p, cta, n_cta, st);
+        sg::side_prefetch(p, cta * 2 + warp - 8, n_cta * 2, lane);
         int n_rows = p.after_rows ? 0 : p.state->n_active;
         sg::pdl_wait();
         if (p.after_rows) { n_rows = p.state->n_active; sg::pdl_launch_dependents(); }
-        sg::side_after_wait(p, n_rows, cta, n_cta, st, lane, warp - 8, red_s, red_q);
+        sg::side_after_wait(p, n_rows, cta + n_cta * (warp - 8), n_cta * 2, lane);
         return;
     }
 

@@ -531,7 +531,9 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
         if (lane == 0) sm_red[warp] = make_float2(s1, s2);
         __syncthreads();
         float t1 = 0.f, t2 = 0.f;
-        for (int w = 0; w < n_warps; ++w) { t1 += sm_red[w].x; t2 += sm_red[w].y; }
+#pragma unroll
+        for (int w = 0; w < kFusedMaxWarps; ++w)
+            if (w < n_warps) { t1 += sm_red[w].x; t2 += sm_red[w].y; }
         const float inv_n = 1.f / d_model;
         const float var = fmaxf((t2 - t1 * t1 * inv_n) * inv_n, 0.f);
         st = make_float2(x0 + t1 * inv_n, rsqrtf(var + ln_eps));
@@ -643,13 +645,31 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
     }
     __syncthreads();
     if (threadIdx.x < kHeadDim) {
-        float big = -INFINITY;
-        for (int w = 0; w < n_warps; ++w) big = fmaxf(big, sm_m[w]);
+        // Unrolled, so that all warps' results are loaded at once (24 layers, 8 / 64 rows, with the same above: 8 / 7 us a step).  fp32,
+        // whose weights take many instructions, is left alone (2 layers, 1 row: 45.7 us a step, unrolled 46.6).
         float lsum = 0.f, a = 0.f;
-        for (int w = 0; w < n_warps; ++w) {
-            const float wgt = (sm_m[w] == -INFINITY) ? 0.f : softmax_weight<CT>(sm_m[w] - big);
-            lsum = fmaf(sm_l[w], wgt, lsum);
-            a = fmaf(sm_acc[w][threadIdx.x], wgt, a);
+        if constexpr (sizeof(CT) < 4) {
+            float mw[kFusedMaxWarps], big = -INFINITY;
+#pragma unroll
+            for (int w = 0; w < kFusedMaxWarps; ++w) {
+                mw[w] = w < n_warps ? sm_m[w] : -INFINITY;
+                big = fmaxf(big, mw[w]);
+            }
+#pragma unroll
+            for (int w = 0; w < kFusedMaxWarps; ++w) {
+                if (w >= n_warps) continue;
+                const float wgt = (mw[w] == -INFINITY) ? 0.f : softmax_weight<CT>(mw[w] - big);
+                lsum = fmaf(sm_l[w], wgt, lsum);
+                a = fmaf(sm_acc[w][threadIdx.x], wgt, a);
+            }
+        } else {
+            float big = -INFINITY;
+            for (int w = 0; w < n_warps; ++w) big = fmaxf(big, sm_m[w]);
+            for (int w = 0; w < n_warps; ++w) {
+                const float wgt = (sm_m[w] == -INFINITY) ? 0.f : softmax_weight<CT>(sm_m[w] - big);
+                lsum = fmaf(sm_l[w], wgt, lsum);
+                a = fmaf(sm_acc[w][threadIdx.x], wgt, a);
+            }
         }
         const float o = a / lsum;
         const size_t off = (size_t)r * ldo + h * kHeadDim + threadIdx.x;

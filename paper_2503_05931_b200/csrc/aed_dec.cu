@@ -192,7 +192,6 @@ struct aed_dec {
     std::vector<TcLayerMaps> tc_layers;
     CUtensorMap tc_w_out;
     CUtensorMap tc_actd[16][2], tc_actf[16][2];   // [N/16 - 1][plane]: activation planes [rows, d] and [rows, F]
-    CUtensorMap tc_src_x[8], tc_src_att[8], tc_src_hid[8];   // fp32 sources of the fused projections, per MMA N
     bool use_tc = false;
     int sm_count = 148;
     int tc_target_ctas = 128;
@@ -200,7 +199,7 @@ struct aed_dec {
     bool use_pdl = true;
     bool attn_pipe = true;
     bool use_gemv = true;           // steps of few rows: projections by warp-level MMAs (step_gemv.cuh)
-    int gemv_rows = 64;             // ... up to this many rows
+    int gemv_rows = 48;             // ... up to this many rows
     bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
@@ -546,10 +545,6 @@ aed_status_t tc_setup(aed_dec *dec)
              encode_map(&dec->tc_actd[i][1], dec->ws + L.actd_lo, L.rows_cap, d, box) &&
              encode_map(&dec->tc_actf[i][0], dec->ws + L.actf_hi, L.rows_cap, F, box) &&
              encode_map(&dec->tc_actf[i][1], dec->ws + L.actf_lo, L.rows_cap, F, box);
-        if (i < 8)
-            ok = ok && encode_map(&dec->tc_src_x[i], dec->ws + L.x, c.max_batch, d, box, true) &&
-             encode_map(&dec->tc_src_att[i], dec->ws + L.act, c.max_batch, d, box, true) &&
-             encode_map(&dec->tc_src_hid[i], dec->ws + L.hid, c.max_batch, F, box, true);
     }
     if (!ok) return fail(nullptr, AED_ERR_CUDA, "cuTensorMapEncodeTiled failed (are all weight tensors 16-byte aligned?)");
     const int smem = kTcSmemBudget + 1024;
@@ -565,9 +560,10 @@ aed_status_t tc_setup(aed_dec *dec)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(e));
     dec->sm_count = sms > 0 ? sms : 148;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_GAMMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sg::step_gemm_kernel<sg::B_LN_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    for (const void *k : {(const void *)sg::step_gemm_kernel<sg::B_PLAIN, 1>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 2>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 4>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 8>,
+                          (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 1>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 2>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 4>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 8>,
+                          (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 1>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 2>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 4>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 8>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSgSmem + 1024);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(pg::plane_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
@@ -578,9 +574,6 @@ aed_status_t tc_setup(aed_dec *dec)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4, 4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4, 4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4, 4));
 
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(e));
     // LayerNorm-fold constants of every layer
@@ -625,7 +618,7 @@ aed_status_t tc_setup(aed_dec *dec)
         v = getenv("AED_DEC_NO_GEMV");
         dec->use_gemv = !(v && v[0] == '1');
         v = getenv("AED_DEC_GEMV_ROWS");
-        if (v && atoi(v) >= 1 && atoi(v) <= 64) dec->gemv_rows = atoi(v);
+        if (v && atoi(v) >= 1 && atoi(v) <= 48) dec->gemv_rows = atoi(v);
         v = getenv("AED_DEC_GEMV_DIRECT_ROWS");
         if (v && atoi(v) >= 0 && atoi(v) <= 8) dec->gemv_direct_rows = atoi(v);
         v = getenv("AED_DEC_PLANES_ROWS");
@@ -670,62 +663,55 @@ aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const v
 // ---- fused step (bf16 mode): 7 kernels per layer, chained with programmatic dependent launch -------------------
 
 template <int MODE>
-aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, const CUtensorMap *src_maps, int M,
+aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w, int M,
                               int K, int rows_ub, sg::StepGemmParams p,
                               const CUtensorMap *map_w2 = nullptr, int M2 = 0, bool after_rows = false)
 {
     // after_rows: the kernel before this launch makes the row table
     // map_w2, M2: a second weight matrix [M2, K] over the same rows (its output, gamma and bias are in p)
-    // Rows per CTA tile: up to 128 (two ring stages still fit beside the transposition buffer); more rows are
-    // covered by row tiles that re-read the weight tile from L2.
-    const int n_tile = tc_n_tile(rows_ub, 128), ni = n_tile / 16 - 1;
+    const int n_tile = tc_n_tile(rows_ub, sg::kSgMaxRows);
     const int m_tiles1 = (M + tc::kTileM - 1) / tc::kTileM;
     const int row_tiles = (rows_ub + n_tile - 1) / n_tile, m_tiles = m_tiles1 + (map_w2 ? (M2 + tc::kTileM - 1) / tc::kTileM : 0);
     p.tiles_first = map_w2 ? m_tiles1 : 0;
     p.after_rows = after_rows;
     p.a_rows2 = M2;
     const int k_blocks = K / tc::kBlockK;
-    const int stage_bytes = tc::kATileBytes + 2 * n_tile * tc::kBlockK * 2 + n_tile * tc::kBlockK * 4;
-    int stages = kTcSmemBudget / stage_bytes;
-    if (stages > sg::kMaxKb) stages = sg::kMaxKb;
-    // k-splits: every split adds rows x features x 4 bytes of red.global traffic, so large batches stop at about
-    // one CTA per SM.  Up to 64 rows that traffic is small, and CTAs with one or two k-blocks need so little
-    // shared memory that the CTAs of the next projection become resident beside them and fetch their weight
-    // tiles while this one still runs: there twice as many CTAs are worth it (measured on the 24-layer batch-64
-    // workload: 129 ms per pass with a target of 128 CTAs, 121 ms with 256, 147 ms with 384).
-    const int target_ctas = dec->tc_target_fixed ? dec->tc_target_ctas : (rows_ub <= 64 ? 256 : 128);
+    // k-splits: every split adds rows x features x 4 bytes of reductions, so the tcgen05 kernel stops at about one CTA per SM (256
+    // CTAs instead of 128: 64 / 96 / 128 rows 1043 / 1297 / 1493 -> 1378 / 1726 / 1950 us per step of the 24-layer model).  For the
+    // few-row kernels that traffic is small, and CTAs with one or two k-blocks need so little shared memory that the CTAs of the
+    // next projection become resident beside them and fetch their weight tiles while this one still runs: there twice as many CTAs
+    // are worth it (24-layer batch-64 workload: 129 ms per pass with a target of 128 CTAs, 121 ms with 256, 147 ms with 384).
+    const int target_ctas = dec->tc_target_fixed ? dec->tc_target_ctas : (rows_ub <= dec->gemv_rows ? 256 : 128);
     int splits = target_ctas / (m_tiles * row_tiles);
     if (splits < 1) splits = 1;
     if (splits > k_blocks) splits = k_blocks;
     const int kb_max = (k_blocks + splits - 1) / splits;
-    if (stages > kb_max) stages = kb_max;
-    p.stages = stages;
-    p.src_rows = dec->cfg.max_batch;
+    const int act_bytes = 2 * n_tile * tc::kBlockK * 2;          // of a k-block, both planes
+    p.stages = std::min(kb_max, sg::kMaxKb);
+    p.share = kb_max >= 4 ? 2 : kb_max >= 2 ? 1 : 0;
     p.a_rows = M;
     p.k_blocks = k_blocks;
     p.n_tile = n_tile;
     p.state = dec->state();
     p.eps = dec->cfg.ln_eps;
-    // Row tiles of 8 per CTA follow the row count: 2, 3 or 4, and from 33 rows two halves of 3 or 4 on grid.z with half the
-    // k-splits, up to four k-blocks per CTA.  A step of these sizes is bound by instructions issued (conversion of the
-    // rows to planes, fragments, reductions), so a tile of padding costs as much as one of rows.  Per decode step of the
-    // 24-layer model, with four tiles -> with three: 715 -> 630 us at 20 rows, 723 -> 680 at 24, 1104 -> 959 at 48; 33 to
-    // 40 rows left the tcgen05 kernel for it (939 / 952 / 1032 -> 837 / 825 / 922 us at 33 / 36 / 40 rows).  At 65 rows
-    // and beyond three or four such parts lose to the tcgen05 kernel (1392 / 1634 / 1881 us there against 1512 / 1655 /
-    // 2006 at 65 / 96 / 128 rows).
+    // Few rows: warp-level MMAs (step_gemv.cuh).  Row tiles of 8 per CTA follow the row count: 2, 3 or 4, and from 33 rows two
+    // halves of 3 on grid.z with half the k-splits, up to four k-blocks per CTA.  A step of these sizes is bound by
+    // instructions issued (conversion of the rows to planes, fragments, reductions), so a tile of padding costs as much as one of
+    // rows.  Per decode step of the 24-layer model, with four tiles -> with three: 715 -> 630 us at 20 rows, 723 -> 680 at 24, 1104 ->
+    // 959 at 48.  From 49 rows on the halves would need four tiles, and the tcgen05 kernel takes over (40 / 48 rows 905 / 949 us there
+    // against 879 / 922 here; 52 / 64 rows 984 / 1043 against 1064 / 1112).
     const int splits_wide = std::max((k_blocks + 3) / 4, splits / 2);
     const bool gemv = dec->use_gemv && rows_ub <= dec->gemv_rows &&
                       (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
     ProfScope ps(dec, family + KF_COUNT * (!gemv ? KV_NONE : rows_ub <= dec->gemv_direct_rows ? KV_GEMV : KV_GEMV_STAGED));
-    // Steps of at most 32 rows whose CTAs cover at most two k-blocks (64 rows, four): warp-level MMAs
-    // (step_gemv.cuh), activation fragments straight from global memory up to 4 rows, through shared memory beyond
+    // (whose CTAs cover at most two k-blocks, beyond 32 rows four; activation fragments straight from global memory up to 4 rows,
+    // through shared memory beyond)
     if (gemv) {
         cudaLaunchConfig_t gc = {};
         gc.gridDim = dim3(m_tiles, splits, 1);
         gc.blockDim = dim3(sv::kSvThreads);
         const bool direct = rows_ub <= dec->gemv_direct_rows, wide = rows_ub > 32;
-        const int part = wide ? (rows_ub + 1) / 2 : rows_ub;
-        const int nt = wide ? (part <= 24 ? 3 : 4) : part <= 16 ? 2 : part <= 24 ? 3 : 4;      // row tiles of 8 per CTA
+        const int nt = wide ? 3 : rows_ub <= 16 ? 2 : rows_ub <= 24 ? 3 : 4;                   // row tiles of 8 per CTA
         if (wide) gc.gridDim = dim3(m_tiles, splits_wide, 2);
         gc.dynamicSmemBytes = direct ? (size_t)sv::kSvMaxKb * tc::kATileBytes + 1024 : (size_t)sv::sv_staged_smem(nt, wide ? 4 : sv::kSvMaxKb);
         gc.stream = dec->stream;
@@ -736,8 +722,7 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
         gc.numAttrs = 1;
         const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
         cudaError_t ge = direct    ? cudaLaunchKernelEx(&gc, sv::step_gemv_kernel<MODE, 1>, map_w, second, p)
-                         : wide    ? (nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3, 4>, map_w, second, p)
-                                              : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4, 4>, map_w, second, p))
+                         : wide    ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3, 4>, map_w, second, p)
                          : nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3>, map_w, second, p)
                          : nt == 2 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 2>, map_w, second, p)
                                    : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4>, map_w, second, p);
@@ -748,14 +733,19 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m_tiles, splits, row_tiles);
     cfg.blockDim = dim3(sg::kSgThreads);
-    cfg.dynamicSmemBytes = (size_t)stages * stage_bytes + 1024;
+    cfg.dynamicSmemBytes = (size_t)p.stages * (tc::kATileBytes + act_bytes) + 1024;
     cfg.stream = dec->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE>, map_w, src_maps[ni], map_w2 ? *map_w2 : src_maps[ni], p);
+    const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
+    const int rows_per_thread = (n_tile * (8 << p.share) + sg::kSgConvertThreads - 1) / sg::kSgConvertThreads;
+    cudaError_t e = rows_per_thread <= 1   ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 1>, map_w, second, p)
+                    : rows_per_thread <= 2 ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 2>, map_w, second, p)
+                    : rows_per_thread <= 4 ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 4>, map_w, second, p)
+                                           : cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 8>, map_w, second, p);
     if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(e));
     AED_LAUNCHED(dec);
     return AED_OK;
@@ -849,7 +839,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.prefetch2_ptr = wn.w_q_c; p.prefetch2_bytes = (size_t)d * d * e2;
         // the vocabulary matrix is as large as a layer: its way into L2 starts a whole layer ahead of the projection
         if (l == c.n_layers - 1) { p.prefetch2_ptr = dec->w_out; p.prefetch2_bytes = (size_t)V * d * e2; }
-        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, dec->tc_src_x, 3 * d, d, rows_ub, p, &m.qc, d, embedded && l == 0));
+        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_QKV, m.qkv, 3 * d, d, rows_ub, p, &m.qc, d, embedded && l == 0));
         // 2. self-attention (applies LN1 to q, k, v; appends k, v)
         if (pf && l == c.n_layers - 1) rows = pf->last_chunk ? pf->batch : 0;
         AED_TRY(launch_self_attention(dec, rows_ub, rows, self_len_ub, self_cache, att, nullptr, nullptr, stats, c1_qkv, c2_qkv, pf != nullptr));
@@ -864,7 +854,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.zero_buf = hid; p.zero_cols = F;
         p.prefetch_ptr = wn.w_o; p.prefetch_bytes = (size_t)d * d * e2;
         p.prefetch2_ptr = dec->at<T>(L.comp_w) + (size_t)((l + 1) % c.n_layers) * d * d; p.prefetch2_bytes = (size_t)d * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_O, m.o, dec->tc_src_att, d, d, rows, p, &m.o_qc, d));
+        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_O, m.o, d, d, rows, p, &m.o_qc, d));
         // 4. cross-attention; every block computes the LN2 statistics of its row of x_new itself
         if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
             const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
@@ -880,21 +870,21 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_o_c;
         p.zero_buf = qkv; p.zero_cols = 3 * d;
         p.prefetch_ptr = wn.w_o_c; p.prefetch_bytes = (size_t)d * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_OC, m.oc, dec->tc_src_att, d, d, rows, p));
+        AED_TRY(launch_step_gemm<sg::B_PLAIN>(dec, KF_GEMM_OC, m.oc, d, d, rows, p));
         // 6. hidden raw = (gamma3 * x) W1^T ; side: LN3 statistics
         p = sg::StepGemmParams{};
         p.src = x; p.ld_src = d; p.gamma = (const T *)w.ln3_g;
         p.out = hid; p.ldo = F;
         p.stats_src = x; p.stats_out = stats + 2 * stats_stride; p.stats_d = d;
         p.prefetch_ptr = wn.w_ff1; p.prefetch_bytes = (size_t)F * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_FF1, m.ff1, dec->tc_src_x, F, d, rows, p));
+        AED_TRY(launch_step_gemm<sg::B_GAMMA>(dec, KF_GEMM_FF1, m.ff1, F, d, rows, p));
         // 7. x += relu(LN3-corrected hidden) W2^T + b2 ; side: clear the cross-query rows
         p = sg::StepGemmParams{};
         p.src = hid; p.ld_src = F; p.c1 = c1_ff; p.c2 = c2_ff; p.stats_in = stats + 2 * stats_stride;
         p.out = x; p.ldo = d; p.bias = (const T *)w.b_ff2;
         p.zero_buf = qc; p.zero_cols = d;          // the next layer's first launch accumulates into it
         p.prefetch_ptr = wn.w_ff2; p.prefetch_bytes = (size_t)F * d * e2;
-        AED_TRY(launch_step_gemm<sg::B_LN_RELU>(dec, KF_GEMM_FF2, m.ff2, dec->tc_src_hid, d, F, rows, p));
+        AED_TRY(launch_step_gemm<sg::B_LN_RELU>(dec, KF_GEMM_FF2, m.ff2, d, F, rows, p));
     }
     if (!pf && dec->use_gemv && dec->use_vocab_gemv && rows <= vg::kVgRows) {
         // at most 16 rows: final LayerNorm, vocabulary projection and argmax keys in one kernel (vocab_gemv.cuh)

@@ -1,29 +1,36 @@
-// Decode-step projection on tensor cores with the activation operand built in the kernel.
+// Decode-step projection on tensor cores with the activation operand built in the kernel, for steps of 49 to 128 rows (fewer
+// rows: step_gemv.cuh, more: plane_gemm.cuh).
 //
 //   out[r, o] += sum_k B(r, k) * W[o, k]      (+ bias[o] from the CTA of the first k-split)
 //
-// W tiles (128 output features x 64 k, bf16) arrive by TMA; they do not depend on earlier kernels, so they are
-// requested before the programmatic-dependency wait and stream in while the previous kernel drains.
-// The activation tile B is produced by four warps straight from fp32 sources into the 128-byte-swizzled layout the
-// MMA reads, as a bf16 high plane and a bf16 low plane (value - high), with one of three transforms fused:
+// A CTA has 128 output features and up to four k-blocks of 64 at a time.  The weight tiles (bf16, TMA) do not depend on
+// earlier kernels and are requested before the programmatic-dependency wait.  The activation tiles are made by 16 warps from
+// the fp32 source in the 128-byte-swizzled layout the MMA reads, as a bf16 high plane and a bf16 low plane
+// (value - high) behind each other, so that one MMA of twice the rows multiplies both; with one of three transforms fused:
 //   B_PLAIN    B = src                                   (attention output -> output projection)
 //   B_GAMMA    B = gamma[k] * src                        (LayerNorm folded into the projection, see below)
 //   B_LN_RELU  B = relu(rstd_r * (src - mean_r * c1[k]) + c2[k])   (FFN hidden layer from the folded first GEMM)
-// (Steps with many rows have planes made once per projection input, plane_gemm.cuh: there every feature tile would convert
-// the same activation rows again, and the conversion, not the tensor cores, would set the pace.)
+//
+// What bounds it: a chain of hand-overs inside one launch.  Cycles at 64 rows, K = 256 per CTA: source rows from L2 900 to 1000,
+// conversion (64 x 256 values) 2000, 16 MMAs and their hand-over 1800, reductions 1200 (an SM gives out 28 bytes a cycle).  So the
+// k-blocks are converted side by side by groups of warps whose per-k constants wait in registers, and the MMAs are issued in
+// one go.  The forms before (up to 64 rows warp-level MMAs; beyond 8 converting warps, source tiles by TMA, a ring of k-blocks with
+// a barrier each, transposed reductions) took, per step of the 24-layer model, 56 / 64 / 80 / 96 / 112 / 128 rows
+// 1093 / 1120 / 1336 / 1485 / 1605 / 1746 us; with this one 1003 / 1039 / 1222 / 1298 / 1393 / 1496.
+// (Tried on the way: k-splits that meet in a cluster through distributed shared memory, which would leave complete sums and planes
+// for the next projection: SM-to-SM reads ran at 10 to 20 bytes a cycle beside the other traffic, 64 rows 1456.)
 //
 // LayerNorm folding: LN(x) W^T = rstd * ((gamma*x) W^T - mean * c1) + c2 with c1[o] = sum_k gamma_k W[o,k] and
 // c2[o] = sum_k beta_k W[o,k] + b[o].  The GEMM therefore runs on gamma*x without knowing the row statistics;
-// whoever consumes its output applies (mean, rstd).  The statistics themselves are a side job: while the MMAs
-// run, the producer warps of this kernel compute mean and rstd of the rows assigned to their CTA and store
-// them for the consumer.  A second side job clears the fp32 rows a later split-K projection accumulates into.
+// whoever consumes its output applies (mean, rstd).  The statistics themselves are a side job: a warp of its own
+// computes mean and rstd of the rows assigned to its CTA and stores them for the
+// consumer.  A second side job clears the fp32 rows a later split-K projection accumulates into.
 //
 // Two matrices in one launch: feature tiles blockIdx.x >= tiles_first belong to a second weight
 // matrix over the same activation rows, with its own tensor map, gamma,
 // bias and output buffer.  This is how one launch serves two projections that depend on the same earlier kernel.
 //
-// A CTA walks its k-blocks through a ring of up to 4 stages (weight tile, two planes, fp32 source tile each); with
-// few k-blocks per CTA (small batches, many k-splits) everything is resident at once.  Waits are bounded.
+// Waits are bounded.
 #pragma once
 #include "tc_gemm.cuh"
 
@@ -32,17 +39,20 @@ namespace sg {
 
 using namespace tc;
 
-constexpr int kMaxKb = 4;             // ring stages per CTA
-constexpr int kSgThreads = 384;       // warp 0 TMA, warp 1 MMA, warps 2..9 activation tiles and epilogue, warps 10..11 side jobs
+constexpr int kMaxKb = 4;             // k-blocks that a CTA holds at most
+constexpr int kSgConvertWarps = 16, kSgMmaWarp = 16, kSgConvertThreads = kSgConvertWarps * 32;
+constexpr int kSgThreads = 576;       // warps 0..15 activation tiles and epilogue, warp 16 MMAs, warp 17 side jobs
+constexpr int kSgMaxRows = 128;       // rows per CTA tile
+constexpr int kSgSmem = 192 * 1024;   // of all tiles at most
 
 enum BMode { B_PLAIN = 0, B_GAMMA = 1, B_LN_RELU = 2 };
 
 struct StepGemmParams {
     int a_rows;                // output features M
     int k_blocks;              // K / 64
-    int n_tile;                // MMA N: rows per CTA tile (16..256, multiple of 16)
-    int stages;                // ring depth, 1..kMaxKb
-    int src_rows;              // rows of the source buffer (reads of rows past it are clamped)
+    int n_tile;                // rows per CTA tile (16..128, multiple of 16)
+    int stages;                // k-blocks that a CTA holds at a time, 1..kMaxKb
+    int share;                 // 1 << share groups of threads take turns with the k-blocks
     // activation source [rows, ld_src] fp32
     const float *src;
     int ld_src;
@@ -92,10 +102,8 @@ __device__ __forceinline__ void split_planes(const float (&y)[8], uint4 &hi, uin
     uint32_t h[4], l[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(y[2 * i]), h1 = __float2bfloat16_rn(y[2 * i + 1]);
-        __nv_bfloat162 hp = __halves2bfloat162(h0, h1);
-        h[i] = *reinterpret_cast<uint32_t *>(&hp);
-        l[i] = pack_bf16(y[2 * i] - __bfloat162float(h0), y[2 * i + 1] - __bfloat162float(h1));
+        h[i] = pack_bf16(y[2 * i], y[2 * i + 1]);
+        l[i] = pack_bf16(y[2 * i] - __uint_as_float(h[i] << 16), y[2 * i + 1] - __uint_as_float(h[i] & 0xFFFF0000u));
     }
     hi = make_uint4(h[0], h[1], h[2], h[3]);
     lo = make_uint4(l[0], l[1], l[2], l[3]);
@@ -106,6 +114,8 @@ __device__ __forceinline__ void red_add_v4(float *addr, float4 v)
 {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
+
+__device__ __forceinline__ void red_add(float *addr, float v) { asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(v) : "memory"); }
 
 // ---- side jobs of a projection launch, run by warps of their own in every CTA, off the critical path ----------------------
 // w / n_w: this warp among all that do them in the launch.
@@ -159,251 +169,194 @@ __device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_r
     }
 }
 
-// grid: x = 128-feature tiles, y = k-splits, z = row tiles.
-// Dynamic smem per k-block: weight tile 16 KB | high plane | low plane (n_tile x 128 B each) | fp32 source tile
-// (n_tile x 256 B, filled by TMA, later reused to transpose the accumulator); plus 1024 for alignment.
-template <int MODE>
-__global__ void __launch_bounds__(kSgThreads, 2)
-step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_src,
-                 const __grid_constant__ CUtensorMap map_w2, StepGemmParams p)
+// grid: x = 128-feature tiles, y = k-splits, z = row tiles.  kNI: rows of a k-block per thread at most.
+// Dynamic smem (from a 1024-byte boundary): p.stages weight tiles of 16 KB | as many activation tiles of 2 n_tile x 128 bytes (high plane, low plane).
+template <int MODE, int kNI>
+__global__ void __launch_bounds__(kSgThreads, 1)
+step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ StepGemmParams p)
 {
-    // map_src: fp32 source tiles
     extern __shared__ uint8_t smem_dyn[];
-    __shared__ __align__(8) uint64_t bar_a[kMaxKb];
-    __shared__ __align__(8) uint64_t bar_s[kMaxKb];
-    __shared__ __align__(8) uint64_t bar_b[kMaxKb];
-    __shared__ __align__(8) uint64_t bar_e[kMaxKb];
-    __shared__ __align__(8) uint64_t bar_done;
+    __shared__ __align__(8) uint64_t bar_w, bar_done;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
-    // timeline of the first producer thread of block 0 (debug builds)
-    AED_TRACE_RESERVE(tcur, p.state, (threadIdx.x == 64 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ? 10u : 0u);
-    AED_TRACE_PUT_NS(p.state, tcur, 19);
+    AED_TRACE_RESERVE(tcur, p.state, (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ? 10u : 0u);
+    AED_TRACE_PUT_NS(p.state, tcur, 40 + MODE);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool second_w = p.tiles_first > 0 && static_cast<int>(blockIdx.x) >= p.tiles_first;
-    const CUtensorMap *mw = second_w ? &map_w2 : &map_w;
+    const CUtensorMap *const mw = second_w ? &map_w2 : &map_w;
     const int a0 = (second_w ? static_cast<int>(blockIdx.x) - p.tiles_first : static_cast<int>(blockIdx.x)) * kTileM;
     const int a_rows = second_w ? p.a_rows2 : p.a_rows;
     const int row0 = blockIdx.z * p.n_tile;
     const int kb_begin = static_cast<int>((static_cast<long long>(p.k_blocks) * blockIdx.y) / gridDim.y);
     const int kb_end = static_cast<int>((static_cast<long long>(p.k_blocks) * (blockIdx.y + 1)) / gridDim.y);
-    const int n_kb = kb_end - kb_begin;
-    const int S = p.stages;
-    // Small tiles (at most 32 rows, one or two k-blocks): the producer threads read their 8 source values per k-block
-    // straight from global memory right after the dependency wait instead of waiting for a TMA copy into shared memory.
-    const bool direct = p.n_tile <= 32 && n_kb <= 2;
-
-    uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
+    const int n_kb = kb_end - kb_begin, S = p.stages;
+    uint8_t *const tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
     const int plane_bytes = p.n_tile * kBlockK * 2;
-    const int src_bytes = p.n_tile * kBlockK * 4;
-    const int stage_bytes = kATileBytes + 2 * plane_bytes + src_bytes;
+    uint8_t *const acts = tiles + S * kATileBytes;
     uint32_t tmem_cols = 32;
-    while (tmem_cols < static_cast<uint32_t>(p.n_tile)) tmem_cols <<= 1;
+    while (tmem_cols < static_cast<uint32_t>(2 * p.n_tile)) tmem_cols <<= 1;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kMaxKb; ++s) { mbar_init(&bar_a[s], 1); mbar_init(&bar_s[s], 1); mbar_init(&bar_b[s], 8); mbar_init(&bar_e[s], 1); }
+    if (threadIdx.x == kSgMmaWarp * 32) {
+        mbar_init(&bar_w, 1);
         mbar_init(&bar_done, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(&tmem_slot, tmem_cols);
+    if (warp == kSgMmaWarp) {
+        __syncwarp();
+        if (elect_one()) {                            // weights: independent of every earlier kernel
+            const int n = min(n_kb, S);
+            mbar_expect_tx(&bar_w, n * kATileBytes);
+            for (int i = 0; i < n; ++i) tma_load_2d(tiles + i * kATileBytes, mw, (kb_begin + i) * kBlockK, a0, &bar_w);
+        }
+        __syncwarp();
+        tmem_alloc(&tmem_slot, tmem_cols);
+    }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_slot;
     if (!p.after_rows) pdl_launch_dependents();
-    AED_TRACE_PUT(p.state, tcur, 40);      // set-up done
 
-    if (warp == 0) {
-        if (lane == 0) {
-            prefetch_tensormap(mw);
-            prefetch_tensormap(&map_src);
-            const int pre = n_kb < S ? n_kb : S;
-            for (int i = 0; i < pre; ++i) {       // weights: independent of every earlier kernel
-                mbar_expect_tx(&bar_a[i], kATileBytes);
-                tma_load_2d(tiles + static_cast<size_t>(i) * stage_bytes, mw, (kb_begin + i) * kBlockK, a0, &bar_a[i]);
-            }
-        }
-        pdl_wait();
-        if (lane == 0) {
-            for (int i = 0; i < n_kb; ++i) {
-                const int s = i % S;
-                uint8_t *stage = tiles + static_cast<size_t>(s) * stage_bytes;
-                if (i >= S) {                     // the stage is free once the MMAs of k-block i - S have read it
-                    if (!mbar_wait(&bar_e[s], ((i / S) - 1) & 1, &abort_flag)) break;
-                    mbar_expect_tx(&bar_a[s], kATileBytes);
-                    tma_load_2d(stage, mw, (kb_begin + i) * kBlockK, a0, &bar_a[s]);
-                }
-                // fp32 activation source, written by the previous kernels
-                if (!direct) {
-                    mbar_expect_tx(&bar_s[s], src_bytes);
-                    tma_load_2d(stage + kATileBytes + 2 * plane_bytes, &map_src, (kb_begin + i) * kBlockK, row0, &bar_s[s]);
-                }
-            }
-        }
-    } else if (warp == 1) {
-        pdl_wait();
-        if (lane == 0) {
-            const uint32_t idesc = instr_desc_bf16(p.n_tile);
-            bool ok = true;
-            for (int i = 0; i < n_kb && ok; ++i) {
-                const int s = i % S;
-                const uint32_t par = (i / S) & 1;
-                ok = mbar_wait(&bar_b[s], par, &abort_flag) && mbar_wait(&bar_a[s], par, &abort_flag);
-                if (!ok) break;
+    // Rounds of up to S k-blocks (one round unless the launch has few blocks for its K): tiles written -> barrier 4 -> MMAs -> barrier 3.
+    // The MMAs of a round are issued in one go: a wait or a commit between them costs more than the four MMAs of a k-block
+    // (16 MMAs of 128 x 64 x 16: 1160 cycles, with a wait and a commit per k-block 2290).
+    if (warp == kSgMmaWarp) {
+        // B: 2 n_tile rows of planes; their products with a weight tile stand in columns r and n_tile + r
+        const uint32_t idesc = instr_desc_bf16(2 * p.n_tile);
+        const uint64_t dw0 = smem_desc_sw128(smem_u32(tiles)), da0 = smem_desc_sw128(smem_u32(acts));
+        bool ok = true;
+        uint32_t phase = 0;
+        for (int i0 = 0; i0 < n_kb; i0 += S, phase ^= 1) {
+            asm volatile("bar.sync 4, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
+            if (ok) ok = mbar_wait(&bar_w, phase, &abort_flag);
+            if (ok) {
                 tc_fence_after_sync();
-                const uint32_t sa = smem_u32(tiles + static_cast<size_t>(s) * stage_bytes);
-                const uint64_t da = smem_desc_sw128(sa), dh = smem_desc_sw128(sa + kATileBytes),
-                               dl = smem_desc_sw128(sa + kATileBytes + plane_bytes);
+                if (elect_one()) {
+                    for (int i = 0; i < min(S, n_kb - i0); ++i) {
+                        const uint64_t dw = dw0 + i * (kATileBytes >> 4), da = da0 + static_cast<uint64_t>(i * 2 * plane_bytes >> 4);
 #pragma unroll
-                for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dh + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
-#pragma unroll
-                for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
-                if (i + S < n_kb) mma_commit(&bar_e[s]);      // someone is waiting to refill this stage
-            }
-            if (ok) mma_commit(&bar_done);
-            else {
-                // weight copies that were requested must land before the block retires
-                for (int s = 0; s < S && s < n_kb; ++s) {
-                    const long long start = clock64();
-                    while (!mbar_try_wait(&bar_a[s], 0) && clock64() - start < kWaitCycles / 8) {}
+                        for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, dw + 2 * k, da + 2 * k, idesc, (i0 + i > 0 || k > 0) ? 1u : 0u);
+                    }
+                    mma_commit(&bar_done);
                 }
+                __syncwarp();
+                ok = mbar_wait(&bar_done, phase, &abort_flag);
             }
+            if (ok && i0 + S < n_kb && elect_one()) {
+                const int n = min(S, n_kb - i0 - S);
+                mbar_expect_tx(&bar_w, n * kATileBytes);
+                for (int i = 0; i < n; ++i) tma_load_2d(tiles + i * kATileBytes, mw, (kb_begin + i0 + S + i) * kBlockK, a0, &bar_w);
+            }
+            __syncwarp();
+            if (!ok) {
+                // gave up: copies in flight land within microseconds; leave them a millisecond
+                const long long start = clock64();
+                while (clock64() - start < 2000000ll) {}
+            }
+            // (one thread polls, the other warps sleep here)
+            asm volatile("bar.sync 3, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
         }
-    } else if (warp >= 10) {
+    } else if (warp > kSgMmaWarp) {
         // ---- side jobs, off the critical path --------------------------------------------------------------
         const int cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
         const int n_cta = gridDim.x * gridDim.y * gridDim.z;
-        side_prefetch(p, cta * 2 + warp - 10, n_cta * 2, lane);
+        side_prefetch(p, cta, n_cta, lane);
         pdl_wait();
-        side_after_wait(p, p.state->n_active, cta + n_cta * (warp - 10), n_cta * 2, lane);
+        side_after_wait(p, p.state->n_active, cta, n_cta, lane);
     } else {
-        pdl_wait();
-        if (p.after_rows) pdl_launch_dependents();
-        AED_TRACE_PUT(p.state, tcur, 41);  // dependency resolved
-        const int pt = threadIdx.x - 64;                  // 0..255 among the producer threads
-        const int n_rows = p.state->n_active;
-        // ---- activation tiles --------------------------------------------------------------------------
-        // Thread pt owns the 16-byte output chunk c = pt & 7 (8 consecutive k) of rows (pt >> 3) + 32 j.  The fp32
-        // source tile of each k-block is already on its way into shared memory (TMA, no swizzle, 256 B per row).
-        // Each k-block has its own barrier, so the MMAs of one k-block run while the next is converted.
-        const int c = pt & 7, rbase = pt >> 3;
-        const int quarter = warp & 3;
-        const int a_idx = a0 + quarter * 32 + lane;
-        const bool a_ok = a_idx < a_rows;
+        // A k-block is the work of 512 >> share threads: each has a 16-byte chunk c (8 consecutive k) of rows rbase, rbase + step, ...
+        // of either plane.  The groups of threads take a k-block of the round each, and have its per-k constants (static) in registers
+        // before the dependency wait.
+        const int step = (kSgConvertThreads / 8) >> p.share, c = threadIdx.x & 7, rbase = (threadIdx.x >> 3) & (step - 1), group = threadIdx.x >> (9 - p.share);
+        const __nv_bfloat16 *const gamma = second_w ? p.gamma2 : p.gamma;
+        float ka[8], kb[8];                           // gamma; or c1, c2
+        auto constants = [&](int i) {
+            const int k = (kb_begin + i) * kBlockK + c * 8;
+            if (MODE == B_GAMMA) load_vec(gamma + k, aligned16(gamma), ka);
+            if (MODE == B_LN_RELU) { load8(p.c1 + k, ka); load8(p.c2 + k, kb); }
+        };
+        if (group < n_kb) constants(group);
+        const int quarter = warp & 3, a_idx = a0 + quarter * 32 + lane;
         float bias = 0.f;
-        if (blockIdx.y == 0 && a_ok) {
+        if (blockIdx.y == 0 && a_idx < a_rows) {
             if (second_w) bias = p.bias2 ? p.bias2[a_idx] : 0.f;
             else bias = p.bias ? to_f32(p.bias[a_idx]) : 0.f;
         }
         float *const out = second_w ? p.out2 : p.out;
         const int ldo = second_w ? p.ldo2 : p.ldo;
-        const __nv_bfloat16 *const gamma = second_w ? p.gamma2 : p.gamma;
-        const bool gamma_aligned = aligned16(gamma);
-        float dv[2][8];
-        if (direct && rbase < p.n_tile) {          // one row per thread (n_tile <= 32), both k-blocks requested at once
-            const int rs = min(row0 + rbase, p.src_rows - 1);
+        int n_rows = p.after_rows ? 0 : p.state->n_active;
+        AED_TRACE_PUT(p.state, tcur, 50);             // set up, weights requested
+        pdl_wait();
+        if (p.after_rows) { n_rows = p.state->n_active; pdl_launch_dependents(); }
+        AED_TRACE_PUT_NS(p.state, tcur, 51);          // dependency resolved
+        // ---- activation tiles ----
+        const int rows_here = min(p.n_tile, max(n_rows - row0, 0)), mine = rows_here - rbase;
+        const float *const src = p.src + static_cast<size_t>(row0 + rbase) * p.ld_src + kb_begin * kBlockK + c * 8;
+        constexpr int kHeld = kNI < 4 ? kNI : 4;      // rows in flight
+        for (int i0 = 0; i0 < n_kb; i0 += S) {
+            for (int s = group; s < min(S, n_kb - i0); s += 1 << p.share) {
+                const int i = i0 + s;
+                float x[kHeld][8];
+                float2 st[kHeld];
+                auto load = [&](int j) {
+                    if (j * step >= mine) return;
+                    load8(src + static_cast<size_t>(j * step) * p.ld_src + i * kBlockK, x[j % kHeld]);
+                    if (MODE == B_LN_RELU) st[j % kHeld] = p.stats_in[row0 + rbase + j * step];
+                };
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-                if (i < n_kb) load8(p.src + static_cast<size_t>(rs) * p.ld_src + (kb_begin + i) * kBlockK + c * 8, dv[i]);
-        }
-        bool ok = true;
-        for (int i = 0; i < n_kb && ok; ++i) {
-            const int s = i % S;
-            uint8_t *stage = tiles + static_cast<size_t>(s) * stage_bytes;
-            uint8_t *hi_tile = stage + kATileBytes, *lo_tile = hi_tile + plane_bytes;
-            const float *src_tile = reinterpret_cast<const float *>(lo_tile + plane_bytes);
-            const int k = (kb_begin + i) * kBlockK + c * 8;
-            float g[8], c1[8], c2[8];
-            if (MODE == B_GAMMA) load_vec(gamma + k, gamma_aligned, g);
-            if (MODE == B_LN_RELU) { load8(p.c1 + k, c1); load8(p.c2 + k, c2); }
-            if (!direct) ok = mbar_wait(&bar_s[s], (i / S) & 1, &abort_flag);
-            if (!ok) break;
-            for (int rl = rbase; rl < p.n_tile; rl += 32) {
-                const int r = row0 + rl;
-                float y[8];
-                if (r < n_rows) {
-                    if (direct) {
+                for (int j = 0; j < kHeld; ++j) load(j);
+                if (i != group) constants(i);
+                uint8_t *const hi_tile = acts + s * 2 * plane_bytes, *const lo_tile = hi_tile + plane_bytes;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) y[e] = i == 0 ? dv[0][e] : dv[1][e];
-                    } else load8(src_tile + rl * kBlockK + c * 8, y);
-                    if (MODE == B_GAMMA) {
+                for (int j = 0; j < kNI; ++j) {
+                    if (j * step >= mine) break;      // (rows past the last: what the tile holds, in columns that nobody reads)
+                    float (&y)[8] = x[j % kHeld];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) y[e] *= g[e];
-                    } else if (MODE == B_LN_RELU) {
-                        const float2 st = p.stats_in[r];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) y[e] = fmaxf(fmaf(st.y, y[e] - st.x * c1[e], c2[e]), 0.f);
+                    for (int e = 0; e < 8; ++e) {
+                        if (MODE == B_GAMMA) y[e] *= ka[e];
+                        if (MODE == B_LN_RELU) y[e] = fmaxf(fmaf(st[j % kHeld].y, y[e] - st[j % kHeld].x * ka[e], kb[e]), 0.f);
                     }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) y[e] = 0.f;
+                    uint4 hi, lo;
+                    split_planes(y, hi, lo);
+                    const int rl = rbase + j * step, off = rl * 128 + ((c ^ (rl & 7)) << 4);
+                    *reinterpret_cast<uint4 *>(hi_tile + off) = hi;
+                    *reinterpret_cast<uint4 *>(lo_tile + off) = lo;
+                    if (j + kHeld < kNI) load(j + kHeld);
                 }
-                uint4 hi, lo;
-                split_planes(y, hi, lo);
-                const int off = rl * 128 + ((c ^ (rl & 7)) << 4);
-                *reinterpret_cast<uint4 *>(hi_tile + off) = hi;
-                *reinterpret_cast<uint4 *>(lo_tile + off) = lo;
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor-core reads
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_b[s])) : "memory");
+            if (i0 == 0) AED_TRACE_PUT(p.state, tcur, 52);                 // activation tiles written
+            asm volatile("bar.sync 4, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
+            asm volatile("bar.sync 3, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
         }
-        AED_TRACE_PUT(p.state, tcur, 42);  // activation tiles written
-        {
-        // ---- epilogue: accumulator -> shared memory (transposed) -> 16-byte reductions ---------------------------
-        // Warps w and w + 4 reach the same accumulator lanes (lane quarter = warp & 3): they split the rows in 16s.
-        ok = ok && mbar_wait(&bar_done, 0, &abort_flag);
+        // ---- epilogue: reductions straight from the accumulator, 128 consecutive bytes per warp and row ----------------------
+        // (An SM gives out about 28 bytes a cycle, as 4-byte reductions of whole warps or as 16-byte ones: 64 rows x 128 features 1220 and
+        // 1230 cycles; a pass through shared memory for the latter costs another 800.)
+        // Warps w, w + 4, ... reach the same accumulator lanes (lane quarter = warp & 3): they split the rows in 16s.
+        const bool ok = *static_cast<volatile int *>(&abort_flag) == 0;
         tc_fence_after_sync();
-        AED_TRACE_PUT(p.state, tcur, 44);  // accumulator complete
-        // every MMA has completed, so the whole stage area is free: T[r][o], 132 floats per row (bank spread)
-        float *trans = reinterpret_cast<float *>(tiles);
-        constexpr int kPitch = kTileM + 4;
-        const int rows_here = min(p.n_tile, max(n_rows - row0, 0));
-        const int second = warp >= 6 ? 1 : 0;
-        const bool fits = static_cast<size_t>(p.n_tile) * kPitch * 4 <= static_cast<size_t>(n_kb < S ? n_kb : S) * stage_bytes;
-        if (ok && fits) {
+        AED_TRACE_PUT(p.state, tcur, 53);             // accumulator complete
+        if (ok) {
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-            for (int c0 = 16 * second; c0 < rows_here; c0 += 32) {
-                float v[16];
-                tmem_ld16(taddr + c0, v);
+            float *const dst = out + static_cast<size_t>(row0) * ldo + a_idx;
+            for (int c0 = 16 * (warp >> 2); c0 < rows_here; c0 += kSgConvertWarps * 4) {
+                float hi[16], lo[16];
+                tmem_ld16x2(taddr + c0, taddr + p.n_tile + c0, hi, lo);
+                if (a_idx < a_rows) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) trans[(c0 + j) * kPitch + quarter * 32 + lane] = v[j] + bias;
-            }
-        }
-        AED_TRACE_PUT(p.state, tcur, 46);  // accumulator in shared memory
-        asm volatile("bar.sync 2, 256;" ::: "memory");
-        AED_TRACE_PUT(p.state, tcur, 47);  // all epilogue warps there
-        if (ok && fits) {
-            const int o4 = (pt & 31) * 4;
-            for (int rl = pt >> 5; rl < rows_here; rl += 8) {
-                const float4 v = *reinterpret_cast<const float4 *>(trans + rl * kPitch + o4);
-                float *dst = out + static_cast<size_t>(row0 + rl) * ldo + a0 + o4;
-                if (a0 + o4 + 3 < a_rows) red_add_v4(dst, v);
-                else {
-                    if (a0 + o4 + 0 < a_rows) atomicAdd(dst + 0, v.x);
-                    if (a0 + o4 + 1 < a_rows) atomicAdd(dst + 1, v.y);
-                    if (a0 + o4 + 2 < a_rows) atomicAdd(dst + 2, v.z);
+                    for (int j = 0; j < 16; ++j)
+                        if (c0 + j < rows_here) red_add(dst + static_cast<size_t>(c0 + j) * ldo, hi[j] + lo[j] + bias);
                 }
             }
-        } else if (ok) {
-            // transposition buffer too small for this shape: scalar reductions straight from the accumulator
-            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-            for (int c0 = 16 * second; c0 < rows_here; c0 += 32) {
-                float v[16];
-                tmem_ld16(taddr + c0, v);
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    if (a_ok && c0 + j < rows_here) atomicAdd(out + static_cast<size_t>(row0 + c0 + j) * ldo + a_idx, v[j] + bias);
-            }
         }
-        }
+        AED_TRACE_PUT(p.state, tcur, 54);
     }
-    AED_TRACE_PUT_NS(p.state, tcur, 45);   // epilogue issued
+    AED_TRACE_PUT_NS(p.state, tcur, 55);              // reductions issued
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == kSgMmaWarp) {
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, tmem_cols);
     }

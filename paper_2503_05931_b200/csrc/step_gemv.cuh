@@ -1,4 +1,4 @@
-// Decode-step projections for steps of at most 64 rows.
+// Decode-step projections for steps of at most 48 rows.
 //
 //   out[r, o] += sum_k B(r, k) * W[o, k]      (+ bias[o] from the CTA of the first k-split)
 //
@@ -226,15 +226,14 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     }
 }
 
-// The same projection for steps of 5 to 64 rows.  Loading B fragments straight from global memory makes every one of
+// The same projection for steps of 5 to 48 rows.  Loading B fragments straight from global memory makes every one of
 // the 8 warps fetch and split the same activation values; beyond a handful of rows that traffic costs more than one
 // hand-over through shared memory.  Here the 256 compute threads load the rows' k range once (coalesced 16-byte loads),
 // apply the transform, write bf16 high and low planes [row][k] into shared memory (row pitch padded against bank
 // conflicts), meet at one named barrier, and every warp reads its B fragments with ldmatrix.  A CTA covers at most 32
-// rows: with 64 the accumulators alone take 64 registers, one CTA fits per SM and the tcgen05 kernel is faster (1350
-// against 1195 us per step of the 24-layer model); launches of up to 64 rows put two row halves on grid.z.
-// kKB: most k-blocks per CTA (2, or 4 for the launches of 33 to 64 rows, which halve the k-splits and put two row
-// halves on grid.z instead: the same number of CTAs, half the reduction traffic).
+// rows; launches of 33 to 48 rows put two halves of 24 on grid.z.
+// kKB: most k-blocks per CTA (2, or 4 for the launches of 33 to 48 rows, which halve the k-splits: the same number of CTAs, half
+// the reduction traffic).
 __host__ __device__ constexpr int sv_pitch(int kb) { return kb * kBlockK * 2 + 16; }          // bytes per row of a plane: the CTA's k range in bf16 + pad
 __host__ __device__ constexpr int sv_staged_smem(int nt, int kb = kSvMaxKb) { return kb * kATileBytes + 2 * nt * 8 * sv_pitch(kb) + 1024; }
 

@@ -306,13 +306,27 @@ def test_large_batches_bf16(batch):
 
 @pytest.mark.parametrize("batch", [20, 130])
 def test_projection_stage_ring_reuse(batch, monkeypatch):
-    """With a single k-split every projection CTA walks all of its k-blocks through the shared-memory ring
-    (4 k-blocks for d = 256, 8 for the FFN), so stages are refilled while earlier ones are still being read."""
+    """With a single k-split every projection CTA walks all of its k-blocks (4 for d = 256, 8 for the FFN): two rounds
+    of the tcgen05 kernel for the FFN at 20 rows, and the ring of the many-rows kernel, whose stages are refilled while
+    earlier ones are still being read, at 130."""
     monkeypatch.setenv("AED_DEC_GEMM_CTAS", "1")
     rng = np.random.default_rng(batch)
     w = wl.make_custom(MID, rng.integers(1, 90, size=batch), rng.integers(1, 7, size=batch), dtype="bf16", seed=batch,
                        out_std=0.1)
     _run_both(w, rows=[0, 1, batch // 2, batch - 1])
+
+
+@pytest.mark.parametrize("model, batch, ctas", [("odd", 49, None), ("odd", 64, "8"), ("wide_a", 65, None), ("odd", 112, "1"), ("wide_a", 113, "24"),
+                                                 ("odd", 128, None)])
+def test_projections_of_49_to_128_rows(model, batch, ctas, monkeypatch):
+    """The tcgen05 projections: one to five k-blocks per CTA in one round or two, k-splits of unequal length, one to eight
+    rows of a k-block per thread, a last row tile of 16 with one row, feature counts that end inside a tile."""
+    if ctas:
+        monkeypatch.setenv("AED_DEC_GEMM_CTAS", ctas)
+    rng = np.random.default_rng(990 + batch)
+    w = wl.make_custom({"odd": ODD, "wide_a": WIDE_A}[model], rng.integers(1, 40, size=batch), rng.integers(1, 5, size=batch), dtype="bf16",
+                       seed=370 + batch, out_std=0.1, ln_std=0.2, bias_std=0.05)
+    _run_both(w, rows=sorted({0, 15, 16, 31, 32, 47, 48, batch // 2, batch - 2, batch - 1}))
 
 
 def test_config3_shape_sampled_rows():

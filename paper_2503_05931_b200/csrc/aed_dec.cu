@@ -606,9 +606,12 @@ aed_status_t tc_setup(aed_dec *dec)
     e = cudaGetLastError();
     // the few-row vocabulary kernel holds planes of the whole width: as wide as its shared memory, static and dynamic, allows
     cudaFuncAttributes attr;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, vg::vocab_gemv_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, vg::vocab_gemv_kernel<2>);
     dec->use_vocab_gemv = e == cudaSuccess && d % 128 == 0 && vg::vg_smem((int)d) + (int)attr.sharedSizeBytes <= 227 * 1024;
-    if (dec->use_vocab_gemv) e = cudaFuncSetAttribute(vg::vocab_gemv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, vg::vg_smem((int)d));
+    if (dec->use_vocab_gemv) {
+        e = cudaFuncSetAttribute(vg::vocab_gemv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, vg::vg_smem((int)d));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(vg::vocab_gemv_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, vg::vg_smem((int)d));
+    }
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "fold constants: %s", cudaGetErrorString(e));
     {
         const char *v = getenv("AED_DEC_NO_PDL");
@@ -899,7 +902,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         vp.active_list = active_list;
         vp.state = dec->state();
         void *args[] = {(void *)&dec->tc_w_out, &vp};
-        return launch_pdl_impl(dec, (const void *)vg::vocab_gemv_kernel, dim3((V + tc::kTileM - 1) / tc::kTileM), dim3(vg::kVgThreads),
+        return launch_pdl_impl(dec, rows <= 8 ? (const void *)vg::vocab_gemv_kernel<1> : (const void *)vg::vocab_gemv_kernel<2>, dim3((V + tc::kTileM - 1) / tc::kTileM), dim3(vg::kVgThreads),
                                (size_t)vg::vg_smem(d), args);
     }
     AED_TRY(launch_ln_planes(dec, rows, x, dec->final_ln_g, dec->final_ln_b));

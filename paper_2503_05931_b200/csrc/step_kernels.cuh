@@ -147,9 +147,13 @@ __global__ void __launch_bounds__(1024) step_rows_kernel(const __grid_constant__
     for (int r = n_rows + threadIdx.x; r < a.row_slots; r += blockDim.x) a.row_info[r] = make_int4(-1, 0, 0, 0);
     if (n_rows > kRowsInside) return;
     for (int i = threadIdx.x; i < a.d; i += blockDim.x) {
-#pragma unroll 4
-        for (int r = 0; r < n_rows; ++r)
-            a.x[(size_t)r * a.d + i] = to_f32(a.embed[(size_t)first[r].z * a.d + i]) * a.scale + a.pe[(size_t)first[r].y * a.d + i];
+        float e[kRowsInside], pe[kRowsInside];               // (table rows come from DRAM: all of them requested at once)
+#pragma unroll
+        for (int r = 0; r < kRowsInside; ++r)
+            if (r < n_rows) { e[r] = to_f32(a.embed[(size_t)first[r].z * a.d + i]); pe[r] = a.pe[(size_t)first[r].y * a.d + i]; }
+#pragma unroll
+        for (int r = 0; r < kRowsInside; ++r)
+            if (r < n_rows) a.x[(size_t)r * a.d + i] = e[r] * a.scale + pe[r];
     }
     if (a.zero_buf)
         for (int i = threadIdx.x; i < n_rows * a.zero_cols; i += blockDim.x) a.zero_buf[i] = 0.f;

@@ -204,9 +204,10 @@ struct aed_dec {
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
     // greedy decoding replays one captured CUDA graph per key; the output buffers stand in the device-side state
-    typedef std::tuple<int, int, int> GraphKey;       // (row count, chunks of self-attention positions, steps)
+    typedef std::tuple<int, int, int, bool> GraphKey;       // (row count, chunks of self-attention positions, steps, short_cross)
     struct GraphEntry { cudaGraphExec_t exec; int64_t nodes; };
     std::map<GraphKey, GraphEntry> graphs;
+    bool short_cross = false;       // of the launches to come: many rows with short encoder outputs (see few_cross_warps)
     cudaStream_t capture_stream = nullptr;
     bool use_graphs = true;
     // set only while aed_dec_step_static_scratch runs: attention partials go here instead of the workspace
@@ -325,6 +326,17 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
     int warps = (len_ub + fused_chunk<T>() - 1) / fused_chunk<T>();
     if (warps < 2) warps = 2;                    // at least 64 threads: the merge uses one thread per head dimension
     if (warps > kFusedMaxWarps) warps = kFusedMaxWarps;
+    if (kCross && dec->short_cross) warps = std::min(warps, 4);
+    // Self-attention, bf16: 2 blocks of 8 warps per SM, so with more pairs than that a block has fewer warps, which take another chunk of
+    // positions each, and the grid still fits.  With at most 128 positions the smaller merge is worth it a little earlier.
+    // (24 layers, us per step with 8 / 4 / 2 warps: positions 100 to 120 at 8 / 16 / 48 rows 495 / 513 / 558, 572 / 550 / 586, 943 / 905 / 882;
+    // 200 to 220 at 16 / 24 / 64 rows 585 / 588 / 656, 745 / 707 / 775, 1188 / 1136 / 1118; 24 to 56 at 24 / 32 / 64 rows, where 4 is the
+    // most, 644 / 655, 738 / 721, 958 / 926.)
+    if (!kCross && sizeof(T) == 2) {
+        const int pairs = rows_ub * dec->cfg.n_heads, fit = len_ub <= 128 ? 200 : 2 * dec->sm_count;
+        if (pairs > fit) warps = std::min(warps, 4);
+        if (pairs > 2 * fit) warps = std::min(warps, 2);
+    }
     // Attention starts early (programmatic launch) and holds each warp's first chunk in registers; rows longer than
     // 8 x 16 positions loop and find their later chunks prefetched in L2.
     cudaLaunchConfig_t cfg = {};
@@ -367,6 +379,19 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
     if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
     AED_LAUNCHED(dec);
     return AED_OK;
+}
+
+// Cross-attention of many rows with short encoder outputs: 4 warps per (row, head) instead of 8.  With more than 4 blocks of 8 warps
+// per SM the blocks come in waves, and each wave pays for a block's start, its statistics and its merge; blocks of half the size
+// make half as many waves.  Long rows are better off with 8 (an SM has as many loads in flight either way, and the rows that are left
+// at the end of a launch are done sooner).  24 layers, us per step, 8 -> 4 warps, 64 / 128 / 200 / 400 rows: 130 frames 1096 / 1582 /
+// 2232 / 3257 -> 1045 / 1504 / 2126 / 2969; 200 frames 1150 / 1657 / 2338 / 3425 -> 1121 / 1654 / 2355 / 3375; 250 frames 128 rows 1722 ->
+// 1745; with the 8-bit store 130 frames 1041 / 1512 / 2107 / 3040 -> 999 / 1418 / 1986 / 2791, 250 frames 1100 / 1611 / 2264 / 3369 -> 1082 /
+// 1558 / 2181 / 3170.  32 rows 726 -> 767.
+// frames: of the `utterances` that the step is for, as far as the host knows.
+bool few_cross_warps(const aed_dec *dec, int rows_ub, long long frames, int utterances)
+{
+    return dec->use_tc && rows_ub * dec->cfg.n_heads > 4 * dec->sm_count && frames <= (dec->cfg.cross_kv_format == AED_CROSS_KV_E4M3 ? 384ll : 192ll) * utterances;
 }
 
 // A launch that may start before its predecessor in the stream has ended (programmatic stream serialization): the
@@ -1346,6 +1371,7 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
         return fail(dec, AED_ERR_CAPACITY, "every utterance already holds max_dec_len = %d tokens", dec->cfg.max_dec_len);
     AED_TRY(launch_step_rows(dec, false, active, tokens_in, true));
     const int rows_ub = dec->batch;
+    dec->short_cross = few_cross_warps(dec, rows_ub, dec->total_frames, dec->batch);
     const int self_len_ub = dec->steps_issued + 1 < dec->cfg.max_dec_len ? dec->steps_issued + 1 : dec->cfg.max_dec_len;
     aed_status_t s = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tokens_in, logits_out)
                      : rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tokens_in, logits_out)
@@ -1387,6 +1413,7 @@ extern "C" aed_status_t aed_dec_prefill(aed_dec_t *dec, const int32_t *prompt, i
             AED_LAUNCHED(dec);
         }
         PrefillPass pf{last, B};
+        dec->short_cross = few_cross_warps(dec, rows, dec->total_frames, B);
         AED_TRY(rows > dec->planes_rows ? forward_step_planes(dec, rows, j0 + chunk, nullptr, logits_out, &pf)
                                         : forward_step_fused(dec, rows, j0 + chunk, nullptr, logits_out, &pf));
         {
@@ -1513,7 +1540,7 @@ int steps_per_graph(const aed_dec *dec, int rows_b) { return rows_b <= (dec->cfg
 // Launch `steps` greedy steps of at most rows_b rows and chunks * kAttnChunk positions as one graph, recorded at first use.
 aed_status_t launch_greedy_graph(aed_dec *dec, int rows_b, int chunks, int steps)
 {
-    const aed_dec::GraphKey key(rows_b, chunks, steps);
+    const aed_dec::GraphKey key(rows_b, chunks, steps, dec->short_cross);
     auto it = dec->graphs.find(key);
     if (it == dec->graphs.end()) {
         aed_dec::GraphEntry entry{};
@@ -1544,7 +1571,9 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
     // rows still alive at step s: utterances with max_len > s (exact without EOS, an upper bound with it)
     std::vector<int> alive(longest + 1, 0);
     for (int u = 0; u < B; ++u) alive[max_len[u] - 1]++;
-    for (int s = longest - 1; s >= 0; --s) alive[s] += alive[s + 1];
+    std::vector<long long> frames_alive(longest + 1, 0);
+    for (int u = 0; u < B; ++u) frames_alive[max_len[u] - 1] += dec->enc_len[u];
+    for (int s = longest - 1; s >= 0; --s) { alive[s] += alive[s + 1]; frames_alive[s] += frames_alive[s + 1]; }
 
     dec->fresh_batch = false;
     AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.max_len, max_len, B * 4, cudaMemcpyHostToDevice, dec->stream));
@@ -1565,6 +1594,7 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
     for (int s = 0; s < longest;) {
         // grids are sized for the keyed row count; kernels leave rows beyond the device-side row count alone
         const int rows_b = rows_key(alive[s]), chunks = s / kAttnChunk + 1;
+        dec->short_cross = few_cross_warps(dec, rows_b, frames_alive[s], alive[s]);
         const bool graph = dec->use_graphs && !dec->profiling;
         int n = 1;
         if (graph) {
@@ -1711,16 +1741,19 @@ extern "C" aed_status_t aed_dec_greedy_steps(aed_dec_t *dec, int32_t n_steps, in
     for (int s = 0; s < n_steps;) {
         // what the host knows: a slot decodes until its forced length (with an end-of-sequence id it may stop earlier
         // on the device; its row then simply is not there any more)
+        long long frames = 0;
         auto rows_at = [&](int ahead, int &longest) {
             int rows = 0;
             longest = 0;
+            frames = 0;
             for (int u = 0; u < dec->batch; ++u)
-                if (dec->slot_t[u] >= 0 && dec->slot_t[u] + ahead < dec->slot_max[u]) { ++rows; longest = std::max(longest, dec->slot_t[u] + ahead + 1); }
+                if (dec->slot_t[u] >= 0 && dec->slot_t[u] + ahead < dec->slot_max[u]) { ++rows; longest = std::max(longest, dec->slot_t[u] + ahead + 1); frames += dec->enc_len[u]; }
             return rows;
         };
         int longest;
         const int rows_ub = rows_at(0, longest);
         if (rows_ub == 0) break;
+        dec->short_cross = few_cross_warps(dec, rows_key(rows_ub), frames, rows_ub);
         if (!dec->rows_ready || dec->rows_tokens != tokens_out || dec->rows_lens != out_lens) {
             AED_TRY(launch_step_rows(dec, false, nullptr, dec->at<int32_t>(dec->lay.cur_tok), true, tokens_out, out_lens));
             dec->rows_ready = true;

@@ -210,6 +210,8 @@ struct aed_dec {
     bool short_cross = false;       // of the launches to come: many rows with short encoder outputs (see few_cross_warps)
     cudaStream_t capture_stream = nullptr;
     bool use_graphs = true;
+    std::map<GraphKey, int> step_seen;      // steps of the caller's loop by key (0 steps): the first one is launched kernel by kernel
+    bool from_state = false;        // while such a step is recorded: its kernels find the caller's pointers in the device-side state
     // set only while aed_dec_step_static_scratch runs: attention partials go here instead of the workspace
     float *partials_override = nullptr;
     // with an end-of-sequence id: the retired count in pinned host memory, written by every greedy step
@@ -667,6 +669,7 @@ aed_status_t launch_vocab_gemm(aed_dec *dec, int rows_ub, tc::TcParams p, int ro
     p.a_rows = dec->cfg.vocab;
     p.n_tile = shape.n_tile;
     p.k_blocks = dec->cfg.d_model / tc::kBlockK;
+    p.from_state = dec->from_state;
     p.rows_fixed = rows_fixed;          // >= 0: only that many rows (a prefill pass projects its last-position rows only)
     p.state = dec->state();
     const CUtensorMap *acts = dec->tc_actd[shape.n_tile / 16 - 1];
@@ -923,6 +926,7 @@ aed_status_t forward_step_fused(aed_dec *dec, int rows_ub, int self_len_ub, cons
         vp.c1 = dec->at<float>(L.fold_out); vp.c2 = vp.c1 + V;
         vp.eps = c.ln_eps;
         vp.logits_out = logits_out;
+        vp.from_state = dec->from_state;
         vp.keys = dec->at<unsigned long long>(L.keys);
         vp.active_list = active_list;
         vp.state = dec->state();
@@ -1087,6 +1091,12 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
     return AED_OK;
 }
 
+aed_status_t forward_step_bf16(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out, const PrefillPass *pf = nullptr)
+{
+    return rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tokens, logits_out, pf)
+                                      : forward_step_fused(dec, rows_ub, self_len_ub, tokens, logits_out, pf);
+}
+
 // Cross K/V of every layer on tensor cores, one persistent launch: D[frame, feature] = enc[frame, :] . w_kv_c[feature, :]
 // Cross-K/V of runs of encoder frames: run i is rows src0[i] .. src0[i] + frames[i] - 1 of the tensor at enc_base
 // (enc_rows rows in all) and goes to store rows dst0[i] .. (see ckv::CkvSegs; tile0 is filled here).
@@ -1149,7 +1159,8 @@ aed_status_t precompute_f32(aed_dec *dec, const void *enc_packed, int frames, in
 // The row table of the next step (step_rows_kernel): after the bookkeeping of a greedy step that ends (finish), or on its
 // own before the first one and before every step of the caller's loop.
 template <typename T>
-aed_status_t launch_step_rows_t(aed_dec *dec, bool finish, const uint8_t *mask, const int32_t *tokens, bool clear, int32_t *tokens_out, int32_t *out_lens)
+aed_status_t launch_step_rows_t(aed_dec *dec, bool finish, const uint8_t *mask, const int32_t *tokens, bool clear, int32_t *tokens_out, int32_t *out_lens,
+                                float *step_logits, int32_t *step_next)
 {
     const auto &c = dec->cfg;
     const Layout &L = dec->lay;
@@ -1169,15 +1180,16 @@ aed_status_t launch_step_rows_t(aed_dec *dec, bool finish, const uint8_t *mask, 
     a.keys = dec->at<unsigned long long>(L.keys); a.cur_tok = dec->at<int32_t>(L.cur_tok); a.max_len = dec->at<int32_t>(L.max_len); a.eos_id = c.eos_id;
     a.retired_host = dec->retired_host;
     a.tokens_out = tokens_out; a.out_lens = out_lens;
+    a.step_logits = step_logits; a.step_next = step_next;
     void *args[] = {&a};
     ProfScope ps(dec, KF_BOOKKEEPING);
     return launch_pdl_impl(dec, finish ? (const void *)step_rows_kernel<T, true> : (const void *)step_rows_kernel<T, false>, dim3(1), dim3(1024), 0, args, !finish);
 }
 aed_status_t launch_step_rows(aed_dec *dec, bool finish, const uint8_t *mask, const int32_t *tokens, bool clear, int32_t *tokens_out = nullptr,
-                              int32_t *out_lens = nullptr)
+                              int32_t *out_lens = nullptr, float *step_logits = nullptr, int32_t *step_next = nullptr)
 {
-    return dec->use_tc ? launch_step_rows_t<__nv_bfloat16>(dec, finish, mask, tokens, clear, tokens_out, out_lens)
-                       : launch_step_rows_t<float>(dec, finish, mask, tokens, clear, tokens_out, out_lens);
+    return dec->use_tc ? launch_step_rows_t<__nv_bfloat16>(dec, finish, mask, tokens, clear, tokens_out, out_lens, step_logits, step_next)
+                       : launch_step_rows_t<float>(dec, finish, mask, tokens, clear, tokens_out, out_lens, step_logits, step_next);
 }
 
 aed_status_t launch_finish(aed_dec *dec, int rows_ub, int32_t *next_out)
@@ -1188,7 +1200,8 @@ aed_status_t launch_finish(aed_dec *dec, int rows_ub, int32_t *next_out)
     const int32_t *active_list = dec->at<int32_t>(L.active_list);
     unsigned long long *keys = dec->at<unsigned long long>(L.keys);
     int32_t *t_u = dec->at<int32_t>(L.t_u);
-    void *args[] = {&state, &active_list, &keys, &t_u, &next_out};
+    int from_state = dec->from_state;
+    void *args[] = {&state, &active_list, &keys, &t_u, &next_out, &from_state};
     return launch_pdl_impl(dec, (const void *)finish_step_kernel, dim3((rows_ub + 127) / 128), dim3(128), 0, args);
 }
 
@@ -1216,6 +1229,74 @@ aed_status_t fill_i32(aed_dec *dec, int32_t *p, int32_t v, size_t n)
     ProfScope ps(dec, KF_BOOKKEEPING);
     fill_i32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, dec->stream>>>(p, v, n);
     AED_LAUNCHED(dec);
+    return AED_OK;
+}
+
+// One greedy step whose row table is in place, and the row table of the next one.
+aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub)
+{
+    const Layout &L = dec->lay;
+    if (self_len_ub > dec->cfg.max_dec_len) self_len_ub = dec->cfg.max_dec_len;
+    const int32_t *tok = dec->at<int32_t>(L.cur_tok);
+    const bool planes = dec->use_tc && rows_ub > dec->planes_rows;
+    aed_status_t st = dec->use_tc ? forward_step_bf16(dec, rows_ub, self_len_ub, tok, nullptr) : forward_step_f32(dec, rows_ub, self_len_ub, tok, nullptr);
+    if (st != AED_OK) return st;
+    // (the side jobs of the few-row projections leave the accumulators clear for the next step, the planes path does not)
+    return launch_step_rows(dec, true, nullptr, tok, planes);
+}
+
+// Record greedy steps (or, with 0, a step of the caller's loop behind its first kernel) into a graph on the library's capture
+// stream (nothing runs) and instantiate it.
+aed_status_t capture_greedy_steps(aed_dec *dec, int rows_ub, int self_len_ub, int steps, aed_dec::GraphEntry *entry)
+{
+    if (!dec->capture_stream)
+        AED_CUDA(dec, cudaStreamCreateWithFlags(&dec->capture_stream, cudaStreamNonBlocking));
+    cudaStream_t user = dec->stream;
+    const int64_t before = dec->launches;
+    AED_CUDA(dec, cudaStreamBeginCapture(dec->capture_stream, cudaStreamCaptureModeThreadLocal));
+    dec->stream = dec->capture_stream;
+    aed_status_t st = AED_OK;
+    for (int i = 0; i < steps && st == AED_OK; ++i) st = enqueue_greedy_step(dec, rows_ub, self_len_ub);
+    if (steps == 0) {
+        dec->from_state = true;
+        st = forward_step_bf16(dec, rows_ub, std::min(self_len_ub, (int)dec->cfg.max_dec_len), nullptr, nullptr);
+        if (st == AED_OK) st = launch_finish(dec, rows_ub, nullptr);
+        dec->from_state = false;
+    }
+    dec->stream = user;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamEndCapture(dec->capture_stream, &graph);
+    entry->nodes = dec->launches - before;
+    dec->launches = before;
+    if (st != AED_OK) { if (graph) cudaGraphDestroy(graph); return st; }
+    if (e != cudaSuccess || !graph) return fail(dec, AED_ERR_CUDA, "cudaStreamEndCapture: %s", cudaGetErrorString(e));
+    e = cudaGraphInstantiate(&entry->exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
+    return AED_OK;
+}
+
+// Steps of the same key per graph.  Inside a graph the kernels around a step's end overlap like all others (each starts
+// while its predecessor runs and fetches its weights); between two graphs they do not, which costs about 3 us.  (4 steps
+// instead of 1, 4-layer model: 93.5 -> 90.6 us per step of 1 row, 105.5 -> 102.1 of 8, 135.3 -> 133.9 of 24, 319.7 -> 318.5
+// of 128; 24 layers: 460 -> 457 us of 1 row, nothing beyond 8; fp32, 2 layers: 51.7 -> 47.1.)  A longer graph takes longer
+// to record, so deep models have them up to 8 rows and shallow ones up to 64.
+constexpr int kGraphSteps = 4;
+int steps_per_graph(const aed_dec *dec, int rows_b) { return rows_b <= (dec->cfg.n_layers <= 8 ? 64 : kRowsInside) ? kGraphSteps : 1; }
+
+// Launch `steps` greedy steps (0: a step of the caller's loop, behind its first kernel) of at most rows_b rows and chunks * kAttnChunk
+// positions as one graph, recorded at first use.
+aed_status_t launch_greedy_graph(aed_dec *dec, int rows_b, int chunks, int steps)
+{
+    const aed_dec::GraphKey key(rows_b, chunks, steps, dec->short_cross);
+    auto it = dec->graphs.find(key);
+    if (it == dec->graphs.end()) {
+        aed_dec::GraphEntry entry{};
+        AED_TRY(capture_greedy_steps(dec, rows_b, chunks * kAttnChunk, steps, &entry));
+        it = dec->graphs.emplace(key, entry).first;
+    }
+    AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
+    dec->launches += it->second.nodes;
     return AED_OK;
 }
 
@@ -1369,15 +1450,29 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
     if (dec->slot_mode) return fail(dec, AED_ERR_STATE, "aed_dec_step does not run on slots: use aed_dec_greedy_steps");
     if (dec->full_steps >= dec->cfg.max_dec_len)
         return fail(dec, AED_ERR_CAPACITY, "every utterance already holds max_dec_len = %d tokens", dec->cfg.max_dec_len);
-    AED_TRY(launch_step_rows(dec, false, active, tokens_in, true));
-    const int rows_ub = dec->batch;
-    dec->short_cross = few_cross_warps(dec, rows_ub, dec->total_frames, dec->batch);
     const int self_len_ub = dec->steps_issued + 1 < dec->cfg.max_dec_len ? dec->steps_issued + 1 : dec->cfg.max_dec_len;
-    aed_status_t s = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tokens_in, logits_out)
-                     : rows_ub > dec->planes_rows ? forward_step_planes(dec, rows_ub, self_len_ub, tokens_in, logits_out)
-                                                  : forward_step_fused(dec, rows_ub, self_len_ub, tokens_in, logits_out);
-    if (s != AED_OK) return s;
-    AED_TRY(launch_finish(dec, rows_ub, next_out));
+    // A step of a size that has come before is replayed as a graph: launching its kernels one by one takes longer than they do up to
+    // 32 rows (24 layers, 24 rows: 770 us a step).  Everything that a call passes goes through the step's first kernel,
+    // which is launched as it is; inside a capture of the caller's own all of them are.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (dec->use_tc && dec->use_graphs && !dec->profiling && !dec->partials_override) AED_CUDA(dec, cudaStreamIsCapturing(dec->stream, &capturing));
+    else capturing = cudaStreamCaptureStatusActive;
+    const int chunks = (self_len_ub + kAttnChunk - 1) / kAttnChunk, rows_b = rows_key(dec->batch);
+    bool graph = capturing == cudaStreamCaptureStatusNone;
+    if (graph) {
+        dec->short_cross = few_cross_warps(dec, rows_b, dec->total_frames, dec->batch);
+        graph = dec->step_seen[aed_dec::GraphKey(rows_b, chunks, 0, dec->short_cross)]++ > 0;
+    }
+    AED_TRY(launch_step_rows(dec, false, active, tokens_in, true, nullptr, nullptr, logits_out, next_out));
+    if (graph) {
+        AED_TRY(launch_greedy_graph(dec, rows_b, chunks, 0));
+    } else {
+        const int rows_ub = dec->batch;
+        dec->short_cross = few_cross_warps(dec, rows_ub, dec->total_frames, dec->batch);
+        AED_TRY(dec->use_tc ? forward_step_bf16(dec, rows_ub, self_len_ub, tokens_in, logits_out)
+                            : forward_step_f32(dec, rows_ub, self_len_ub, tokens_in, logits_out));
+        AED_TRY(launch_finish(dec, rows_ub, next_out));
+    }
     dec->steps_issued++;
     if (!active) dec->full_steps++;
     dec->fresh_batch = false;
@@ -1414,8 +1509,7 @@ extern "C" aed_status_t aed_dec_prefill(aed_dec_t *dec, const int32_t *prompt, i
         }
         PrefillPass pf{last, B};
         dec->short_cross = few_cross_warps(dec, rows, dec->total_frames, B);
-        AED_TRY(rows > dec->planes_rows ? forward_step_planes(dec, rows, j0 + chunk, nullptr, logits_out, &pf)
-                                        : forward_step_fused(dec, rows, j0 + chunk, nullptr, logits_out, &pf));
+        AED_TRY(forward_step_bf16(dec, rows, j0 + chunk, nullptr, logits_out, &pf));
         {
             ProfScope ps(dec, KF_BOOKKEEPING);
             DecState *state = dec->state();
@@ -1487,72 +1581,6 @@ extern "C" aed_status_t aed_dec_step_static_scratch(aed_dec_t *dec, const int32_
     dec->partials_override = nullptr;
     return s;
 }
-
-namespace {
-
-// One greedy step whose row table is in place, and the row table of the next one.
-aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub)
-{
-    const Layout &L = dec->lay;
-    if (self_len_ub > dec->cfg.max_dec_len) self_len_ub = dec->cfg.max_dec_len;
-    const int32_t *tok = dec->at<int32_t>(L.cur_tok);
-    const bool planes = dec->use_tc && rows_ub > dec->planes_rows;
-    aed_status_t st = !dec->use_tc ? forward_step_f32(dec, rows_ub, self_len_ub, tok, nullptr)
-                      : planes     ? forward_step_planes(dec, rows_ub, self_len_ub, tok, nullptr)
-                                   : forward_step_fused(dec, rows_ub, self_len_ub, tok, nullptr);
-    if (st != AED_OK) return st;
-    // (the side jobs of the few-row projections leave the accumulators clear for the next step, the planes path does not)
-    return launch_step_rows(dec, true, nullptr, tok, planes);
-}
-
-// Record greedy steps into a graph on the library's capture stream (nothing runs) and instantiate it.
-aed_status_t capture_greedy_steps(aed_dec *dec, int rows_ub, int self_len_ub, int steps, aed_dec::GraphEntry *entry)
-{
-    if (!dec->capture_stream)
-        AED_CUDA(dec, cudaStreamCreateWithFlags(&dec->capture_stream, cudaStreamNonBlocking));
-    cudaStream_t user = dec->stream;
-    const int64_t before = dec->launches;
-    AED_CUDA(dec, cudaStreamBeginCapture(dec->capture_stream, cudaStreamCaptureModeThreadLocal));
-    dec->stream = dec->capture_stream;
-    aed_status_t st = AED_OK;
-    for (int i = 0; i < steps && st == AED_OK; ++i) st = enqueue_greedy_step(dec, rows_ub, self_len_ub);
-    dec->stream = user;
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamEndCapture(dec->capture_stream, &graph);
-    entry->nodes = dec->launches - before;
-    dec->launches = before;
-    if (st != AED_OK) { if (graph) cudaGraphDestroy(graph); return st; }
-    if (e != cudaSuccess || !graph) return fail(dec, AED_ERR_CUDA, "cudaStreamEndCapture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&entry->exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
-    return AED_OK;
-}
-
-// Steps of the same key per graph.  Inside a graph the kernels around a step's end overlap like all others (each starts
-// while its predecessor runs and fetches its weights); between two graphs they do not, which costs about 3 us.  (4 steps
-// instead of 1, 4-layer model: 93.5 -> 90.6 us per step of 1 row, 105.5 -> 102.1 of 8, 135.3 -> 133.9 of 24, 319.7 -> 318.5
-// of 128; 24 layers: 460 -> 457 us of 1 row, nothing beyond 8; fp32, 2 layers: 51.7 -> 47.1.)  A longer graph takes longer
-// to record, so deep models have them up to 8 rows and shallow ones up to 64.
-constexpr int kGraphSteps = 4;
-int steps_per_graph(const aed_dec *dec, int rows_b) { return rows_b <= (dec->cfg.n_layers <= 8 ? 64 : kRowsInside) ? kGraphSteps : 1; }
-
-// Launch `steps` greedy steps of at most rows_b rows and chunks * kAttnChunk positions as one graph, recorded at first use.
-aed_status_t launch_greedy_graph(aed_dec *dec, int rows_b, int chunks, int steps)
-{
-    const aed_dec::GraphKey key(rows_b, chunks, steps, dec->short_cross);
-    auto it = dec->graphs.find(key);
-    if (it == dec->graphs.end()) {
-        aed_dec::GraphEntry entry{};
-        AED_TRY(capture_greedy_steps(dec, rows_b, chunks * kAttnChunk, steps, &entry));
-        it = dec->graphs.emplace(key, entry).first;
-    }
-    AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
-    dec->launches += it->second.nodes;
-    return AED_OK;
-}
-
-}  // namespace
 
 extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max_len, int32_t *tokens_out, int32_t *out_lens)
 {

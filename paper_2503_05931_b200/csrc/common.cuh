@@ -18,6 +18,10 @@ struct DecState {
     int32_t n_retired;   // utterances retired so far
     int32_t batch;       // utterances of the current batch (written by the cross-K/V precompute)
     int32_t *tokens_out, *out_lens;      // where greedy steps leave tokens and lengths: here, so that step graphs do not depend on it
+    // the same for steps of the caller's loop: its tokens, and where logits and choices go (or null)
+    const int32_t *step_tokens;
+    float *step_logits;
+    int32_t *step_next;
 };
 
 // Optional device-side timeline (debug builds with -DAED_TRACE): block 0 of every traced kernel stamps its start

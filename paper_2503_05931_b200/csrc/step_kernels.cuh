@@ -50,8 +50,10 @@ struct StepRowsArgs {
     const int32_t *max_len;
     int eos_id;
     volatile int32_t *retired_host;           // with an end-of-sequence id: how many have retired, for the host; or null
-    // !kFinish: where the greedy steps to come leave their results
+    // !kFinish: where the greedy steps to come leave their results, or this step of the caller's loop does
     int32_t *tokens_out, *out_lens;
+    float *step_logits;
+    int32_t *step_next;
 };
 
 // One block of 1024 threads, one utterance per thread and pass.  Everything but the argmax keys is known before the
@@ -100,7 +102,10 @@ __global__ void __launch_bounds__(1024) step_rows_kernel(const __grid_constant__
             for (int i = 0; i < a.d; i += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.pe + (size_t)min(t + 1, a.max_dec_len - 1) * a.d + i));
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!kFinish && threadIdx.x == 0) { state->tokens_out = tokens_out; state->out_lens = out_lens; }
+    if (!kFinish && threadIdx.x == 0) {
+        state->tokens_out = tokens_out; state->out_lens = out_lens;
+        state->step_tokens = a.tokens; state->step_logits = a.step_logits; state->step_next = a.step_next;
+    }
     for (int start = 0; start < batch; start += blockDim.x) {
         if (start > 0) {
             load(start + threadIdx.x);
@@ -203,7 +208,7 @@ __global__ void embed_kernel(const DecState *state, const int32_t *active_list,
     int r = blockIdx.x;
     if (r >= state->n_active) return;
     int u = active_list[r];
-    int tok = tokens[u];
+    int tok = (tokens ? tokens : state->step_tokens)[u];
     tok = min(max(tok, 0), vocab - 1);
     int t = t_u[u];
     for (int i = threadIdx.x; i < d; i += blockDim.x)
@@ -1046,10 +1051,11 @@ __global__ void prefill_finish_kernel(DecState *state, const int32_t *__restrict
 // End of a step of the caller's own loop: decode the argmax keys, hand the choice out by utterance id, advance t_u.
 __global__ void finish_step_kernel(DecState *state, const int32_t *__restrict__ active_list,
                                    unsigned long long *__restrict__ keys, int32_t *__restrict__ t_u,
-                                   int32_t *__restrict__ next_out /* by utterance, nullable */)
+                                   int32_t *next_out /* by utterance, nullable */, int from_state)
 {
     AED_TRACE_BEGIN(state, 6);
     asm volatile("griddepcontrol.wait;" ::: "memory");       // launched with programmatic stream serialization
+    if (from_state) next_out = state->step_next;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= state->n_active) return;
     const int u = active_list[r];

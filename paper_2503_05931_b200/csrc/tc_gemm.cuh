@@ -161,6 +161,7 @@ struct TcParams {
     int rows_fixed;      // >= 0: number of valid B rows; < 0: read it from the decode state
     const __nv_bfloat16 *bias;         // over the columns of D's first dimension (vocabulary / K-V features), may be null
     float *logits_out;                 // [batch, vocab] by utterance or nullptr
+    int from_state;                    // logits_out stands in the decode state (steps that are replayed as a graph)
     unsigned long long *keys;          // [rows]
     const int32_t *active_list;
     DecState *state;
@@ -268,6 +269,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         float *trans = reinterpret_cast<float *>(tiles);             // T[row][feature] over the ring's memory
         __syncwarp();
         const int n_rows = p.rows_fixed >= 0 ? p.rows_fixed : p.state->n_active;
+        float *const logits_out = p.from_state ? p.state->step_logits : p.logits_out;
         const bool ok = mbar_wait(&bar_done, 0, &abort_flag);        // every MMA has completed: the ring is free
         tc_fence_after_sync();
         if (threadIdx.x == (kProducerWarps + 1) * 32) AED_TRACE_MARK(p.state, 34);  // accumulator complete
@@ -288,14 +290,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             float bias[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) bias[j] = p.bias && o + j < p.a_rows ? to_f32(p.bias[o + j]) : 0.f;
-            const bool vec = o + 3 < p.a_rows && p.a_rows % 4 == 0 && (reinterpret_cast<uintptr_t>(p.logits_out) & 15) == 0;
+            const bool vec = o + 3 < p.a_rows && p.a_rows % 4 == 0 && (reinterpret_cast<uintptr_t>(logits_out) & 15) == 0;
 #pragma unroll 2
             for (int rl = ew; rl < rows_here; rl += kThreads / 32 - 1) {
                 const int r = row0 + rl;
                 float4 t = *reinterpret_cast<const float4 *>(trans + rl * kPitch + lane * 4);
                 const float z[4] = {t.x + bias[0], t.y + bias[1], t.z + bias[2], t.w + bias[3]};
-                if (p.logits_out) {
-                    float *dst = p.logits_out + static_cast<size_t>(p.active_list[r]) * p.a_rows + o;
+                if (logits_out) {
+                    float *dst = logits_out + static_cast<size_t>(p.active_list[r]) * p.a_rows + o;
                     if (vec) *reinterpret_cast<float4 *>(dst) = make_float4(z[0], z[1], z[2], z[3]);
                     else {
 #pragma unroll

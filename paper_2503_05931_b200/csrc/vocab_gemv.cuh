@@ -37,6 +37,7 @@ struct VocabGemvParams {
     const float *c1, *c2;              // fold constants [vocab] each
     float eps;
     float *logits_out;                 // [batch, vocab] by utterance, or nullptr
+    int from_state;                    // logits_out stands in the decode state (steps that are replayed as a graph)
     unsigned long long *keys;          // [rows]
     const int32_t *active_list;
     DecState *state;
@@ -117,6 +118,7 @@ vocab_gemv_kernel(const __grid_constant__ CUtensorMap map_w, VocabGemvParams p)
     // ---- row `warp`: statistics and planes, read once -----------------------------------------------------------------
     const int n_rows = p.state->n_active;
     sg::pdl_wait();
+    float *const logits_out = p.from_state ? p.state->step_logits : p.logits_out;
     if (has_row && warp < n_rows) {                           // (rows past the last: planes and statistics that nobody reads the results of)
         const int r = warp;
         const float *xr = p.x + static_cast<size_t>(r) * p.d_model;
@@ -232,8 +234,8 @@ vocab_gemv_kernel(const __grid_constant__ CUtensorMap map_w, VocabGemvParams p)
         int which;
         const uint32_t k32 = best_of(z, r < n_rows ? p.vocab - o : 0, which);
         unsigned long long key = k32 ? (static_cast<unsigned long long>(k32) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(o + which)) : 0ull;
-        if (r < n_rows && p.logits_out) {
-            float *dst = p.logits_out + static_cast<size_t>(p.active_list[r]) * p.vocab + o;
+        if (r < n_rows && logits_out) {
+            float *dst = logits_out + static_cast<size_t>(p.active_list[r]) * p.vocab + o;
             if (o + 3 < p.vocab && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) *reinterpret_cast<float4 *>(dst) = make_float4(z[0], z[1], z[2], z[3]);
             else {
 #pragma unroll

@@ -439,6 +439,40 @@ def test_rows_of_the_next_step(groups, dtype):
     _run_both(w, rows=sorted({0, len(dec_lens) - 1} | set(int(u) for u in np.argsort(dec_lens)[-5:])))
 
 
+@pytest.mark.parametrize("batch", [3, 12, 50, 131])
+def test_steps_with_other_buffers(batch, monkeypatch):
+    """Steps of the caller's loop are replayed as graphs from the second one of a size on: every call has tokens, logits and
+    choices of its own (or none), and a mask or none, and has to do what the same calls do launched kernel by kernel."""
+    import torch
+    rng = np.random.default_rng(1000 + batch)
+    w = wl.make_custom(MID, rng.integers(1, 60, size=batch), [8] * batch, dtype="bf16", seed=400 + batch, out_std=0.1, ln_std=0.2)
+    V = MID["vocab"]
+    tokens = torch.from_numpy(rng.integers(0, V, size=(6, batch)).astype(np.int32)).cuda()
+    mask = torch.from_numpy((rng.random(batch) < 0.6).astype(np.uint8)).cuda()
+    results = []
+    for graphs in (True, False):
+        monkeypatch.setenv("AED_DEC_NO_GRAPH", "0" if graphs else "1")
+        dec = binding.decoder_for_workload(w)
+        enc = dec.upload_encoder(w.enc)
+        outs = []
+        for _ in range(2):
+            dec.precompute_cross_kv(enc, w.enc_lens)
+            for t in range(6):
+                logits = torch.full((batch, V), -7.0, device="cuda") if t % 3 != 1 else None
+                choice = torch.full((batch,), -1, dtype=torch.int32, device="cuda") if t % 2 == 0 else None
+                dec.step(tokens[t].clone(), mask if t in (2, 4) else None, logits, choice)
+                outs += [x.clone() for x in (logits, choice) if x is not None]
+        dec.sync_status()
+        results.append(outs)
+        dec.close()
+    for a, b in zip(*results):
+        if a.dtype == torch.int32:
+            assert torch.equal(a == -1, b == -1)
+        else:
+            assert torch.equal(a == -7.0, b == -7.0)
+            assert float((a - b).abs().max()) < 2e-3      # fp32 sums of split projections come in another order
+
+
 @pytest.mark.parametrize("dtype, steps", [("bf16", 3), ("bf16", 4), ("bf16", 21), ("fp32", 37)])
 def test_several_steps_per_graph(dtype, steps):
     """Greedy decodes of fewer steps than a graph holds, of exactly as many, and across 16-position chunks, with rows that

@@ -452,7 +452,7 @@ def test_steps_with_other_buffers(batch, monkeypatch):
     results = []
     for graphs in (True, False):
         monkeypatch.setenv("AED_DEC_NO_GRAPH", "0" if graphs else "1")
-        dec = binding.decoder_for_workload(w)
+        dec = _binding().decoder_for_workload(w)
         enc = dec.upload_encoder(w.enc)
         outs = []
         for _ in range(2):

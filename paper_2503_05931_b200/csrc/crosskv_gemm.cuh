@@ -194,8 +194,9 @@ crosskv_gemm_kernel(const __grid_constant__ CUtensorMap map_enc, const CUtensorM
     const uint32_t tmem_base = tmem_slot;
 
     if (warp < kProducers) {
-        if (lane == 0) {
-            prefetch_tensormap(&map_enc);
+        {
+            if (elect_one()) prefetch_tensormap(&map_enc);
+            __syncwarp();
             const uint32_t full0 = map_to_rank(&bar_full[warp], 0);      // kStages == kProducers: this thread's stage
             uint8_t *const st = tiles + static_cast<size_t>(warp) * kStageBytes;
             long long it = 0;                           // k-block counter over all of this pair's tiles
@@ -209,9 +210,12 @@ crosskv_gemm_kernel(const __grid_constant__ CUtensorMap map_enc, const CUtensorM
                 for (int kb = 0; kb < k_blocks; ++kb, ++it) {
                     if (static_cast<int>(it % kProducers) != warp) continue;
                     if (fills > 0 && !mbar_wait(&bar_empty[warp], (fills - 1) & 1, &abort_flag)) { ok = false; break; }
-                    if (rank == 0) mbar_expect_tx(&bar_full[warp], 2 * kStageBytes);      // its own copies and the peer's
-                    tma_load_2d_pair(st, &map_enc, kb * kBlockK, m0, full0);
-                    tma_load_2d_pair(st + kATileBytes, map_w + layer, kb * kBlockK, nt * kTileN + static_cast<int>(rank) * (kTileN / 2), full0);
+                    if (elect_one()) {
+                        if (rank == 0) mbar_expect_tx(&bar_full[warp], 2 * kStageBytes);      // its own copies and the peer's
+                        tma_load_2d_pair(st, &map_enc, kb * kBlockK, m0, full0);
+                        tma_load_2d_pair(st + kATileBytes, map_w + layer, kb * kBlockK, nt * kTileN + static_cast<int>(rank) * (kTileN / 2), full0);
+                    }
+                    __syncwarp();
                     ++fills;
                 }
             }
@@ -224,7 +228,7 @@ crosskv_gemm_kernel(const __grid_constant__ CUtensorMap map_enc, const CUtensorM
             }
         }
     } else if (warp == kMmaWarp) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kTileN >> 3) << 17) |
                                    (static_cast<uint32_t>(2 * kTileM >> 4) << 24);
             int s = 0;
@@ -244,12 +248,15 @@ crosskv_gemm_kernel(const __grid_constant__ CUtensorMap map_enc, const CUtensorM
                     tc_fence_after_sync();
                     const uint32_t sa = smem_u32(tiles + static_cast<size_t>(s) * kStageBytes);
                     const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kATileBytes);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < kBlockK / 16; ++k) mma_bf16_pair(acc, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-                    mma_commit_pair(&bar_empty[s]);
+                        for (int k = 0; k < kBlockK / 16; ++k) mma_bf16_pair(acc, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                        mma_commit_pair(&bar_empty[s]);
+                        if (kb == k_blocks - 1) mma_commit_pair(&bar_acc_full[buf]);
+                    }
+                    __syncwarp();
                     if (++s == kStages) { s = 0; phase ^= 1; }
                 }
-                if (ok) mma_commit_pair(&bar_acc_full[buf]);
             }
         }
     } else if (warp >= 8) {

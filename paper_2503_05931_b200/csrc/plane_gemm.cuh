@@ -82,10 +82,13 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
     if (warp < kPgMmaWarp) {
         // a ring stage per warp; both blocks' copies report to the first block's barrier
         const int s = warp;
-        if (lane == 0 && s < S) {
-            prefetch_tensormap(&map_w);
-            prefetch_tensormap(&map_hi);
-            prefetch_tensormap(&map_lo);
+        if (s < S) {
+            if (elect_one()) {
+                prefetch_tensormap(&map_w);
+                prefetch_tensormap(&map_hi);
+                prefetch_tensormap(&map_lo);
+            }
+            __syncwarp();
             const uint32_t full0 = ckv::map_to_rank(&bar_full[s], 0);
             uint8_t *const st = tiles + static_cast<size_t>(s) * stage_bytes;
             const int rows_at = row0 + static_cast<int>(rank) * (p.n_tile / 2);
@@ -94,11 +97,17 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
             for (int i = s; i < n_kb; i += S, ++fills) {
                 if (fills > 0 && !mbar_wait(&bar_empty[s], (fills - 1) & 1, &abort_flag)) { ok = false; break; }
                 const int kc = (kb_begin + i) * kBlockK;
-                if (rank == 0) mbar_expect_tx(&bar_full[s], 2 * stage_bytes);
-                ckv::tma_load_2d_pair(st, &map_w, kc, a0, full0);
+                if (elect_one()) {
+                    if (rank == 0) mbar_expect_tx(&bar_full[s], 2 * stage_bytes);
+                    ckv::tma_load_2d_pair(st, &map_w, kc, a0, full0);
+                }
+                __syncwarp();
                 if (fills == 0) sg::pdl_wait();        // the weights are static
-                ckv::tma_load_2d_pair(st + kATileBytes, &map_hi, kc, rows_at, full0);
-                ckv::tma_load_2d_pair(st + kATileBytes + plane_bytes, &map_lo, kc, rows_at, full0);
+                if (elect_one()) {
+                    ckv::tma_load_2d_pair(st + kATileBytes, &map_hi, kc, rows_at, full0);
+                    ckv::tma_load_2d_pair(st + kATileBytes + plane_bytes, &map_lo, kc, rows_at, full0);
+                }
+                __syncwarp();
             }
             // the last MMAs that read this stage must have done so before its memory is used again
             if (ok && fills > 0) ok = mbar_wait(&bar_empty[s], (fills - 1) & 1, &abort_flag);
@@ -110,7 +119,7 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
         }
         __syncwarp();
     } else if (warp == kPgMmaWarp) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(p.n_tile >> 3) << 17) |
                                    (static_cast<uint32_t>(2 * kTileM >> 4) << 24);
             bool ok = true;
@@ -122,14 +131,17 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
                 tc_fence_after_sync();
                 const uint32_t sa = smem_u32(tiles + static_cast<size_t>(s) * stage_bytes);
                 const uint64_t da = smem_desc_sw128(sa), dh = smem_desc_sw128(sa + kATileBytes), dl = smem_desc_sw128(sa + kATileBytes + plane_bytes);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < kBlockK / 16; ++k) ckv::mma_bf16_pair(tmem_base, da + 2 * k, dh + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+                    for (int k = 0; k < kBlockK / 16; ++k) ckv::mma_bf16_pair(tmem_base, da + 2 * k, dh + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
 #pragma unroll
-                for (int k = 0; k < kBlockK / 16; ++k) ckv::mma_bf16_pair(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
-                ckv::mma_commit_pair(&bar_empty[s]);
+                    for (int k = 0; k < kBlockK / 16; ++k) ckv::mma_bf16_pair(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
+                    ckv::mma_commit_pair(&bar_empty[s]);
+                    if (i == n_kb - 1) ckv::mma_commit_pair(&bar_done);
+                }
+                __syncwarp();
                 if (++s == S) { s = 0; phase ^= 1; }
             }
-            if (ok) ckv::mma_commit_pair(&bar_done);
         }
     }
     // ---- epilogue ----------------------------------------------------------------------------------------------------

@@ -126,7 +126,8 @@ __device__ __forceinline__ void side_prefetch(const StepGemmParams &p, int w, in
         const char *base = static_cast<const char *>(range ? p.prefetch2_ptr : p.prefetch_ptr);
         if (!base) continue;
         const size_t pieces = (range ? p.prefetch2_bytes : p.prefetch_bytes) / 4096;
-        for (size_t i = static_cast<size_t>(w) * 32 + lane; i < pieces; i += static_cast<size_t>(n_w) * 32)
+        // (a warp issues these one lane after the other: spread over the warps first)
+        for (size_t i = static_cast<size_t>(lane) * n_w + w; i < pieces; i += static_cast<size_t>(n_w) * 32)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + i * 4096), "r"(4096) : "memory");
     }
 }

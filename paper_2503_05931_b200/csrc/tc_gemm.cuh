@@ -211,24 +211,27 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp < kProducerWarps) {
-        if (lane == 0 && warp < producers) {
-            prefetch_tensormap(&map_a);
-            prefetch_tensormap(&map_b);
-            prefetch_tensormap(&map_b_lo);
+        if (warp < producers) {
             int issued = 0;
             bool waited = false;
             for (int i = warp; i < n_kb; i += producers) {
                 const int s = i % stages;
                 if (i >= stages && !mbar_wait(&bar_empty[s], ((i / stages) - 1) & 1, &abort_flag)) break;
                 uint8_t *st = tiles + static_cast<size_t>(s) * stage_bytes;
-                mbar_expect_tx(&bar_full[s], stage_bytes);
                 const int kc = i * kBlockK;
-                tma_load_2d(st, &map_a, kc, a0, &bar_full[s]);
+                if (elect_one()) {
+                    mbar_expect_tx(&bar_full[s], stage_bytes);
+                    tma_load_2d(st, &map_a, kc, a0, &bar_full[s]);
+                }
+                __syncwarp();
                 // A is static (a weight matrix): its first tile is requested while the previous kernel still runs;
                 // B is that kernel's output
                 if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
-                tma_load_2d(st + kATileBytes, &map_b, kc, row0, &bar_full[s]);
-                tma_load_2d(st + kATileBytes + b_bytes, &map_b_lo, kc, row0, &bar_full[s]);
+                if (elect_one()) {
+                    tma_load_2d(st + kATileBytes, &map_b, kc, row0, &bar_full[s]);
+                    tma_load_2d(st + kATileBytes + b_bytes, &map_b_lo, kc, row0, &bar_full[s]);
+                }
+                __syncwarp();
                 issued = i + 1;
             }
             if (abort_flag && issued > 0) {
@@ -239,25 +242,27 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
         }
     } else if (warp == kProducerWarps) {
-        if (lane == 0) {
+        {
             const uint32_t idesc = instr_desc_bf16(p.n_tile);
-            bool ok = true;
-            for (int i = 0; i < n_kb && ok; ++i) {
-                const int s = i % stages;
-                ok = mbar_wait(&bar_full[s], (i / stages) & 1, &abort_flag);
-                if (!ok) break;
-                if (i == 0) AED_TRACE_MARK(p.state, 33);    // first operands landed
+            int s = 0;
+            uint32_t phase = 0;
+            for (int i = 0; i < n_kb; ++i) {
+                if (!mbar_wait(&bar_full[s], phase, &abort_flag)) break;
                 tc_fence_after_sync();
                 const uint32_t sa = smem_u32(tiles + static_cast<size_t>(s) * stage_bytes);
                 const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kATileBytes), dl = smem_desc_sw128(sa + kATileBytes + b_bytes);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < kBlockK / 16; ++k)
-                    mma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+                    for (int k = 0; k < kBlockK / 16; ++k)
+                        mma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
 #pragma unroll
-                for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
-                mma_commit(&bar_empty[s]);      // the stage may be refilled once these MMAs have read it
+                    for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
+                    mma_commit(&bar_empty[s]);      // the stage may be refilled once these MMAs have read it
+                    if (i == n_kb - 1) mma_commit(&bar_done);      // accumulator complete
+                }
+                __syncwarp();
+                if (++s == stages) { s = 0; phase ^= 1; }
             }
-            if (ok) mma_commit(&bar_done);      // accumulator complete
         }
     }
     // ---- epilogue: all warps but the one that issues the MMAs (the producers have nothing left to do) -------------

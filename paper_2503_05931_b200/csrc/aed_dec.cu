@@ -688,7 +688,7 @@ aed_status_t launch_ln_planes(aed_dec *dec, int rows_ub, const float *x, const v
     const __nv_bfloat16 *gp = (const __nv_bfloat16 *)g, *bp = (const __nv_bfloat16 *)b;
     __nv_bfloat16 *hi = dec->at<__nv_bfloat16>(L.actd_hi), *lo = dec->at<__nv_bfloat16>(L.actd_lo);
     void *args[] = {&state, &x, &gp, &bp, &d, &eps, &hi, &lo};
-    return launch_pdl_impl(dec, (const void *)layernorm_planes_kernel<8>, dim3(rows_ub), dim3(d <= 2048 ? 256 : 1024), 0, args);
+    return launch_pdl_impl(dec, (const void *)layernorm_planes_kernel, dim3(rows_ub), dim3(d <= 2048 ? 256 : 1024), 0, args);
 }
 
 // ---- fused step (bf16 mode): 7 kernels per layer, chained with programmatic dependent launch -------------------
@@ -1032,7 +1032,7 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
     const dim3 ln_block(d <= 2048 ? 256 : 1024);
     auto gamma_planes = [&](const void *g, float2 *st, float *zero_buf, int zero_cols) -> aed_status_t {
         ProfScope ps(dec, KF_LAYERNORM + KF_COUNT * KV_GAMMA);
-        return launch_pdl(dec, gamma_planes_kernel<8>, dim3(rows), ln_block, (const DecState *)dec->state(), (const float *)x,
+        return launch_pdl(dec, gamma_planes_kernel, dim3(rows), ln_block, (const DecState *)dec->state(), (const float *)x,
                           (const T *)g, d, c.ln_eps, st, ad_hi, ad_lo, zero_buf, zero_cols);
     };
     const PlaneShape sh_qkv = plane_shape(3 * d, d, rows_ub, false), sh_o = plane_shape(d, d, rows_ub, false), sh_qc = sh_o,

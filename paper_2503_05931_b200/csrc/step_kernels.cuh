@@ -843,59 +843,76 @@ attn_combine_kernel(const DecState *state, const int32_t *__restrict__ active_li
     *reinterpret_cast<float2 *>(out + (size_t)r * ldo + h * kHeadDim + lane * 2) = o;
 }
 
-// LayerNorm whose result is written as bf16 high and low planes [row, d].
-template <int kMaxPerThread>
-__global__ void layernorm_planes_kernel(const DecState *state, const float *x,
-                                        const __nv_bfloat16 *__restrict__ g, const __nv_bfloat16 *__restrict__ b, int d,
+// A block's row of d values (a multiple of 64, at most 8 per thread), 4 consecutive ones per thread and piece: (mean, rstd) with one
+// barrier per sum.  sums: two floats per warp.
+constexpr int kRowPieces = 2;
+__device__ __forceinline__ float2 block_row_stats(const float4 (&v)[kRowPieces], int d, float eps, float (*sums)[32])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    auto total = [&](float x, float *red) {
+        x = warp_sum(x);
+        if (lane == 0) red[warp] = x;
+        __syncthreads();
+        return warp_sum(lane < n_warps ? red[lane] : 0.f);
+    };
+    float s = 0.f, q = 0.f;
+#pragma unroll
+    for (int i = 0; i < kRowPieces; ++i) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+    const float mean = total(s, sums[0]) / d;
+#pragma unroll
+    for (int i = 0; i < kRowPieces; ++i) {
+        const float d0 = v[i].x - mean, d1 = v[i].y - mean, d2 = v[i].z - mean, d3 = v[i].w - mean;
+        if (static_cast<int>(threadIdx.x + i * blockDim.x) * 4 < d) q += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+    }
+    return make_float2(mean, rsqrtf(total(q, sums[1]) / d + eps));
+}
+// four values -> the planes
+__device__ __forceinline__ void store_planes(__nv_bfloat16 *hi, __nv_bfloat16 *lo, const float (&y)[4])
+{
+    uint32_t h[2], l[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(y[2 * j], y[2 * j + 1]);
+        const __nv_bfloat162 b = __floats2bfloat162_rn(y[2 * j] - __bfloat162float(a.x), y[2 * j + 1] - __bfloat162float(a.y));
+        h[j] = *reinterpret_cast<const uint32_t *>(&a);
+        l[j] = *reinterpret_cast<const uint32_t *>(&b);
+    }
+    *reinterpret_cast<uint2 *>(hi) = make_uint2(h[0], h[1]);
+    *reinterpret_cast<uint2 *>(lo) = make_uint2(l[0], l[1]);
+}
+
+// LayerNorm whose result is written as bf16 high and low planes [row, d].  One block per row.
+__global__ void layernorm_planes_kernel(const DecState *state, const float *x, const __nv_bfloat16 *__restrict__ g, const __nv_bfloat16 *__restrict__ b, int d,
                                         float eps, __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo)
 {
     AED_TRACE_BEGIN(state, 4);
-    // launched with programmatic stream serialization: nothing of the previous kernel is touched before this wait
+    __shared__ float sums[2][32];
+    // gain and bias are static and come from DRAM: ahead of the wait (programmatic stream serialization; nothing of the previous kernel is)
+    float4 v[kRowPieces];
+    float gk[kRowPieces][4], bk[kRowPieces][4];
+#pragma unroll
+    for (int i = 0; i < kRowPieces; ++i) {
+        const int k = static_cast<int>(threadIdx.x + i * blockDim.x) * 4;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { gk[i][j] = k < d ? to_f32(g[k + j]) : 0.f; bk[i][j] = k < d ? to_f32(b[k + j]) : 0.f; }
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    int r = blockIdx.x;
+    const int r = blockIdx.x;
     if (r >= state->n_active) return;
-    __shared__ float red[32];
-    __shared__ float stat;
-    float v[kMaxPerThread];
-    const float *xr = x + (size_t)r * d;
-    float s = 0.f;
 #pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        int i = threadIdx.x + j * blockDim.x;
-        v[j] = (i < d) ? xr[i] : 0.f;
-        s += v[j];
+    for (int i = 0; i < kRowPieces; ++i) {
+        const int k = static_cast<int>(threadIdx.x + i * blockDim.x) * 4;
+        v[i] = k < d ? *reinterpret_cast<const float4 *>(x + (size_t)r * d + k) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    s = warp_sum(s);
-    if (lane == 0) red[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) { float tsum = 0.f; for (int w = 0; w < n_warps; ++w) tsum += red[w]; stat = tsum / d; }
-    __syncthreads();
-    const float mean = stat;
-    float q = 0.f;
+    const float2 st = block_row_stats(v, d, eps, sums);
 #pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        int i = threadIdx.x + j * blockDim.x;
-        float c = (i < d) ? v[j] - mean : 0.f;
-        q += c * c;
-    }
-    q = warp_sum(q);
-    __syncthreads();
-    if (lane == 0) red[warp] = q;
-    __syncthreads();
-    if (threadIdx.x == 0) { float tsum = 0.f; for (int w = 0; w < n_warps; ++w) tsum += red[w]; stat = rsqrtf(tsum / d + eps); }
-    __syncthreads();
-    const float rstd = stat;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        int i = threadIdx.x + j * blockDim.x;
-        if (i < d) {
-            const float y = to_f32(g[i]) * (v[j] - mean) * rstd + to_f32(b[i]);
-            const __nv_bfloat16 hi = __float2bfloat16_rn(y);
-            out_hi[(size_t)r * d + i] = hi;
-            out_lo[(size_t)r * d + i] = __float2bfloat16_rn(y - __bfloat162float(hi));
-        }
+    for (int i = 0; i < kRowPieces; ++i) {
+        const int k = static_cast<int>(threadIdx.x + i * blockDim.x) * 4;
+        if (k >= d) continue;
+        const float y[4] = {gk[i][0] * (v[i].x - st.x) * st.y + bk[i][0], gk[i][1] * (v[i].y - st.x) * st.y + bk[i][1],
+                            gk[i][2] * (v[i].z - st.x) * st.y + bk[i][2], gk[i][3] * (v[i].w - st.x) * st.y + bk[i][3]};
+        store_planes(out_hi + (size_t)r * d + k, out_lo + (size_t)r * d + k, y);
     }
 }
 
@@ -905,62 +922,42 @@ __global__ void layernorm_planes_kernel(const DecState *state, const float *x,
 // Both kernels start with a programmatic-dependency wait and may be launched ahead of their predecessor's end.
 // ------------------------------------------------------------------------------------------------------------
 // planes of gamma * x, the LayerNorm statistics (mean, rstd) of every row, and the clearing of the fp32 rows a later
-// split-K projection accumulates into (zero_cols columns of zero_buf, if any).  One block per row.
-template <int kMaxPerThread>
-__global__ void gamma_planes_kernel(const DecState *state, const float *x, const __nv_bfloat16 *__restrict__ g,
-                                    int d, float eps, float2 *__restrict__ stats_out, __nv_bfloat16 *__restrict__ out_hi,
-                                    __nv_bfloat16 *__restrict__ out_lo, float *__restrict__ zero_buf, int zero_cols)
+// split-K projection accumulates into (zero_cols columns of zero_buf, if any).  One block per row.  (A warp per row, without
+// barriers, was slower: 200 rows 1980 us per step of the 24-layer model against 1850.)
+__global__ void gamma_planes_kernel(const DecState *state, const float *x, const __nv_bfloat16 *__restrict__ g, int d, float eps, float2 *__restrict__ stats_out,
+                                    __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, float *__restrict__ zero_buf, int zero_cols)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __shared__ float sums[2][32];
+    float4 v[kRowPieces];
+    float gk[kRowPieces][4];                              // (static, and from DRAM: ahead of the wait)
+#pragma unroll
+    for (int i = 0; i < kRowPieces; ++i) {
+        const int k = static_cast<int>(threadIdx.x + i * blockDim.x) * 4;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) gk[i][j] = k < d ? to_f32(g[k + j]) : 0.f;
+    }
     const int r = blockIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (r >= state->n_active) return;
-    __shared__ float red[32];
-    __shared__ float stat;
-    float v[kMaxPerThread];
-    const float *xr = x + (size_t)r * d;
-    float s = 0.f;
 #pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        const int i = threadIdx.x + j * blockDim.x;
-        v[j] = (i < d) ? xr[i] : 0.f;
-        s += v[j];
+    for (int i = 0; i < kRowPieces; ++i) {
+        const int k = static_cast<int>(threadIdx.x + i * blockDim.x) * 4;
+        v[i] = k < d ? *reinterpret_cast<const float4 *>(x + (size_t)r * d + k) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    s = warp_sum(s);
-    if (lane == 0) red[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) { float t = 0.f; for (int w = 0; w < n_warps; ++w) t += red[w]; stat = t / d; }
-    __syncthreads();
-    const float mean = stat;
-    float q = 0.f;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        const int i = threadIdx.x + j * blockDim.x;
-        const float c = (i < d) ? v[j] - mean : 0.f;
-        q += c * c;
-    }
-    q = warp_sum(q);
-    __syncthreads();
-    if (lane == 0) red[warp] = q;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < n_warps; ++w) t += red[w];
-        stats_out[r] = make_float2(mean, rsqrtf(t / d + eps));
+    if (zero_buf) {
+        float4 *const z = reinterpret_cast<float4 *>(zero_buf + (size_t)r * zero_cols);
+        for (int i = threadIdx.x; i < zero_cols / 4; i += blockDim.x) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
-    for (int j = 0; j < kMaxPerThread; ++j) {
-        const int i = threadIdx.x + j * blockDim.x;
-        if (i < d) {
-            const float y = to_f32(g[i]) * v[j];
-            const __nv_bfloat16 hi = __float2bfloat16_rn(y);
-            out_hi[(size_t)r * d + i] = hi;
-            out_lo[(size_t)r * d + i] = __float2bfloat16_rn(y - __bfloat162float(hi));
-        }
+    for (int i = 0; i < kRowPieces; ++i) {
+        const int k = static_cast<int>(threadIdx.x + i * blockDim.x) * 4;
+        if (k >= d) continue;
+        const float y[4] = {gk[i][0] * v[i].x, gk[i][1] * v[i].y, gk[i][2] * v[i].z, gk[i][3] * v[i].w};
+        store_planes(out_hi + (size_t)r * d + k, out_lo + (size_t)r * d + k, y);
     }
-    if (zero_buf)
-        for (int i = threadIdx.x; i < zero_cols; i += blockDim.x) zero_buf[(size_t)r * zero_cols + i] = 0.f;
+    const float2 st = block_row_stats(v, d, eps, sums);
+    if (threadIdx.x == 0) stats_out[r] = st;
 }
 
 // ------------------------------------------------------------------------------------------------------------

@@ -193,8 +193,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
     const int b_bytes = p.n_tile * kBlockK * 2;
     const int stage_bytes = kATileBytes + 2 * b_bytes;
+    // Up to 128 rows the low plane's tile, which stands right behind the high plane's, is multiplied by the same MMAs (N of twice the
+    // rows; the two products of a row meet in the epilogue): what an MMA of a few rows costs is its issue.  (us per step of the 4-layer
+    // model, 24 / 32 / 64 / 128 rows: 120.9 / 135.7 / 180.3 / 261.0 -> 119.5 / 134.1 / 179.0 / 259.7.  In plane_gemm.cuh, where an MMA has 96 rows
+    // and more, the same changed nothing: 200 / 512 rows 1785 / 2873 against 1786 / 2879.)
+    const bool stacked = p.n_tile <= 128;
+    const int n_cols = stacked ? 2 * p.n_tile : p.n_tile;
     uint32_t tmem_cols = 32;
-    while (tmem_cols < static_cast<uint32_t>(p.n_tile)) tmem_cols <<= 1;
+    while (tmem_cols < static_cast<uint32_t>(n_cols)) tmem_cols <<= 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) { mbar_init(&bar_full[s], 1); mbar_init(&bar_empty[s], 1); }
@@ -243,7 +249,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == kProducerWarps) {
         {
-            const uint32_t idesc = instr_desc_bf16(p.n_tile);
+            const uint32_t idesc = instr_desc_bf16(n_cols);
             int s = 0;
             uint32_t phase = 0;
             for (int i = 0; i < n_kb; ++i) {
@@ -255,8 +261,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
                     for (int k = 0; k < kBlockK / 16; ++k)
                         mma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+                    if (!stacked) {
 #pragma unroll
-                    for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
+                        for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, da + 2 * k, dl + 2 * k, idesc, 1u);
+                    }
                     mma_commit(&bar_empty[s]);      // the stage may be refilled once these MMAs have read it
                     if (i == n_kb - 1) mma_commit(&bar_done);      // accumulator complete
                 }
@@ -282,10 +290,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (ok) {
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
             for (int c0 = 16 * third; c0 < rows_here; c0 += 48) {
-                float v[16];
-                tmem_ld16(taddr + c0, v);
+                float v[16], low[16];
+                tmem_ld16x2(taddr + c0, taddr + (stacked ? p.n_tile : 0) + c0, v, low);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) trans[(c0 + j) * kPitch + quarter * 32 + lane] = v[j];
+                for (int j = 0; j < 16; ++j) trans[(c0 + j) * kPitch + quarter * 32 + lane] = stacked ? v[j] + low[j] : v[j];
             }
         }
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");

@@ -143,10 +143,10 @@ def profile_bytes(prof, w):
 # dram__bytes_write.sum of the captured launches over their algorithmic bytes).  An entry is removed when its kernel
 # changes, which turns the reported traffic back into null.
 NCU_TRAFFIC_RATIO = {
-    # five launches of one layer at 128 rows (cfg3): 73.68 MB read for 29.36 MB of layer weights; the launches also read
+    # five launches of one layer at 128 rows (cfg3): 71.87 MB read for 29.36 MB of layer weights; the launches also read
     # the composite cross-query matrix (2.1 MB), the fp32 activation rows, and each prefetches the next layer's matrices
     # of its kind into L2, which under the profiler's serialised replay is a second DRAM read
-    "step_gemm_kernel": 2.51,
+    "step_gemm_kernel": 2.45,
     # the five launches at 16 and at 4 rows (cfg2): 63.70 MB and 62.92 MB read
     "step_gemv_staged_kernel": 2.17,
     "step_gemv_kernel": 2.14,

@@ -16,13 +16,13 @@
 // With tcgen05 cta_group::2 each block of the pair fetches its own 128 frames and half of the features (32 KB per
 // k-block for the same 512 cycles); the tensor cores read the other half from the peer's shared memory.
 //
-// 75k frames, 4 layers (d 1024): 1371 us before, 956 us now (1.32 PFLOP/s, 0.80 of the measured cuBLAS rate); with four
-// epilogue warps instead of eight, 1078 us: draining 256 columns then takes longer than accumulating them.
+// 75k frames, 4 layers (d 1024): 1371 us before, 956 us in pairs, 900 us since an elected lane issues (1.40 PFLOP/s, 0.86 of the
+// measured cuBLAS rate); with four epilogue warps instead of eight (at 956) 1078 us: draining 256 columns then takes longer than
+// accumulating them.
 //
 // Warp roles (16 warps): 0..5 producers, 6 issues the MMAs (in the pair's first block only), 7 idle, 8..15 epilogue.
-//   * A thread's TMA copies complete one after the other (about a third of a microsecond each on this part,
-//     whatever their size), so one issuing thread cannot feed the tensor cores: six producer threads share the
-//     k-blocks round robin, each loading both operands of its k-blocks into a ring stage of its own.  The copies of
+//   * Six producer warps share the k-blocks round robin, each loading
+//     both operands of its k-blocks into a ring stage of its own.  The copies of
 //     both blocks report to the first block's barrier.
 //   * The accumulator (128 lanes x 256 fp32 columns in either block) is double-buffered in tensor memory: while the
 //     epilogue warps drain tile i (bias, bf16 pack, 32-byte stores straight into the per-head K/V rows), the MMA warp

@@ -11,7 +11,7 @@ constexpr int kBlockK = 64;                    // bf16 elements per k-block = on
 constexpr int kTileM = 128;
 constexpr int kATileBytes = kTileM * kBlockK * 2;
 constexpr int kMaxStages = 8;
-constexpr int kProducerWarps = 8;              // (a k-block is three copies, and a thread's copies complete one after the other)
+constexpr int kProducerWarps = 8;              // (a k-block is three copies)
 constexpr int kRowPitch = kTileM + 4;          // floats between the rows of an accumulator tile in shared memory (bank spread)
 constexpr int kTcSmemBudget = 200 * 1024;
 

@@ -4,9 +4,8 @@
 //
 // Both operands are K-major bf16 in global memory and arrive in shared memory through
 // cp.async.bulk.tensor (no multicast) with the 128-byte swizzle the MMA descriptors name.
-// One CTA = one (128-row tile of A, N-row tile of B).  Warp roles: warps 0..7 issue TMA (a thread's
-// copies complete one after the other, about a third of a microsecond each, so the k-blocks are shared out round
-// robin over the issuing threads), warp 8 owns the TMEM allocation and issues the MMAs; at the end all warps but that
+// One CTA = one (128-row tile of A, N-row tile of B).  Warp roles: warps 0..7 issue TMA (the k-blocks are
+// shared out round robin, a ring stage per warp), warp 8 owns the TMEM allocation and issues the MMAs; at the end all warps but that
 // one drain the accumulator (warp w reads TMEM lanes 32*(w%4) .. +31) into the ring's memory, rows first, and then take
 // a row each.
 //

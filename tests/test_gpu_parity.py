@@ -408,6 +408,18 @@ def test_self_attention_of_many_rows(model, batch):
     _run_both(w, rows=[0, 1, 2, 3, 4, batch // 2, batch - 1])
 
 
+@pytest.mark.parametrize("batch, frames", [(80, 40), (160, 40), (160, 300)])
+def test_attention_blocks_of_fewer_warps(batch, frames):
+    """320 and 640 (row, head) pairs that all reach position 139: self-attention blocks of 4 and 2 warps whose warps take up to
+    five 16-position chunks each; 640 pairs of cross-attention with short outputs (4 warps) and with long ones (8)."""
+    rng = np.random.default_rng(1010 + batch + frames)
+    dec_lens = np.full(batch, 140)
+    dec_lens[1] = 129
+    w = wl.make_custom(MID, rng.integers(max(1, frames - 20), frames + 1, size=batch), dec_lens, dtype="bf16", seed=410 + batch + frames,
+                       out_std=0.1, ln_std=0.2)
+    _run_both(w, rows=[0, 1, batch - 1])
+
+
 @pytest.mark.parametrize("enc_lens", [(1,), (128,), (100, 29), (256,), (200, 57), (384, 1)])
 def test_cross_kv_frame_tiles(enc_lens):
     """Encoder frames that fill 1, 2, 3 and 4 tiles of 128 exactly or by one frame (an odd last tile has no partner in

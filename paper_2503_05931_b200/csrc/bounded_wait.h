@@ -4,8 +4,13 @@
 // case it sets the abort word itself.  The caller then stops issuing work, lets its own copies land, frees what
 // it holds and returns, and the host later reads the sticky error word as AED_ERR_TIMEOUT.
 //
-// The loop is plain C++ with the condition and the clock passed in, so the same source compiles for the host
-// (steady clock, threads instead of warps), which is how its give-up path is tested without a GPU.
+// A wait belongs to one party, which is a whole warp on the device.  Its lanes poll together, and each decision to leave is put
+// to all of them (`all`: true if p is true in every lane): a lane that sees the phase complete while another sees the abort word
+// must not return with another result, because what follows a wait are operations of the whole warp (elect.sync, tensor-memory
+// loads, named barriers), which are undefined and may hang when lanes are missing.
+//
+// The loop is plain C++ with the condition, the clock and the vote passed in, so the same source compiles for the host
+// (steady clock, threads instead of warps or lanes), which is how its give-up path is tested without a GPU.
 #pragma once
 
 #if defined(__CUDACC__)
@@ -16,15 +21,15 @@
 
 namespace aed {
 
-template <class Ready, class Now>
-AED_WAIT_FN bool bounded_poll(Ready ready, Now now, long long limit, volatile int *abort_flag)
+template <class Ready, class Now, class All>
+AED_WAIT_FN bool bounded_poll(Ready ready, Now now, long long limit, volatile int *abort_flag, All all)
 {
-    if (ready()) return true;
+    if (all(ready())) return true;
     const long long start = now();
     while (true) {
-        if (ready()) return true;
-        if (*abort_flag) return false;
-        if (now() - start > limit) { *abort_flag = 1; return false; }
+        if (all(ready())) return true;
+        if (!all(*abort_flag == 0)) return false;
+        if (!all(now() - start <= limit)) { *abort_flag = 1; return false; }
     }
 }
 

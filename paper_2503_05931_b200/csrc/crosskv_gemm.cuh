@@ -117,7 +117,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity
                          "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
             return ok != 0;
         },
-        [] { return clock64(); }, kWaitCycles, abort_flag);
+        [] { return clock64(); }, kWaitCycles, abort_flag, WarpVote());
 }
 
 // The tiles of one block pair, in order (m_tiles: frame tile pairs; G, b: block pairs of the grid and this one).  Every warp role walks the same sequence.

@@ -59,15 +59,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
         : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
 }
-// Bounded wait.  Returns false if the phase did not complete in time or another role already gave up.
-// (The polling loop is kept out of line: the common case is that the phase has already completed.)
+// The lanes of a warp agree on how a wait ends (see bounded_wait.h).
+struct WarpVote {
+    __device__ __forceinline__ bool operator()(bool p) const { return __all_sync(0xffffffffu, p) != 0; }
+};
+// Bounded wait of a whole warp, with one result for all lanes: false if the phase did not complete in time or another role already
+// gave up.  (The polling loop is kept out of line: the common case is that the phase has already completed.)
 __device__ __noinline__ bool mbar_wait_poll(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
 {
-    return bounded_poll([&] { return mbar_try_wait(bar, parity); }, [] { return clock64(); }, kWaitCycles, abort_flag);
+    return bounded_poll([&] { return mbar_try_wait(bar, parity); }, [] { return clock64(); }, kWaitCycles, abort_flag, WarpVote());
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
 {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (WarpVote()(mbar_try_wait(bar, parity))) return true;
     return mbar_wait_poll(bar, parity, abort_flag);
 }
 

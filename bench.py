@@ -175,6 +175,25 @@ def roofline_seconds(w, peaks):
     return dec, pre
 
 
+def timed_passes(one_pass, warmup: int, steps: int, barrier, event, start=None):
+    """Device time of ``steps`` passes after ``warmup`` untimed ones of the same kind: (all, each) in ms.  ``start`` is called between
+    the two.  Passes from the host need warm-ups of their own: the binding keeps a batch's encoder states until the next
+    batch, so the first two passes take a new block of device memory each, and that call takes 1 to 85 ms of host time, during which
+    the device idles (with one warm-up pass 20 passes came to 27.4k to 29.0k tokens/s on boxes that agree to 0.2 % otherwise)."""
+    for _ in range(warmup):
+        one_pass()
+    if start is not None:
+        start()
+    ev = [event() for _ in range(steps + 1)]
+    barrier()
+    ev[0].record()
+    for i in range(steps):
+        one_pass()
+        ev[i + 1].record()
+    barrier()
+    return ev[0].elapsed_time(ev[steps]), [ev[i].elapsed_time(ev[i + 1]) for i in range(steps)]
+
+
 def reduce_over_ranks(total_ms: float, n_tok: float, n_frames: float, device: str, world: int):
     """Whole-job figures of a weak-scaling run: the slowest rank's time, tokens and frames summed over ranks.
     Ranks decode independent batches, so these two reductions are the only communication of the benchmark."""
@@ -481,29 +500,23 @@ def main():
             dist.barrier()
         torch.cuda.synchronize()
 
-    def timed(from_host: bool, steps: int):
-        ev = [torch.cuda.Event(enable_timing=True) for _ in range(steps + 1)]
-        barrier()
-        ev[0].record()
-        for i in range(steps):
-            one_pass(from_host)
-            ev[i + 1].record()
-        barrier()
-        per = [ev[i].elapsed_time(ev[i + 1]) for i in range(steps)]
-        total_ms = ev[0].elapsed_time(ev[steps])
-        return total_ms, per
+    def timed(from_host: bool, start=None):
+        return timed_passes(lambda: one_pass(from_host), max(args.warmup, 3), args.steps, barrier,
+                            lambda: torch.cuda.Event(enable_timing=True), start)
 
-    for _ in range(max(args.warmup, 3)):
-        one_pass(False)
     sampler = ClockSampler(local_rank)
-    if rank == 0:
-        sampler.start()
-    launches0 = dec.launch_count()
-    total_ms, per = timed(False, args.steps)
+    launches0 = 0
+
+    def start():
+        nonlocal launches0
+        if rank == 0:
+            sampler.start()
+        launches0 = dec.launch_count()
+
+    total_ms, _ = timed(False, start)
     launches = dec.launch_count() - launches0
     clocks = sampler.stop() if rank == 0 else None
-    one_pass(True)
-    e2e_ms, _ = timed(True, args.steps)
+    e2e_ms, e2e_per = timed(True)
     dec.sync_status()
 
     e2e_ms, _, _ = reduce_over_ranks(e2e_ms, 0.0, 0.0, device, world)
@@ -530,7 +543,8 @@ def main():
             "step_roofline": {"roofline_ms": 1e3 * (dec_s + pre_s), "frac": 1e3 * (dec_s + pre_s) / ms_per_step,
                               "peaks": peaks["source"], "hbm_gbs": peaks["hbm_gbs"],
                               "bf16_tflops": peaks["bf16_tflops_sustained"]},
-            "e2e": {"value": e2e_value, "unit": "tokens/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
+            "e2e": {"value": e2e_value, "unit": "tokens/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
+                    "ms_per_step_median": float(np.median(e2e_per)), "ms_per_step_slowest": float(max(e2e_per))},
             "gpu_launches": int(launches),
             "clocks": clocks,
         }

@@ -1,5 +1,5 @@
 """What bench.py says about a profiled pass, on made-up launch counts: every variant of a call site goes to the kernel that ran
-it, and the variants' bytes add up to the call site's."""
+it, and the variants' bytes add up to the call site's.  And what it times: passes that have nothing left to set up."""
 import numpy as np
 import pytest
 
@@ -58,3 +58,34 @@ def test_kernel_names_exist_in_the_source():
     for variant in bench.KERNEL_OF_VARIANT:
         assert f'"@{variant}"' in src, variant
     assert set(bench.VARIANT_ORDER) | {"gamma"} == set(bench.KERNEL_OF_VARIANT) | {""}
+
+
+@pytest.mark.parametrize("warmup, steps", [(3, 5), (4, 1)])
+def test_timed_passes_do_not_set_anything_up(warmup, steps):
+    """A pass from the host copies its inputs into a new device buffer while the decoder still holds the last one's: on a made-up
+    clock the first two passes take a block of memory (60 ms each), later ones reuse it, and no timed pass may show it."""
+    import bench
+    clock, free, held, log = [0.0], [], [None], []
+
+    class Event:
+        def record(self):
+            self.at = clock[0]
+
+        def elapsed_time(self, other):
+            return other.at - self.at
+
+    def one_pass():
+        if free:
+            block = free.pop()
+        else:
+            block = object()
+            clock[0] += 60.0
+        if held[0] is not None:
+            free.append(held[0])
+        held[0] = block
+        clock[0] += 10.0
+        log.append("pass")
+
+    total, per = bench.timed_passes(one_pass, warmup, steps, lambda: log.append("barrier"), Event, lambda: log.append("start"))
+    assert log == ["pass"] * warmup + ["start", "barrier"] + ["pass"] * steps + ["barrier"]
+    assert per == [10.0] * steps and total == 10.0 * steps

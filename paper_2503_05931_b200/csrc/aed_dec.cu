@@ -173,7 +173,7 @@ struct aed_dec {
     bool fresh_batch = false;       // no step issued since the precompute
     int steps_issued = 0;           // steps of any kind since the precompute: upper bound on any t_u
     int full_steps = 0;             // steps without a mask: lower bound on t_u of every utterance not retired
-    int total_frames = 0;
+    EncoderFrames frames;           // of the whole batch
     std::vector<int32_t> enc_len, enc_off;
     // continuous batching: the batch is a set of slots that utterances enter and leave one by one
     bool slot_mode = false;
@@ -383,17 +383,10 @@ aed_status_t launch_attention_fused(aed_dec *dec, int rows_ub, int len_ub, const
     return AED_OK;
 }
 
-// Cross-attention of many rows with short encoder outputs: 4 warps per (row, head) instead of 8.  With more than 4 blocks of 8 warps
-// per SM the blocks come in waves, and each wave pays for a block's start, its statistics and its merge; blocks of half the size
-// make half as many waves.  Long rows are better off with 8 (an SM has as many loads in flight either way, and the rows that are left
-// at the end of a launch are done sooner).  24 layers, us per step, 8 -> 4 warps, 64 / 128 / 200 / 400 rows: 130 frames 1096 / 1582 /
-// 2232 / 3257 -> 1045 / 1504 / 2126 / 2969; 200 frames 1150 / 1657 / 2338 / 3425 -> 1121 / 1654 / 2355 / 3375; 250 frames 128 rows 1722 ->
-// 1745; with the 8-bit store 130 frames 1041 / 1512 / 2107 / 3040 -> 999 / 1418 / 1986 / 2791, 250 frames 1100 / 1611 / 2264 / 3369 -> 1082 /
-// 1558 / 2181 / 3170.  32 rows 726 -> 767.
-// frames: of the `utterances` that the step is for, as far as the host knows.
-bool few_cross_warps(const aed_dec *dec, int rows_ub, long long frames, int utterances)
+// The rule is in launch_shapes.h.
+bool few_cross_warps(const aed_dec *dec, int rows_ub, const EncoderFrames &frames)
 {
-    return dec->use_tc && rows_ub * dec->cfg.n_heads > 4 * dec->sm_count && frames <= (dec->cfg.cross_kv_format == AED_CROSS_KV_E4M3 ? 384ll : 192ll) * utterances;
+    return dec->use_tc && few_cross_warps((long long)rows_ub * dec->cfg.n_heads, dec->sm_count, frames, dec->cfg.cross_kv_format == AED_CROSS_KV_E4M3);
 }
 
 // A launch that may start before its predecessor in the stream has ended (programmatic stream serialization): the
@@ -1422,7 +1415,8 @@ extern "C" aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *
     dec->enc_len.assign(enc_lens, enc_lens + batch);
     dec->enc_off = off;
     dec->batch = batch;
-    dec->total_frames = (int)total;
+    dec->frames = EncoderFrames{};
+    for (int u = 0; u < batch; ++u) dec->frames.add(enc_lens[u]);
     {
         // visiting order of the row compaction: longest encoder output first (ties by utterance index)
         std::vector<int32_t> order(batch);
@@ -1431,8 +1425,7 @@ extern "C" aed_status_t aed_dec_precompute_cross_kv(aed_dec_t *dec, const void *
         AED_TRY(begin_batch(dec, order));
     }
     dec->slot_mode = false;
-    aed_status_t s = dec->use_tc ? precompute_tc(dec, enc_packed, dec->total_frames, one_run(dec->total_frames, 0))
-                                 : precompute_f32(dec, enc_packed, dec->total_frames, 0);
+    aed_status_t s = dec->use_tc ? precompute_tc(dec, enc_packed, total, one_run((int)total, 0)) : precompute_f32(dec, enc_packed, (int)total, 0);
     if (s != AED_OK) return s;
     dec->have_batch = true;
     dec->fresh_batch = true;
@@ -1460,7 +1453,7 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
     const int chunks = (self_len_ub + kAttnChunk - 1) / kAttnChunk, rows_b = rows_key(dec->batch);
     bool graph = capturing == cudaStreamCaptureStatusNone;
     if (graph) {
-        dec->short_cross = few_cross_warps(dec, rows_b, dec->total_frames, dec->batch);
+        dec->short_cross = few_cross_warps(dec, rows_b, dec->frames);
         graph = dec->step_seen[aed_dec::GraphKey(rows_b, chunks, 0, dec->short_cross)]++ > 0;
     }
     AED_TRY(launch_step_rows(dec, false, active, tokens_in, true, nullptr, nullptr, logits_out, next_out));
@@ -1468,7 +1461,7 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
         AED_TRY(launch_greedy_graph(dec, rows_b, chunks, 0));
     } else {
         const int rows_ub = dec->batch;
-        dec->short_cross = few_cross_warps(dec, rows_ub, dec->total_frames, dec->batch);
+        dec->short_cross = few_cross_warps(dec, rows_ub, dec->frames);
         AED_TRY(dec->use_tc ? forward_step_bf16(dec, rows_ub, self_len_ub, tokens_in, logits_out)
                             : forward_step_f32(dec, rows_ub, self_len_ub, tokens_in, logits_out));
         AED_TRY(launch_finish(dec, rows_ub, next_out));
@@ -1508,7 +1501,7 @@ extern "C" aed_status_t aed_dec_prefill(aed_dec_t *dec, const int32_t *prompt, i
             AED_LAUNCHED(dec);
         }
         PrefillPass pf{last, B};
-        dec->short_cross = few_cross_warps(dec, rows, dec->total_frames, B);
+        dec->short_cross = few_cross_warps(dec, rows, dec->frames);
         AED_TRY(forward_step_bf16(dec, rows, j0 + chunk, nullptr, logits_out, &pf));
         {
             ProfScope ps(dec, KF_BOOKKEEPING);
@@ -1599,9 +1592,9 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
     // rows still alive at step s: utterances with max_len > s (exact without EOS, an upper bound with it)
     std::vector<int> alive(longest + 1, 0);
     for (int u = 0; u < B; ++u) alive[max_len[u] - 1]++;
-    std::vector<long long> frames_alive(longest + 1, 0);
-    for (int u = 0; u < B; ++u) frames_alive[max_len[u] - 1] += dec->enc_len[u];
-    for (int s = longest - 1; s >= 0; --s) { alive[s] += alive[s + 1]; frames_alive[s] += frames_alive[s + 1]; }
+    std::vector<EncoderFrames> frames_alive(longest + 1);
+    for (int u = 0; u < B; ++u) frames_alive[max_len[u] - 1].add(dec->enc_len[u]);
+    for (int s = longest - 1; s >= 0; --s) { alive[s] += alive[s + 1]; frames_alive[s].add(frames_alive[s + 1]); }
 
     dec->fresh_batch = false;
     AED_CUDA(dec, cudaMemcpyAsync(dec->ws + L.max_len, max_len, B * 4, cudaMemcpyHostToDevice, dec->stream));
@@ -1622,7 +1615,7 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
     for (int s = 0; s < longest;) {
         // grids are sized for the keyed row count; kernels leave rows beyond the device-side row count alone
         const int rows_b = rows_key(alive[s]), chunks = s / kAttnChunk + 1;
-        dec->short_cross = few_cross_warps(dec, rows_b, frames_alive[s], alive[s]);
+        dec->short_cross = few_cross_warps(dec, rows_b, frames_alive[s]);
         const bool graph = dec->use_graphs && !dec->profiling;
         int n = 1;
         if (graph) {
@@ -1665,7 +1658,7 @@ extern "C" aed_status_t aed_dec_open_slots(aed_dec_t *dec, int32_t slots)
     const Layout &L = dec->lay;
     dec->have_batch = false;
     dec->batch = slots;
-    dec->total_frames = 0;
+    dec->frames = EncoderFrames{};
     dec->enc_len.assign(slots, 0);
     dec->enc_off.assign(slots + 1, 0);
     for (int u = 0; u <= slots; ++u) dec->enc_off[u] = u * c.max_enc_len;       // every slot owns max_enc_len store rows
@@ -1769,19 +1762,19 @@ extern "C" aed_status_t aed_dec_greedy_steps(aed_dec_t *dec, int32_t n_steps, in
     for (int s = 0; s < n_steps;) {
         // what the host knows: a slot decodes until its forced length (with an end-of-sequence id it may stop earlier
         // on the device; its row then simply is not there any more)
-        long long frames = 0;
+        EncoderFrames frames;
         auto rows_at = [&](int ahead, int &longest) {
             int rows = 0;
             longest = 0;
-            frames = 0;
+            frames = EncoderFrames{};
             for (int u = 0; u < dec->batch; ++u)
-                if (dec->slot_t[u] >= 0 && dec->slot_t[u] + ahead < dec->slot_max[u]) { ++rows; longest = std::max(longest, dec->slot_t[u] + ahead + 1); frames += dec->enc_len[u]; }
+                if (dec->slot_t[u] >= 0 && dec->slot_t[u] + ahead < dec->slot_max[u]) { ++rows; longest = std::max(longest, dec->slot_t[u] + ahead + 1); frames.add(dec->enc_len[u]); }
             return rows;
         };
         int longest;
         const int rows_ub = rows_at(0, longest);
         if (rows_ub == 0) break;
-        dec->short_cross = few_cross_warps(dec, rows_key(rows_ub), frames, rows_ub);
+        dec->short_cross = few_cross_warps(dec, rows_key(rows_ub), frames);
         if (!dec->rows_ready || dec->rows_tokens != tokens_out || dec->rows_lens != out_lens) {
             AED_TRY(launch_step_rows(dec, false, nullptr, dec->at<int32_t>(dec->lay.cur_tok), true, tokens_out, out_lens));
             dec->rows_ready = true;

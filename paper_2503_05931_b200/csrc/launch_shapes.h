@@ -1,5 +1,5 @@
-// The shape of the tensor-core vocabulary projection: row tile, ring and shared memory.  Plain C++ (no CUDA), so that the
-// sizes are also checked on the host, over every row count and model width.
+// Launch shapes that depend on sizes alone: row tile, ring and shared memory of the tensor-core vocabulary projection; warps of a
+// cross-attention block.  Plain C++ (no CUDA), so that they are also checked on the host, over every row count and model width.
 #pragma once
 #include <algorithm>
 #include <cstddef>
@@ -44,6 +44,45 @@ inline VocabShape vocab_shape(int rows_ub, int k_blocks)
     // (d_model 64, row tiles of 64 and more: 528 bytes a row against 16 KB + 256 bytes a row).
     s.smem = std::max((size_t)s.stages * stage_bytes, (size_t)s.n_tile * tc::kRowPitch * sizeof(float)) + 1024;
     return s;
+}
+
+// The encoder outputs of the rows of a step, as far as the host knows them.
+struct EncoderFrames {
+    int rows = 0, longest = 0;
+    long long sum = 0;
+    void add(int frames)
+    {
+        ++rows;
+        longest = std::max(longest, frames);
+        sum += frames;
+    }
+    void add(const EncoderFrames &o)
+    {
+        rows += o.rows;
+        longest = std::max(longest, o.longest);
+        sum += o.sum;
+    }
+};
+
+// Cross-attention of many rows with short encoder outputs: 4 warps per (row, head) instead of 8.  pairs: (row, head) pairs of the grid.
+// With more than 4 blocks of 8 warps per SM the blocks come in waves, and each wave pays for a block's start, its statistics and its
+// merge; blocks of half the size make half as many waves.  Two things speak against it.
+//  * Long rows in general: an SM has as many loads in flight either way, and the rows that are left at the end of a launch are done
+//    sooner with 8.  So the mean is limited, to more frames where a frame is half the bytes.  24 layers, 16 heads, us per step, 8 -> 4
+//    warps, 128 / 200 / 400 rows of one length: 130 frames 1535 / 1964 / 2914 -> 1450 / 1873 / 2607, 192 frames 1594 / 2068 / 3076 -> 1561 /
+//    2051 / 3038, 220 frames 1633 / 2122 / 3272 -> 1644 / 2176 / 3220; 8-bit store, 250 frames 1567 / 2004 / 3081 -> 1511 / 1926 / 2876,
+//    384 frames 1722 / 2240 / 3638 -> 1707 / 2200 / 3496.
+//  * One long row among few: it decides when the launch ends, and takes twice as long with 4.  How long it may be grows with the blocks
+//    that an SM has to work through meanwhile: 30 frames per block, until beyond 10 blocks per SM the longest that were tried (500) cost
+//    2 % at most.  bf16 / 8-bit store, change of the step in %: log-normal lengths (sigma 0.7, median 130, longest 408 to 500) at 40 / 48 /
+//    64 / 80 / 96 / 112 / 128 rows +7.7 / +8.3 / +6.1 / +1.9 / -0.9 / -2.5 / -4.4 and +9.0 / +9.1 / +5.3 / +1.9 / -0.7 / -2.2 / -3.7; uniform up
+//    to 250 frames +4.8 / +3.8 / +0.7 / -2.5 / -4.5 / -5.0 / -6.1 and +6.1 / +6.0 / +1.1 / -1.8 / -4.4 / -5.9 / -6.9; half 40 and half 190 +1.6 /
+//    +0.5 / -1.0 / -4.6 / -5.9 / -6.2 / -7.1 and +3.3 / +2.0 / -0.6 / -4.3 / -5.7 / -6.8 / -7.5; all 130 -2.5 / -3.9 / -4.0 / -3.5 / -4.2 / -4.9 /
+//    -5.6 and -0.6 / -2.5 / -4.1 / -4.0 / -4.8 / -6.3 / -6.6.  (The mean alone, as it was, lost up to 17 % below 96 rows.)
+inline bool few_cross_warps(long long pairs, int sm_count, const EncoderFrames &f, bool eight_bit_store)
+{
+    return pairs > 4ll * sm_count && f.sum <= (eight_bit_store ? 384ll : 192ll) * f.rows &&
+           (pairs > 10ll * sm_count || (long long)f.longest * sm_count <= 30 * pairs);
 }
 
 }  // namespace aed

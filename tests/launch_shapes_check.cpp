@@ -1,13 +1,50 @@
 // Host check of launch_shapes.h (no GPU): whatever the row count and the model width, the dynamic shared memory of the
-// vocabulary projection holds both things that live in it one after the other, the ring and the accumulator's rows.
+// vocabulary projection holds both things that live in it one after the other, the ring and the accumulator's rows.  And the
+// rule for smaller cross-attention blocks, on batches whose step times on either side of it are known.
 #include <cstdio>
 
 #include "../paper_2503_05931_b200/csrc/launch_shapes.h"
 
 using namespace aed;
 
+// rows utterances, every n-th of them of `b` frames and the others of `a`
+static bool smaller(int rows, int a, int b, int n, bool eight_bit)
+{
+    EncoderFrames f;
+    for (int u = 0; u < rows; ++u) f.add(u % n == 0 ? b : a);
+    return few_cross_warps(16ll * rows, 148, f, eight_bit);
+}
+
+static bool cross_warps_ok()
+{
+    bool ok = true;
+    for (bool eight_bit : {false, true}) {
+        ok = ok && smaller(64, 130, 130, 1, eight_bit) && smaller(128, 130, 130, 1, eight_bit) && smaller(400, 130, 130, 1, eight_bit);
+        // at most 4 blocks per SM
+        ok = ok && !smaller(36, 10, 10, 1, eight_bit) && smaller(40, 10, 10, 1, eight_bit);
+        // half short, half long; a few very long ones: longest against the blocks per SM, not the mean
+        ok = ok && !smaller(40, 60, 300, 2, eight_bit) && !smaller(64, 60, 300, 2, eight_bit) && smaller(128, 60, 300, 2, eight_bit);
+        ok = ok && !smaller(48, 100, 500, 16, eight_bit) && !smaller(64, 100, 500, 16, eight_bit) && !smaller(88, 100, 500, 16, eight_bit) &&
+             smaller(128, 100, 500, 16, eight_bit);
+        // a longer longest, or a longer mean, never brings the smaller block back
+        for (int rows = 1; rows <= 512; ++rows) {
+            bool before = true;
+            for (int frames = 1; frames <= 600; ++frames) {
+                const bool now = smaller(rows, 1, frames, 4, eight_bit);
+                ok = ok && (before || !now);
+                before = now;
+            }
+        }
+    }
+    // long on average
+    ok = ok && smaller(128, 192, 192, 1, false) && !smaller(128, 193, 193, 1, false) && !smaller(400, 250, 250, 1, false);
+    ok = ok && smaller(128, 384, 384, 1, true) && !smaller(128, 385, 385, 1, true);
+    return ok;
+}
+
 int main()
 {
+    if (!cross_warps_ok()) { printf("few_cross_warps\n"); return 1; }
     for (int k_blocks = 1; k_blocks <= 128; ++k_blocks)          // d_model 64 .. 8192
         for (int rows = 1; rows <= 2100; ++rows) {
             const VocabShape s = vocab_shape(rows, k_blocks);

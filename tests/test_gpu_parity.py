@@ -453,36 +453,48 @@ def test_rows_of_the_next_step(groups, dtype):
 
 @pytest.mark.parametrize("batch", [3, 12, 50, 131])
 def test_steps_with_other_buffers(batch, monkeypatch):
-    """Steps of the caller's loop are replayed as graphs from the second one of a size on: every call has tokens, logits and
-    choices of its own (or none), and a mask or none, and has to do what the same calls do launched kernel by kernel."""
+    """Steps of the caller's loop of a size that keeps coming are replayed as graphs (enough of them here that the last passes are):
+    every call has tokens, logits and choices of its own (or none), and a mask or none, and has to do what the same calls do
+    launched kernel by kernel."""
     import torch
     rng = np.random.default_rng(1000 + batch)
     w = wl.make_custom(MID, rng.integers(1, 60, size=batch), [8] * batch, dtype="bf16", seed=400 + batch, out_std=0.1, ln_std=0.2)
     V = MID["vocab"]
     tokens = torch.from_numpy(rng.integers(0, V, size=(6, batch)).astype(np.int32)).cuda()
     mask = torch.from_numpy((rng.random(batch) < 0.6).astype(np.uint8)).cuda()
-    results = []
-    for graphs in (True, False):
+
+    def run(graphs, passes, everything):
         monkeypatch.setenv("AED_DEC_NO_GRAPH", "0" if graphs else "1")
         dec = _binding().decoder_for_workload(w)
         enc = dec.upload_encoder(w.enc)
         outs = []
-        for _ in range(2):
+        for _ in range(passes):
             dec.precompute_cross_kv(enc, w.enc_lens)
             for t in range(6):
-                logits = torch.full((batch, V), -7.0, device="cuda") if t % 3 != 1 else None
-                choice = torch.full((batch,), -1, dtype=torch.int32, device="cuda") if t % 2 == 0 else None
+                logits = torch.full((batch, V), -7.0, device="cuda") if everything or t % 3 != 1 else None
+                choice = torch.full((batch,), -1, dtype=torch.int32, device="cuda") if everything or t % 2 == 0 else None
                 dec.step(tokens[t].clone(), mask if t in (2, 4) else None, logits, choice)
-                outs += [x.clone() for x in (logits, choice) if x is not None]
+                outs.append([x.clone() if x is not None else None for x in (logits, choice)])
         dec.sync_status()
-        results.append(outs)
         dec.close()
-    for a, b in zip(*results):
-        if a.dtype == torch.int32:
-            assert torch.equal(a == -1, b == -1)
-        else:
-            assert torch.equal(a == -7.0, b == -7.0)
-            assert float((a - b).abs().max()) < 2e-3      # fp32 sums of split projections come in another order
+        return outs
+
+    # fp32 sums of split projections come in another order, so logits may differ by `tol`, and choices only where the two best
+    # entries are closer than twice that
+    tol, decided, choices = 2e-3, 0, 0
+    want = run(False, 1, True)
+    for i, (logits, choice) in enumerate(run(True, 8, False)):
+        full, best = want[i % 6]
+        if logits is not None:
+            assert torch.equal(logits == -7.0, full == -7.0)
+            assert float((logits - full).abs().max()) < tol
+        if choice is not None:
+            assert torch.equal(choice == -1, best == -1)
+            top = full.topk(2, dim=1).values
+            sure = (top[:, 0] - top[:, 1] > 2 * tol) & (best != -1)
+            assert torch.equal(choice[sure], best[sure])
+            decided, choices = decided + int(sure.sum()), choices + int((best != -1).sum())
+    assert decided > 0.9 * choices
 
 
 @pytest.mark.parametrize("dtype, steps", [("bf16", 3), ("bf16", 4), ("bf16", 21), ("fp32", 37)])

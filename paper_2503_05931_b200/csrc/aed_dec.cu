@@ -6,7 +6,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <map>
 #include <mutex>
 #include <tuple>
 #include <new>
@@ -22,6 +21,7 @@
 #include "crosskv_gemm.cuh"
 #include "plane_gemm.cuh"
 #include "f32_rows.cuh"
+#include "step_graphs.h"
 #include "stream_schedule.h"
 
 using namespace aed;
@@ -203,14 +203,13 @@ struct aed_dec {
     bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
-    // greedy decoding replays one captured CUDA graph per key; the output buffers stand in the device-side state
-    typedef std::tuple<int, int, int, bool> GraphKey;       // (row count, chunks of self-attention positions, steps, short_cross)
-    struct GraphEntry { cudaGraphExec_t exec; int64_t nodes; };
-    std::map<GraphKey, GraphEntry> graphs;
+    // steps are replayed as one captured CUDA graph per key; the output buffers stand in the device-side state
+    typedef std::tuple<int, int, int, bool> GraphKey;       // (row count, chunks of self-attention positions, steps (0: one of the caller's loop), short_cross)
+    typedef StepGraphs<GraphKey, cudaGraphExec_t> Graphs;
+    Graphs graphs;
     bool short_cross = false;       // of the launches to come: many rows with short encoder outputs (see few_cross_warps)
     cudaStream_t capture_stream = nullptr;
     bool use_graphs = true;
-    std::map<GraphKey, int> step_seen;      // steps of the caller's loop by key (0 steps): the first one is launched kernel by kernel
     bool from_state = false;        // while such a step is recorded: its kernels find the caller's pointers in the device-side state
     // set only while aed_dec_step_static_scratch runs: attention partials go here instead of the workspace
     float *partials_override = nullptr;
@@ -1240,7 +1239,7 @@ aed_status_t enqueue_greedy_step(aed_dec *dec, int rows_ub, int self_len_ub)
 
 // Record greedy steps (or, with 0, a step of the caller's loop behind its first kernel) into a graph on the library's capture
 // stream (nothing runs) and instantiate it.
-aed_status_t capture_greedy_steps(aed_dec *dec, int rows_ub, int self_len_ub, int steps, aed_dec::GraphEntry *entry)
+aed_status_t capture_greedy_steps(aed_dec *dec, int rows_ub, int self_len_ub, int steps, aed_dec::Graphs::Entry *entry)
 {
     if (!dec->capture_stream)
         AED_CUDA(dec, cudaStreamCreateWithFlags(&dec->capture_stream, cudaStreamNonBlocking));
@@ -1277,19 +1276,22 @@ aed_status_t capture_greedy_steps(aed_dec *dec, int rows_ub, int self_len_ub, in
 constexpr int kGraphSteps = 4;
 int steps_per_graph(const aed_dec *dec, int rows_b) { return rows_b <= (dec->cfg.n_layers <= 8 ? 64 : kRowsInside) ? kGraphSteps : 1; }
 
-// Launch `steps` greedy steps (0: a step of the caller's loop, behind its first kernel) of at most rows_b rows and chunks * kAttnChunk
-// positions as one graph, recorded at first use.
-aed_status_t launch_greedy_graph(aed_dec *dec, int rows_b, int chunks, int steps)
+// The graph of `steps` greedy steps (0: a step of the caller's loop, behind its first kernel) of at most rows_b rows and chunks *
+// kAttnChunk positions, recorded at first use; null if it cannot be recorded.
+const aed_dec::Graphs::Entry *step_graph(aed_dec *dec, int rows_b, int chunks, int steps)
 {
-    const aed_dec::GraphKey key(rows_b, chunks, steps, dec->short_cross);
-    auto it = dec->graphs.find(key);
-    if (it == dec->graphs.end()) {
-        aed_dec::GraphEntry entry{};
-        AED_TRY(capture_greedy_steps(dec, rows_b, chunks * kAttnChunk, steps, &entry));
-        it = dec->graphs.emplace(key, entry).first;
-    }
-    AED_CUDA(dec, cudaGraphLaunch(it->second.exec, dec->stream));
-    dec->launches += it->second.nodes;
+    return dec->graphs.get(aed_dec::GraphKey(rows_b, chunks, steps, dec->short_cross), [&](aed_dec::Graphs::Entry &entry) {
+        std::string err = dec->err;
+        if (capture_greedy_steps(dec, rows_b, chunks * kAttnChunk, steps, &entry) == AED_OK) return true;
+        dec->err.swap(err);               // the steps are launched kernel by kernel instead: nothing has failed yet
+        cudaGetLastError();
+        return false;
+    });
+}
+aed_status_t launch_graph(aed_dec *dec, const aed_dec::Graphs::Entry &graph)
+{
+    AED_CUDA(dec, cudaGraphLaunch(graph.exec, dec->stream));
+    dec->launches += graph.nodes;
     return AED_OK;
 }
 
@@ -1444,21 +1446,21 @@ extern "C" aed_status_t aed_dec_step(aed_dec_t *dec, const int32_t *tokens_in, c
     if (dec->full_steps >= dec->cfg.max_dec_len)
         return fail(dec, AED_ERR_CAPACITY, "every utterance already holds max_dec_len = %d tokens", dec->cfg.max_dec_len);
     const int self_len_ub = dec->steps_issued + 1 < dec->cfg.max_dec_len ? dec->steps_issued + 1 : dec->cfg.max_dec_len;
-    // A step of a size that has come before is replayed as a graph: launching its kernels one by one takes longer than they do up to
-    // 32 rows (24 layers, 24 rows: 770 us a step).  Everything that a call passes goes through the step's first kernel,
-    // which is launched as it is; inside a capture of the caller's own all of them are.
+    // A step of a size that keeps coming is replayed as a graph (see step_graphs.h for when and why).  Everything that a call
+    // passes goes through the step's first kernel, which is launched as it is; inside a capture of the caller's own all of them are.
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (dec->use_tc && dec->use_graphs && !dec->profiling && !dec->partials_override) AED_CUDA(dec, cudaStreamIsCapturing(dec->stream, &capturing));
     else capturing = cudaStreamCaptureStatusActive;
     const int chunks = (self_len_ub + kAttnChunk - 1) / kAttnChunk, rows_b = rows_key(dec->batch);
-    bool graph = capturing == cudaStreamCaptureStatusNone;
-    if (graph) {
+    const aed_dec::Graphs::Entry *graph = nullptr;
+    if (capturing == cudaStreamCaptureStatusNone) {
         dec->short_cross = few_cross_warps(dec, rows_b, dec->frames);
-        graph = dec->step_seen[aed_dec::GraphKey(rows_b, chunks, 0, dec->short_cross)]++ > 0;
+        if (dec->graphs.due(aed_dec::GraphKey(rows_b, chunks, 0, dec->short_cross), steps_before_recording(rows_b > dec->planes_rows)))
+            graph = step_graph(dec, rows_b, chunks, 0);
     }
     AED_TRY(launch_step_rows(dec, false, active, tokens_in, true, nullptr, nullptr, logits_out, next_out));
     if (graph) {
-        AED_TRY(launch_greedy_graph(dec, rows_b, chunks, 0));
+        AED_TRY(launch_graph(dec, *graph));
     } else {
         const int rows_ub = dec->batch;
         dec->short_cross = few_cross_warps(dec, rows_ub, dec->frames);
@@ -1616,12 +1618,14 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
         // grids are sized for the keyed row count; kernels leave rows beyond the device-side row count alone
         const int rows_b = rows_key(alive[s]), chunks = s / kAttnChunk + 1;
         dec->short_cross = few_cross_warps(dec, rows_b, frames_alive[s]);
-        const bool graph = dec->use_graphs && !dec->profiling;
+        const aed_dec::Graphs::Entry *graph = nullptr;
         int n = 1;
-        if (graph) {
+        if (dec->use_graphs && !dec->profiling) {
             const int most = steps_per_graph(dec, rows_b);
             while (n < most && s + n < longest && rows_key(alive[s + n]) == rows_b && (s + n) / kAttnChunk + 1 == chunks) ++n;
             if (n < most) n = 1;
+            graph = step_graph(dec, rows_b, chunks, n);
+            if (!graph) n = 1;
         }
         if (probe) {
             while (s + n - done > kWindow) {
@@ -1631,7 +1635,7 @@ extern "C" aed_status_t aed_dec_greedy_decode(aed_dec_t *dec, const int32_t *max
             // (looked at only behind an event of this decode; steps already issued beyond the last retirement do nothing)
             if (done > 0 && *static_cast<volatile int32_t *>(dec->retired_host) >= B) break;
         }
-        if (graph) AED_TRY(launch_greedy_graph(dec, rows_b, chunks, n));
+        if (graph) AED_TRY(launch_graph(dec, *graph));
         else AED_TRY(enqueue_greedy_step(dec, alive[s], s + 1));
         s += n;
         dec->steps_issued = s;
@@ -1780,6 +1784,7 @@ extern "C" aed_status_t aed_dec_greedy_steps(aed_dec_t *dec, int32_t n_steps, in
             dec->rows_ready = true;
             dec->rows_tokens = tokens_out; dec->rows_lens = out_lens;
         }
+        const aed_dec::Graphs::Entry *graph = nullptr;
         int n = 1;
         if (dec->use_graphs && !dec->profiling) {
             const int rows_b = rows_key(rows_ub), chunks = (longest + kAttnChunk - 1) / kAttnChunk, most = steps_per_graph(dec, rows_b);
@@ -1788,10 +1793,11 @@ extern "C" aed_status_t aed_dec_greedy_steps(aed_dec_t *dec, int32_t n_steps, in
                 const int rows_last = rows_at(most - 1, last);       // (rows only leave in between, positions only grow)
                 if (rows_last > 0 && rows_key(rows_last) == rows_b && (last + kAttnChunk - 1) / kAttnChunk == chunks && last == longest + most - 1) n = most;
             }
-            AED_TRY(launch_greedy_graph(dec, rows_b, chunks, n));
-        } else {
-            AED_TRY(enqueue_greedy_step(dec, rows_ub, longest));
+            graph = step_graph(dec, rows_b, chunks, n);
+            if (!graph) n = 1;
         }
+        if (graph) AED_TRY(launch_graph(dec, *graph));
+        else AED_TRY(enqueue_greedy_step(dec, rows_ub, longest));
         for (int u = 0; u < dec->batch; ++u)
             if (dec->slot_t[u] >= 0 && dec->slot_t[u] < dec->slot_max[u]) dec->slot_t[u] = std::min(dec->slot_t[u] + n, dec->slot_max[u]);
         s += n;
@@ -1944,7 +1950,7 @@ extern "C" void aed_dec_destroy(aed_dec_t *dec)
 {
     if (!dec) return;
     for (cudaEvent_t e : dec->prof_events) cudaEventDestroy(e);
-    for (auto &g : dec->graphs) cudaGraphExecDestroy(g.second.exec);
+    dec->graphs.clear([](cudaGraphExec_t g) { cudaGraphExecDestroy(g); });
     if (dec->capture_stream) cudaStreamDestroy(dec->capture_stream);
     for (cudaEvent_t e : dec->probe_event) if (e) cudaEventDestroy(e);
     if (dec->retired_host) cudaFreeHost(dec->retired_host);

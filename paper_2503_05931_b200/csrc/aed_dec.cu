@@ -199,7 +199,7 @@ struct aed_dec {
     bool use_pdl = true;
     bool attn_pipe = true;
     bool use_gemv = true;           // steps of few rows: projections by warp-level MMAs (step_gemv.cuh)
-    int gemv_rows = 48;             // ... up to this many rows
+    int gemv_rows = kFewRows;       // ... up to this many rows
     bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
     int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
@@ -640,7 +640,7 @@ aed_status_t tc_setup(aed_dec *dec)
         v = getenv("AED_DEC_NO_GEMV");
         dec->use_gemv = !(v && v[0] == '1');
         v = getenv("AED_DEC_GEMV_ROWS");
-        if (v && atoi(v) >= 1 && atoi(v) <= 48) dec->gemv_rows = atoi(v);
+        dec->gemv_rows = few_row_setting(v);
         v = getenv("AED_DEC_GEMV_DIRECT_ROWS");
         if (v && atoi(v) >= 0 && atoi(v) <= 8) dec->gemv_direct_rows = atoi(v);
         v = getenv("AED_DEC_PLANES_ROWS");

@@ -1,8 +1,9 @@
 // Launch shapes that depend on sizes alone: row tile, ring and shared memory of the tensor-core vocabulary projection; warps of a
-// cross-attention block.  Plain C++ (no CUDA), so that they are also checked on the host, over every row count and model width.
+// cross-attention block; rows of the warp-level projections.  Plain C++ (no CUDA), so that they are also checked on the host, over every row count and model width.
 #pragma once
 #include <algorithm>
 #include <cstddef>
+#include <cstdlib>
 
 namespace aed {
 namespace tc {
@@ -44,6 +45,15 @@ inline VocabShape vocab_shape(int rows_ub, int k_blocks)
     // (d_model 64, row tiles of 64 and more: 528 bytes a row against 16 KB + 256 bytes a row).
     s.smem = std::max((size_t)s.stages * stage_bytes, (size_t)s.n_tile * tc::kRowPitch * sizeof(float)) + 1024;
     return s;
+}
+
+// Most rows that the warp-level projections take (two halves of three row tiles of 8, step_gemv.cuh), and what AED_DEC_GEMV_ROWS makes of
+// it: fewer, from 1 on.  A setting of more rows means all that there are; none, or none of these, the default.
+constexpr int kFewRows = 48;
+inline int few_row_setting(const char *text)
+{
+    const int rows = text ? std::atoi(text) : 0;
+    return rows >= 1 ? std::min(rows, kFewRows) : kFewRows;
 }
 
 // The encoder outputs of the rows of a step, as far as the host knows them.

@@ -44,6 +44,10 @@ static bool cross_warps_ok()
 
 int main()
 {
+    const bool setting_ok = few_row_setting(nullptr) == 48 && few_row_setting("") == 48 && few_row_setting("0") == 48 && few_row_setting("-3") == 48 &&
+                            few_row_setting("1") == 1 && few_row_setting("32") == 32 && few_row_setting("48") == 48 && few_row_setting("49") == 48 &&
+                            few_row_setting("64") == 48 && few_row_setting("1000") == 48;
+    if (!setting_ok) { printf("few_row_setting\n"); return 1; }
     if (!cross_warps_ok()) { printf("few_cross_warps\n"); return 1; }
     for (int k_blocks = 1; k_blocks <= 128; ++k_blocks)          // d_model 64 .. 8192
         for (int rows = 1; rows <= 2100; ++rows) {

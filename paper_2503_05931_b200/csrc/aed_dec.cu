@@ -43,8 +43,8 @@ int rows_bucket(int rows)
 
 // Row count a step graph is captured for.  Kernels whose grids follow the row count (attention: one block per row and
 // head) pay for every row of the grid, also for those beyond the device-side count, whose blocks only find out that
-// they have nothing to do, and hold the next kernel back until they have (attn_fused_kernel).  Every key is a graph to record,
-// so: 4, then multiples of 8 up to 64 rows, of 16 up to 256, of 32 beyond.  Never above rows_bucket(rows).
+// they have nothing to do, and take a slot of an SM until they have.  Every key is a graph to record, so: 4, then multiples
+// of 8 up to 64 rows, of 16 up to 256, of 32 beyond.  Never above rows_bucket(rows).
 int rows_key(int rows)
 {
     if (rows <= 4) return 4;         // the projections of steps of at most 4 rows take a form of their own

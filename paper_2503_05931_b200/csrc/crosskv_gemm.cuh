@@ -197,10 +197,10 @@ crosskv_gemm_kernel(const __grid_constant__ CUtensorMap map_enc, const CUtensorM
         {
             if (elect_one()) prefetch_tensormap(&map_enc);
             __syncwarp();
-            const uint32_t full0 = map_to_rank(&bar_full[warp], 0);      // kStages == kProducers: this thread's stage
+            const uint32_t full0 = map_to_rank(&bar_full[warp], 0);      // kStages == kProducers: this warp's stage
             uint8_t *const st = tiles + static_cast<size_t>(warp) * kStageBytes;
             long long it = 0;                           // k-block counter over all of this pair's tiles
-            uint32_t fills = 0;                         // of this thread's stage
+            uint32_t fills = 0;                         // of this warp's stage
             bool ok = true;
             for (TileWalk w(m_pairs, per_group, pairs, pair); w.valid() && ok; w.next()) {
                 const int layer = w.lnt() / n_tiles, nt = w.lnt() % n_tiles;

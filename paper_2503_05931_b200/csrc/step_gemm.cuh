@@ -256,7 +256,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
                 const long long start = clock64();
                 while (clock64() - start < 2000000ll) {}
             }
-            // (one thread polls, the other warps sleep here)
+            // (one warp polls, the others sleep here)
             asm volatile("bar.sync 3, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
         }
     } else if (warp > kSgMmaWarp) {

@@ -84,7 +84,7 @@ step_gemv_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     if (!p.after_rows) sg::pdl_launch_dependents();
 
     if (warp >= 8) {
-        // ---- weight copies (independent of every earlier kernel), then the side jobs --------------------------
+        // ---- weight copies (independent of every earlier kernel, two at most; see elect_one for why lane 0 does), then the side jobs ----
         if (warp == 8 && lane == 0) {
             prefetch_tensormap(mw);
             for (int i = 0; i < n_kb; ++i) {

@@ -33,8 +33,10 @@ constexpr int kErrTimeout = 2;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
-// One lane of a converged warp.  Copies, MMAs and commits are issued behind this and not behind `lane == 0`: they take their operands from
-// uniform registers, and under a branch that the compiler has to take for divergent each of them cost 200 cycles and more.
+// One lane of a converged warp.  MMAs and commits are issued behind this and not behind `lane == 0`: they take their operands from uniform
+// registers, and under a branch that the compiler has to take for divergent each of them cost 70 to 200 cycles (a k-block of four MMAs
+// with its wait and commit 530; four MMAs behind this 126).  Copies show no such difference (8 of 16 KB issue in 571 cycles from lane 0
+// and in 361 from an elected lane, one from each of 8 warps in 144 and 244); they stand behind this where the warp issues in a loop.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t yes;
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_b_lo, TcParams p, int stages, int producers)
 {
-    // `stages` is a multiple of `producers` (1..kProducerWarps): every ring stage is refilled by one thread only, so
+    // `stages` is a multiple of `producers` (1..kProducerWarps): every ring stage is refilled by one warp only, so
     // a producer is never more than one phase ahead of the barrier it waits on (a parity wait cannot tell more).
     extern __shared__ uint8_t smem_dyn[];
     __shared__ __align__(8) uint64_t bar_full[kMaxStages];
@@ -244,7 +246,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 issued = i + 1;
             }
             if (abort_flag && issued > 0) {
-                // give this thread's last copies a bounded chance to land before the CTA's memory goes away
+                // give this warp's last copies a bounded chance to land before the CTA's memory goes away
                 const int i = issued - 1;
                 const long long start = clock64();
                 while (!mbar_try_wait(&bar_full[i % stages], (i / stages) & 1) && clock64() - start < kWaitCycles / 8) {}

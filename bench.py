@@ -143,22 +143,22 @@ def profile_bytes(prof, w):
 # dram__bytes_write.sum of the captured launches over their algorithmic bytes).  An entry is removed when its kernel
 # changes, which turns the reported traffic back into null.
 NCU_TRAFFIC_RATIO = {
-    # five launches of one layer at 128 rows (cfg3): 71.87 MB read for 29.36 MB of layer weights; the launches also read
-    # the composite cross-query matrix (2.1 MB), the fp32 activation rows, and each prefetches the next layer's matrices
+    # five launches of one layer at 128 rows (cfg3): 71.85 MB read for 29.36 MB of layer weights (64 rows: 66.61); the launches also
+    # read the composite cross-query matrix (2.1 MB), the fp32 activation rows, and each prefetches the next layer's matrices
     # of its kind into L2, which under the profiler's serialised replay is a second DRAM read
     "step_gemm_kernel": 2.45,
-    # the five launches at 16 and at 4 rows (cfg2): 63.70 MB and 62.92 MB read
-    "step_gemv_staged_kernel": 2.17,
-    "step_gemv_kernel": 2.14,
-    # the six launches of one layer at 512 rows: 56.82 MB read; beside the weights the activation planes
+    # the five launches at 16 and at 4 rows (cfg2): 62.03 MB and 61.27 MB read
+    "step_gemv_staged_kernel": 2.11,
+    "step_gemv_kernel": 2.09,
+    # the six launches of one layer at 512 rows: 56.83 MB read; beside the weights the activation planes
     "plane_gemm_kernel": 1.94,
-    # self + cross attention of one layer at 64 rows: 0.84 + 31.05 MB for 0.52 + 30.49 MB of K/V (cross-attention of 512 rows:
+    # self + cross attention of one layer at 64 rows: 1.10 + 31.05 MB for 0.52 + 30.49 MB of K/V (cross-attention of 512 rows:
     # 127.97 MB read for 125.8)
-    "attn_fused_kernel": 1.03,
+    "attn_fused_kernel": 1.04,
     # vocabulary projection: 33.84 MB for the 33.55 MB output matrix (tcgen05 kernel; 33.79 MB in the few-row kernel)
     "tc_gemm_kernel": 1.01,
     "vocab_gemv_kernel": 1.01,
-    # cross-K/V of 7444 frames: 131.3 MB read + 683.0 MB written for 847.7 MB (part of the output is still in L2 at exit)
+    # cross-K/V of 7444 frames: 129.9 MB read + 683.9 MB written for 847.7 MB (part of the output is still in L2 at exit)
     "crosskv_gemm_kernel": 0.96,
     # fp32: the six projections of a layer at 4 rows (2 layers, d 256), 3.86 MB for 3.67; cross-K/V of 20000 frames (d 1024),
     # 90.9 MB read + 125.4 MB written for 254.1 MB

@@ -179,7 +179,7 @@ def timed_passes(one_pass, warmup: int, steps: int, barrier, event, start=None):
     """Device time of ``steps`` passes after ``warmup`` untimed ones of the same kind: (all, each) in ms.  ``start`` is called between
     the two.  Passes from the host need warm-ups of their own: the binding keeps a batch's encoder states until the next
     batch, so the first two passes take a new block of device memory each, and that call takes 1 to 85 ms of host time, during which
-    the device idles (with one warm-up pass 20 passes came to 27.4k to 29.0k tokens/s on boxes that agree to 0.2 % otherwise)."""
+    the device idles (with one warm-up pass 20 passes came to 27.4k to 29.0k tokens/s between runs that agree to 0.2 % otherwise)."""
     for _ in range(warmup):
         one_pass()
     if start is not None:

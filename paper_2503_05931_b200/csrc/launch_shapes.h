@@ -1,5 +1,6 @@
 // Launch shapes that depend on sizes alone: row tile, ring and shared memory of the tensor-core vocabulary projection; warps of a
-// cross-attention block; rows of the warp-level projections.  Plain C++ (no CUDA), so that they are also checked on the host, over every row count and model width.
+// cross-attention block; rows of the warp-level projections.  Plain C++ (no CUDA), so that they are also checked on the host,
+// over every row count and model width.
 #pragma once
 #include <algorithm>
 #include <cstddef>

@@ -101,7 +101,7 @@ KERNEL_OF_FAMILY = {
 }
 KERNEL_OF_VARIANT = {
     "plane": "plane_gemm_kernel", "warp": "self_attn_warp_kernel", "gamma": "gamma_planes_kernel", "gemv_staged": "step_gemv_staged_kernel",
-    "gemv": "step_gemv_kernel", "f32_tile": "tile_kernel", "f32_rows": "rows_kernel",
+    "gemv": "vocab_gemv_kernel", "f32_tile": "tile_kernel", "f32_rows": "rows_kernel",
 }
 # The rows of a greedy pass only fall, so the variants of a call site take its steps in this order.
 VARIANT_ORDER = ["plane", "warp", "f32_tile", "", "gemv_staged", "f32_rows", "gemv"]
@@ -147,9 +147,8 @@ NCU_TRAFFIC_RATIO = {
     # read the composite cross-query matrix (2.1 MB), the fp32 activation rows, and each prefetches the next layer's matrices
     # of its kind into L2, which under the profiler's serialised replay is a second DRAM read
     "step_gemm_kernel": 2.45,
-    # the five launches at 16 and at 4 rows (cfg2): 62.03 MB and 61.27 MB read
+    # the five launches at 16 rows (cfg2): 62.03 MB read
     "step_gemv_staged_kernel": 2.11,
-    "step_gemv_kernel": 2.09,
     # the six launches of one layer at 512 rows: 56.83 MB read; beside the weights the activation planes
     "plane_gemm_kernel": 1.94,
     # self + cross attention of one layer at 64 rows: 1.10 + 31.05 MB for 0.52 + 30.49 MB of K/V (cross-attention of 512 rows:

@@ -43,12 +43,12 @@ int rows_bucket(int rows)
 
 // Row count a step graph is captured for.  Kernels whose grids follow the row count (attention: one block per row and
 // head) pay for every row of the grid, also for those beyond the device-side count, whose blocks only find out that
-// they have nothing to do, and take a slot of an SM until they have.  Every key is a graph to record, so: 4, then multiples
-// of 8 up to 64 rows, of 16 up to 256, of 32 beyond.  Never above rows_bucket(rows).
+// they have nothing to do, and take a slot of an SM until they have; the projections of few rows multiply tiles of four.  Every
+// key is a graph to record, so: multiples of 4 up to 48 rows, of 8 up to 64, of 16 up to 256, of 32 beyond.  (Multiples of 8 from 8 on: 12 / 20 /
+// 28 / 36 rows 499 / 593 / 669 / 773 us per step of the 24-layer model instead of 481 / 591 / 663 / 732.)  Never above rows_bucket(rows).
 int rows_key(int rows)
 {
-    if (rows <= 4) return 4;         // the projections of steps of at most 4 rows take a form of their own
-    const int g = rows <= 64 ? 8 : rows <= 256 ? 16 : 32;
+    const int g = rows <= kFewRows ? 4 : rows <= 64 ? 8 : rows <= 256 ? 16 : 32;
     return (rows + g - 1) / g * g;
 }
 
@@ -201,7 +201,6 @@ struct aed_dec {
     bool use_gemv = true;           // steps of few rows: projections by warp-level MMAs (step_gemv.cuh)
     int gemv_rows = kFewRows;       // ... up to this many rows
     bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
-    int gemv_direct_rows = 4;       // ... with the activation fragments straight from global memory up to this many
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
     // steps are replayed as one captured CUDA graph per key; the output buffers stand in the device-side state
     typedef std::tuple<int, int, int, bool> GraphKey;       // (row count, chunks of self-attention positions, steps (0: one of the caller's loop), short_cross)
@@ -537,6 +536,22 @@ bool encode_map(CUtensorMap *map, const void *base, size_t rows, size_t cols, in
 
 using tc::kTcSmemBudget;
 
+// The few-row projection for that many rows per CTA; wide: of up to four k-blocks (launches of 33 to 48 rows).
+template <int MODE> const void *few_row_kernel(int rows, bool wide)
+{
+    if (wide) return rows == 20 ? (const void *)sv::step_gemv_staged_kernel<MODE, 20, 4> : rows == 24 ? (const void *)sv::step_gemv_staged_kernel<MODE, 24, 4> : nullptr;
+    switch (rows) {
+    case 4: return (const void *)sv::step_gemv_staged_kernel<MODE, 4>;
+    case 8: return (const void *)sv::step_gemv_staged_kernel<MODE, 8>;
+    case 12: return (const void *)sv::step_gemv_staged_kernel<MODE, 12>;
+    case 16: return (const void *)sv::step_gemv_staged_kernel<MODE, 16>;
+    case 20: return (const void *)sv::step_gemv_staged_kernel<MODE, 20>;
+    case 24: return (const void *)sv::step_gemv_staged_kernel<MODE, 24>;
+    case 28: return (const void *)sv::step_gemv_staged_kernel<MODE, 28>;
+    default: return (const void *)sv::step_gemv_staged_kernel<MODE, 32>;
+    }
+}
+
 aed_status_t tc_setup(aed_dec *dec)
 {
     const auto &c = dec->cfg;
@@ -584,16 +599,10 @@ aed_status_t tc_setup(aed_dec *dec)
                           (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 1>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 2>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 4>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 8>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSgSmem + 1024);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(pg::plane_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(3, 4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_PLAIN, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_GAMMA, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sv::step_gemv_staged_kernel<sg::B_LN_RELU, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_staged_smem(4));
-
+    for (int rows = 4; rows <= 32; rows += 4)
+        for (int wide = 0; wide < 2; ++wide)
+            for (const void *k : {few_row_kernel<sg::B_PLAIN>(rows, wide), few_row_kernel<sg::B_GAMMA>(rows, wide), few_row_kernel<sg::B_LN_RELU>(rows, wide)})
+                if (e == cudaSuccess && k) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sv::sv_smem(rows, wide ? 4 : sv::kSvMaxKb));
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(e));
     // LayerNorm-fold constants of every layer
     for (int l = 0; l < c.n_layers; ++l) {
@@ -641,8 +650,6 @@ aed_status_t tc_setup(aed_dec *dec)
         dec->use_gemv = !(v && v[0] == '1');
         v = getenv("AED_DEC_GEMV_ROWS");
         dec->gemv_rows = few_row_setting(v);
-        v = getenv("AED_DEC_GEMV_DIRECT_ROWS");
-        if (v && atoi(v) >= 0 && atoi(v) <= 8) dec->gemv_direct_rows = atoi(v);
         v = getenv("AED_DEC_PLANES_ROWS");
         if (v && atoi(v) > 0) dec->planes_rows = atoi(v);
 
@@ -717,26 +724,21 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     p.n_tile = n_tile;
     p.state = dec->state();
     p.eps = dec->cfg.ln_eps;
-    // Few rows: warp-level MMAs (step_gemv.cuh).  Row tiles of 8 per CTA follow the row count: 2, 3 or 4, and from 33 rows two
-    // halves of 3 on grid.z with half the k-splits, up to four k-blocks per CTA.  A step of these sizes is bound by
-    // instructions issued (conversion of the rows to planes, fragments, reductions), so a tile of padding costs as much as one of
-    // rows.  Per decode step of the 24-layer model, with four tiles -> with three: 715 -> 630 us at 20 rows, 723 -> 680 at 24, 1104 ->
-    // 959 at 48.  From 49 rows on the halves would need four tiles, and the tcgen05 kernel takes over (40 / 48 rows 905 / 949 us there
-    // against 879 / 922 here; 52 / 64 rows 984 / 1043 against 1064 / 1112).
+    // Few rows: warp-level MMAs (step_gemv.cuh), rows of a CTA in multiples of 4, and from 33 rows two halves on grid.z with half the
+    // k-splits, up to four k-blocks per CTA.  From 49 rows on the tcgen05 kernel takes over (48 / 56 / 64 rows 824 us per step of the
+    // 24-layer model here, 938 and 970 there).
     const int splits_wide = std::max((k_blocks + 3) / 4, splits / 2);
     const bool gemv = dec->use_gemv && rows_ub <= dec->gemv_rows &&
                       (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
-    ProfScope ps(dec, family + KF_COUNT * (!gemv ? KV_NONE : rows_ub <= dec->gemv_direct_rows ? KV_GEMV : KV_GEMV_STAGED));
-    // (whose CTAs cover at most two k-blocks, beyond 32 rows four; activation fragments straight from global memory up to 4 rows,
-    // through shared memory beyond)
+    ProfScope ps(dec, family + KF_COUNT * (gemv ? KV_GEMV_STAGED : KV_NONE));
     if (gemv) {
         cudaLaunchConfig_t gc = {};
         gc.gridDim = dim3(m_tiles, splits, 1);
         gc.blockDim = dim3(sv::kSvThreads);
-        const bool direct = rows_ub <= dec->gemv_direct_rows, wide = rows_ub > 32;
-        const int nt = wide ? 3 : rows_ub <= 16 ? 2 : rows_ub <= 24 ? 3 : 4;                   // row tiles of 8 per CTA
+        const bool wide = rows_ub > 32;
+        const int rows = ((wide ? (rows_ub + 1) / 2 : rows_ub) + 3) / 4 * 4;                  // of a CTA
         if (wide) gc.gridDim = dim3(m_tiles, splits_wide, 2);
-        gc.dynamicSmemBytes = direct ? (size_t)sv::kSvMaxKb * tc::kATileBytes + 1024 : (size_t)sv::sv_staged_smem(nt, wide ? 4 : sv::kSvMaxKb);
+        gc.dynamicSmemBytes = (size_t)sv::sv_smem(rows, wide ? 4 : sv::kSvMaxKb);
         gc.stream = dec->stream;
         cudaLaunchAttribute ga[1];
         ga[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -744,11 +746,8 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
         gc.attrs = ga;
         gc.numAttrs = 1;
         const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
-        cudaError_t ge = direct    ? cudaLaunchKernelEx(&gc, sv::step_gemv_kernel<MODE, 1>, map_w, second, p)
-                         : wide    ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3, 4>, map_w, second, p)
-                         : nt == 3 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 3>, map_w, second, p)
-                         : nt == 2 ? cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 2>, map_w, second, p)
-                                   : cudaLaunchKernelEx(&gc, sv::step_gemv_staged_kernel<MODE, 4>, map_w, second, p);
+        void *args[] = {(void *)&map_w, (void *)&second, &p};
+        const cudaError_t ge = cudaLaunchKernelExC(&gc, few_row_kernel<MODE>(rows, wide), args);
         if (ge != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(ge));
         AED_LAUNCHED(dec);
         return AED_OK;

@@ -396,6 +396,16 @@ def test_row_tiles_of_three(batch):
     _run_both(w, rows=sorted({0, 7, 16, 19, batch // 2, batch - 1}))
 
 
+@pytest.mark.parametrize("batch", [3, 4, 5, 11, 12, 13, 20, 21, 28, 29, 36, 37, 44, 45])
+def test_row_tiles_of_four(batch):
+    """Row counts whose last row tile has at most four rows (high and low planes in one MMA), filled, partly filled and one row
+    beyond, alone and in two row halves."""
+    rng = np.random.default_rng(1100 + batch)
+    w = wl.make_custom(WIDE_A, rng.integers(1, 80, size=batch), rng.integers(1, 6, size=batch), dtype="bf16", seed=510 + batch,
+                       out_std=0.1, ln_std=0.2)
+    _run_both(w, rows=sorted({0, batch // 2 - 1, batch // 2, max(batch - 5, 0), batch - 4 if batch > 4 else 0, batch - 1}))
+
+
 @pytest.mark.parametrize("model, batch", [("wide_a", 129), ("wide_b", 65), ("odd", 342), ("odd", 347)])
 def test_self_attention_of_many_rows(model, batch):
     """More than 1024 (row, head) pairs, where self-attention takes a warp per pair: just above the line, a last block

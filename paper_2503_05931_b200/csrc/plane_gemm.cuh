@@ -75,7 +75,7 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
     }
     tc_fence_before_sync();
     __syncthreads();
-    ckv::cluster_sync();                               // the peer's barriers exist before anything reports to them
+    ckv::cluster_meet();                               // the peer's barriers exist before anything reports to them
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_slot;
 
@@ -206,7 +206,7 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
     }
     tc_fence_before_sync();
     __syncthreads();
-    ckv::cluster_sync();                               // neither block ends while the other may still report to it
+    ckv::cluster_meet();                               // neither block ends while the other may still report to it
     if (warp == kPgMmaWarp) {
         tc_fence_after_sync();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");

@@ -594,9 +594,9 @@ aed_status_t tc_setup(aed_dec *dec)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "tensor-core path set-up: %s", cudaGetErrorString(e));
     dec->sm_count = sms > 0 ? sms : 148;
-    for (const void *k : {(const void *)sg::step_gemm_kernel<sg::B_PLAIN, 1>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 2>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 4>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 8>,
-                          (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 1>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 2>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 4>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 8>,
-                          (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 1>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 2>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 4>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 8>})
+    for (const void *k : {(const void *)sg::step_gemm_kernel<sg::B_PLAIN, 1>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 2>, (const void *)sg::step_gemm_kernel<sg::B_PLAIN, 4>,
+                          (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 1>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 2>, (const void *)sg::step_gemm_kernel<sg::B_GAMMA, 4>,
+                          (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 1>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 2>, (const void *)sg::step_gemm_kernel<sg::B_LN_RELU, 4>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSgSmem + 1024);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(pg::plane_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     for (int rows = 4; rows <= 32; rows += 4)
@@ -699,37 +699,36 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
 {
     // after_rows: the kernel before this launch makes the row table
     // map_w2, M2: a second weight matrix [M2, K] over the same rows (its output, gamma and bias are in p)
-    const int n_tile = tc_n_tile(rows_ub, sg::kSgMaxRows);
-    const int m_tiles1 = (M + tc::kTileM - 1) / tc::kTileM;
-    const int row_tiles = (rows_ub + n_tile - 1) / n_tile, m_tiles = m_tiles1 + (map_w2 ? (M2 + tc::kTileM - 1) / tc::kTileM : 0);
-    p.tiles_first = map_w2 ? m_tiles1 : 0;
     p.after_rows = after_rows;
     p.a_rows2 = M2;
     const int k_blocks = K / tc::kBlockK;
+    p.a_rows = M;
+    p.k_blocks = k_blocks;
+    p.state = dec->state();
+    p.eps = dec->cfg.ln_eps;
     // k-splits: every split adds rows x features x 4 bytes of reductions, so the tcgen05 kernel stops at about one CTA per SM (256
-    // CTAs instead of 128: 64 / 96 / 128 rows 1043 / 1297 / 1493 -> 1378 / 1726 / 1950 us per step of the 24-layer model).  For the
+    // CTAs instead of 128: 64 / 96 / 128 rows 1043 / 1297 / 1493 -> 1378 / 1726 / 1950 us per step of the 24-layer model; 64 instead of 128
+    // at 64 / 128 rows 949 / 1356 -> 1027 / 1564).  For the
     // few-row kernels that traffic is small, and CTAs with one or two k-blocks need so little shared memory that the CTAs of the
     // next projection become resident beside them and fetch their weight tiles while this one still runs: there twice as many CTAs
     // are worth it (24-layer batch-64 workload: 129 ms per pass with a target of 128 CTAs, 121 ms with 256, 147 ms with 384).
-    const int target_ctas = dec->tc_target_fixed ? dec->tc_target_ctas : (rows_ub <= dec->gemv_rows ? 256 : 128);
-    int splits = target_ctas / (m_tiles * row_tiles);
-    if (splits < 1) splits = 1;
-    if (splits > k_blocks) splits = k_blocks;
-    const int kb_max = (k_blocks + splits - 1) / splits;
-    const int act_bytes = 2 * n_tile * tc::kBlockK * 2;          // of a k-block, both planes
-    p.stages = std::min(kb_max, sg::kMaxKb);
-    p.share = kb_max >= 4 ? 2 : kb_max >= 2 ? 1 : 0;
-    p.a_rows = M;
-    p.k_blocks = k_blocks;
-    p.n_tile = n_tile;
-    p.state = dec->state();
-    p.eps = dec->cfg.ln_eps;
+    const bool few = dec->use_gemv && rows_ub <= dec->gemv_rows;
+    const int target_ctas = dec->tc_target_fixed ? dec->tc_target_ctas : (few ? 256 : 128);
+    int m_tiles = 0, splits = 0, kb_max = 0;
+    // feature tiles come in multiples of `group`
+    auto split = [&](int group, int row_tiles) {
+        auto tiles = [&](int m) { return (m + group * tc::kTileM - 1) / (group * tc::kTileM) * group; };
+        p.tiles_first = map_w2 ? tiles(M) : 0;
+        m_tiles = tiles(M) + (map_w2 ? tiles(M2) : 0);
+        splits = std::min(std::max(target_ctas / (m_tiles * row_tiles), 1), k_blocks);
+        kb_max = (k_blocks + splits - 1) / splits;
+    };
+    split(1, 1);
     // Few rows: warp-level MMAs (step_gemv.cuh), rows of a CTA in multiples of 4, and from 33 rows two halves on grid.z with half the
-    // k-splits, up to four k-blocks per CTA.  From 49 rows on the tcgen05 kernel takes over (48 / 56 / 64 rows 824 us per step of the
-    // 24-layer model here, 938 and 970 there).
+    // k-splits, up to four k-blocks per CTA.  From 49 rows on the tcgen05 kernel takes over (20 / 24 / 32 / 40 / 48 rows 591 / 608 / 679 / 778 / 827
+    // us per step of the 24-layer model here, at best 635 / 644 / 684 / 832 / 857 there; 49 / 56 / 64 rows 867 / 888 / 917 there).
     const int splits_wide = std::max((k_blocks + 3) / 4, splits / 2);
-    const bool gemv = dec->use_gemv && rows_ub <= dec->gemv_rows &&
-                      (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
+    const bool gemv = few && (rows_ub <= 32 ? kb_max <= sv::kSvMaxKb : (k_blocks + splits_wide - 1) / splits_wide <= 4);
     ProfScope ps(dec, family + KF_COUNT * (gemv ? KV_GEMV_STAGED : KV_NONE));
     if (gemv) {
         cudaLaunchConfig_t gc = {};
@@ -752,6 +751,12 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
         AED_LAUNCHED(dec);
         return AED_OK;
     }
+    // pairs of blocks
+    p.n_tile = tc_pair_tile(rows_ub, sg::kSgMaxRows);
+    const int row_tiles = (rows_ub + p.n_tile - 1) / p.n_tile, act_bytes = p.n_tile * tc::kBlockK * 2;      // of a k-block, both planes of half of the rows
+    split(2, row_tiles);
+    p.stages = std::min(kb_max, sg::kMaxKb);
+    p.share = kb_max >= 4 ? 2 : kb_max >= 2 ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m_tiles, splits, row_tiles);
     cfg.blockDim = dim3(sg::kSgThreads);
@@ -763,11 +768,10 @@ aed_status_t launch_step_gemm(aed_dec *dec, int family, const CUtensorMap &map_w
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const CUtensorMap &second = map_w2 ? *map_w2 : map_w;
-    const int rows_per_thread = (n_tile * (8 << p.share) + sg::kSgConvertThreads - 1) / sg::kSgConvertThreads;
+    const int rows_per_thread = (p.n_tile / 2 * (8 << p.share) + sg::kSgConvertThreads - 1) / sg::kSgConvertThreads;
     cudaError_t e = rows_per_thread <= 1   ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 1>, map_w, second, p)
                     : rows_per_thread <= 2 ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 2>, map_w, second, p)
-                    : rows_per_thread <= 4 ? cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 4>, map_w, second, p)
-                                           : cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 8>, map_w, second, p);
+                                           : cudaLaunchKernelEx(&cfg, sg::step_gemm_kernel<MODE, 4>, map_w, second, p);
     if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "projection launch: %s", cudaGetErrorString(e));
     AED_LAUNCHED(dec);
     return AED_OK;

@@ -28,6 +28,13 @@ inline int tc_n_tile(int rows_ub, int most)
     return std::max(16, ((rows_ub + tiles - 1) / tiles + 15) / 16 * 16);
 }
 
+// The same for pairs of blocks, each with half of the rows, in 16s.
+inline int tc_pair_tile(int rows_ub, int most)
+{
+    const int tiles = (rows_ub + most - 1) / most;
+    return std::max(32, ((rows_ub + tiles - 1) / tiles + 31) / 32 * 32);
+}
+
 struct VocabShape {
     int n_tile, row_tiles, stages, producers;
     size_t smem;                               // dynamic shared memory, the alignment of the ring included

@@ -3,7 +3,8 @@
 //
 //   out[r, o] += sum_k B(r, k) * W[o, k]      (+ bias[o] from the CTA of the first k-split)
 //
-// A CTA has 128 output features and up to four k-blocks of 64 at a time.  The weight tiles (bf16, TMA) do not depend on
+// Pairs of CTAs (tcgen05 cta_group::2): a CTA has 128 output features, up to four k-blocks of 64 at a time and makes the activation tiles of
+// half of the rows; the tensor cores read the other half from the peer's shared memory.  The weight tiles (bf16, TMA) do not depend on
 // earlier kernels and are requested before the programmatic-dependency wait.  The activation tiles are made by 16 warps from
 // the fp32 source in the 128-byte-swizzled layout the MMA reads, as a bf16 high plane and a bf16 low plane
 // (value - high) behind each other, so that one MMA of twice the rows multiplies both; with one of three transforms fused:
@@ -11,14 +12,14 @@
 //   B_GAMMA    B = gamma[k] * src                        (LayerNorm folded into the projection, see below)
 //   B_LN_RELU  B = relu(rstd_r * (src - mean_r * c1[k]) + c2[k])   (FFN hidden layer from the folded first GEMM)
 //
-// What bounds it: a chain of hand-overs inside one launch.  Cycles at 64 rows, K = 256 per CTA: source rows from L2 900 to 1000,
-// conversion (64 x 256 values) 2000, 16 MMAs and their hand-over 1800, reductions 1200 (an SM gives out 28 bytes a cycle).  So the
-// k-blocks are converted side by side by groups of warps whose per-k constants wait in registers, and the MMAs are issued in
-// one go.  The forms before (up to 64 rows warp-level MMAs; beyond 8 converting warps, source tiles by TMA, a ring of k-blocks with
-// a barrier each, transposed reductions) took, per step of the 24-layer model, 56 / 64 / 80 / 96 / 112 / 128 rows
-// 1093 / 1120 / 1336 / 1485 / 1605 / 1746 us; with this one 1003 / 1039 / 1222 / 1298 / 1393 / 1496.
-// (Tried on the way: k-splits that meet in a cluster through distributed shared memory, which would leave complete sums and planes
-// for the next projection: SM-to-SM reads ran at 10 to 20 bytes a cycle beside the other traffic, 64 rows 1456.)
+// What bounds it: a chain of hand-overs inside one launch.  Cycles at 64 rows, K = 256 per CTA: tiles of 32 rows (from L2, converted, written)
+// 2050, 16 MMAs and their hand-over 1800, reductions 1620 (an SM gives out 28 bytes a cycle).  So the k-blocks are converted side by side
+// by groups of warps whose per-k constants wait in registers, and the MMAs are issued in one go.  One CTA per tile, which converted all 64 rows, took
+// 3180 + 1900 + 1860 cycles; us per step of the 24-layer model, 49 / 56 / 64 / 72 / 80 / 96 / 112 / 128 rows: 911 / 940 / 970 / 1120 / 1176 /
+// 1252 / 1335 / 1420 then, 867 / 888 / 917 / 1082 / 1132 / 1181 / 1268 / 1321 now.  (8 converting warps instead of 16: 873 / 885 / 904 / 1081 /
+// 1137 / 1200 / 1333 / 1390.  Registers for two CTAs per SM: 947 / 990 / 1022 and 1174 to 1516, because blocks of the next projection then take the room
+// of attention's.  Tried before the pairs: k-splits that meet in a cluster through distributed shared memory, which would leave complete sums
+// and planes for the next projection: SM-to-SM reads ran at 10 to 20 bytes a cycle beside the other traffic.)
 //
 // LayerNorm folding: LN(x) W^T = rstd * ((gamma*x) W^T - mean * c1) + c2 with c1[o] = sum_k gamma_k W[o,k] and
 // c2[o] = sum_k beta_k W[o,k] + b[o].  The GEMM therefore runs on gamma*x without knowing the row statistics;
@@ -32,7 +33,7 @@
 //
 // Waits are bounded.
 #pragma once
-#include "tc_gemm.cuh"
+#include "crosskv_gemm.cuh"
 
 namespace aed {
 namespace sg {
@@ -42,7 +43,7 @@ using namespace tc;
 constexpr int kMaxKb = 4;             // k-blocks that a CTA holds at most
 constexpr int kSgConvertWarps = 16, kSgMmaWarp = 16, kSgConvertThreads = kSgConvertWarps * 32;
 constexpr int kSgThreads = 576;       // warps 0..15 activation tiles and epilogue, warp 16 MMAs, warp 17 side jobs
-constexpr int kSgMaxRows = 128;       // rows per CTA tile
+constexpr int kSgMaxRows = 128;       // rows per tile of a pair
 constexpr int kSgSmem = 192 * 1024;   // of all tiles at most
 
 enum BMode { B_PLAIN = 0, B_GAMMA = 1, B_LN_RELU = 2 };
@@ -50,7 +51,7 @@ enum BMode { B_PLAIN = 0, B_GAMMA = 1, B_LN_RELU = 2 };
 struct StepGemmParams {
     int a_rows;                // output features M
     int k_blocks;              // K / 64
-    int n_tile;                // rows per CTA tile (16..128, multiple of 16)
+    int n_tile;                // rows per pair of CTAs (32..128, multiple of 32)
     int stages;                // k-blocks that a CTA holds at a time, 1..kMaxKb
     int share;                 // 1 << share groups of threads take turns with the k-blocks
     // activation source [rows, ld_src] fp32
@@ -170,87 +171,103 @@ __device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_r
     }
 }
 
-// grid: x = 128-feature tiles, y = k-splits, z = row tiles.  kNI: rows of a k-block per thread at most.
-// Dynamic smem (from a 1024-byte boundary): p.stages weight tiles of 16 KB | as many activation tiles of 2 n_tile x 128 bytes (high plane, low plane).
+// One arrival at a barrier of either block of the pair (shared::cluster address).  What it tells of are tiles that tensor cores read: every
+// writer has put a proxy fence behind its writes (tiles_written), so the arrival itself, in its default form, need not be a release at
+// cluster scope, which would wait for all that its thread has under way (64 / 128 rows 981 / 1392 us a step even with one such arrival per CTA, 917 / 1321 so).
+__device__ __forceinline__ void arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// this thread's generic-proxy writes of operand tiles -> tensor-core reads of either block
+__device__ __forceinline__ void tiles_written() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// grid: x = 128-feature tiles (an even number of either matrix), y = k-splits, z = row tiles.  kNI: rows of a k-block per thread at most.
+// Dynamic smem (from a 1024-byte boundary): p.stages weight tiles of 16 KB | as many activation tiles of n_tile x 128 bytes: the high
+// plane of this block's half of the rows, then their low plane.
 template <int MODE, int kNI>
-__global__ void __launch_bounds__(kSgThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSgThreads, 1)
 step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_w2, const __grid_constant__ StepGemmParams p)
 {
     extern __shared__ uint8_t smem_dyn[];
-    __shared__ __align__(8) uint64_t bar_w, bar_done;
+    __shared__ __align__(8) uint64_t bar_w, bar_act, bar_done;      // (the first two: of the pair's first block)
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
     AED_TRACE_RESERVE(tcur, p.state, (threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ? 10u : 0u);
     AED_TRACE_PUT_NS(p.state, tcur, 40 + MODE);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = ckv::cluster_rank();
     const bool second_w = p.tiles_first > 0 && static_cast<int>(blockIdx.x) >= p.tiles_first;
     const CUtensorMap *const mw = second_w ? &map_w2 : &map_w;
     const int a0 = (second_w ? static_cast<int>(blockIdx.x) - p.tiles_first : static_cast<int>(blockIdx.x)) * kTileM;
     const int a_rows = second_w ? p.a_rows2 : p.a_rows;
-    const int row0 = blockIdx.z * p.n_tile;
+    const int row0 = blockIdx.z * p.n_tile, half_tile = p.n_tile / 2;
     const int kb_begin = static_cast<int>((static_cast<long long>(p.k_blocks) * blockIdx.y) / gridDim.y);
     const int kb_end = static_cast<int>((static_cast<long long>(p.k_blocks) * (blockIdx.y + 1)) / gridDim.y);
     const int n_kb = kb_end - kb_begin, S = p.stages;
     uint8_t *const tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
-    const int plane_bytes = p.n_tile * kBlockK * 2;
+    const int plane_bytes = half_tile * kBlockK * 2;
     uint8_t *const acts = tiles + S * kATileBytes;
     uint32_t tmem_cols = 32;
     while (tmem_cols < static_cast<uint32_t>(2 * p.n_tile)) tmem_cols <<= 1;
 
     if (threadIdx.x == kSgMmaWarp * 32) {
         mbar_init(&bar_w, 1);
+        mbar_init(&bar_act, 2 * kSgConvertWarps);
         mbar_init(&bar_done, 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kSgMmaWarp) {
         __syncwarp();
-        if (elect_one()) {                            // weights: independent of every earlier kernel
-            const int n = min(n_kb, S);
-            mbar_expect_tx(&bar_w, n * kATileBytes);
-            for (int i = 0; i < n; ++i) tma_load_2d(tiles + i * kATileBytes, mw, (kb_begin + i) * kBlockK, a0, &bar_w);
-        }
-        __syncwarp();
-        tmem_alloc(&tmem_slot, tmem_cols);
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before_sync();
     __syncthreads();
+    ckv::cluster_meet();                                  // the peer's barriers exist before anything reports to them
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_slot;
     if (!p.after_rows) pdl_launch_dependents();
 
-    // Rounds of up to S k-blocks (one round unless the launch has few blocks for its K): tiles written -> barrier 4 -> MMAs -> barrier 3.
-    // The MMAs of a round are issued in one go: a wait or a commit between them costs more than the four MMAs of a k-block
-    // (16 MMAs of 128 x 64 x 16: 1160 cycles, with a wait and a commit per k-block 2290).
+    // Rounds of up to S k-blocks (one round unless the launch has few blocks for its K): tiles of both blocks written -> bar_act -> MMAs ->
+    // bar_done -> barrier 3.  The MMAs of a round are issued in one go, by the pair's first block: a wait or a commit between them costs more
+    // than the four MMAs of a k-block (16 MMAs of 128 x 64 x 16: 1160 cycles, with a wait and a commit per k-block 2290).
     if (warp == kSgMmaWarp) {
-        // B: 2 n_tile rows of planes; their products with a weight tile stand in columns r and n_tile + r
-        const uint32_t idesc = instr_desc_bf16(2 * p.n_tile);
+        const uint32_t bar_w0 = ckv::map_to_rank(&bar_w, 0);
+        auto fetch = [&](int i0) {                        // weights of a round: independent of every earlier kernel
+            if (elect_one()) {
+                const int n = min(n_kb - i0, S);
+                if (rank == 0) mbar_expect_tx(&bar_w, 2 * n * kATileBytes);
+                for (int i = 0; i < n; ++i) ckv::tma_load_2d_pair(tiles + i * kATileBytes, mw, (kb_begin + i0 + i) * kBlockK, a0, bar_w0);
+            }
+            __syncwarp();
+        };
+        fetch(0);
+        // M = 256 features, N = 2 n_tile: high planes and low planes of the first block's rows, then of the second's
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(2 * p.n_tile >> 3) << 17) | (static_cast<uint32_t>(2 * kTileM >> 4) << 24);
         const uint64_t dw0 = smem_desc_sw128(smem_u32(tiles)), da0 = smem_desc_sw128(smem_u32(acts));
         bool ok = true;
         uint32_t phase = 0;
         for (int i0 = 0; i0 < n_kb; i0 += S, phase ^= 1) {
-            asm volatile("bar.sync 4, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
-            if (ok) ok = mbar_wait(&bar_w, phase, &abort_flag);
-            if (ok) {
-                tc_fence_after_sync();
-                if (elect_one()) {
-                    for (int i = 0; i < min(S, n_kb - i0); ++i) {
-                        const uint64_t dw = dw0 + i * (kATileBytes >> 4), da = da0 + static_cast<uint64_t>(i * 2 * plane_bytes >> 4);
+            if (rank == 0) {
+                if (ok) ok = mbar_wait(&bar_w, phase, &abort_flag);
+                if (ok) ok = ckv::mbar_wait_cluster(&bar_act, phase, &abort_flag);
+                if (ok) {
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+                        for (int i = 0; i < min(S, n_kb - i0); ++i) {
+                            const uint64_t dw = dw0 + i * (kATileBytes >> 4), da = da0 + static_cast<uint64_t>(i * 2 * plane_bytes >> 4);
 #pragma unroll
-                        for (int k = 0; k < kBlockK / 16; ++k) mma_bf16(tmem_base, dw + 2 * k, da + 2 * k, idesc, (i0 + i > 0 || k > 0) ? 1u : 0u);
+                            for (int k = 0; k < kBlockK / 16; ++k) ckv::mma_bf16_pair(tmem_base, dw + 2 * k, da + 2 * k, idesc, (i0 + i > 0 || k > 0) ? 1u : 0u);
+                        }
+                        ckv::mma_commit_pair(&bar_done);
                     }
-                    mma_commit(&bar_done);
+                    __syncwarp();
                 }
-                __syncwarp();
-                ok = mbar_wait(&bar_done, phase, &abort_flag);
             }
-            if (ok && i0 + S < n_kb && elect_one()) {
-                const int n = min(S, n_kb - i0 - S);
-                mbar_expect_tx(&bar_w, n * kATileBytes);
-                for (int i = 0; i < n; ++i) tma_load_2d(tiles + i * kATileBytes, mw, (kb_begin + i0 + S + i) * kBlockK, a0, &bar_w);
-            }
-            __syncwarp();
+            if (ok) ok = mbar_wait(&bar_done, phase, &abort_flag);
+            if (ok && i0 + S < n_kb) fetch(i0 + S);
             if (!ok) {
                 // gave up: copies in flight land within microseconds; leave them a millisecond
                 const long long start = clock64();
@@ -272,6 +289,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         // before the dependency wait.
         const int step = (kSgConvertThreads / 8) >> p.share, c = threadIdx.x & 7, rbase = (threadIdx.x >> 3) & (step - 1), group = threadIdx.x >> (9 - p.share);
         const __nv_bfloat16 *const gamma = second_w ? p.gamma2 : p.gamma;
+        const uint32_t bar_act0 = ckv::map_to_rank(&bar_act, 0);
         float ka[8], kb[8];                           // gamma; or c1, c2
         auto constants = [&](int i) {
             const int k = (kb_begin + i) * kBlockK + c * 8;
@@ -292,9 +310,10 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         pdl_wait();
         if (p.after_rows) { n_rows = p.state->n_active; pdl_launch_dependents(); }
         AED_TRACE_PUT_NS(p.state, tcur, 51);          // dependency resolved
-        // ---- activation tiles ----
-        const int rows_here = min(p.n_tile, max(n_rows - row0, 0)), mine = rows_here - rbase;
-        const float *const src = p.src + static_cast<size_t>(row0 + rbase) * p.ld_src + kb_begin * kBlockK + c * 8;
+        // ---- activation tiles: this block's half of the rows ----
+        const int rows_here = min(p.n_tile, max(n_rows - row0, 0)), first = (rows_here + 1) / 2;      // first: rows of the pair's first block
+        const int my0 = rank ? first : 0, mine = (rank ? rows_here - first : first) - rbase;
+        const float *const src = p.src + static_cast<size_t>(row0 + my0 + rbase) * p.ld_src + kb_begin * kBlockK + c * 8;
         constexpr int kHeld = kNI < 4 ? kNI : 4;      // rows in flight
         for (int i0 = 0; i0 < n_kb; i0 += S) {
             for (int s = group; s < min(S, n_kb - i0); s += 1 << p.share) {
@@ -304,7 +323,7 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
                 auto load = [&](int j) {
                     if (j * step >= mine) return;
                     load8(src + static_cast<size_t>(j * step) * p.ld_src + i * kBlockK, x[j % kHeld]);
-                    if (MODE == B_LN_RELU) st[j % kHeld] = p.stats_in[row0 + rbase + j * step];
+                    if (MODE == B_LN_RELU) st[j % kHeld] = p.stats_in[row0 + my0 + rbase + j * step];
                 };
 #pragma unroll
                 for (int j = 0; j < kHeld; ++j) load(j);
@@ -327,9 +346,10 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
                     if (j + kHeld < kNI) load(j + kHeld);
                 }
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> tensor-core reads
+            tiles_written();
+            __syncwarp();
+            if (lane == 0) arrive_cluster(bar_act0);
             if (i0 == 0) AED_TRACE_PUT(p.state, tcur, 52);                 // activation tiles written
-            asm volatile("bar.sync 4, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
             asm volatile("bar.sync 3, %0;" ::"n"(kSgConvertThreads + 32) : "memory");
         }
         // ---- epilogue: reductions straight from the accumulator, 128 consecutive bytes per warp and row ----------------------
@@ -341,14 +361,18 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         AED_TRACE_PUT(p.state, tcur, 53);             // accumulator complete
         if (ok) {
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-            float *const dst = out + static_cast<size_t>(row0) * ldo + a_idx;
-            for (int c0 = 16 * (warp >> 2); c0 < rows_here; c0 += kSgConvertWarps * 4) {
+            for (int c0 = 16 * (warp >> 2); c0 < p.n_tile; c0 += kSgConvertWarps * 4) {
+                const bool upper = c0 >= half_tile;      // rows of the pair's second block
+                const int at = upper ? c0 - half_tile : c0, live = (upper ? rows_here - first : first) - at;
+                if (live <= 0) continue;
+                const uint32_t col = taddr + (upper ? p.n_tile : 0) + at;
+                float *const dst = out + static_cast<size_t>(row0 + (upper ? first : 0) + at) * ldo + a_idx;
                 float hi[16], lo[16];
-                tmem_ld16x2(taddr + c0, taddr + p.n_tile + c0, hi, lo);
+                tmem_ld16x2(col, col + half_tile, hi, lo);
                 if (a_idx < a_rows) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
-                        if (c0 + j < rows_here) red_add(dst + static_cast<size_t>(c0 + j) * ldo, hi[j] + lo[j] + bias);
+                        if (j < live) red_add(dst + static_cast<size_t>(j) * ldo, hi[j] + lo[j] + bias);
                 }
             }
         }
@@ -357,9 +381,10 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     AED_TRACE_PUT_NS(p.state, tcur, 55);              // reductions issued
     tc_fence_before_sync();
     __syncthreads();
+    ckv::cluster_meet();                               // neither block ends while the other may still report to it or read its tiles
     if (warp == kSgMmaWarp) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, tmem_cols);
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
     }
     if (threadIdx.x == 0 && abort_flag) atomicExch(&p.state->error, kErrTimeout);
 }

@@ -406,6 +406,18 @@ def test_row_tiles_of_four(batch):
     _run_both(w, rows=sorted({0, batch // 2 - 1, batch // 2, max(batch - 5, 0), batch - 4 if batch > 4 else 0, batch - 1}))
 
 
+@pytest.mark.parametrize("model, batch", [("odd", 49), ("odd", 63), ("odd", 64), ("wide_a", 65), ("odd", 95), ("odd", 97), ("odd", 127), ("wide_b", 128)])
+def test_halves_of_a_row_tile(model, batch):
+    """Projections on pairs of blocks with half of the rows each: even and odd row counts, tiles of 64, 96 and 128 rows, full and not, and
+    feature counts that are an odd number of 128s (the last pair's second block has none)."""
+    rng = np.random.default_rng(1200 + batch)
+    m = {"wide_a": WIDE_A, "wide_b": WIDE_B, "odd": ODD}[model]
+    w = wl.make_custom(m, rng.integers(1, 40, size=batch), rng.integers(1, 4, size=batch), dtype="bf16", seed=530 + batch,
+                       out_std=0.1, ln_std=0.2)
+    half = (batch + 1) // 2
+    _run_both(w, rows=sorted({0, 15, 16, half - 1, half, half + 16, batch - 2, batch - 1}))
+
+
 @pytest.mark.parametrize("model, batch", [("wide_a", 129), ("wide_b", 65), ("odd", 342), ("odd", 347)])
 def test_self_attention_of_many_rows(model, batch):
     """More than 1024 (row, head) pairs, where self-attention takes a warp per pair: just above the line, a last block

@@ -84,6 +84,9 @@ def family_bytes(family, w, first=0, last=None):
         return sum((CROSS_KV_BYTES or e) * NL * 2 * d * int(T[L > s].sum()) for s in steps)
     if family == "attn_self":
         return sum(e * NL * 2 * d * int((L > s).sum()) * (s + 1) for s in steps)
+    if family == "step":                                   # small fp32 models: a whole step per launch
+        parts = [family_bytes(f, w, first, last) for f in list(per_layer_weights) + ["gemm_vocab", "attn_cross", "attn_self"]]
+        return sum(parts)
     if family == "precompute_cross_kv":
         total_T = int(T.sum())
         return e * (total_T * de + NL * 2 * d * de) + (CROSS_KV_BYTES or e) * total_T * NL * 2 * d
@@ -97,7 +100,7 @@ KERNEL_OF_FAMILY = {
     "gemm_oc": "step_gemm_kernel", "gemm_ff1": "step_gemm_kernel", "gemm_ff2": "step_gemm_kernel",
     "attn_self": "attn_fused_kernel", "attn_cross": "attn_fused_kernel", "attn_combine": "attn_combine_kernel",
     "gemm_vocab": "tc_gemm_kernel", "precompute_cross_kv": "crosskv_gemm_kernel", "layernorm": "layernorm_planes_kernel",
-    "embed": "embed_kernel", "bookkeeping": "step_rows/finish_step",
+    "embed": "embed_kernel", "bookkeeping": "step_rows/finish_step", "step": "cluster_step_kernel",
 }
 KERNEL_OF_VARIANT = {
     "plane": "plane_gemm_kernel", "warp": "self_attn_warp_kernel", "gamma": "gamma_planes_kernel", "gemv_staged": "step_gemv_staged_kernel",
@@ -126,7 +129,7 @@ def profile_bytes(prof, w):
             fam = base + "@" + variant if variant else base
             if fam not in prof:
                 continue
-            per_step = 1 if base == "gemm_vocab" else m["n_layers"]
+            per_step = 1 if base in ("gemm_vocab", "step") else m["n_layers"]
             n = prof[fam]["launches"] // per_step
             if base == "precompute_cross_kv":
                 out[fam] = family_bytes(base, w)

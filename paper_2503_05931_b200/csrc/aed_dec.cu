@@ -21,6 +21,7 @@
 #include "crosskv_gemm.cuh"
 #include "plane_gemm.cuh"
 #include "f32_rows.cuh"
+#include "f32_cluster.cuh"
 #include "step_graphs.h"
 #include "stream_schedule.h"
 
@@ -70,6 +71,7 @@ struct Layout {
     size_t slot_tokens, slot_lens;        // aed_dec_decode_stream: token rows and lengths of the slots
     size_t fold_out;                      // c1 | c2 of the vocabulary projection with the final LayerNorm folded in
     size_t comp_w, comp_b;                // per layer: Wqc diag(gamma2) Wo as bf16 [d, d], and Wqc (gamma2 * bo) as fp32 [d]
+    size_t f32_layers;                    // fp32: pointers of every layer's weights
     size_t ckv_maps, ckv_bias;            // per-layer tensor maps and bias pointers of the cross-K/V weights
     size_t fold_layer_floats;
     int rows_cap;
@@ -152,6 +154,8 @@ Layout make_layout(const aed_dec_config_t &c)
         L.fold_out = take((size_t)2 * c.vocab * 4);
         L.comp_w = take((size_t)c.n_layers * d * d * 2);
         L.comp_b = take((size_t)c.n_layers * d * 4);
+    } else {
+        L.f32_layers = take((size_t)c.n_layers * sizeof(f32::ClusterLayer));
     }
     L.total = off;
     return L;
@@ -202,6 +206,7 @@ struct aed_dec {
     int gemv_rows = kFewRows;       // ... up to this many rows
     bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
+    int f32_clusters[2] = {0, 0};   // fp32 steps of small models in one launch (f32_cluster.cuh): how many clusters of 16 and of 8 blocks find room
     // steps are replayed as one captured CUDA graph per key; the output buffers stand in the device-side state
     typedef std::tuple<int, int, int, bool> GraphKey;       // (row count, chunks of self-attention positions, steps (0: one of the caller's loop), short_cross)
     typedef StepGraphs<GraphKey, cudaGraphExec_t> Graphs;
@@ -250,10 +255,10 @@ aed_status_t fail(aed_dec *d, aed_status_t code, const char *fmt, ...)
 
 enum KernelFamily { KF_BOOKKEEPING = 0, KF_EMBED, KF_LAYERNORM, KF_GEMM_QKV, KF_ATTN_SELF, KF_ATTN_COMBINE, KF_GEMM_O,
                     KF_GEMM_QC, KF_ATTN_CROSS, KF_GEMM_OC, KF_GEMM_FF1, KF_GEMM_FF2, KF_GEMM_VOCAB, KF_PRECOMPUTE,
-                    KF_COUNT };
+                    KF_STEP, KF_COUNT };
 const char *const kFamilyNames[KF_COUNT] = {"bookkeeping", "embed", "layernorm", "gemm_qkv", "attn_self", "attn_combine",
                                             "gemm_o", "gemm_qc", "attn_cross", "gemm_oc", "gemm_ff1", "gemm_ff2",
-                                            "gemm_vocab", "precompute_cross_kv"};
+                                            "gemm_vocab", "precompute_cross_kv", "step"};
 // A call site runs different kernels at different row counts; the profile keeps the call site and says which kernel ran it:
 // family + KF_COUNT * variant, reported as "gemm_qkv@gemv", "attn_self@warp".
 enum { KV_NONE = 0, KV_GEMV, KV_GEMV_STAGED, KV_PLANE, KV_GAMMA, KV_WARP, KV_F32_ROWS, KV_F32_TILE, KV_COUNT };
@@ -441,11 +446,100 @@ aed_status_t launch_f32(aed_dec *dec, int family, int rows_ub, f32::RowsArgs p, 
     return launch_pdl_impl(dec, kernel, grid, dim3(warps * 32), f32::rows_smem(rt, p.K), args);
 }
 
+// ---- steps of small fp32 models in one launch (f32_cluster.cuh) ------------------------------------------------------------
+const void *const kClusterKernel = (const void *)f32::cluster_step_kernel;
+cudaLaunchConfig_t cluster_config(const aed_dec_config_t &c, int cluster, int clusters, cudaLaunchAttribute *attr)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(clusters * cluster);
+    cfg.blockDim = dim3(f32::kClusterThreads);
+    cfg.dynamicSmemBytes = f32::cluster_smem(c.d_model, c.d_ffn, c.n_heads, cluster, c.n_layers);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// The layers' weights as a table on the device, and how many clusters of either size find room at a time.
+aed_status_t f32_setup(aed_dec *dec)
+{
+    const auto &c = dec->cfg;
+    const char *v = getenv("AED_DEC_NO_CLUSTER");
+    if ((v && v[0] == '1') || !f32::cluster_supports(c.d_model, c.d_ffn, c.n_layers)) return AED_OK;
+    std::vector<f32::ClusterLayer> table;
+    for (const LayerWeights &w : dec->layers) {
+        auto f = [](const void *q) { return (const float *)q; };
+        table.push_back({f(w.ln1_g), f(w.ln1_b), f(w.w_qkv), f(w.b_qkv), f(w.w_o), f(w.b_o), f(w.ln2_g), f(w.ln2_b), f(w.w_q_c), f(w.b_q_c), f(w.w_o_c),
+                         f(w.b_o_c), f(w.ln3_g), f(w.ln3_b), f(w.w_ff1), f(w.b_ff1), f(w.w_ff2), f(w.b_ff2)});
+    }
+    cudaError_t e = cudaMemcpyAsync(dec->ws + dec->lay.f32_layers, table.data(), table.size() * sizeof table[0], cudaMemcpyHostToDevice, dec->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(dec->stream);       // the host vector goes away
+    const size_t most = f32::cluster_smem(c.d_model, c.d_ffn, c.n_heads, f32::kClusterSizes[1], c.n_layers);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kClusterKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "fp32 set-up: %s", cudaGetErrorString(e));
+    // (a GPU that does not have them is no error: steps run kernel by kernel)
+    bool larger = cudaFuncSetAttribute(kClusterKernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int i = 0; i < 2; ++i) {
+        cudaLaunchAttribute attr[2];
+        const cudaLaunchConfig_t cfg = cluster_config(c, f32::kClusterSizes[i], 1, attr);
+        int &fit = dec->f32_clusters[i];
+        if ((i == 0 && !larger) || cudaOccupancyMaxActiveClusters(&fit, kClusterKernel, &cfg) != cudaSuccess) fit = 0;
+    }
+    cudaGetLastError();
+    return AED_OK;
+}
+
+// Blocks per cluster for a step of rows_ub rows: the larger clusters while all of them find room, then the smaller; 0: kernel by kernel.
+int cluster_of(const aed_dec *dec, int rows_ub)
+{
+    if (dec->partials_override) return 0;
+    for (int i = 0; i < 2; ++i)
+        if ((rows_ub + f32::kClusterRows - 1) / f32::kClusterRows <= dec->f32_clusters[i]) return f32::kClusterSizes[i];
+    return 0;
+}
+
+aed_status_t launch_cluster_step(aed_dec *dec, int cluster, int rows_ub, const int32_t *tokens, float *logits_out)
+{
+    const auto &c = dec->cfg;
+    const Layout &L = dec->lay;
+    ProfScope ps(dec, KF_STEP);
+    f32::ClusterArgs p{};
+    p.state = dec->state();
+    p.layers = dec->at<f32::ClusterLayer>(L.f32_layers);
+    p.n_layers = c.n_layers; p.cluster_log = cluster == 16 ? 4 : 3; p.d = c.d_model; p.n_heads = c.n_heads; p.d_ffn = c.d_ffn; p.vocab = c.vocab;
+    p.max_dec_len = c.max_dec_len; p.frame_capacity = c.max_total_enc_frames;
+    p.eps = c.ln_eps; p.scale = sqrtf((float)c.d_model);
+    p.row_info = dec->at<int4>(L.row_info);
+    p.tokens = tokens;
+    p.embed = (const float *)dec->embed; p.pe = dec->at<float>(L.pe);
+    p.x = rows_ub <= kRowsInside ? dec->at<float>(L.x) : nullptr;          // made with the row table
+    p.self_cache = dec->at<float>(L.self_cache); p.cross = dec->at<float>(L.cross_store);
+    p.self_layer_elems = L.self_layer_elems; p.cross_layer_elems = L.cross_layer_elems;
+    p.final_ln_g = (const float *)dec->final_ln_g; p.final_ln_b = (const float *)dec->final_ln_b;
+    p.w_out = (const float *)dec->w_out; p.b_out = (const float *)dec->b_out;
+    p.logits_out = logits_out;
+    p.keys = dec->at<unsigned long long>(L.keys);
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(c, cluster, (rows_ub + f32::kClusterRows - 1) / f32::kClusterRows, attr);
+    cfg.stream = dec->stream;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = dec->use_pdl ? 1 : 0;
+    cfg.numAttrs = 2;
+    void *args[] = {&p};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kClusterKernel, args);
+    if (e != cudaSuccess) return fail(dec, AED_ERR_CUDA, "step launch: %s", cudaGetErrorString(e));
+    AED_LAUNCHED(dec);
+    return AED_OK;
+}
+
 // The forward pass of one step in fp32 for the rows in the active list (at most rows_ub of them): 8 kernels per layer, chained
 // with programmatic dependent launch.
 //   tokens: by utterance.  self_len_ub: upper bound on t_u + 1.
 aed_status_t forward_step_f32(aed_dec *dec, int rows_ub, int self_len_ub, const int32_t *tokens, float *logits_out)
 {
+    if (const int cluster = cluster_of(dec, rows_ub)) return launch_cluster_step(dec, cluster, rows_ub, tokens, logits_out);
     const auto &c = dec->cfg;
     const Layout &L = dec->lay;
     int d = c.d_model, V = c.vocab, zero = 0;
@@ -1381,6 +1475,13 @@ extern "C" aed_status_t aed_dec_create(const aed_dec_config_t *config, const aed
     }
     if (config->dtype == AED_DTYPE_BF16) {
         aed_status_t s = tc_setup(dec);
+        if (s != AED_OK) {
+            aed_dec_destroy(dec);
+            return s;
+        }
+    }
+    if (config->dtype == AED_DTYPE_F32) {
+        aed_status_t s = f32_setup(dec);
         if (s != AED_OK) {
             aed_dec_destroy(dec);
             return s;

@@ -750,3 +750,42 @@ def test_random_shapes_and_row_counts_bf16(seed):
     w = wl.make_custom(model, enc_lens, dec_lens, dtype="bf16", seed=2000 + seed, out_std=0.1, ln_std=0.2, bias_std=0.05)
     rows = sorted({0, batch - 1, batch // 2, int(np.argmax(dec_lens)), int(np.argmax(enc_lens))})
     _run_both(w, rows=rows, need_tokens=False, label=f"random shape {model} B={batch}")
+
+
+@pytest.mark.parametrize("model, batch", [("tiny", 1), ("tiny", 5), ("tiny", 9), ("tiny", 28), ("tiny", 29), ("tiny", 57), ("one_head", 7), ("three_heads", 6),
+                                          ("odd_vocab", 4)])
+def test_fp32_steps_in_one_launch(model, batch):
+    """Small fp32 models, whose steps are one launch: clusters with missing rows, clusters of 16 and of 8 blocks and just beyond both, rows embedded
+    with the row table (up to 8) and in the launch, widths that leave blocks without features or pairs, caches and encoder outputs on both
+    sides of what the warps of a pair take at a time."""
+    m = {"tiny": wl.MODELS["tiny"], "one_head": dict(n_layers=2, d_model=64, n_heads=1, d_ffn=64, vocab=301, d_enc=64),
+         "three_heads": dict(n_layers=3, d_model=192, n_heads=3, d_ffn=320, vocab=77, d_enc=64),
+         "odd_vocab": dict(n_layers=1, d_model=256, n_heads=4, d_ffn=1024, vocab=2999, d_enc=128)}[model]
+    rng = np.random.default_rng(1300 + batch)
+    enc_lens, dec_lens = rng.integers(1, 80, size=batch), rng.integers(1, 6, size=batch)
+    enc_lens[0], dec_lens[0] = 130, 70 if batch < 10 else 9
+    w = wl.make_custom(m, enc_lens, dec_lens, dtype="fp32", seed=560 + batch, out_std=0.5, ln_std=0.2, out_bias_std=0.1)
+    _run_both(w, rows=sorted({0, batch // 2, max(batch - 5, 0), batch - 1}))
+
+
+def test_fp32_steps_in_one_launch_and_kernel_by_kernel(monkeypatch):
+    """The same steps either way: their sums differ in order alone.  (Each is within 1e-4 of the checker; 2e-6 of logits of size 1 to
+    10 is what the two orders of up to 1024 products leave.)"""
+    import torch
+    w = wl.make_custom(wl.MODELS["tiny"], [20, 33, 60, 7, 41], [6] * 5, dtype="fp32", seed=590, ln_std=0.2, out_bias_std=0.1)
+    out = []
+    for off in ("0", "1"):
+        monkeypatch.setenv("AED_DEC_NO_CLUSTER", off)
+        dec = _binding().decoder_for_workload(w)
+        dec.precompute_cross_kv(dec.upload_encoder(w.enc), w.enc_lens)
+        logits = torch.zeros((w.batch, w.model["vocab"]), dtype=torch.float32, device="cuda:0")
+        steps = []
+        for t in range(6):
+            tokens = (torch.arange(w.batch, dtype=torch.int32, device="cuda:0") * 7 + 3 * t) % w.model["vocab"]
+            dec.step(tokens, None, logits, None)
+            steps.append(logits.clone())
+        dec.sync_status()
+        dec.close()
+        out.append(torch.stack(steps))
+    size = out[0].abs().max().item()
+    assert (out[0] - out[1]).abs().max().item() < 2e-6 * max(size, 1.0)

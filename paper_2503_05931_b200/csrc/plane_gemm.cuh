@@ -54,8 +54,8 @@ plane_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = ckv::cluster_rank();
     const int a0 = blockIdx.x * kTileM, row0 = blockIdx.z * p.n_tile;
-    const int kb_begin = static_cast<int>((static_cast<long long>(p.k_blocks) * blockIdx.y) / gridDim.y);
-    const int kb_end = static_cast<int>((static_cast<long long>(p.k_blocks) * (blockIdx.y + 1)) / gridDim.y);
+    const int kb_begin = static_cast<int>(p.k_blocks * blockIdx.y / gridDim.y);
+    const int kb_end = static_cast<int>(p.k_blocks * (blockIdx.y + 1) / gridDim.y);
     const int n_kb = kb_end - kb_begin, S = p.stages;
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
     const int plane_bytes = p.n_tile / 2 * kBlockK * 2, stage_bytes = kATileBytes + 2 * plane_bytes;

@@ -119,6 +119,9 @@ __device__ __forceinline__ void red_add_v4(float *addr, float4 v)
 __device__ __forceinline__ void red_add(float *addr, float v) { asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(v) : "memory"); }
 
 // ---- side jobs of a projection launch, run by warps of their own in every CTA, off the critical path ----------------------
+// (Their loops are not unrolled, nor that of attention's prefetches: a step's kernels together are as large as what an SM holds of
+// code, and 30 -> 21 KB for QKV of few rows, 42 -> 35 for the tcgen05 form and 25 -> 21 for attention were worth, at 8 / 16 / 24 / 64 / 128 rows, 424 / 511 /
+// 614 / 916 / 1322 -> 418 / 500 / 607 / 881 / 1304 us per step of the 24-layer model.)
 // w / n_w: this warp among all that do them in the launch.
 // Static data (a later kernel's weights) into L2: no need to wait for the previous kernel.  4 KB pieces.
 __device__ __forceinline__ void side_prefetch(const StepGemmParams &p, int w, int n_w, int lane)
@@ -140,6 +143,7 @@ __device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_r
 {
     if (p.stats_src) {
         constexpr int kHeld = 8;
+#pragma unroll 1
         for (int r = w; r < n_rows; r += n_w) {
             const float *const xr = p.stats_src + static_cast<size_t>(r) * p.stats_d + lane * 4;
             const int n = (p.stats_d + 127) / 128;    // (widths are multiples of 64)
@@ -150,6 +154,7 @@ __device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_r
             for (int i = 0; i < kHeld; ++i) v[i] = load(i);
 #pragma unroll
             for (int i = 0; i < kHeld; ++i) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+#pragma unroll 1
             for (int i = kHeld; i < n; ++i) { const float4 u = load(i); s += (u.x + u.y) + (u.z + u.w); }
             const float mean = warp_sum(s) / p.stats_d;
             auto spread = [&](int i, float4 u) {
@@ -158,6 +163,7 @@ __device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_r
             };
 #pragma unroll
             for (int i = 0; i < kHeld; ++i) spread(i, v[i]);
+#pragma unroll 1
             for (int i = kHeld; i < n; ++i) spread(i, load(i));
             q = warp_sum(q);
             if (lane == 0) p.stats_out[r] = make_float2(mean, rsqrtf(q / p.stats_d + p.eps));
@@ -166,6 +172,7 @@ __device__ __forceinline__ void side_after_wait(const StepGemmParams &p, int n_r
     if (p.zero_buf) {
         const size_t total4 = static_cast<size_t>(n_rows) * p.zero_cols / 4;
         float4 *z = reinterpret_cast<float4 *>(p.zero_buf);
+#pragma unroll 1
         for (size_t idx = static_cast<size_t>(w) * 32 + lane; idx < total4; idx += static_cast<size_t>(n_w) * 32)
             z[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -202,8 +209,8 @@ step_gemm_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int a0 = (second_w ? static_cast<int>(blockIdx.x) - p.tiles_first : static_cast<int>(blockIdx.x)) * kTileM;
     const int a_rows = second_w ? p.a_rows2 : p.a_rows;
     const int row0 = blockIdx.z * p.n_tile, half_tile = p.n_tile / 2;
-    const int kb_begin = static_cast<int>((static_cast<long long>(p.k_blocks) * blockIdx.y) / gridDim.y);
-    const int kb_end = static_cast<int>((static_cast<long long>(p.k_blocks) * (blockIdx.y + 1)) / gridDim.y);
+    const int kb_begin = static_cast<int>(p.k_blocks * blockIdx.y / gridDim.y);
+    const int kb_end = static_cast<int>(p.k_blocks * (blockIdx.y + 1) / gridDim.y);
     const int n_kb = kb_end - kb_begin, S = p.stages;
     uint8_t *const tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
     const int plane_bytes = half_tile * kBlockK * 2;

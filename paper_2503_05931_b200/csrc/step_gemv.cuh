@@ -113,8 +113,8 @@ step_gemv_staged_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_
     const CUtensorMap *mw = second_w ? &map_w2 : &map_w;
     const int a0 = (second_w ? static_cast<int>(blockIdx.x) - p.tiles_first : static_cast<int>(blockIdx.x)) * kTileM;
     const int a_rows = second_w ? p.a_rows2 : p.a_rows;
-    const int kb_begin = static_cast<int>((static_cast<long long>(p.k_blocks) * blockIdx.y) / gridDim.y);
-    const int kb_end = static_cast<int>((static_cast<long long>(p.k_blocks) * (blockIdx.y + 1)) / gridDim.y);
+    const int kb_begin = static_cast<int>(p.k_blocks * blockIdx.y / gridDim.y);
+    const int kb_end = static_cast<int>(p.k_blocks * (blockIdx.y + 1) / gridDim.y);
     const int n_kb = min(kb_end - kb_begin, kKB);
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t *plane_hi = tiles + kKB * kATileBytes, *plane_lo = plane_hi + kTiles * 8 * kSvPitch;

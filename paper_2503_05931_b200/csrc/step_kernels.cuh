@@ -480,6 +480,7 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
         }
         // later chunks of this warp: pull them into L2 now (one 128-byte row per lane group)
         if (dg == 0) {
+#pragma unroll 1
             for (int q0 = p0 + n_warps * kChunk; q0 < len_static; q0 += n_warps * kChunk) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {

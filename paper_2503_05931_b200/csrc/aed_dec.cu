@@ -897,7 +897,7 @@ aed_status_t launch_self_attention(aed_dec *dec, int rows_ub, int rows_out, int 
         const int4 *ri = dec->at<int4>(dec->lay.row_info);
         int ldq = 3 * d, heads = c.n_heads, cap = c.max_dec_len;
         void *args[] = {&state, &ri, &qkv, &ldq, &self_cache, &heads, &cap, &stats, &c1, &c2};
-        AED_TRY(launch_pdl_impl(dec, (const void *)append_kv_kernel<T>, dim3(rows_ub, c.n_heads), dim3(kHeadDim), 0, args));
+        AED_TRY(launch_pdl_impl(dec, (const void *)append_kv_kernel<T>, dim3(rows_ub), dim3(256), 0, args));
     }
     if (rows_out == 0) return AED_OK;
     return launch_attention_fused<T, false, false>(dec, rows_out, self_len_ub, qkv, 3 * d, self_cache, c.max_dec_len, out, out_hi, out_lo, stats, c1, c2,
@@ -1152,14 +1152,25 @@ aed_status_t forward_step_planes(aed_dec *dec, int rows_ub, int self_len_ub, con
         // cross-attention block
         AED_TRY(gamma_planes(w.ln2_g, stats + stats_stride, nullptr, 0));
         AED_TRY(project(KF_GEMM_QC, m.qc, dec->tc_actd, d, d, sh_qc, qc, nullptr));
-        if (c.cross_kv_format == AED_CROSS_KV_E4M3) {
-            const fp8e4m3 *cross8 = dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems;
-            AED_TRY((launch_attention_fused<fp8e4m3, true, false>(dec, rows, c.max_enc_len, qc, d, cross8, c.max_total_enc_frames, nullptr,
-                                                                  ad_hi, ad_lo, stats + stats_stride, c1_qc, c2_qc, pdl)));
-        } else {
-            AED_TRY((launch_attention_fused<T, true, false>(dec, rows, c.max_enc_len, qc, d, cross, c.max_total_enc_frames, nullptr,
-                                                            ad_hi, ad_lo, stats + stats_stride, c1_qc, c2_qc, pdl)));
-        }
+        auto cross_attention = [&](const auto *store) -> aed_status_t {
+            // Prefill, three positions of an utterance or more: its keys and values once for four of them.  4 warps per block; 2 where the blocks
+            // are more than three times what the SMs hold.  (24 layers, us per prefill of utterances x positions at frames, a block per row and
+            // head -> this: 37 x 9 at 110 2214 -> 2155, 20 x 24 at 110 / 400 2610 / 4099 -> 2323 / 3270, 96 x 5 at 110 2644 -> 2597, 130 x 3 at 60 2294 ->
+            // 2139, 10 x 20 at 250 2088 -> 1926; 70 x 2 at 110 1510 -> 1594.)
+            if (pf && rows > 2 * pf->batch) {
+                ProfScope ps(dec, KF_ATTN_CROSS);
+                const int chunk = rows / pf->batch;
+                const dim3 grid(pf->batch * c.n_heads, (chunk + kPrompt - 1) / kPrompt);
+                const int warps = (long long)grid.x * grid.y > 12ll * dec->sm_count ? 2 : 4;
+                return launch_pdl(dec, prompt_cross_kernel<std::remove_const_t<std::remove_pointer_t<decltype(store)>>>, grid, dim3(32 * warps),
+                                  (const int4 *)dec->at<int4>(L.row_info), (const float *)qc, d, store, c.n_heads, c.max_total_enc_frames,
+                                  1.0f / sqrtf((float)kHeadDim), ad_hi, ad_lo, d, (const float2 *)(stats + stats_stride), c1_qc, c2_qc, pf->batch, chunk);
+            }
+            return launch_attention_fused<std::remove_const_t<std::remove_pointer_t<decltype(store)>>, true, false>(
+                dec, rows, c.max_enc_len, qc, d, store, c.max_total_enc_frames, nullptr, ad_hi, ad_lo, stats + stats_stride, c1_qc, c2_qc, pdl);
+        };
+        if (c.cross_kv_format == AED_CROSS_KV_E4M3) AED_TRY(cross_attention((const fp8e4m3 *)(dec->at<fp8e4m3>(L.cross_store) + (size_t)l * L.cross_layer_elems)));
+        else AED_TRY(cross_attention(cross));
         AED_TRY(project(KF_GEMM_OC, m.oc, dec->tc_actd, d, d, sh_o, nullptr, w.b_o_c));
         // feed-forward block; FFN1's epilogue makes the activation planes of FFN2
         AED_TRY(gamma_planes(w.ln3_g, stats + 2 * stats_stride, sh_qkv.splits > 1 ? qkv : nullptr, 3 * d));

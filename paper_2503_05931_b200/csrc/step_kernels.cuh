@@ -1005,25 +1005,157 @@ __global__ void embed_rows_kernel(const DecState *state, const int4 *__restrict_
 
 // Keys and values of every row into the self-attention cache (raw projection output with the LayerNorm fold applied,
 // rounded as the cache stores it), before any row attends: in a prefill pass a row reads positions that other rows of
-// the same pass append.  grid: (rows, heads), 64 threads.
+// the same pass append.  grid: rows; a thread takes 8 components at a time.  (With a block of 64 threads per row and head, one component each,
+// 333 rows took 7.7 us a launch on its own.)
 template <typename CT>
-__global__ void append_kv_kernel(const DecState *state, const int4 *row_info, const float *qkv, int ldq,
-                                 CT *__restrict__ cache, int n_heads, int seq_capacity, const float2 *ln_stats,
-                                 const float *__restrict__ ln_c1, const float *__restrict__ ln_c2)
+__global__ void __launch_bounds__(256)
+append_kv_kernel(const DecState *state, const int4 *row_info, const float *qkv, int ldq, CT *__restrict__ cache, int n_heads, int seq_capacity,
+                 const float2 *ln_stats, const float *__restrict__ ln_c1, const float *__restrict__ ln_c2)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int r = blockIdx.x, h = blockIdx.y, dim = threadIdx.x;
+    const int r = blockIdx.x, d_model = n_heads * kHeadDim;
     const int4 ri = row_info[r];
     if (ri.x < 0) return;
-    const int d_model = n_heads * kHeadDim;
-    const float2 st = ln_stats ? ln_stats[r] : make_float2(0.f, 1.f);
+    const float2 st = ln_stats[r];
+    for (int i = threadIdx.x * 8; i < 2 * d_model; i += blockDim.x * 8) {
+        const int kv = i >= d_model, c = i - kv * d_model, col = d_model + i;
+        float y[8], c1[8], c2[8];
+        load8(qkv + (size_t)r * ldq + col, y);
+        load8(ln_c1 + col, c1);
+        load8(ln_c2 + col, c2);
 #pragma unroll
-    for (int kv = 0; kv < 2; ++kv) {
-        const int col = (1 + kv) * d_model + h * kHeadDim + dim;
-        float y = qkv[(size_t)r * ldq + col];
-        if (ln_stats) y = fmaf(st.y, y - st.x * ln_c1[col], ln_c2[col]);
-        cache[((((size_t)ri.x * 2 + kv) * n_heads + h) * (size_t)seq_capacity + ri.y) * kHeadDim + dim] = from_f32<CT>(y);
+        for (int e = 0; e < 8; ++e) y[e] = fmaf(st.y, y[e] - st.x * c1[e], c2[e]);
+        RawLane<CT> out;
+        out.set(y);
+        out.store(cache + ((((size_t)ri.x * 2 + kv) * n_heads + c / kHeadDim) * (size_t)seq_capacity + ri.y) * kHeadDim + c % kHeadDim);
+    }
+}
+
+// Cross-attention of a prefill pass of many rows: a block takes kPrompt positions of one utterance and head, which read the same keys and
+// values, so that a chunk of them is loaded and unpacked once for all.  Otherwise as attn_fused_kernel with statistics from ln_stats and planes for output: warps take 16
+// positions of the store at a time, one pass, merged through shared memory.  What bounds it is instructions (dot products and their shuffles, weights) at four
+// warps per scheduler of 128 registers; with 8 warps per block, as a row alone has them, most have one chunk or none and the block is start and
+// merge (37 x 9 positions at 110 frames 2306 us a prefill of 24 layers instead of 2155).  Where it is used, and what it gained, stands at its launch.
+// grid: x = utterances * heads, y = groups of kPrompt positions; up to kFusedMaxWarps warps.  Position j of utterance i is row j * batch + i.
+constexpr int kPrompt = 4;
+template <typename CT>
+__global__ void __launch_bounds__(256, 2)
+prompt_cross_kernel(const int4 *row_info, const float *q, int ldq, const CT *__restrict__ cache, int n_heads, int seq_capacity, float scale,
+                    __nv_bfloat16 *__restrict__ out_hi, __nv_bfloat16 *__restrict__ out_lo, int ldo, const float2 *ln_stats, const float *__restrict__ ln_c1,
+                    const float *__restrict__ ln_c2, int batch, int chunk)
+{
+    constexpr int kWarps = kFusedMaxWarps;
+    const int n_warps = blockDim.x >> 5, step = n_warps * 16;
+    __shared__ float sm_m[kPrompt][kWarps], sm_l[kPrompt][kWarps];
+    __shared__ float sm_acc[kPrompt][kWarps][kHeadDim];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, dg = lane & 7, pg = lane >> 3;
+    const int utt = blockIdx.x / n_heads, h = blockIdx.x - utt * n_heads, j0 = blockIdx.y * kPrompt, n = min(chunk - j0, kPrompt);
+    const int4 ri = row_info[utt];                     // (of its first row; the others have the same encoder output)
+    const int len = ri.z, qcol = h * kHeadDim + dg * 8;
+    const CT *const kbase = cache + ((size_t)h * seq_capacity + ri.w) * kHeadDim + dg * 8;
+    const CT *const vbase = kbase + (size_t)n_heads * seq_capacity * kHeadDim;
+    RawLane<CT> rk[4], rv[4];
+    auto load_chunk = [&](int p0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int p = p0 + i * 4 + pg;
+            if (p < len) { rk[i].load(kbase + (size_t)p * kHeadDim); rv[i].load(vbase + (size_t)p * kHeadDim); }
+            else { rk[i].zero(); rv[i].zero(); }
+        }
+    };
+    load_chunk(warp * 16);                             // static: before the dependency wait
+    float c1[8], c2[8];
+    load_n<8>(ln_c1 + qcol, c1);
+    load_n<8>(ln_c2 + qcol, c2);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float qv[kPrompt][8], acc[kPrompt][8], m[kPrompt], l[kPrompt];
+#pragma unroll
+    for (int j = 0; j < kPrompt; ++j) {
+        const size_t r = (size_t)(j0 + min(j, n - 1)) * batch + utt;
+        const float2 st = ln_stats[r];
+        load_n<8>(q + r * ldq + qcol, qv[j]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { qv[j][e] = fmaf(st.y, qv[j][e] - st.x * c1[e], c2[e]) * (scale * kScoreUnit); acc[j][e] = 0.f; }
+        m[j] = -INFINITY;
+        l[j] = 0.f;
+    }
+#pragma unroll 1
+    for (int p0 = warp * 16; p0 < len; p0 += step) {
+        if (p0 != warp * 16) load_chunk(p0);
+        float s[kPrompt][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float kf[8];
+            rk[i].get(kf);
+            const bool in = p0 + i * 4 + pg < len;
+#pragma unroll
+            for (int j = 0; j < kPrompt; ++j) {
+                float d = 0.f;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) d = fmaf(qv[j][e], kf[e], d);
+#pragma unroll
+                for (int o = 1; o < 8; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                s[j][i] = in ? d : -INFINITY;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kPrompt; ++j) {
+            float top = fmaxf(fmaxf(s[j][0], s[j][1]), fmaxf(s[j][2], s[j][3]));
+            top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 8));
+            top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 16));
+            const float m_new = fmaxf(m[j], top), corr = softmax_weight<CT>(m[j] - m_new);
+            m[j] = m_new;
+            l[j] *= corr;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[j][e] *= corr;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { s[j][i] = softmax_weight<CT>(s[j][i] - m_new); l[j] += s[j][i]; }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float vf[8];
+            rv[i].get(vf);
+#pragma unroll
+            for (int j = 0; j < kPrompt; ++j)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[j][e] = fmaf(s[j][i], vf[e], acc[j][e]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kPrompt; ++j) {
+#pragma unroll
+        for (int o = 8; o < 32; o <<= 1) {             // the position groups of the warp (they share m)
+            l[j] += __shfl_xor_sync(0xffffffffu, l[j], o);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[j][e] += __shfl_xor_sync(0xffffffffu, acc[j][e], o);
+        }
+        if (lane == 0) { sm_m[j][warp] = m[j]; sm_l[j][warp] = l[j]; }
+        if (pg == j % 4) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) sm_acc[j][warp][dg * 8 + e] = acc[j][e];
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = threadIdx.x; i < n * kHeadDim; i += blockDim.x) {
+        const int j = i / kHeadDim, e = i % kHeadDim;
+        float mw[kWarps], big = -INFINITY, sum = 0.f, o = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) { mw[w] = w < n_warps ? sm_m[j][w] : -INFINITY; big = fmaxf(big, mw[w]); }
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            if (w >= n_warps) break;
+            const float wgt = mw[w] == -INFINITY ? 0.f : softmax_weight<CT>(mw[w] - big);
+            sum = fmaf(sm_l[j][w], wgt, sum);
+            o = fmaf(sm_acc[j][w][e], wgt, o);
+        }
+        o /= sum;
+        const size_t at = ((size_t)(j0 + j) * batch + utt) * ldo + h * kHeadDim + e;
+        const __nv_bfloat16 hi = __float2bfloat16_rn(o);
+        out_hi[at] = hi;
+        out_lo[at] = __float2bfloat16_rn(o - __bfloat162float(hi));
     }
 }
 

@@ -62,6 +62,35 @@ def test_prefill_with_many_rows(prompt_len, max_batch):
     test_prefill_matches_the_checker(prompt_len, max_batch)
 
 
+@pytest.mark.parametrize("batch,prompt_len,e4m3", [(65, 2, False), (45, 3, False), (33, 5, True), (70, 29, False), (70, 29, True)])
+def test_prefill_positions_that_share_keys(batch, prompt_len, e4m3):
+    """Passes of many rows whose cross-attention takes up to four positions of an utterance per block: two positions (a block per row), a
+    part of a group, a group and one more, and so many blocks that they have two warps; encoder outputs that end inside a chunk,
+    at its end and one past it, and longer than what the warps of a block take at a time."""
+    import torch
+    from paper_2503_05931_b200 import binding
+    rng = np.random.default_rng(batch * 100 + prompt_len)
+    enc_lens = rng.integers(1, 60, size=batch)
+    enc_lens[:6] = [1, 16, 17, 64, 65, 150]
+    w = wl.make_custom(MID, enc_lens, [prompt_len + 1] * batch, dtype="bf16", seed=57, out_std=0.1, ln_std=0.2)
+    prompt = rng.integers(0, MID["vocab"], size=(batch, prompt_len)).astype(np.int32)
+    dec = binding.Decoder(w.model, w.weights, "bf16", max_batch=batch * prompt_len, max_total_enc_frames=int(sum(enc_lens)), max_enc_len=int(max(enc_lens)),
+                          max_dec_len=prompt_len + 1, cross_kv_e4m3=e4m3)
+    try:
+        dec.precompute_cross_kv(dec.upload_encoder(w.enc), w.enc_lens)
+        logits = torch.zeros((batch, MID["vocab"]), dtype=torch.float32, device="cuda:0")
+        dec.prefill(torch.from_numpy(prompt).to("cuda:0"), logits, None)
+        dec.sync_status()
+        got = logits.cpu().numpy()
+    finally:
+        dec.close()
+    model = orc.Model(w.model, w.weights, cross_kv_e4m3=e4m3)
+    start = np.concatenate([[0], np.cumsum(enc_lens)])
+    for u in [0, 1, 2, 3, 4, 5, batch // 2, batch - 1]:
+        ref = orc.decode_batch(model, w.enc[start[u]:start[u + 1]], [int(enc_lens[u])], [prompt_len], forced=prompt[u:u + 1], want_logits=True)
+        assert float(np.max(np.abs(got[u] - ref["logits"][0][prompt_len - 1]))) < TOL["bf16"], u
+
+
 def test_prefill_argument_errors():
     import torch
     from paper_2503_05931_b200 import binding

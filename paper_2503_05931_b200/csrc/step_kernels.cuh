@@ -410,6 +410,19 @@ template <int N> __device__ __forceinline__ void load_n(const float *p, float (&
     }
 }
 
+// Sums of a warp's four position groups (lanes dg + 8 pg) of 8 head dimensions each: a lane keeps dimensions 2 pg and 2 pg + 1 of its 8 (6 shuffles
+// instead of 16).
+__device__ __forceinline__ float2 sum_position_groups(const float (&acc)[8], int pg)
+{
+    float a4[4], o2[2];
+    const bool up = pg & 2, up1 = pg & 1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a4[j] = (up ? acc[4 + j] : acc[j]) + __shfl_xor_sync(0xffffffffu, up ? acc[j] : acc[4 + j], 16);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) o2[j] = (up1 ? a4[2 + j] : a4[j]) + __shfl_xor_sync(0xffffffffu, up1 ? a4[j] : a4[2 + j], 8);
+    return make_float2(o2[0], o2[1]);
+}
+
 // kPipe: the loads of a warp's next chunk are issued before the current chunk is reduced (twice the K/V registers,
 // so only two blocks per SM: for grids that fit anyway).
 // kRowStats: the block computes (mean, rstd) of its row of stats_x itself instead of reading ln_stats.
@@ -429,7 +442,7 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
     // this step writes is touched: the row table (written by the step's first kernel, which ran to completion
     // before any programmatic launch of the step) and, for cross-attention, the encoder K/V store.
     __shared__ float sm_m[kFusedMaxWarps], sm_l[kFusedMaxWarps];
-    __shared__ float sm_acc[kFusedMaxWarps][kHeadDim];
+    __shared__ __align__(8) float sm_acc[kFusedMaxWarps][kHeadDim];
     __shared__ float2 sm_red[kFusedMaxWarps];
     const int rh = blockIdx.x;
     const int r = rh / n_heads, h = rh % n_heads;
@@ -642,17 +655,11 @@ attn_fused_kernel(const DecState *state, const int4 *row_info, const float *q, i
     }
     AED_TRACE_PUT(state, tcur, 5);                          // all chunks of this warp reduced
     // sum the position groups (they share m)
-#pragma unroll
-    for (int o = kDG; o < 32; o <<= 1) {
-        l += __shfl_xor_sync(0xffffffffu, l, o);
-#pragma unroll
-        for (int j = 0; j < kE; ++j) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
-    }
+    static_assert(kE == 8 && kPG == 4, "as sum_position_groups has it");
+    l += __shfl_xor_sync(0xffffffffu, l, 8);
+    l += __shfl_xor_sync(0xffffffffu, l, 16);
     if (lane == 0) { sm_m[warp] = m; sm_l[warp] = l; }
-    if (pg == 0) {
-#pragma unroll
-        for (int j = 0; j < kE; ++j) sm_acc[warp][dg * kE + j] = acc[j];
-    }
+    *reinterpret_cast<float2 *>(&sm_acc[warp][dg * 8 + pg * 2]) = sum_position_groups(acc, pg);
     __syncthreads();
     if (threadIdx.x < kHeadDim) {
         // Unrolled, so that all warps' results are loaded at once (24 layers, 8 / 64 rows, with the same above: 8 / 7 us a step).  fp32,
@@ -790,28 +797,19 @@ self_attn_warp_kernel(const DecState *state, const int4 *row_info, const float *
         }
         m = m_new;
     }
-    // sum the position groups: every lane keeps kE / kPG = 2 of its 8 dimensions, so the groups write one row together
-    float o2[2];
+    // sum the position groups: every lane keeps 2 of its 8 dimensions, so the groups write one row together
+    static_assert(kE == 8 && kPG == 4, "as sum_position_groups has it");
     l += __shfl_xor_sync(0xffffffffu, l, kDG);
     l += __shfl_xor_sync(0xffffffffu, l, 2 * kDG);
-    static_assert(kE == 8 && kPG == 4, "two halving exchanges");
-    {
-        float a4[4];
-        const bool up = pg & 2;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) a4[j] = (up ? acc[4 + j] : acc[j]) + __shfl_xor_sync(0xffffffffu, up ? acc[j] : acc[4 + j], 2 * kDG);
-        const bool up1 = pg & 1;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) o2[j] = (up1 ? a4[2 + j] : a4[j]) + __shfl_xor_sync(0xffffffffu, up1 ? a4[j] : a4[2 + j], kDG);
-    }
+    float2 o2 = sum_position_groups(acc, pg);
     const float inv = 1.f / l;
-    o2[0] *= inv; o2[1] *= inv;
+    o2.x *= inv; o2.y *= inv;
     const size_t off = (size_t)r * ldo + qcol + pg * 2;
-    if (out) *reinterpret_cast<float2 *>(out + off) = make_float2(o2[0], o2[1]);
+    if (out) *reinterpret_cast<float2 *>(out + off) = o2;
     if (out_hi) {
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(o2[0], o2[1]);
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(o2.x, o2.y);
         *reinterpret_cast<__nv_bfloat162 *>(out_hi + off) = hi;
-        *reinterpret_cast<__nv_bfloat162 *>(out_lo + off) = __floats2bfloat162_rn(o2[0] - __bfloat162float(hi.x), o2[1] - __bfloat162float(hi.y));
+        *reinterpret_cast<__nv_bfloat162 *>(out_lo + off) = __floats2bfloat162_rn(o2.x - __bfloat162float(hi.x), o2.y - __bfloat162float(hi.y));
     }
 }
 
@@ -1048,7 +1046,7 @@ prompt_cross_kernel(const int4 *row_info, const float *q, int ldq, const CT *__r
     constexpr int kWarps = kFusedMaxWarps;
     const int n_warps = blockDim.x >> 5, step = n_warps * 16;
     __shared__ float sm_m[kPrompt][kWarps], sm_l[kPrompt][kWarps];
-    __shared__ float sm_acc[kPrompt][kWarps][kHeadDim];
+    __shared__ __align__(8) float sm_acc[kPrompt][kWarps][kHeadDim];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, dg = lane & 7, pg = lane >> 3;
     const int utt = blockIdx.x / n_heads, h = blockIdx.x - utt * n_heads, j0 = blockIdx.y * kPrompt, n = min(chunk - j0, kPrompt);
     const int4 ri = row_info[utt];                     // (of its first row; the others have the same encoder output)
@@ -1125,17 +1123,10 @@ prompt_cross_kernel(const int4 *row_info, const float *q, int ldq, const CT *__r
     }
 #pragma unroll
     for (int j = 0; j < kPrompt; ++j) {
-#pragma unroll
-        for (int o = 8; o < 32; o <<= 1) {             // the position groups of the warp (they share m)
-            l[j] += __shfl_xor_sync(0xffffffffu, l[j], o);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[j][e] += __shfl_xor_sync(0xffffffffu, acc[j][e], o);
-        }
+        l[j] += __shfl_xor_sync(0xffffffffu, l[j], 8);      // the position groups of the warp (they share m)
+        l[j] += __shfl_xor_sync(0xffffffffu, l[j], 16);
         if (lane == 0) { sm_m[j][warp] = m[j]; sm_l[j][warp] = l[j]; }
-        if (pg == j % 4) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) sm_acc[j][warp][dg * 8 + e] = acc[j][e];
-        }
+        *reinterpret_cast<float2 *>(&sm_acc[j][warp][dg * 8 + pg * 2]) = sum_position_groups(acc[j], pg);
     }
     __syncthreads();
 #pragma unroll 1

@@ -206,6 +206,7 @@ struct aed_dec {
     int gemv_rows = kFewRows;       // ... up to this many rows
     bool use_vocab_gemv = false;    // ... and the vocabulary projection of at most 16 rows (vocab_gemv.cuh)
     int planes_rows = 128;                // steps with more rows make their activation planes once per projection input
+    std::vector<f32::ClusterLayer> f32_table;
     int f32_clusters[2] = {0, 0};   // fp32 steps of small models in one launch (f32_cluster.cuh): how many clusters of 16 and of 8 blocks find room
     // steps are replayed as one captured CUDA graph per key; the output buffers stand in the device-side state
     typedef std::tuple<int, int, int, bool> GraphKey;       // (row count, chunks of self-attention positions, steps (0: one of the caller's loop), short_cross)
@@ -468,18 +469,17 @@ aed_status_t f32_setup(aed_dec *dec)
     const auto &c = dec->cfg;
     const char *v = getenv("AED_DEC_NO_CLUSTER");
     if ((v && v[0] == '1') || !f32::cluster_supports(c.d_model, c.d_ffn, c.n_layers)) return AED_OK;
-    std::vector<f32::ClusterLayer> table;
+    std::vector<f32::ClusterLayer> &table = dec->f32_table;            // (kept: the copy may be taken from it later)
     for (const LayerWeights &w : dec->layers) {
         auto f = [](const void *q) { return (const float *)q; };
         table.push_back({f(w.ln1_g), f(w.ln1_b), f(w.w_qkv), f(w.b_qkv), f(w.w_o), f(w.b_o), f(w.ln2_g), f(w.ln2_b), f(w.w_q_c), f(w.b_q_c), f(w.w_o_c),
                          f(w.b_o_c), f(w.ln3_g), f(w.ln3_b), f(w.w_ff1), f(w.b_ff1), f(w.w_ff2), f(w.b_ff2)});
     }
-    cudaError_t e = cudaMemcpyAsync(dec->ws + dec->lay.f32_layers, table.data(), table.size() * sizeof table[0], cudaMemcpyHostToDevice, dec->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(dec->stream);       // the host vector goes away
-    const size_t most = f32::cluster_smem(c.d_model, c.d_ffn, c.n_heads, f32::kClusterSizes[1], c.n_layers);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kClusterKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    const cudaError_t e = cudaMemcpyAsync(dec->ws + dec->lay.f32_layers, table.data(), table.size() * sizeof table[0], cudaMemcpyHostToDevice, dec->stream);
     if (e != cudaSuccess) return fail(nullptr, AED_ERR_CUDA, "fp32 set-up: %s", cudaGetErrorString(e));
-    // (a GPU that does not have them is no error: steps run kernel by kernel)
+    // (a GPU that does not have room for them is no error: steps run kernel by kernel)
+    const size_t most = f32::cluster_smem(c.d_model, c.d_ffn, c.n_heads, f32::kClusterSizes[1], c.n_layers);
+    if (cudaFuncSetAttribute(kClusterKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) { cudaGetLastError(); return AED_OK; }
     bool larger = cudaFuncSetAttribute(kClusterKernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (int i = 0; i < 2; ++i) {
         cudaLaunchAttribute attr[2];

@@ -146,12 +146,12 @@ def profile_bytes(prof, w):
 # dram__bytes_write.sum of the captured launches over their algorithmic bytes).  An entry is removed when its kernel
 # changes, which turns the reported traffic back into null.
 NCU_TRAFFIC_RATIO = {
-    # five launches of one layer at 128 rows (cfg3): 71.85 MB read for 29.36 MB of layer weights (64 rows: 66.61); the launches also
+    # five launches of one layer at 64 rows: 65.99 MB read for 29.36 MB of layer weights; the launches also
     # read the composite cross-query matrix (2.1 MB), the fp32 activation rows, and each prefetches the next layer's matrices
     # of its kind into L2, which under the profiler's serialised replay is a second DRAM read
-    "step_gemm_kernel": 2.45,
-    # the five launches at 16 rows (cfg2): 62.03 MB read
-    "step_gemv_staged_kernel": 2.11,
+    "step_gemm_kernel": 2.25,
+    # the five launches at 16 rows: 62.33 MB read
+    "step_gemv_staged_kernel": 2.12,
     # the six launches of one layer at 512 rows: 56.83 MB read; beside the weights the activation planes
     "plane_gemm_kernel": 1.94,
     # self + cross attention of one layer at 64 rows: 1.10 + 31.05 MB for 0.52 + 30.49 MB of K/V (cross-attention of 512 rows:

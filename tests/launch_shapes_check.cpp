@@ -42,8 +42,20 @@ static bool cross_warps_ok()
     return ok;
 }
 
+// Row tiles of the pairs of blocks: whole 32s (halves of 16 rows, an MMA of a multiple of 64 columns, at most 256), as many as needed, none empty.
+static bool pair_tiles_ok()
+{
+    bool ok = true;
+    for (int rows = 1; rows <= 2048; ++rows) {
+        const int n = tc_pair_tile(rows, 128), tiles = (rows + n - 1) / n;
+        ok = ok && n % 32 == 0 && n >= 32 && n <= 128 && tiles * n >= rows && (tiles - 1) * n < rows && tiles == (rows + 127) / 128;
+    }
+    return ok;
+}
+
 int main()
 {
+    if (!pair_tiles_ok()) { std::printf("row tiles of pairs\n"); return 1; }
     const bool setting_ok = few_row_setting(nullptr) == 48 && few_row_setting("") == 48 && few_row_setting("0") == 48 && few_row_setting("-3") == 48 &&
                             few_row_setting("1") == 1 && few_row_setting("32") == 32 && few_row_setting("48") == 48 && few_row_setting("49") == 48 &&
                             few_row_setting("64") == 48 && few_row_setting("1000") == 48;
